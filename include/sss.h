@@ -64,15 +64,14 @@ typedef enum sss_status {
 #define SSS_FLAG_MERGE_TREE 0x10u /* merge: pairwise LCP-merge tree over whole
                                   buckets instead of second-level sub-buckets
                                   merged inside one CTA each */
-#define SSS_FLAG_GRAPH 0x40u /* local sort: run its round loop as one CUDA graph
-                                  launch (a conditional while node whose body is a
-                                  device-planned round); sss_sort_batch: the whole
-                                  call (identity order, device-side classification
-                                  of the instances, first finishers, round loop,
-                                  instance-local order) is one graph launch after
-                                  the instance-table upload.  Graphs are kept in the
-                                  context (up to four) and relaunched while the
-                                  call's pointers and sizes are unchanged */
+#define SSS_FLAG_GRAPH 0x40u /* local sort: its rounds (a conditional while node whose
+                                  body is a device-planned round), finishers and
+                                  seams are one CUDA graph launch.  That is how every
+                                  sort runs unless kernel timing is on (sss_set_timing),
+                                  which launches the same kernels one by one; with this
+                                  flag it is a graph launch then too.  The graphs (up to
+                                  eight per context) read the call's pointers and sizes
+                                  from device memory: they serve any inputs */
 #define SSS_FLAG_NO_CTA_ROUNDS 0x80u /* doubling: launch the per-round kernels for
                                   every round instead of running the rounds that
                                   test at most 4096 keys inside one CTA (hash-table
@@ -151,8 +150,9 @@ const char* sss_last_error(sss_ctx* ctx);
  *                indices in sorted order (equal strings by index).
  * out_run_lcp  : uint32_t[n]; out_run_lcp[q] = lcp(run[q-1], run[q]) within a
  *                partition, 0 at every partition start.
- * Synchronises the stream once per round of segments larger than cta_cap
- * (never with SSS_FLAG_GRAPH, whose round loop runs on the device). */
+ * Does not synchronise the stream: the round loop runs on the device (with
+ * kernel timing on and no SSS_FLAG_GRAPH, once per round of segments larger
+ * than cta_cap). */
 sss_status sss_local_sort(sss_ctx* ctx, const uint8_t* chars, uint64_t n_chars,
                           const uint64_t* offsets, const uint32_t* lengths, uint32_t n,
                           uint32_t p, const sss_params* params,

@@ -172,7 +172,14 @@ sss_status sss_create(sss_ctx** out, int device, void* stream) {
         delete ctx;
         return SSS_ERR_OOM;
     }
+    if (cudaMalloc(&ctx->d_ls, ls_dev_bytes()) != cudaSuccess) {
+        cudaFree(ctx->d_small);
+        cudaFree(ctx->d_err);
+        delete ctx;
+        return SSS_ERR_OOM;
+    }
     if (cudaMallocHost(&ctx->h_small, 64) != cudaSuccess) {
+        cudaFree(ctx->d_ls);
         cudaFree(ctx->d_small);
         cudaFree(ctx->d_err);
         delete ctx;
@@ -195,6 +202,7 @@ sss_status sss_destroy(sss_ctx* ctx) {
     if (ctx->h_pin) cudaFreeHost(ctx->h_pin);
     if (ctx->d_err) cudaFree(ctx->d_err);
     if (ctx->d_small) cudaFree(ctx->d_small);
+    if (ctx->d_ls) cudaFree(ctx->d_ls);
     if (ctx->h_small) cudaFreeHost(ctx->h_small);
     for (auto& lg : ctx->ls_graphs) {
         if (lg.exec) cudaGraphExecDestroy(lg.exec);
@@ -202,6 +210,9 @@ sss_status sss_destroy(sss_ctx* ctx) {
     }
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     if (ctx->cap_stream2) cudaStreamDestroy(ctx->cap_stream2);
+    if (ctx->cap_stream3) cudaStreamDestroy(ctx->cap_stream3);
+    for (cudaEvent_t e : ctx->cap_event)
+        if (e) cudaEventDestroy(e);
     if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
     for (cudaEvent_t e : ctx->chunk_events) cudaEventDestroy(e);
     if (ctx->pin_event) cudaEventDestroy(ctx->pin_event);
@@ -628,8 +639,6 @@ sss_status sss_sort_batch(sss_ctx* ctx, const uint8_t* chars, uint64_t n_chars, 
     SSS_TRY(sss_upload(ctx, d_inst, pin, sizeof(Seg) * m));
     size_t off = (ar.off + 255) & ~size_t(255);
     Arena sa{ws + off, need - off, 0};
-    if (prm.flags & SSS_FLAG_GRAPH)  // the whole sort as one graph launch
-        return impl_sort_batch_graph(ctx, sa, in, d_inst, m, prm, out_perm, out_lcp, out_dist);
     SSS_TRY(impl_sort_segments(ctx, sa, in, segs, prm, out_perm, out_lcp));
     return impl_batch_finish(ctx, d_inst, m, lengths, out_perm, out_lcp, out_dist);
 }

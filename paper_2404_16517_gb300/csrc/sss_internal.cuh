@@ -82,21 +82,18 @@ struct sss_ctx {
     std::string timing_filter;
     std::vector<PendingTiming> pending;
     std::vector<cudaEvent_t> event_pool;
-    // graphs of the local sort's round loop (SSS_FLAG_GRAPH and the merge's sample
-    // sorts), each reused while its key (every pointer and size baked into it) is
-    // unchanged; the least recently used of LS_GRAPHS is replaced
+    // graphs of the local sort (rounds, finishers, seams), one per grid class and
+    // bucket CTA; their kernels read the call's pointers and sizes from d_ls
+    void* d_ls = nullptr;
     bool capturing = false;
-    cudaStream_t cap_stream = nullptr;
-    cudaStream_t cap_stream2 = nullptr;  // captures a graph's loop body while cap_stream captures the graph
+    cudaStream_t cap_stream = nullptr, cap_stream2 = nullptr, cap_stream3 = nullptr;
+    cudaEvent_t cap_event[3] = {};
     struct LsGraph {
-        std::string key;
         cudaGraph_t graph = nullptr;
         cudaGraphExec_t exec = nullptr;
-        uint64_t used = 0;
     };
-    static constexpr int LS_GRAPHS = 4;
+    static constexpr int LS_GRAPHS = 8;
     LsGraph ls_graphs[LS_GRAPHS];
-    uint64_t ls_clock = 0;
     // kernel-statistics name of the next round-loop graph launches (timed like a
     // kernel when timing is on); set by a caller for its own sorts
     const char* graph_tag = "ls_graph";
@@ -195,9 +192,8 @@ sss_status impl_part_extents(sss_ctx* ctx, const StrIn& in, uint32_t p, unsigned
 sss_status impl_suffix_views(sss_ctx* ctx, uint32_t n, uint32_t max_len, uint64_t* offs, uint32_t* lens);
 sss_status impl_batch_finish(sss_ctx* ctx, const Seg* d_inst, uint32_t m, const uint32_t* lens, uint32_t* perm,
                              const uint32_t* lcp, uint32_t* dist);
-// The batched sort of the m instances d_inst (device table) as one graph launch.
-sss_status impl_sort_batch_graph(sss_ctx* ctx, Arena& ar, const StrIn& in, const Seg* d_inst, uint32_t m,
-                                 const sss_params& prm, uint32_t* perm, uint32_t* lcp, uint32_t* dist);
+// bytes of the local sort's device state (sss_ctx::d_ls)
+size_t ls_dev_bytes();
 
 // Finish segments of positions whose strings share their first `depth`
 // characters (stage A's CTA finisher): perm[start..start+size) is sorted by the

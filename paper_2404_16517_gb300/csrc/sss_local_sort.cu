@@ -42,94 +42,64 @@ constexpr int BK_T = 512, BK_CAP = 4096;        // bucket sort CTA (bucket targe
 constexpr int BKS_T = 256, BKS_CAP = 2048;      // bucket sort CTA for targets <= BKS_CAP / 2 (4 CTAs per SM)
 constexpr int DIRECT_T = 1024, DIRECT_CAP = 8192;  // whole-segment sort CTA (segments <= direct_cap)
 
-struct SegLists {
-    Seg* tiny;
-    Seg* med;
-    Seg* large;
-    uint32_t* cnt;  // [0] tiny, [1] med, [2] large, [3] warp, [4] small, [5] quad
-    uint32_t cap_tiny, cap_med, cap_large;
-    Seg* warp;
-    uint32_t cap_warp;
-    Seg* small;
-    uint32_t cap_small;
-    uint32_t warp_max, med_max;  // classes: warp <= warp_max < tiny <= TINY_CAP < small <= SM_CAP < med <= med_max < large
-};
+// size class of a segment of >= 2 strings: quad <= QUAD_W, warp <= warp_max <
+// tiny <= TINY_CAP < small <= SM_CAP < med <= med_max < large
+__device__ __forceinline__ uint32_t seg_class(const LsArgs& A, uint32_t size) {
+    if (size <= A.warp_max) return size <= (uint32_t)QUAD_W ? LC_QUAD : LC_WARP;
+    if (size <= (uint32_t)TINY_CAP) return LC_TINY;
+    if (size <= A.med_max) return size <= (uint32_t)SM_CAP ? LC_SMALL : LC_MED;
+    return LC_LARGE;
+}
 
-__device__ __forceinline__ void push_seg(const SegLists& L, uint32_t start, uint32_t size, uint32_t depth,
-                                         unsigned* err) {
-    Seg s{start, size, depth, 0};
-    if (size <= L.warp_max) {
-        // one array for both short classes: segments of <= QUAD_W strings from
-        // the bottom (count cnt[5]), the others from the top (count cnt[3]); the
-        // two never meet, as the segments of a round are disjoint and hold >= 2
-        // strings each (the finishers check it)
-        if (size <= (uint32_t)QUAD_W) {
-            uint32_t i = atomicAdd(&L.cnt[5], 1u);
-            if (i < L.cap_warp) L.warp[i] = s; else atomicOr(err, ERRBIT_OVERFLOW);
-        } else {
-            uint32_t i = atomicAdd(&L.cnt[3], 1u);
-            if (i < L.cap_warp) L.warp[L.cap_warp - 1u - i] = s; else atomicOr(err, ERRBIT_OVERFLOW);
-        }
-    } else if (size <= (uint32_t)TINY_CAP) {
-        uint32_t i = atomicAdd(&L.cnt[0], 1u);
-        if (i < L.cap_tiny) L.tiny[i] = s; else atomicOr(err, ERRBIT_OVERFLOW);
-    } else if (size <= (uint32_t)SM_CAP && size <= L.med_max) {
-        uint32_t i = atomicAdd(&L.cnt[4], 1u);
-        if (i < L.cap_small) L.small[i] = s; else atomicOr(err, ERRBIT_OVERFLOW);
-    } else if (size <= L.med_max) {
-        uint32_t i = atomicAdd(&L.cnt[1], 1u);
-        if (i < L.cap_med) L.med[i] = s; else atomicOr(err, ERRBIT_OVERFLOW);
-    } else {
-        uint32_t i = atomicAdd(&L.cnt[2], 1u);
-        if (i < L.cap_large) L.large[i] = s; else atomicOr(err, ERRBIT_OVERFLOW);
+// Entry i of list c.  The two short classes share one array, quad from the
+// bottom and warp from the top; they never meet, as the segments on the short
+// lists are disjoint over all rounds (a short segment is final: its positions
+// never return to the large list) and hold >= 2 strings each.
+__device__ __forceinline__ void put_seg(const LsArgs& A, uint32_t c, uint32_t i, const Seg& sg, unsigned* err) {
+    if (i >= A.cap[c]) {
+        atomicOr(err, ERRBIT_OVERFLOW);
+        return;
     }
+    Seg* at = A.list[c];
+    if (c == LC_WARP) at -= i;
+    else at += i;
+    *at = sg;
+}
+
+__device__ __forceinline__ void push_seg(const LsArgs& A, uint32_t* cnt, uint32_t start, uint32_t size,
+                                         uint32_t depth, unsigned* err) {
+    const uint32_t c = seg_class(A, size);
+    put_seg(A, c, atomicAdd(&cnt[c], 1u), Seg{start, size, depth, 0}, err);
 }
 
 // push_seg for a whole warp: every lane calls it (converged) and the lanes
 // with `want` push their segment.  Lanes pushing to the same list share one
 // atomic on its counter: a round can emit millions of short segments, and one
 // atomic per segment on the few list counters serialises in L2.
-__device__ __forceinline__ void push_seg_warp(const SegLists& L, bool want, uint32_t start, uint32_t size,
+__device__ __forceinline__ void push_seg_warp(const LsArgs& A, uint32_t* cnt, bool want, uint32_t start, uint32_t size,
                                               uint32_t depth, unsigned* err) {
     if (__ballot_sync(SSS_FULL, want) == 0) return;
-    // list of the segment: 0 quad, 1 warp, 2 tiny, 3 small, 4 med, 5 large; 6 none
-    uint32_t cls = 6u;
-    if (want) {
-        if (size <= L.warp_max) cls = size <= (uint32_t)QUAD_W ? 0u : 1u;
-        else if (size <= (uint32_t)TINY_CAP) cls = 2u;
-        else if (size <= (uint32_t)SM_CAP && size <= L.med_max) cls = 3u;
-        else if (size <= L.med_max) cls = 4u;
-        else cls = 5u;
-    }
+    const uint32_t cls = want ? seg_class(A, size) : (uint32_t)LC_COUNT;
     const unsigned peers = __match_any_sync(SSS_FULL, cls);
     if (!want) return;
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t leader = (uint32_t)__ffs(peers) - 1u;
     const uint32_t rank = (uint32_t)__popc(peers & ((1u << lane) - 1u));
-    const uint32_t cidx = (0x214035u >> (4u * cls)) & 0xFu;  // counter of the list: 5 3 0 4 1 2
     uint32_t base = 0;
-    if (lane == leader) base = atomicAdd(&L.cnt[cidx], (uint32_t)__popc(peers));
+    if (lane == leader) base = atomicAdd(&cnt[cls], (uint32_t)__popc(peers));
     base = __shfl_sync(peers, base, leader);
-    const uint32_t i = base + rank;
-    const Seg sg{start, size, depth, 0};
-    bool ok;
-    switch (cls) {
-        case 0: ok = i < L.cap_warp; if (ok) L.warp[i] = sg; break;
-        case 1: ok = i < L.cap_warp; if (ok) L.warp[L.cap_warp - 1u - i] = sg; break;
-        case 2: ok = i < L.cap_tiny; if (ok) L.tiny[i] = sg; break;
-        case 3: ok = i < L.cap_small; if (ok) L.small[i] = sg; break;
-        case 4: ok = i < L.cap_med; if (ok) L.med[i] = sg; break;
-        default: ok = i < L.cap_large; if (ok) L.large[i] = sg; break;
-    }
-    if (!ok) atomicOr(err, ERRBIT_OVERFLOW);
+    put_seg(A, cls, base + rank, Seg{start, size, depth, 0}, err);
 }
 
 // Dynamic work distribution: the next unit for the whole CTA (units vary a lot
-// in cost, so a static block-to-unit map leaves a long tail).
+// in cost, so a static block-to-unit map leaves a long tail).  A CTA's first
+// unit is its own index, the counter hands out the ones past the grid: a grid
+// larger than its work ends without touching the counter (10^4 atomics on one
+// address take 9 us).
 __device__ __forceinline__ uint32_t cta_next_unit(uint32_t* counter) {
     __shared__ uint32_t s_unit;
     __syncthreads();
-    if (threadIdx.x == 0) s_unit = atomicAdd(counter, 1u);
+    if (threadIdx.x == 0) s_unit = gridDim.x + atomicAdd(counter, 1u);
     __syncthreads();
     return s_unit;
 }
@@ -155,12 +125,55 @@ __device__ __forceinline__ uint32_t ref_pick(uint32_t start, uint32_t cnt, uint3
     return cnt > 1 ? ref_mix(start, cnt, depth, t) % cnt : 0u;
 }
 
-// identity order and LCP 0 over positions q0 .. q0 + n (perm and lcp point at q0)
-__global__ void k_init_perm(uint32_t* perm, uint32_t* lcp, uint32_t n, uint32_t q0) {
-    uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q < n) {
-        perm[q] = q0 + q;
-        lcp[q] = 0;
+// Start of a sort: the call's arguments into the context's device state,
+// identity order and LCP 0 over positions q0 .. q1, no LCPs to recompute, and
+// the given initial segments (`table`, in device memory, goes through
+// k_ls_classify instead) on their lists.  One launch in place of an upload per
+// list, two memsets and the identity kernel.
+constexpr uint32_t LS_INLINE = 64;  // initial segments passed by value
+struct LsInit {
+    Seg seg[LS_INLINE];
+    uint32_t n;
+};
+constexpr uint32_t BG_T = 256, BG_PER = 4;
+
+__global__ void __launch_bounds__(BG_T) k_ls_begin(LsDev* __restrict__ S, const __grid_constant__ LsArgs A,
+                                                   const __grid_constant__ LsInit init,
+                                                   unsigned* err) {
+    const uint32_t q0 = A.q0, q1 = A.q1;
+    const uint32_t base = blockIdx.x * BG_T * BG_PER + threadIdx.x;
+#pragma unroll
+    for (uint32_t k = 0; k < BG_PER; ++k) {
+        const uint32_t i = base + k * BG_T;
+        if (i < q1 - q0) {
+            A.perm[q0 + i] = q0 + i;
+            A.lcp[q0 + i] = 0;
+        }
+    }
+    // the words holding the bits of q0 .. q1 - 1 (at most one word per 32
+    // positions and one more: every block clears its share)
+    const uint32_t w0 = q0 >> 5, nw = ((q1 - 1) >> 5) - w0 + 1;
+    for (uint32_t w = blockIdx.x * BG_T + threadIdx.x; w < nw; w += gridDim.x * BG_T) A.fixmap[w0 + w] = 0;
+    if (blockIdx.x != 0) return;
+    if (threadIdx.x < 8) S->cnt[threadIdx.x] = S->work[threadIdx.x] = 0;
+    if (threadIdx.x == 0) {
+        S->args = A;
+        S->rounds = 0;
+    }
+    __syncthreads();
+    if (threadIdx.x < init.n) {
+        const Seg s = init.seg[threadIdx.x];
+        push_seg(A, S->cnt, s.start, s.size, s.depth, err);
+    }
+}
+
+// every segment of >= 2 strings of a device table onto its list
+__global__ void __launch_bounds__(BG_T) k_ls_classify(LsDev* __restrict__ S, const Seg* __restrict__ table, uint32_t m,
+                                                      unsigned* err) {
+    for (uint32_t k0 = blockIdx.x * BG_T; k0 < m; k0 += gridDim.x * BG_T) {
+        const uint32_t k = k0 + threadIdx.x;
+        const Seg s = k < m ? table[k] : Seg{0, 0, 0, 0};
+        push_seg_warp(S->args, S->cnt, s.size >= 2, s.start, s.size, s.depth, err);
     }
 }
 
@@ -350,29 +363,63 @@ __device__ __forceinline__ void finish_segment(const Seg sg, const uint8_t* __re
     for (uint32_t i = tid; i < m; i += THREADS) perm[sg.start + i] = sV[i];
 }
 
-// Segments segs[0 .. count) (count from the device when d_count is given,
-// clamped to count), one CTA at a time.
-template <int THREADS, int CAP>
-__global__ void __launch_bounds__(THREADS) k_finish(const Seg* __restrict__ segs, const uint32_t* __restrict__ d_count,
-                                                    uint32_t count, uint32_t* work, const uint8_t* __restrict__ chars,
-                                                    const uint64_t* __restrict__ offs,
-                                                    const uint32_t* __restrict__ lens, uint32_t* __restrict__ perm,
-                                                    uint32_t* __restrict__ lcp, unsigned* err) {
-    const uint32_t nseg = d_count ? min(*d_count, count) : count;
-    for (uint32_t i = cta_next_unit(work); i < nseg; i = cta_next_unit(work))
-        finish_segment<THREADS, CAP>(segs[i], chars, offs, lens, perm, lcp, err);
+// Where a finisher's segments and strings are: list `cls` of the context's
+// device state (S), or explicit arrays (S == NULL).
+struct FinIn {
+    const LsDev* S;
+    uint32_t cls;
+    GPtr<const Seg> segs;
+    uint32_t count;
+    GPtr<uint32_t> work;
+    GPtr<const uint8_t> chars;
+    GPtr<const uint64_t> offs;
+    GPtr<const uint32_t> lens;
+    GPtr<uint32_t> perm;
+    GPtr<uint32_t> lcp;
+};
+
+// the same with the state's pointers filled in; count = 0 if a list overran
+__device__ __forceinline__ FinIn fin_resolve(FinIn f, unsigned* err) {
+    if (f.S) {
+        const LsArgs& A = f.S->args;
+        f.segs.p = A.list[f.cls];
+        f.count = f.S->cnt[f.cls];
+        f.work.p = const_cast<uint32_t*>(&f.S->work[f.cls]);
+        f.chars.p = A.chars;
+        f.offs.p = A.offs;
+        f.lens.p = A.lens;
+        f.perm.p = A.perm;
+        f.lcp.p = A.lcp;
+        // the short classes share an array of cap[] entries
+        const uint32_t used = f.cls <= LC_WARP ? f.S->cnt[LC_QUAD] + f.S->cnt[LC_WARP] : f.count;
+        if (used > A.cap[f.cls] || f.count > A.cap[f.cls]) {
+            if (threadIdx.x == 0) atomicOr(err, ERRBIT_OVERFLOW);
+            f.count = 0;
+        }
+    }
+    return f;
 }
 
-// k_finish held to two CTAs per SM (the 512-thread class: 63 registers)
+// Segments, one CTA at a time.
 template <int THREADS, int CAP>
-__global__ void __launch_bounds__(THREADS, 2) k_finish2(const Seg* __restrict__ segs, const uint32_t* __restrict__ d_count,
-                                                    uint32_t count, uint32_t* work, const uint8_t* __restrict__ chars,
-                                                    const uint64_t* __restrict__ offs,
-                                                    const uint32_t* __restrict__ lens, uint32_t* __restrict__ perm,
-                                                    uint32_t* __restrict__ lcp, unsigned* err) {
-    const uint32_t nseg = d_count ? min(*d_count, count) : count;
-    for (uint32_t i = cta_next_unit(work); i < nseg; i = cta_next_unit(work))
-        finish_segment<THREADS, CAP>(segs[i], chars, offs, lens, perm, lcp, err);
+__device__ __forceinline__ void finish_list(const FinIn& in, unsigned* err) {
+    __shared__ FinIn f;  // in shared memory: its pointers would cost the loop 10 registers
+    if (threadIdx.x == 0) f = fin_resolve(in, err);
+    __syncthreads();
+    const uint32_t nseg = f.count;
+    for (uint32_t i = blockIdx.x; i < nseg; i = cta_next_unit(f.work))
+        finish_segment<THREADS, CAP>(f.segs[i], f.chars, f.offs, f.lens, f.perm, f.lcp, err);
+}
+
+template <int THREADS, int CAP>
+__global__ void __launch_bounds__(THREADS) k_finish(const FinIn in, unsigned* err) {
+    finish_list<THREADS, CAP>(in, err);
+}
+
+// k_finish held to two CTAs per SM (the 512-thread class)
+template <int THREADS, int CAP>
+__global__ void __launch_bounds__(THREADS, 2) k_finish2(const FinIn in, unsigned* err) {
+    finish_list<THREADS, CAP>(in, err);
 }
 
 // Group finisher: W consecutive lanes of a warp (W = 32, or QUAD_W for the
@@ -506,37 +553,25 @@ __device__ __forceinline__ void finish_group_segment(const Seg sg, bool has, con
     if (live) perm[sg.start + gl] = e;
 }
 
-// Short segments, 32 / W per warp: segment i is segs[i] (top == 0) or
-// segs[top - 1 - i] (a list filled from the top of its array); count from the
-// device when d_count is given, clamped to count.  d_other, when given, is the
-// count of the list that fills the same array from the other end: the two must
-// not overlap.
+// Short segments, 32 / W per warp: segment i is segs[i], or segs[-i] for the
+// class that fills its array downwards.  A warp's first segments are those of
+// its own index, the counter hands out the rest.
 template <int W>
-__global__ void __launch_bounds__(32 * WF_WARPS) k_finish_group(const Seg* __restrict__ segs,
-                                                                const uint32_t* __restrict__ d_count,
-                                                                const uint32_t* __restrict__ d_other, uint32_t count,
-                                                                uint32_t top, uint32_t* work,
-                                                                const uint8_t* __restrict__ chars,
-                                                                const uint64_t* __restrict__ offs,
-                                                                const uint32_t* __restrict__ lens,
-                                                                uint32_t* __restrict__ perm,
-                                                                uint32_t* __restrict__ lcp, unsigned* err) {
+__global__ void __launch_bounds__(32 * WF_WARPS, 4) k_finish_group(const FinIn in, unsigned* err) {
     constexpr uint32_t G = 32u / W;
-    uint32_t nseg = d_count ? min(*d_count, count) : count;
-    if (d_count && d_other && (uint64_t)*d_count + *d_other > count) {
-        if (threadIdx.x == 0) atomicOr(err, ERRBIT_OVERFLOW);
-        nseg = 0;
-    }
+    __shared__ FinIn f;
+    if (threadIdx.x == 0) f = fin_resolve(in, err);
+    __syncthreads();
+    const uint32_t nseg = f.count;
     const uint32_t lane = threadIdx.x & 31;
-    for (;;) {
-        uint32_t i0 = 0;
-        if (lane == 0) i0 = atomicAdd(work, G);
-        i0 = __shfl_sync(SSS_FULL, i0, 0);
-        if (i0 >= nseg) break;
+    const uint32_t nwarps = gridDim.x * WF_WARPS;
+    for (uint32_t i0 = (blockIdx.x * WF_WARPS + (threadIdx.x >> 5)) * G; i0 < nseg;) {
         const uint32_t i = i0 + lane / W;
         const bool has = i < nseg;
-        const Seg sg = has ? segs[top ? top - 1u - i : i] : Seg{0, 0, 0, 0};
-        finish_group_segment<W>(sg, has, chars, offs, lens, perm, lcp, err);
+        const Seg sg = has ? (f.cls == LC_WARP ? *(f.segs - i) : f.segs[i]) : Seg{0, 0, 0, 0};
+        finish_group_segment<W>(sg, has, f.chars, f.offs, f.lens, f.perm, f.lcp, err);
+        if (lane == 0) i0 = nwarps * G + atomicAdd(f.work, G);
+        i0 = __shfl_sync(SSS_FULL, i0, 0);
     }
 }
 
@@ -553,15 +588,23 @@ __device__ __noinline__ uint32_t lcp_full_w_outline(const uint8_t* a, uint32_t l
     return lcp_full_w(a, la, b, lb, d, w);
 }
 
-__device__ __forceinline__ void lg_ext_tile(const LgTile tl, const LgSegInfo* __restrict__ info,
-                                            const uint8_t* __restrict__ chars, const uint64_t* __restrict__ offs,
-                                            const uint32_t* __restrict__ lens, const uint32_t* __restrict__ perm,
-                                            uint64_t* __restrict__ K, uint32_t* __restrict__ segfmt) {
+// A tile of k_lg_ext.  What the member loop needs of the call and the tile sits
+// in shared memory: in registers next to the word stream it spills at the six
+// CTAs per SM this kernel lives on.
+struct ExtTile {
+    GPtr<const uint8_t> chars;
+    GPtr<const uint64_t> offs;
+    GPtr<const uint32_t> lens;
+    GPtr<const uint32_t> perm;
+    GPtr<uint64_t> K;
+    GPtr<const uint8_t> rs;  // the reference and its length
+    uint32_t rl, f, refpos, end;
+};
+__device__ __forceinline__ void lg_ext_tile(uint32_t sidx, const Seg seg, uint32_t begin, ExtTile& P,
+                                            uint32_t* segfmt) {
     constexpr uint32_t NREF = 68;  // 64 words (512 chars) plus a 4-word block of slack
     __shared__ uint64_t refw[NREF];
-    __shared__ uint32_t s_refpos;
-    LgSegInfo si = info[tl.s];
-    const uint32_t d = si.seg.depth;
+    const uint32_t d = seg.depth;
     // The reference of a large segment: the longest of REF_CAND pseudo-random
     // members (the earliest candidate on ties).  A member's LCP with the
     // reference is capped by the reference's length, so a short reference
@@ -572,10 +615,10 @@ __device__ __forceinline__ void lg_ext_tile(const LgTile tl, const LgSegInfo* __
         constexpr uint32_t REF_CAND = 8;
         const uint32_t t = threadIdx.x;
         uint64_t best = 0;
-        uint32_t pos = si.seg.start;
+        uint32_t pos = seg.start;
         if (t < REF_CAND) {
-            pos = si.seg.start + ref_pick(si.seg.start, si.seg.size, d, t);
-            best = ((uint64_t)lens[perm[pos]] << 32) | (uint64_t)(REF_CAND - t);
+            pos = seg.start + ref_pick(seg.start, seg.size, d, t);
+            best = ((uint64_t)P.lens[P.perm[pos]] << 32) | (uint64_t)(REF_CAND - t);
         }
 #pragma unroll
         for (uint32_t o = 16; o > 0; o >>= 1) {
@@ -584,46 +627,57 @@ __device__ __forceinline__ void lg_ext_tile(const LgTile tl, const LgSegInfo* __
         }
         const uint32_t win = REF_CAND - (uint32_t)best;  // the winning candidate's t
         const uint32_t wpos = __shfl_sync(SSS_FULL, pos, win);
-        if (t == 0) s_refpos = wpos;
+        if (t == 0) {
+            const uint32_t r = P.perm[wpos];
+            const uint32_t rl = (uint32_t)(best >> 32);
+            const uint32_t f = key_fmt(rl, d);
+            P.rs.p = P.chars + P.offs[r];
+            P.rl = rl;
+            P.f = f;
+            P.refpos = wpos;
+            P.end = min(begin + (uint32_t)LG_TILE, seg.start + seg.size);
+            if (begin == seg.start) segfmt[sidx] = f;
+        }
     }
     __syncthreads();
-    const uint32_t refpos = s_refpos;
-    uint32_t r = perm[refpos];
-    const uint8_t* rs = chars + offs[r];
-    uint32_t rl = lens[r];
-    const uint32_t f = key_fmt(rl, d);
-    if (threadIdx.x == 0 && tl.begin == si.seg.start) segfmt[tl.s] = f;
-    for (uint32_t i = threadIdx.x; i < NREF; i += LG_T) refw[i] = load_word_be(rs, rl, d + 8 * i);
+    for (uint32_t i = threadIdx.x; i < NREF; i += LG_T) refw[i] = load_word_be(P.rs, P.rl, d + 8 * i);
     __syncthreads();
-    for (uint32_t q = tl.begin + threadIdx.x; q < tl.end; q += LG_T) {
+    for (uint32_t q = begin + threadIdx.x; q < P.end; q += LG_T) {
+        const uint32_t rl = P.rl;
         uint64_t w;
         uint32_t v;
-        if (q == refpos) {
+        if (q == P.refpos) {
             v = rl > d ? rl - d : 0u;
             v = v < VCAP ? v : VCAP;
-            w = load_word_be(rs, rl, d + v);
+            w = load_word_be(P.rs, rl, d + v);
         } else {
-            uint32_t e = perm[q];
-            uint32_t le = lens[e];
+            uint32_t e = P.perm[q];
+            uint32_t le = P.lens[e];
             uint32_t mlen = le < rl ? le : rl;
-            v = (mlen <= d + 8 * (NREF - 4)) ? lcp_full_w_ref(chars + offs[e], le, rl, refw, d, &w)
-                                             : lcp_full_w_outline(chars + offs[e], le, rs, rl, d, &w);
+            v = (mlen <= d + 8 * (NREF - 4)) ? lcp_full_w_ref(P.chars + P.offs[e], le, rl, refw, d, &w)
+                                             : lcp_full_w_outline(P.chars + P.offs[e], le, P.rs, rl, d, &w);
         }
         uint32_t rho = (v >> 3) < NREF ? (uint32_t)(refw[v >> 3] >> (56 - 8 * (v & 7))) & 0xFFu
-                                       : (uint32_t)(load_word_be(rs, rl, d + v) >> 56);
-        K[q] = ref_key(v, w, rho, f);
+                                       : (uint32_t)(load_word_be(P.rs, rl, d + v) >> 56);
+        P.K[q] = ref_key(v, w, rho, P.f);
     }
 }
 
-__global__ void __launch_bounds__(LG_T, 6) k_lg_ext(const LsPlan* __restrict__ plan, const LgTile* __restrict__ tiles,
-                                                 const LgSegInfo* __restrict__ info,
-                                                 const uint8_t* __restrict__ chars, const uint64_t* __restrict__ offs,
-                                                 const uint32_t* __restrict__ lens, const uint32_t* __restrict__ perm,
-                                                 uint64_t* __restrict__ K, uint32_t* __restrict__ segfmt) {
-    const uint32_t nt = plan->ntiles;
+__global__ void __launch_bounds__(LG_T, 6) k_lg_ext(const LsDev* __restrict__ S) {
+    __shared__ ExtTile P;
+    const LsArgs& A = S->args;
+    if (threadIdx.x == 0) {
+        P.chars.p = A.chars;
+        P.offs.p = A.offs;
+        P.lens.p = A.lens;
+        P.perm.p = A.perm;
+        P.K.p = A.K;
+    }
+    const uint32_t nt = S->plan.ntiles;
     for (uint32_t g = blockIdx.x; g < nt; g += gridDim.x) {
         __syncthreads();
-        lg_ext_tile(tiles[g], info, chars, offs, lens, perm, K, segfmt);
+        const LgTile tl = lg_tile(A, S->plan.ns, g);
+        lg_ext_tile(tl.s, A.info[tl.s].seg, tl.begin, P, A.segfmt);
     }
 }
 
@@ -631,20 +685,41 @@ __global__ void __launch_bounds__(LG_T, 6) k_lg_ext(const LsPlan* __restrict__ p
 // keys and indices back, set the LCP at every key change (d + key_lcp) and emit
 // the groups of equal keys: runs of equal strings get lcp = length, other groups
 // become segments at depth d + v + C.  The first position's LCP is left alone.
-// Reads srcK/srcV fully before writing K/perm.
-template <int THREADS, int CAP>
-__device__ void sort_emit(unsigned char* smem, uint32_t bs, uint32_t m, uint32_t d, uint32_t f, const uint64_t* srcK,
-                          const uint32_t* srcV, const uint32_t* __restrict__ lens, uint64_t* K, uint32_t* perm,
-                          uint32_t* __restrict__ lcp, const SegLists& L, unsigned* err) {
+// Reads tK/tV (FROM_T) or K/perm fully before writing K/perm.
+template <int THREADS, int CAP, bool FROM_T>
+__device__ __forceinline__ void sort_emit(unsigned char* smem, uint32_t bs, uint32_t m, uint32_t d, uint32_t f,
+                                          LsDev* S, unsigned* err) {
+    const LsArgs& A = S->args;  // S and err are kernel parameters: no registers held through the sort
+    __shared__ uint32_t s_d, s_f;
+    if (threadIdx.x == 0) {
+        s_d = d;
+        s_f = f;
+    }
     constexpr int ITEMS = CAP / THREADS;
     uint64_t* sHi = reinterpret_cast<uint64_t*>(smem);
     uint64_t* sLo = sHi + CAP;
     uint32_t* sA = reinterpret_cast<uint32_t*>(sLo + CAP);
     uint32_t* sN = sA + CAP;
     __shared__ uint32_t sh_warp[32];
-    for (uint32_t i = threadIdx.x; i < m; i += THREADS) {
-        sHi[i] = srcK[bs + i];
-        sA[i] = srcV[bs + i];
+    {
+        const uint64_t* srcK = FROM_T ? A.tK : A.K;
+        const uint32_t* srcV = FROM_T ? A.tV : A.perm;
+        uint64_t k[ITEMS];
+        uint32_t v[ITEMS];
+#pragma unroll
+        for (int t = 0; t < ITEMS; ++t) {
+            const uint32_t i = threadIdx.x + t * THREADS;
+            k[t] = i < m ? srcK[bs + i] : 0ull;
+            v[t] = i < m ? srcV[bs + i] : 0u;
+        }
+#pragma unroll
+        for (int t = 0; t < ITEMS; ++t) {
+            const uint32_t i = threadIdx.x + t * THREADS;
+            if (i < m) {
+                sHi[i] = k[t];
+                sA[i] = v[t];
+            }
+        }
     }
     __syncthreads();
     // A segment's members arrive in index order (every sort of an earlier round
@@ -662,6 +737,11 @@ __device__ void sort_emit(unsigned char* smem, uint32_t bs, uint32_t m, uint32_t
         __syncthreads();
         block_merge_sort128_fit<THREADS, ITEMS>(sHi, sLo, m);
     }
+    uint64_t* K = A.K;
+    uint32_t* perm = A.perm;
+    uint32_t* lcp = A.lcp;
+    d = s_d;
+    f = s_f;
     for (uint32_t i = threadIdx.x; i < CAP; i += THREADS) {
         uint32_t v = 0;
         if (i < m) {
@@ -691,33 +771,31 @@ __device__ void sort_emit(unsigned char* smem, uint32_t bs, uint32_t m, uint32_t
             if (c >= 2) {
                 const uint64_t k = sHi[i];
                 if (key_ended(k, f)) {
-                    if (i != g) lcp[bs + i] = lens[(uint32_t)sLo[i]];
+                    if (i != g) lcp[bs + i] = A.lens[(uint32_t)sLo[i]];
                 } else if (i == g) {
                     want = true;
                     dn = d + key_v(k, f) + fmt_chars(f);
                 }
             }
         }
-        push_seg_warp(L, want, bs + i, c, dn, err);
+        push_seg_warp(A, S->cnt, want, bs + i, c, dn, err);
     }
 }
 
 // One CTA per (segment, bucket).  Range buckets are sorted in shared memory;
 // groups of equal keys become new segments at depth d + v + C.
 template <int THREADS, int CAP>
-__device__ __forceinline__ void lg_bucket(uint32_t g, uint32_t ns, const LgSegInfo* __restrict__ info,
-                                          const uint32_t* __restrict__ bst, const uint32_t* __restrict__ segfmt,
-                                          const uint64_t* __restrict__ tK, const uint32_t* __restrict__ tV,
-                                          const uint32_t* __restrict__ lens, uint64_t* __restrict__ K,
-                                          uint32_t* __restrict__ perm, uint32_t* __restrict__ lcp, const SegLists& L,
-                                          unsigned* err, uint8_t* __restrict__ fixmark) {
+__device__ __forceinline__ void lg_bucket(uint32_t g, uint32_t npart, LsDev* S, unsigned* err) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const uint32_t sidx = segment_of_bucket(info, ns, g);
-    LgSegInfo si = info[sidx];
-    uint32_t b = g - si.bk_base;
-    uint32_t nbk = 2 * si.nb - 1;
+    const LsArgs& A = S->args;
+    uint32_t* cnt = S->cnt;
+    const uint32_t sidx = warp_last_le(A.bk0, npart, g);
+    const LgSegInfo si = A.info[sidx];
+    const uint32_t b = g - A.bk0[sidx];
+    const uint32_t nbk = 2 * si.nb - 1;
     if (b >= nbk) return;
-    uint32_t bs = bst[si.bst_base + b], be = bst[si.bst_base + b + 1];
+    const uint32_t* bst = A.bst + (size_t)sidx * (LG_NBMAX + 1);
+    uint32_t bs = bst[b], be = bst[b + 1];
     if (bs < si.seg.start || be > si.seg.start + si.seg.size || be < bs) {
         if (threadIdx.x == 0) atomicOr(err, ERRBIT_OVERFLOW);
         return;
@@ -725,111 +803,116 @@ __device__ __forceinline__ void lg_bucket(uint32_t g, uint32_t ns, const LgSegIn
     uint32_t m = be - bs;
     if (m == 0) return;
     uint32_t d = si.seg.depth;
-    const uint32_t f = segfmt[sidx];
+    const uint32_t f = A.segfmt[sidx];
     bool eq = (b & 1u) != 0;
     if (eq || m > (uint32_t)CAP) {
         for (uint32_t q = bs + threadIdx.x; q < be; q += THREADS) {
-            K[q] = tK[q];
-            perm[q] = tV[q];
+            A.K[q] = A.tK[q];
+            A.perm[q] = A.tV[q];
         }
         if (threadIdx.x == 0) {
             if (eq) {
-                uint64_t k = tK[bs];
-                if (m >= 2 && !key_ended(k, f)) push_seg(L, bs, m, d + key_v(k, f) + fmt_chars(f), err);
+                uint64_t k = A.tK[bs];
+                if (m >= 2 && !key_ended(k, f)) push_seg(A, cnt, bs, m, d + key_v(k, f) + fmt_chars(f), err);
             } else {
                 // oversized range bucket: another round at this depth.  Its members
                 // have distinct keys, so the LCPs across its two ends depend on which
                 // members end up first and last: recomputed after the last round.
-                push_seg(L, bs, m, d, err);
-                if (bs > si.seg.start) fixmark[bs] = 1;
-                if (be < si.seg.start + si.seg.size) fixmark[be] = 1;
+                push_seg(A, cnt, bs, m, d, err);
+                if (bs > si.seg.start) atomicOr(&A.fixmap[bs >> 5], 1u << (bs & 31u));
+                if (be < si.seg.start + si.seg.size) atomicOr(&A.fixmap[be >> 5], 1u << (be & 31u));
             }
         }
-        if (eq && m >= 2 && key_ended(tK[bs], f)) {
+        if (eq && m >= 2 && key_ended(A.tK[bs], f)) {
             // a run of equal strings: lcp = length inside the run
-            for (uint32_t q = bs + 1 + threadIdx.x; q < be; q += THREADS) lcp[q] = lens[tV[q]];
+            for (uint32_t q = bs + 1 + threadIdx.x; q < be; q += THREADS) A.lcp[q] = A.lens[A.tV[q]];
         }
         return;
     }
-    sort_emit<THREADS, CAP>(smem, bs, m, d, f, tK, tV, lens, K, perm, lcp, L, err);
+    sort_emit<THREADS, CAP, true>(smem, bs, m, d, f, S, err);
 }
 
 template <int THREADS, int CAP>
-__global__ void __launch_bounds__(THREADS, 65536 / (64 * THREADS)) k_lg_buckets(const LsPlan* __restrict__ plan,
-                                                     const LgSegInfo* __restrict__ info,
-                                                     const uint32_t* __restrict__ bst,
-                                                     const uint32_t* __restrict__ segfmt,
-                                                     const uint64_t* __restrict__ tK, const uint32_t* __restrict__ tV,
-                                                     const uint32_t* __restrict__ lens, uint64_t* __restrict__ K,
-                                                     uint32_t* __restrict__ perm, uint32_t* __restrict__ lcp,
-                                                     SegLists L, unsigned* err, uint8_t* __restrict__ fixmark,
-                                                     uint32_t* work) {
-    const uint32_t nb = plan->pbuckets, npart = plan->npart;
-    for (uint32_t g = cta_next_unit(work); g < nb; g = cta_next_unit(work))
-        lg_bucket<THREADS, CAP>(g, npart, info, bst, segfmt, tK, tV, lens, K, perm, lcp, L, err, fixmark);
+__global__ void __launch_bounds__(THREADS, 65536 / (64 * THREADS)) k_lg_buckets(LsDev* S, unsigned* err) {
+    const uint32_t nb = S->plan.pbuckets;
+    for (uint32_t g = blockIdx.x; g < nb; g = cta_next_unit(&S->work[5]))
+        lg_bucket<THREADS, CAP>(g, S->plan.npart, S, err);
 }
 
-// Large segments of at most DIRECT_CAP strings: one CTA sorts the whole segment
-// by its keys (no sampling, classification or scatter).
-// (segments of more than min_size strings; CAP bounds the size)
+// LCP at the first position of every non-first, non-empty bucket of segment s.
+__device__ __forceinline__ void lg_seams(const LsArgs& A, uint32_t s) {
+    const LgSegInfo si = A.info[s];
+    const uint32_t* bst = A.bst + (size_t)s * (LG_NBMAX + 1);
+    const uint32_t nbk = 2 * si.nb - 1;
+    const uint32_t f = A.segfmt[s];
+    for (uint32_t b = threadIdx.x; b < nbk; b += blockDim.x) {
+        const uint32_t bs = bst[b], be = bst[b + 1];
+        if (be > bs && bs > si.seg.start && be <= si.seg.start + si.seg.size)
+            A.lcp[bs] = si.seg.depth + key_lcp(A.K[bs - 1], A.K[bs], f);
+    }
+}
+
+// The last kernel of a round.  Bucket seams of the partitioned segments (their
+// buckets are sorted by now), then the large segments of at most DIRECT_CAP
+// strings: one CTA sorts a whole segment by its keys (no sampling,
+// classification or scatter).  The last CTA to end decides whether the round
+// loop goes on: another round while segments were pushed, the round limit
+// holds and no capacity error occurred (loop = 1: inside a captured loop).
 template <int THREADS, int CAP>
-__global__ void __launch_bounds__(THREADS) k_lg_direct(const LsPlan* __restrict__ plan,
-                                                       const LgSegInfo* __restrict__ info,
-                                                       const uint32_t* __restrict__ segfmt,
-                                                       const uint32_t* __restrict__ lens, uint64_t* __restrict__ K,
-                                                       uint32_t* __restrict__ perm, uint32_t* __restrict__ lcp,
-                                                       SegLists L, unsigned* err, uint32_t* work, uint32_t min_size) {
+__global__ void __launch_bounds__(THREADS) k_lg_direct(LsDev* S, unsigned* err, cudaGraphConditionalHandle h,
+                                                       int loop) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const uint32_t ns = plan->ns, npart = plan->npart;
-    for (uint32_t sidx = npart + cta_next_unit(work); sidx < ns; sidx = npart + cta_next_unit(work)) {
-        const LgSegInfo si = info[sidx];
-        if (si.seg.size <= min_size || si.seg.size > (uint32_t)CAP) continue;
-        sort_emit<THREADS, CAP>(smem, si.seg.start, si.seg.size, si.seg.depth, segfmt[sidx], K, perm, lens, K, perm,
-                                lcp, L, err);
+    const LsArgs& A = S->args;
+    const uint32_t ns = S->plan.ns, npart = S->plan.npart;
+    for (uint32_t s = blockIdx.x; s < npart; s += gridDim.x) lg_seams(A, s);
+    for (uint32_t i = blockIdx.x; npart + i < ns; i = cta_next_unit(&S->work[6])) {
+        const uint32_t sidx = npart + i;
+        const LgSegInfo si = A.info[sidx];
+        if (si.seg.size > (uint32_t)CAP) continue;
+        sort_emit<THREADS, CAP, false>(smem, si.seg.start, si.seg.size, si.seg.depth, A.segfmt[sidx], S, err);
     }
-}
-
-// LCP at the first position of every non-first, non-empty bucket.
-__global__ void __launch_bounds__(512) k_lg_seams(const LsPlan* __restrict__ plan, const LgSegInfo* __restrict__ info,
-                                                  const uint32_t* __restrict__ bst, const uint32_t* __restrict__ segfmt,
-                                                  const uint64_t* __restrict__ K, uint32_t* __restrict__ lcp) {
-    const uint32_t npart = plan->npart;
-    for (uint32_t s = blockIdx.x; s < npart; s += gridDim.x) {
-        LgSegInfo si = info[s];
-        uint32_t nbk = 2 * si.nb - 1;
-        uint32_t d = si.seg.depth;
-        const uint32_t f = segfmt[s];
-        for (uint32_t b = threadIdx.x; b < nbk; b += 512) {
-            uint32_t bs = bst[si.bst_base + b], be = bst[si.bst_base + b + 1];
-            if (be > bs && bs > si.seg.start && be <= si.seg.start + si.seg.size)
-                lcp[bs] = d + key_lcp(K[bs - 1], K[bs], f);
-        }
+    if (!loop) return;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    __threadfence();
+    if (atomicAdd(&S->work[7], 1u) + 1u != gridDim.x) return;
+    const uint32_t r = ++S->rounds;
+    bool more = atomicAdd(&S->cnt[LC_LARGE], 0u) > 0;
+    if (more && r >= A.limit) {
+        atomicOr(err, ERRBIT_OVERFLOW);
+        more = false;
     }
+    if (*(volatile unsigned*)err & ERRBIT_OVERFLOW) more = false;
+    cudaGraphSetConditional(h, more ? 1u : 0u);
 }
 
 // LCP with the predecessor at the positions marked by k_lg_buckets, from the
 // final order (full comparison; there are at most two per oversized bucket).
-__global__ void k_fix_seams(const uint8_t* __restrict__ fixmark, uint32_t n, const uint8_t* __restrict__ chars,
-                            const uint64_t* __restrict__ offs, const uint32_t* __restrict__ lens,
-                            const uint32_t* __restrict__ perm, uint32_t* __restrict__ lcp) {
-    for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
-        if (!fixmark[q] || q == 0) continue;
-        uint32_t a = perm[q - 1], b = perm[q];
-        uint32_t la = lens[a], lb = lens[b];
-        uint32_t m = la < lb ? la : lb;
-        WordStream A, B;
-        A.init(chars + offs[a], la, 0);
-        B.init(chars + offs[b], lb, 0);
-        uint32_t r = m;
-        for (uint32_t k = 0; k < m; k += 8) {
-            uint64_t x = A.next() ^ B.next();
-            if (x) {
-                uint32_t c = k + ((uint32_t)__clzll((long long)x) >> 3);
-                r = c < m ? c : m;
-                break;
+// One bit per position: a scan of n / 8 bytes.  The first position sorted keeps
+// its 0.
+__global__ void __launch_bounds__(256) k_fix_seams(const LsDev* __restrict__ S) {
+    const LsArgs& A = S->args;
+    const uint32_t q0 = A.q0, q1 = A.q1;
+    for (uint32_t w = (q0 >> 5) + blockIdx.x * 256 + threadIdx.x; w <= (q1 - 1) >> 5; w += gridDim.x * 256) {
+        for (uint32_t m = A.fixmap[w]; m; m &= m - 1) {
+            const uint32_t q = 32 * w + (uint32_t)__ffs(m) - 1;
+            if (q <= q0 || q >= q1) continue;
+            const uint32_t a = A.perm[q - 1], b = A.perm[q];
+            const uint32_t la = A.lens[a], lb = A.lens[b], n = la < lb ? la : lb;
+            WordStream sa, sb;
+            sa.init(A.chars + A.offs[a], la, 0);
+            sb.init(A.chars + A.offs[b], lb, 0);
+            uint32_t r = n;
+            for (uint32_t k = 0; k < n; k += 8) {
+                const uint64_t x = sa.next() ^ sb.next();
+                if (x) {
+                    const uint32_t c = k + ((uint32_t)__clzll((long long)x) >> 3);
+                    r = c < n ? c : n;
+                    break;
+                }
             }
+            A.lcp[q] = r;
         }
-        lcp[q] = r;
     }
 }
 
@@ -862,24 +945,6 @@ __global__ void k_check_input(const uint8_t* __restrict__ chars, uint64_t n_char
         }
 }
 
-// Work memory layout of the local sort.
-struct LsBufs {
-    uint64_t* K;
-    uint64_t* tK;
-    uint32_t* tV;
-    Seg* warp;
-    Seg* tiny;
-    Seg* small;
-    Seg* med;
-    Seg* large;
-    uint32_t* cnt;
-    uint32_t* work;  // dynamic work counters: [0] warp, [1] tiny, [2] med, [3] buckets, [4] direct
-    uint32_t* segfmt;
-    uint8_t* fixmark;
-    SpBufs sp;
-    uint32_t cap_warp, cap_tiny, cap_small, cap_med, cap_large;
-};
-
 // The size-class knobs of the local sort; 0 (e.g. internal callers passing
 // sss_params{}) means the default.  Values are clamped by the API already.
 struct LsKnobs {
@@ -895,81 +960,79 @@ static LsKnobs ls_knobs(const sss_params& prm) {
     return k;
 }
 
-void carve_ls(Arena& ar, uint32_t n, uint32_t p, const sss_params& prm, LsBufs& b) {
+// Work memory of the local sort: fills the pointers and capacities of a.
+void carve_ls(Arena& ar, uint32_t n, uint32_t p, const sss_params& prm, LsArgs& a) {
     const LsKnobs kn = ls_knobs(prm);
-    b.cap_warp = n / 2 + 2;
-    b.cap_tiny = n / (kn.warp_cap + 1) + 2;
-    b.cap_small = n / (TINY_CAP + 1) + 2;
-    b.cap_med = n / (SM_CAP + 1) + 2;
-    b.cap_large = n / (kn.cta_cap + 1) + p + 2;  // every large segment holds > cta_cap strings
-    b.K = ar.take<uint64_t>(n);
-    b.tK = ar.take<uint64_t>(n);
-    b.tV = ar.take<uint32_t>(n);
-    b.warp = ar.take<Seg>(b.cap_warp);
-    b.tiny = ar.take<Seg>(b.cap_tiny);
-    b.small = ar.take<Seg>(b.cap_small);
-    b.med = ar.take<Seg>(b.cap_med);
-    b.large = ar.take<Seg>(b.cap_large);
-    b.cnt = ar.take<uint32_t>(8);
-    b.work = ar.take<uint32_t>(8);
-    b.segfmt = ar.take<uint32_t>(b.cap_large);
-    b.fixmark = ar.take<uint8_t>(n);
-    carve_sp(ar, n, b.cap_large, b.sp);
+    a.cap[LC_QUAD] = a.cap[LC_WARP] = n / 2 + 2;
+    a.cap[LC_TINY] = n / (kn.warp_cap + 1) + 2;
+    a.cap[LC_SMALL] = n / (TINY_CAP + 1) + 2;
+    a.cap[LC_MED] = n / (SM_CAP + 1) + 2;
+    a.cap[LC_LARGE] = n / (kn.cta_cap + 1) + p + 2;  // every large segment holds > cta_cap strings
+    a.K = ar.take<uint64_t>(n);
+    a.tK = ar.take<uint64_t>(n);
+    a.tV = ar.take<uint32_t>(n);
+    a.list[LC_QUAD] = ar.take<Seg>(a.cap[LC_QUAD]);
+    a.list[LC_WARP] = a.list[LC_QUAD] ? a.list[LC_QUAD] + (a.cap[LC_WARP] - 1) : nullptr;
+    for (uint32_t c = LC_TINY; c <= LC_LARGE; ++c) a.list[c] = ar.take<Seg>(a.cap[c]);
+    a.segfmt = ar.take<uint32_t>(a.cap[LC_LARGE]);
+    a.fixmap = ar.take<uint32_t>(n / 32 + 1);
+    carve_sp(ar, n, a.cap[LC_LARGE], a);
+    a.warp_max = kn.warp_cap;
+    a.med_max = kn.cta_cap;
+    a.direct_max = kn.direct_cap;
+    a.target = kn.bucket_target;
+    a.limit = 100000u;
+    a.use_tiles = 0;
 }
 
-// The finishers over their lists: host counts, or (d_cnt != NULL) the device
-// counters of the round that just ran (d_cnt[5] quad, [3] warp, [0] tiny,
-// [4] small, [1] med).
-sss_status run_finishers(sss_ctx* ctx, const LsBufs& B, const uint32_t* d_cnt, uint32_t nquad, uint32_t nwarp,
-                         uint32_t ntiny, uint32_t nsmall, uint32_t nmed, const StrIn& in, uint32_t* perm,
-                         uint32_t* lcp) {
-    const uint32_t sm = (uint32_t)std::max(1, ctx->sm_count);
-    uint32_t gq, gw, gt, gs, gm;
-    if (d_cnt) {
-        nquad = nwarp = B.cap_warp;
-        ntiny = B.cap_tiny;
-        nsmall = B.cap_small;
-        nmed = B.cap_med;
-        gq = sm * 8;
-        gw = sm * 8;
-        gt = sm * 16;
-        gs = sm * 8;
-        gm = sm * 2;
-    } else {
-        if ((uint64_t)nquad + nwarp > B.cap_warp) return sss_fail(ctx, SSS_ERR_CUDA, "local sort: internal capacity exceeded");
-        const uint32_t qpb = WF_WARPS * (32 / QUAD_W);  // quad segments per CTA step
-        gq = std::min((nquad + qpb - 1) / qpb, sm * 8);
-        gw = std::min((nwarp + WF_WARPS - 1) / WF_WARPS, sm * 16);
-        gt = std::min(ntiny, sm * 32);
-        gs = std::min(nsmall, sm * 16);
-        gm = std::min(nmed, sm * 4);
+// Grid sizes follow the number of strings in four steps: a launch of more CTAs
+// than there is work costs up to 3 us for a grid that only finds nothing to do.
+// s is the share of the full grid: 1/8 up to 2^17 strings, then 1/4, 1/2, 1.
+struct LsGrid {
+    uint32_t sm, div;
+    uint32_t of(uint32_t per_sm) const { return std::max(1u, sm * per_sm / div); }
+};
+uint32_t ls_grid_class(uint32_t nr) { return nr <= (1u << 17) ? 0u : nr <= (1u << 18) ? 1u : nr <= (1u << 19) ? 2u : 3u; }
+LsGrid ls_grid(sss_ctx* ctx, uint32_t cls) { return LsGrid{(uint32_t)std::max(1, ctx->sm_count), 8u >> cls}; }
+
+// One finisher: grid CTAs over `in`.
+sss_status launch_finisher(sss_ctx* ctx, uint32_t cls, uint32_t grid, const FinIn& in) {
+    switch (cls) {
+        case LC_QUAD:
+            return sss_launch(ctx, "ls_finish_quad", k_finish_group<QUAD_W>, dim3(grid), dim3(32 * WF_WARPS), 0, in, ctx->d_err);
+        case LC_WARP:
+            return sss_launch(ctx, "ls_finish_warp", k_finish_group<32>, dim3(grid), dim3(32 * WF_WARPS), 0, in, ctx->d_err);
+        case LC_TINY:
+            return sss_launch(ctx, "ls_finish_tiny", k_finish<TINY_T, TINY_CAP>, dim3(grid), dim3(TINY_T),
+                              finish_smem(TINY_CAP), in, ctx->d_err);
+        case LC_SMALL:
+            return sss_launch(ctx, "ls_finish_small", k_finish<SM_T, SM_CAP>, dim3(grid), dim3(SM_T),
+                              finish_smem(SM_CAP), in, ctx->d_err);
+        default:
+            return sss_launch(ctx, "ls_finish_cta", k_finish2<MED_T, MED_CAP>, dim3(grid), dim3(MED_T),
+                              finish_smem(MED_CAP), in, ctx->d_err);
     }
-    SSS_TRY(sss_launch(ctx, "ls_finish_quad", k_finish_group<QUAD_W>, dim3(gq), dim3(32 * WF_WARPS), 0,
-                       (const Seg*)B.warp, d_cnt ? d_cnt + 5 : (const uint32_t*)nullptr,
-                       d_cnt ? d_cnt + 3 : (const uint32_t*)nullptr, nquad, 0u, B.work + 4, in.chars, in.offs,
-                       in.lens, perm, lcp, ctx->d_err));
-    SSS_TRY(sss_launch(ctx, "ls_finish_warp", k_finish_group<32>, dim3(gw), dim3(32 * WF_WARPS), 0,
-                       (const Seg*)B.warp, d_cnt ? d_cnt + 3 : (const uint32_t*)nullptr,
-                       (const uint32_t*)nullptr, nwarp, B.cap_warp, B.work + 0, in.chars, in.offs, in.lens, perm,
-                       lcp, ctx->d_err));
-    SSS_TRY(sss_launch(ctx, "ls_finish_tiny", k_finish<TINY_T, TINY_CAP>, dim3(gt), dim3(TINY_T),
-                       finish_smem(TINY_CAP), (const Seg*)B.tiny, d_cnt ? d_cnt + 0 : (const uint32_t*)nullptr, ntiny,
-                       B.work + 1, in.chars, in.offs, in.lens, perm, lcp, ctx->d_err));
-    SSS_TRY(sss_launch(ctx, "ls_finish_small", k_finish<SM_T, SM_CAP>, dim3(gs), dim3(SM_T), finish_smem(SM_CAP),
-                       (const Seg*)B.small, d_cnt ? d_cnt + 4 : (const uint32_t*)nullptr, nsmall, B.work + 6, in.chars,
-                       in.offs, in.lens, perm, lcp, ctx->d_err));
-    SSS_TRY(sss_launch(ctx, "ls_finish_cta", k_finish2<MED_T, MED_CAP>, dim3(gm), dim3(MED_T), finish_smem(MED_CAP),
-                       (const Seg*)B.med, d_cnt ? d_cnt + 1 : (const uint32_t*)nullptr, nmed, B.work + 2, in.chars,
-                       in.offs, in.lens, perm, lcp, ctx->d_err));
-    return SSS_OK;
+}
+
+FinIn list_input(sss_ctx* ctx, uint32_t cls) {
+    FinIn f{};
+    f.S = static_cast<const LsDev*>(ctx->d_ls);
+    f.cls = cls;
+    return f;
+}
+
+// CTAs of a finisher after a round loop (the counts are on the device)
+uint32_t finisher_grid(const LsGrid& g, uint32_t cls) {
+    static const uint32_t per_sm[5] = {8, 8, 16, 8, 2};
+    return g.of(per_sm[cls]);
 }
 
 }  // namespace
 
 size_t need_local_sort(uint32_t n, uint32_t p, const sss_params& prm) {
     Arena ar;
-    LsBufs b;
-    carve_ls(ar, n, p, prm, b);
+    LsArgs a{};
+    carve_ls(ar, n, p, prm, a);
     return ar.off + 256;
 }
 
@@ -1006,126 +1069,109 @@ sss_status impl_local_sort(sss_ctx* ctx, Arena& ar, const StrIn& in, uint32_t p,
 
 // One round of the multi-CTA path, planned on the device from the segments the
 // previous round pushed: keys, partition of the large segments, bucket sorts,
-// seams, whole-segment sorts, then the finishers of every segment pushed.
-static sss_status launch_round(sss_ctx* ctx, const LsBufs& B, const LsKnobs& kn, const SegLists& L,
-                               const StrIn& in, uint32_t* perm, uint32_t* lcp) {
-    const uint32_t sm = (uint32_t)std::max(1, ctx->sm_count);
-    SSS_TRY(sss_launch(ctx, "ls_lg_plan", k_lg_plan, dim3(1), dim3(1024), 0, (const Seg*)B.large, B.cnt, B.work,
-                       kn.direct_cap, kn.bucket_target, B.sp.cap_segs, B.sp.cap_tiles, B.sp.cap_hist, B.sp.info,
-                       B.sp.plan, ctx->d_err));
-    SSS_TRY(sss_launch(ctx, "ls_lg_tiles", k_lg_tiles, dim3(sm * 4), dim3(256), 0, (const LsPlan*)B.sp.plan,
-                       (const LgSegInfo*)B.sp.info, B.sp.tiles));
-    SSS_TRY(sss_launch(ctx, "ls_lg_ext", k_lg_ext, dim3(sm * 6), dim3(LG_T), 0, (const LsPlan*)B.sp.plan,
-                       (const LgTile*)B.sp.tiles, (const LgSegInfo*)B.sp.info, in.chars, in.offs, in.lens,
-                       (const uint32_t*)perm, B.K, B.segfmt));
-    SSS_TRY(launch_sp(ctx, B.sp, B.K, perm, B.tK, B.tV, "ls_lg_samples", "ls_lg_classify", "ls_lg_offsets",
-                      "ls_lg_scatter"));
-    if (kn.bucket_target <= (uint32_t)BKS_CAP / 2) {
-        SSS_TRY(sss_launch(ctx, "ls_lg_buckets", k_lg_buckets<BKS_T, BKS_CAP>, dim3(sm * 4), dim3(BKS_T),
-                           emit_smem(BKS_T, BKS_CAP), (const LsPlan*)B.sp.plan, (const LgSegInfo*)B.sp.info,
-                           (const uint32_t*)B.sp.bst, (const uint32_t*)B.segfmt, (const uint64_t*)B.tK,
-                           (const uint32_t*)B.tV, in.lens, B.K, perm, lcp, L, ctx->d_err, B.fixmark, B.work + 3));
-    } else {
-        SSS_TRY(sss_launch(ctx, "ls_lg_buckets", k_lg_buckets<BK_T, BK_CAP>, dim3(sm * 2), dim3(BK_T),
-                           emit_smem(BK_T, BK_CAP), (const LsPlan*)B.sp.plan, (const LgSegInfo*)B.sp.info,
-                           (const uint32_t*)B.sp.bst, (const uint32_t*)B.segfmt, (const uint64_t*)B.tK,
-                           (const uint32_t*)B.tV, in.lens, B.K, perm, lcp, L, ctx->d_err, B.fixmark, B.work + 3));
-    }
-    SSS_TRY(sss_launch(ctx, "ls_lg_seams", k_lg_seams, dim3(sm * 2), dim3(512), 0, (const LsPlan*)B.sp.plan,
-                       (const LgSegInfo*)B.sp.info, (const uint32_t*)B.sp.bst, (const uint32_t*)B.segfmt,
-                       (const uint64_t*)B.K, lcp));
-    SSS_TRY(sss_launch(ctx, "ls_lg_direct", k_lg_direct<DIRECT_T, DIRECT_CAP>, dim3(sm), dim3(DIRECT_T),
-                       emit_smem(DIRECT_T, DIRECT_CAP), (const LsPlan*)B.sp.plan, (const LgSegInfo*)B.sp.info,
-                       (const uint32_t*)B.segfmt, in.lens, B.K, perm, lcp, L, ctx->d_err, B.work + 5, 0u));
-    return run_finishers(ctx, B, B.cnt, 0, 0, 0, 0, 0, in, perm, lcp);
+// seams and whole-segment sorts.  Segments up to cta_cap strings stay on their
+// lists: they are finished once, after the last round (one launch per class
+// over all rounds' segments in place of one per round).
+static sss_status launch_round(sss_ctx* ctx, const LsGrid& g, bool small_buckets, cudaGraphConditionalHandle h,
+                               int loop) {
+    LsDev* S = static_cast<LsDev*>(ctx->d_ls);
+    const LsDev* cS = S;
+    SSS_TRY(sss_launch(ctx, "ls_lg_plan", k_lg_plan, dim3(1), dim3(1024), 0, S, ctx->d_err));
+    if (g.div == 1)
+        SSS_TRY(sss_launch(ctx, "ls_lg_tiles", k_lg_tiles, dim3(g.of(4)), dim3(256), 0, cS));
+    SSS_TRY(sss_launch(ctx, "ls_lg_ext", k_lg_ext, dim3(g.of(6)), dim3(LG_T), 0, cS));
+    SSS_TRY(sss_launch(ctx, "ls_lg_samples", k_lg_samples, dim3(g.of(2)), dim3(512), 0, cS));
+    SSS_TRY(sss_launch(ctx, "ls_lg_classify", k_lg_classify, dim3(g.of(6)), dim3(LG_T), 0, cS));
+    SSS_TRY(sss_launch(ctx, "ls_lg_offsets", k_lg_rowscan, dim3(g.of(4)), dim3(256), 0, cS));
+    SSS_TRY(sss_launch(ctx, "ls_lg_scatter", k_lg_scatter, dim3(g.of(8)), dim3(LG_T), 0, cS, ctx->d_err));
+    if (small_buckets)
+        SSS_TRY(sss_launch(ctx, "ls_lg_buckets", k_lg_buckets<BKS_T, BKS_CAP>, dim3(std::max(g.sm, g.of(4))),
+                           dim3(BKS_T), emit_smem(BKS_T, BKS_CAP), S, ctx->d_err));
+    else
+        SSS_TRY(sss_launch(ctx, "ls_lg_buckets", k_lg_buckets<BK_T, BK_CAP>, dim3(std::max(g.sm, g.of(2))),
+                           dim3(BK_T), emit_smem(BK_T, BK_CAP), S, ctx->d_err));
+    return sss_launch(ctx, "ls_lg_direct", k_lg_direct<DIRECT_T, DIRECT_CAP>, dim3(g.sm), dim3(DIRECT_T),
+                      emit_smem(DIRECT_T, DIRECT_CAP), S, ctx->d_err, h, loop);
 }
 
-// Loop condition of the captured round loop: another round while segments were
-// pushed, the round limit is not reached and no capacity error occurred.
-__global__ void k_ls_cond(const uint32_t* __restrict__ cnt, uint32_t* rounds, uint32_t limit, unsigned* err,
-                          cudaGraphConditionalHandle h) {
-    const uint32_t r = ++*rounds;
-    bool more = cnt[2] > 0;
-    if (more && r >= limit) {
-        atomicOr(err, ERRBIT_OVERFLOW);
-        more = false;
+// The rounds, the finishers and the seam fix as one graph: a while node whose
+// body is one round, the finishers as parallel branches after it, then the
+// seams.  Its kernels take the context's device state only, so one graph per
+// grid class and bucket CTA (eight at most, kept in the context) serves every
+// call; captured per call address, a sort of new inputs paid for a capture.
+static sss_status sort_graph(sss_ctx* ctx, uint32_t gcls, bool small_buckets, cudaGraphExec_t* out) {
+    sss_ctx::LsGraph& slot = ctx->ls_graphs[2 * gcls + (small_buckets ? 1 : 0)];
+    if (slot.exec) {
+        *out = slot.exec;
+        return SSS_OK;
     }
-    if (*(volatile unsigned*)err & ERRBIT_OVERFLOW) more = false;
-    cudaGraphSetConditional(h, more ? 1u : 0u);
-}
-
-// The round loop as one graph launch: a while node whose body is one round plus
-// k_ls_cond.  Built on first use and kept in the context (a few graphs, least
-// recently used replaced) under a key of every pointer and size its kernels take.
-static sss_status run_rounds_graph(sss_ctx* ctx, const LsBufs& B, const LsKnobs& kn, const SegLists& L,
-                                   const StrIn& in, uint32_t* perm, uint32_t* lcp, uint32_t limit) {
-    char keyb[512];
-    std::snprintf(keyb, sizeof(keyb), "%p %p %p %u %p %p %p %p %p %u %u %u %u %d %u", (const void*)in.chars,
-                  (const void*)in.offs, (const void*)in.lens, in.n, (void*)perm, (void*)lcp, (void*)B.K,
-                  (void*)B.large, (void*)B.sp.plan, kn.warp_cap, kn.cta_cap, kn.direct_cap, kn.bucket_target,
-                  ctx->sm_count, limit);
-    uint32_t* rounds = reinterpret_cast<uint32_t*>(ctx->d_err) + 1;  // a spare word of the context
-    sss_ctx::LsGraph* slot = nullptr;
-    for (auto& lg : ctx->ls_graphs)
-        if (lg.exec && lg.key == keyb) slot = &lg;
-    if (!slot) {
-        slot = &ctx->ls_graphs[0];  // an empty entry, else the least recently used
-        for (auto& lg : ctx->ls_graphs)
-            if (!lg.exec ? slot->exec != nullptr : (slot->exec && lg.used < slot->used)) slot = &lg;
-        if (slot->exec) cudaGraphExecDestroy(slot->exec);
-        if (slot->graph) cudaGraphDestroy(slot->graph);
-        slot->exec = nullptr;
-        slot->graph = nullptr;
-        slot->key.clear();
-        if (!ctx->cap_stream) SSS_CUDA(cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
-        cudaGraph_t g;
-        SSS_CUDA(cudaGraphCreate(&g, 0));
-        cudaGraphConditionalHandle h;
-        SSS_CUDA(cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault));
-        cudaGraphNodeParams cp{};
-        cp.type = cudaGraphNodeTypeConditional;
-        cp.conditional.handle = h;
-        cp.conditional.type = cudaGraphCondTypeWhile;
-        cp.conditional.size = 1;
-        cudaGraphNode_t node;
-        SSS_CUDA(cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &cp));
+    for (cudaStream_t* s : {&ctx->cap_stream, &ctx->cap_stream2, &ctx->cap_stream3})
+        if (!*s) SSS_CUDA(cudaStreamCreateWithFlags(s, cudaStreamNonBlocking));
+    for (cudaEvent_t& e : ctx->cap_event)
+        if (!e) SSS_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    const LsGrid g = ls_grid(ctx, gcls);
+    cudaGraph_t graph;
+    SSS_CUDA(cudaGraphCreate(&graph, 0));
+    cudaStream_t saved = ctx->stream;
+    ctx->capturing = true;
+    sss_status st = SSS_OK;
+    cudaGraphConditionalHandle h;
+    cudaGraphNodeParams cp{};
+    cp.type = cudaGraphNodeTypeConditional;
+    cp.conditional.type = cudaGraphCondTypeWhile;
+    cp.conditional.size = 1;
+    cudaGraphNode_t node = nullptr;
+    cudaError_t ce = cudaGraphConditionalHandleCreate(&h, graph, 1, cudaGraphCondAssignDefault);
+    cp.conditional.handle = h;
+    if (ce == cudaSuccess) ce = cudaGraphAddNode(&node, graph, nullptr, nullptr, 0, &cp);
+    // the body: one round
+    if (ce == cudaSuccess) {
         cudaGraph_t body = cp.conditional.phGraph_out[0];
-        cudaStream_t saved = ctx->stream;
-        ctx->stream = ctx->cap_stream;
-        ctx->capturing = true;
-        sss_status st = SSS_OK;
-        cudaError_t ce = cudaStreamBeginCaptureToGraph(ctx->cap_stream, body, nullptr, nullptr, 0,
-                                                       cudaStreamCaptureModeThreadLocal);
+        ce = cudaStreamBeginCaptureToGraph(ctx->cap_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
         if (ce == cudaSuccess) {
-            st = launch_round(ctx, B, kn, L, in, perm, lcp);
-            if (st == SSS_OK)
-                st = sss_launch(ctx, "ls_cond", k_ls_cond, dim3(1), dim3(1), 0, (const uint32_t*)B.cnt, rounds, limit,
-                                ctx->d_err, h);
-            cudaGraph_t out = body;
-            cudaError_t ee = cudaStreamEndCapture(ctx->cap_stream, &out);
+            ctx->stream = ctx->cap_stream;
+            st = launch_round(ctx, g, small_buckets, h, 1);
+            const cudaError_t ee = cudaStreamEndCapture(ctx->cap_stream, &body);
             if (ce == cudaSuccess) ce = ee;
         }
-        ctx->capturing = false;
-        ctx->stream = saved;
-        if (st != SSS_OK || ce != cudaSuccess) {
-            cudaGetLastError();
-            cudaGraphDestroy(g);
-            return st != SSS_OK ? st : sss_fail(ctx, SSS_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(ce));
-        }
-        cudaGraphExec_t ex;
-        ce = cudaGraphInstantiate(&ex, g, 0);
-        if (ce != cudaSuccess) {
-            cudaGetLastError();
-            cudaGraphDestroy(g);
-            return sss_fail(ctx, SSS_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(ce));
-        }
-        slot->graph = g;
-        slot->exec = ex;
-        slot->key = keyb;
     }
-    slot->used = ++ctx->ls_clock;
-    SSS_CUDA(cudaMemsetAsync(rounds, 0, sizeof(uint32_t), ctx->stream));
-    return sss_graph_launch(ctx, ctx->graph_tag, slot->exec);
+    // after it: the finishers side by side, then the seams
+    if (st == SSS_OK && ce == cudaSuccess) {
+        ce = cudaStreamBeginCaptureToGraph(ctx->cap_stream, graph, &node, nullptr, 1, cudaStreamCaptureModeThreadLocal);
+        if (ce == cudaSuccess) {
+            cudaStream_t br[3] = {ctx->cap_stream, ctx->cap_stream2, ctx->cap_stream3};
+            static const uint32_t order[3][2] = {{LC_MED, LC_COUNT}, {LC_SMALL, LC_TINY}, {LC_WARP, LC_QUAD}};
+            ce = cudaEventRecord(ctx->cap_event[0], br[0]);
+            for (int b = 1; b < 3 && ce == cudaSuccess; ++b) ce = cudaStreamWaitEvent(br[b], ctx->cap_event[0], 0);
+            for (int b = 0; b < 3 && st == SSS_OK; ++b) {
+                ctx->stream = br[b];
+                for (uint32_t c : order[b])
+                    if (c != LC_COUNT && st == SSS_OK) st = launch_finisher(ctx, c, finisher_grid(g, c), list_input(ctx, c));
+            }
+            for (int b = 1; b < 3; ++b) {
+                if (ce == cudaSuccess) ce = cudaEventRecord(ctx->cap_event[b], br[b]);
+                if (ce == cudaSuccess) ce = cudaStreamWaitEvent(br[0], ctx->cap_event[b], 0);
+            }
+            ctx->stream = br[0];
+            if (st == SSS_OK)
+                st = sss_launch(ctx, "ls_fix_seams", k_fix_seams, dim3(g.of(4)), dim3(256), 0,
+                                static_cast<const LsDev*>(ctx->d_ls));
+            const cudaError_t ee = cudaStreamEndCapture(ctx->cap_stream, &graph);
+            if (ce == cudaSuccess) ce = ee;
+        }
+    }
+    ctx->capturing = false;
+    ctx->stream = saved;
+    cudaGraphExec_t ex = nullptr;
+    if (st == SSS_OK && ce == cudaSuccess) ce = cudaGraphInstantiate(&ex, graph, 0);
+    if (st != SSS_OK || ce != cudaSuccess) {
+        cudaGetLastError();
+        cudaGraphDestroy(graph);
+        return st != SSS_OK ? st : sss_fail(ctx, SSS_ERR_CUDA, std::string("sort graph: ") + cudaGetErrorString(ce));
+    }
+    slot.graph = graph;
+    slot.exec = *out = ex;
+    return SSS_OK;
 }
 
 sss_status impl_sort_segments(sss_ctx* ctx, Arena& ar, const StrIn& in, const std::vector<Seg>& init,
@@ -1138,227 +1184,86 @@ sss_status impl_sort_segments_range(sss_ctx* ctx, Arena& ar, const StrIn& in, co
     const uint32_t n = in.n;
     if (n == 0 || q1 <= q0) return SSS_OK;
     const uint32_t nr = q1 - q0;
-    LsBufs B;
-    carve_ls(ar, n, 1, prm, B);
-    const LsKnobs kn = ls_knobs(prm);
-    const uint32_t warp_max = kn.warp_cap, med_max = kn.cta_cap;
+    LsArgs A{};
+    carve_ls(ar, n, 1, prm, A);
+    A.chars = in.chars;
+    A.offs = in.offs;
+    A.lens = in.lens;
+    A.perm = perm;
+    A.lcp = lcp;
+    A.q0 = q0;
+    A.q1 = q1;
+    const uint32_t gcls = ls_grid_class(nr);
+    A.use_tiles = ls_grid(ctx, gcls).div == 1;
     SSS_TRY(set_ls_attributes(ctx));
-    SSS_TRY(sss_launch(ctx, "ls_init", k_init_perm, dim3((nr + 255) / 256), dim3(256), 0, perm + q0, lcp + q0, nr,
-                       q0));
+    LsDev* S = static_cast<LsDev*>(ctx->d_ls);
 
-    // initial segments (partitions or instances), by size class
-    std::vector<Seg> quad, warp, tiny, small, med, large;
+    // initial segments (partitions or instances), counted by size class
+    uint32_t have[LC_COUNT] = {}, m = 0;
+    LsInit li{};
     for (const Seg& s : init) {
         if (s.size < 2) continue;
-        if (s.size <= warp_max && s.size <= (uint32_t)QUAD_W) quad.push_back(s);
-        else if (s.size <= warp_max) warp.push_back(s);
-        else if (s.size <= (uint32_t)TINY_CAP) tiny.push_back(s);
-        else if (s.size <= (uint32_t)SM_CAP && s.size <= med_max) small.push_back(s);
-        else if (s.size <= med_max) med.push_back(s);
-        else large.push_back(s);
+        const uint32_t c = s.size <= A.warp_max    ? (s.size <= (uint32_t)QUAD_W ? LC_QUAD : LC_WARP)
+                           : s.size <= (uint32_t)TINY_CAP ? LC_TINY
+                           : s.size <= A.med_max   ? (s.size <= (uint32_t)SM_CAP ? LC_SMALL : LC_MED)
+                                                   : LC_LARGE;
+        ++have[c];
+        if (m < LS_INLINE) li.seg[m] = s;
+        ++m;
     }
-    if (large.size() > B.cap_large || quad.size() + warp.size() > B.cap_warp)
-        return sss_fail(ctx, SSS_ERR_CUDA, "local sort: internal capacity exceeded");
-    // the warp class fills its array from the top: segment i at cap_warp - 1 - i
-    std::reverse(warp.begin(), warp.end());
-    // pinned staging: counters, then the initial lists
-    void* pin;
-    SSS_TRY(sss_pinned(ctx, 64 + sizeof(Seg) * (init.size() + 4), &pin));
-    uint32_t* h_cnt = reinterpret_cast<uint32_t*>(pin);
-    Seg* hq = reinterpret_cast<Seg*>(reinterpret_cast<char*>(pin) + 64);
-    Seg* hw = hq + quad.size();
-    Seg* ht = hw + warp.size();
-    Seg* hs = ht + tiny.size();
-    Seg* hm = hs + small.size();
-    Seg* hl = hm + med.size();
-    std::copy(quad.begin(), quad.end(), hq);
-    std::copy(warp.begin(), warp.end(), hw);
-    std::copy(tiny.begin(), tiny.end(), ht);
-    std::copy(small.begin(), small.end(), hs);
-    std::copy(med.begin(), med.end(), hm);
-    std::copy(large.begin(), large.end(), hl);
-    for (int k = 0; k < 8; ++k) h_cnt[k] = 0;
-    h_cnt[2] = (uint32_t)large.size();
-    SSS_TRY(sss_upload(ctx, B.warp, hq, sizeof(Seg) * quad.size()));
-    SSS_TRY(sss_upload(ctx, B.warp + (B.cap_warp - warp.size()), hw, sizeof(Seg) * warp.size()));
-    SSS_TRY(sss_upload(ctx, B.tiny, ht, sizeof(Seg) * tiny.size()));
-    SSS_TRY(sss_upload(ctx, B.small, hs, sizeof(Seg) * small.size()));
-    SSS_TRY(sss_upload(ctx, B.med, hm, sizeof(Seg) * med.size()));
-    SSS_TRY(sss_upload(ctx, B.large, hl, sizeof(Seg) * large.size()));
-    SSS_TRY(sss_upload(ctx, B.cnt, h_cnt, sizeof(uint32_t) * 8));
-    SSS_CUDA(cudaMemsetAsync(B.work, 0, sizeof(uint32_t) * 8, ctx->stream));
-    SSS_TRY(run_finishers(ctx, B, nullptr, (uint32_t)quad.size(), (uint32_t)warp.size(), (uint32_t)tiny.size(),
-                          (uint32_t)small.size(), (uint32_t)med.size(), in, perm, lcp));
-    if (large.empty()) return SSS_OK;
-
-    SSS_CUDA(cudaMemsetAsync(B.fixmark + q0, 0, nr, ctx->stream));
-    SegLists L{B.tiny, B.med, B.large, B.cnt, B.cap_tiny, B.cap_med, B.cap_large, B.warp, B.cap_warp, B.small,
-               B.cap_small, warp_max, med_max};
-    if (prm.flags & SSS_FLAG_GRAPH) {
-        SSS_TRY(run_rounds_graph(ctx, B, kn, L, in, perm, lcp, 100000u));
-    } else {
+    li.n = m <= LS_INLINE ? m : 0u;
+    SSS_TRY(sss_launch(ctx, "ls_init", k_ls_begin, dim3((nr + BG_T * BG_PER - 1) / (BG_T * BG_PER)), dim3(BG_T), 0, S,
+                       A, li, ctx->d_err));
+    if (m > LS_INLINE) {
+        // more than fit in the launch's arguments: through the second key array,
+        // free until the first scatter (every one holds >= 2 strings of 8 bytes there)
+        void* pin;
+        SSS_TRY(sss_pinned(ctx, sizeof(Seg) * (size_t)m, &pin));
+        Seg* h = static_cast<Seg*>(pin);
+        for (const Seg& s : init)
+            if (s.size >= 2) *h++ = s;
+        Seg* table = reinterpret_cast<Seg*>(A.tK.p);
+        SSS_TRY(sss_upload(ctx, table, pin, sizeof(Seg) * (size_t)m));
+        SSS_TRY(sss_launch(ctx, "ls_classify", k_ls_classify,
+                           dim3(std::min((m + BG_T - 1) / BG_T, (uint32_t)ctx->sm_count)), dim3(BG_T), 0, S,
+                           (const Seg*)table, m, ctx->d_err));
+    }
+    if (have[LC_LARGE] == 0) {
+        // nothing for the rounds: the finishers over the initial segments
+        const uint32_t sm = (uint32_t)std::max(1, ctx->sm_count);
+        const uint32_t qpb = WF_WARPS * (32 / QUAD_W);
+        const uint32_t grid[5] = {std::min((have[LC_QUAD] + qpb - 1) / qpb, sm * 8),
+                                  std::min((have[LC_WARP] + WF_WARPS - 1) / WF_WARPS, sm * 16),
+                                  std::min(have[LC_TINY], sm * 32), std::min(have[LC_SMALL], sm * 16),
+                                  std::min(have[LC_MED], sm * 4)};
+        for (uint32_t c = LC_MED + 1; c-- > LC_QUAD;) SSS_TRY(launch_finisher(ctx, c, grid[c], list_input(ctx, c)));
+        return SSS_OK;
+    }
+    const bool small_buckets = A.target <= (uint32_t)BKS_CAP / 2;
+    if (!ctx->timing || (prm.flags & SSS_FLAG_GRAPH)) {
+        cudaGraphExec_t ex;
+        SSS_TRY(sort_graph(ctx, gcls, small_buckets, &ex));
+        return sss_graph_launch(ctx, ctx->graph_tag, ex);
+    }
+    // kernel timing is on: the same kernels launched one by one, with the next
+    // round's segment count and the error word read back after every round
+    const LsGrid g = ls_grid(ctx, gcls);
     uint32_t* h_next = reinterpret_cast<uint32_t*>(ctx->h_small);
     for (uint32_t rounds = 1;; ++rounds) {
-        if (rounds > 100000u) return sss_fail(ctx, SSS_ERR_CUDA, "local sort: round limit exceeded");
-        SSS_TRY(launch_round(ctx, B, kn, L, in, perm, lcp));
-        // segments pushed for the next round, and the sticky error word
-        SSS_CUDA(cudaMemcpyAsync(h_next, B.cnt + 2, sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
+        if (rounds > A.limit) return sss_fail(ctx, SSS_ERR_CUDA, "local sort: round limit exceeded");
+        SSS_TRY(launch_round(ctx, g, small_buckets, cudaGraphConditionalHandle{}, 0));
+        SSS_CUDA(cudaMemcpyAsync(h_next, &S->cnt[LC_LARGE], sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
         SSS_CUDA(cudaMemcpyAsync(h_next + 1, ctx->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
         SSS_CUDA(cudaStreamSynchronize(ctx->stream));
         if (h_next[1] & ERRBIT_OVERFLOW) return sss_fail(ctx, SSS_ERR_CUDA, "local sort: device capacity check failed");
         if (h_next[0] == 0) break;
     }
-    }
-    // (over the sorted range only; its first position keeps lcp 0)
-    SSS_TRY(sss_launch(ctx, "ls_fix_seams", k_fix_seams, dim3(std::min((nr + 255) / 256, 4096u)), dim3(256), 0,
-                       (const uint8_t*)(B.fixmark + q0), nr, in.chars, in.offs, in.lens,
-                       (const uint32_t*)(perm + q0), lcp + q0));
-    return SSS_OK;
+    for (uint32_t c = LC_QUAD; c <= LC_MED; ++c)
+        SSS_TRY(launch_finisher(ctx, c, finisher_grid(g, c), list_input(ctx, c)));
+    return sss_launch(ctx, "ls_fix_seams", k_fix_seams, dim3(g.of(4)), dim3(256), 0, (const LsDev*)S);
 }
 
-// ---------------------------------------------------------------------------
-// The batched sort as one graph launch (sss_sort_batch with SSS_FLAG_GRAPH).
-// The instances are classified into the size-class lists on the device, so no
-// step needs the host: identity order, classification, the first finishers,
-// the round loop (a conditional WHILE node around one planned round) and the
-// instance-local permutation are all nodes of one graph, kept in the context
-// under a key of every pointer and size its kernels take.
-
-// every instance of >= 2 strings becomes a segment of its size class
-__global__ void k_batch_classify(const Seg* __restrict__ inst, uint32_t m, SegLists L, unsigned* err) {
-    for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
-        const Seg s = inst[k];
-        if (s.size >= 2) push_seg(L, s.start, s.size, 0, err);
-    }
-}
-
-// the round loop runs at least once only if an instance is large
-__global__ void k_ls_cond0(const uint32_t* __restrict__ cnt, cudaGraphConditionalHandle h) {
-    cudaGraphSetConditional(h, cnt[2] > 0 ? 1u : 0u);
-}
-
-sss_status impl_sort_batch_graph(sss_ctx* ctx, Arena& ar, const StrIn& in, const Seg* d_inst, uint32_t m,
-                                 const sss_params& prm, uint32_t* perm, uint32_t* lcp, uint32_t* dist) {
-    const uint32_t n = in.n;
-    if (n == 0 || m == 0) return SSS_OK;
-    LsBufs B;
-    carve_ls(ar, n, 1, prm, B);
-    const LsKnobs kn = ls_knobs(prm);
-    SSS_TRY(set_ls_attributes(ctx));
-    const SegLists L{B.tiny, B.med, B.large, B.cnt, B.cap_tiny, B.cap_med, B.cap_large, B.warp, B.cap_warp, B.small,
-                     B.cap_small, kn.warp_cap, kn.cta_cap};
-    const uint32_t limit = 100000u;
-    char keyb[512];
-    std::snprintf(keyb, sizeof(keyb), "batch %p %p %p %u %p %p %p %p %u %p %p %p %u %u %u %u %d", (const void*)in.chars,
-                  (const void*)in.offs, (const void*)in.lens, n, (void*)perm, (void*)lcp, (void*)dist,
-                  (const void*)d_inst, m, (void*)B.K, (void*)B.large, (void*)B.sp.plan, kn.warp_cap, kn.cta_cap,
-                  kn.direct_cap, kn.bucket_target, ctx->sm_count);
-    uint32_t* rounds = reinterpret_cast<uint32_t*>(ctx->d_err) + 1;  // a spare word of the context
-    sss_ctx::LsGraph* slot = nullptr;
-    for (auto& lg : ctx->ls_graphs)
-        if (lg.exec && lg.key == keyb) slot = &lg;
-    if (!slot) {
-        slot = &ctx->ls_graphs[0];  // an empty entry, else the least recently used
-        for (auto& lg : ctx->ls_graphs)
-            if (!lg.exec ? slot->exec != nullptr : (slot->exec && lg.used < slot->used)) slot = &lg;
-        if (slot->exec) cudaGraphExecDestroy(slot->exec);
-        if (slot->graph) cudaGraphDestroy(slot->graph);
-        slot->exec = nullptr;
-        slot->graph = nullptr;
-        slot->key.clear();
-        if (!ctx->cap_stream) SSS_CUDA(cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
-        if (!ctx->cap_stream2) SSS_CUDA(cudaStreamCreateWithFlags(&ctx->cap_stream2, cudaStreamNonBlocking));
-        cudaGraph_t g;
-        SSS_CUDA(cudaGraphCreate(&g, 0));
-        cudaGraphConditionalHandle h;
-        SSS_CUDA(cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault));
-        const uint32_t sm = (uint32_t)std::max(1, ctx->sm_count);
-        cudaStream_t saved = ctx->stream;
-        ctx->capturing = true;
-        sss_status st = SSS_OK;
-        cudaError_t ce = cudaStreamBeginCaptureToGraph(ctx->cap_stream, g, nullptr, nullptr, 0,
-                                                       cudaStreamCaptureModeThreadLocal);
-        if (ce == cudaSuccess) {
-            ctx->stream = ctx->cap_stream;
-            // A: identity order, the instances' segments by size class, their finishers
-            ce = cudaMemsetAsync(rounds, 0, sizeof(uint32_t), ctx->stream);
-            if (ce == cudaSuccess) ce = cudaMemsetAsync(B.cnt, 0, sizeof(uint32_t) * 8, ctx->stream);
-            if (ce == cudaSuccess) ce = cudaMemsetAsync(B.work, 0, sizeof(uint32_t) * 8, ctx->stream);
-            if (ce == cudaSuccess) ce = cudaMemsetAsync(B.fixmark, 0, n, ctx->stream);
-            if (ce == cudaSuccess) {
-                st = sss_launch(ctx, "ls_init", k_init_perm, dim3((n + 255) / 256), dim3(256), 0, perm, lcp, n, 0u);
-                if (st == SSS_OK)
-                    st = sss_launch(ctx, "batch_classify", k_batch_classify, dim3(std::min((m + 255) / 256, sm * 4)),
-                                    dim3(256), 0, d_inst, m, L, ctx->d_err);
-                if (st == SSS_OK) st = run_finishers(ctx, B, B.cnt, 0, 0, 0, 0, 0, in, perm, lcp);
-                if (st == SSS_OK)
-                    st = sss_launch(ctx, "ls_cond", k_ls_cond0, dim3(1), dim3(1), 0, (const uint32_t*)B.cnt, h);
-            }
-            // B: the round loop, a while node after everything captured so far
-            cudaGraphNode_t wnode = nullptr;
-            if (st == SSS_OK && ce == cudaSuccess) {
-                cudaStreamCaptureStatus cs;
-                cudaGraph_t cg;
-                const cudaGraphNode_t* deps = nullptr;
-                size_t ndeps = 0;
-                ce = cudaStreamGetCaptureInfo(ctx->cap_stream, &cs, nullptr, &cg, &deps, nullptr, &ndeps);
-                cudaGraphNodeParams cp{};
-                cp.type = cudaGraphNodeTypeConditional;
-                cp.conditional.handle = h;
-                cp.conditional.type = cudaGraphCondTypeWhile;
-                cp.conditional.size = 1;
-                if (ce == cudaSuccess) ce = cudaGraphAddNode(&wnode, cg, deps, nullptr, ndeps, &cp);
-                if (ce == cudaSuccess)
-                    ce = cudaStreamUpdateCaptureDependencies(ctx->cap_stream, &wnode, nullptr, 1,
-                                                             cudaStreamSetCaptureDependencies);
-                if (ce == cudaSuccess) {
-                    cudaGraph_t body = cp.conditional.phGraph_out[0];
-                    ce = cudaStreamBeginCaptureToGraph(ctx->cap_stream2, body, nullptr, nullptr, 0,
-                                                       cudaStreamCaptureModeThreadLocal);
-                    if (ce == cudaSuccess) {
-                        ctx->stream = ctx->cap_stream2;
-                        st = launch_round(ctx, B, kn, L, in, perm, lcp);
-                        if (st == SSS_OK)
-                            st = sss_launch(ctx, "ls_cond", k_ls_cond, dim3(1), dim3(1), 0, (const uint32_t*)B.cnt,
-                                            rounds, limit, ctx->d_err, h);
-                        cudaGraph_t out = body;
-                        cudaError_t ee = cudaStreamEndCapture(ctx->cap_stream2, &out);
-                        if (ce == cudaSuccess) ce = ee;
-                        ctx->stream = ctx->cap_stream;
-                    }
-                }
-            }
-            // C: LCPs across re-sorted buckets, instance-local order, dist
-            if (st == SSS_OK && ce == cudaSuccess) {
-                st = sss_launch(ctx, "ls_fix_seams", k_fix_seams, dim3(std::min((n + 255) / 256, 4096u)), dim3(256), 0,
-                                (const uint8_t*)B.fixmark, n, in.chars, in.offs, in.lens, (const uint32_t*)perm, lcp);
-                if (st == SSS_OK) st = impl_batch_finish(ctx, d_inst, m, in.lens, perm, lcp, dist);
-            }
-            cudaGraph_t out = g;
-            cudaError_t ee = cudaStreamEndCapture(ctx->cap_stream, &out);
-            if (ce == cudaSuccess) ce = ee;
-        }
-        ctx->capturing = false;
-        ctx->stream = saved;
-        if (st != SSS_OK || ce != cudaSuccess) {
-            cudaGetLastError();
-            cudaGraphDestroy(g);
-            return st != SSS_OK ? st : sss_fail(ctx, SSS_ERR_CUDA, std::string("batch graph: ") + cudaGetErrorString(ce));
-        }
-        cudaGraphExec_t ex;
-        ce = cudaGraphInstantiate(&ex, g, 0);
-        if (ce != cudaSuccess) {
-            cudaGetLastError();
-            cudaGraphDestroy(g);
-            return sss_fail(ctx, SSS_ERR_CUDA, std::string("batch graph instantiate: ") + cudaGetErrorString(ce));
-        }
-        slot->graph = g;
-        slot->exec = ex;
-        slot->key = keyb;
-    }
-    slot->used = ++ctx->ls_clock;
-    return sss_graph_launch(ctx, "batch_graph", slot->exec);
-}
+size_t ls_dev_bytes() { return sizeof(LsDev); }
 
 sss_status impl_finish_segments(sss_ctx* ctx, const Seg* tiny, uint32_t ntiny, const Seg* med, uint32_t nmed,
                                 const StrIn& in, uint32_t* perm, uint32_t* lcp) {
@@ -1366,13 +1271,13 @@ sss_status impl_finish_segments(sss_ctx* ctx, const Seg* tiny, uint32_t ntiny, c
     const uint32_t sm = (uint32_t)std::max(1, ctx->sm_count);
     uint32_t* work = reinterpret_cast<uint32_t*>(ctx->d_err) + 2;  // two spare words of the context
     SSS_CUDA(cudaMemsetAsync(work, 0, sizeof(uint32_t) * 2, ctx->stream));
-    SSS_TRY(sss_launch(ctx, "ls_finish_tiny", k_finish<TINY_T, TINY_CAP>, dim3(std::min(ntiny, sm * 32)), dim3(TINY_T),
-                       finish_smem(TINY_CAP), tiny, (const uint32_t*)nullptr, ntiny, work, in.chars, in.offs, in.lens,
-                       perm, lcp, ctx->d_err));
-    SSS_TRY(sss_launch(ctx, "ls_finish_cta", k_finish2<MED_T, MED_CAP>, dim3(std::min(nmed, sm * 4)), dim3(MED_T),
-                       finish_smem(MED_CAP), med, (const uint32_t*)nullptr, nmed, work + 1, in.chars, in.offs, in.lens,
-                       perm, lcp, ctx->d_err));
-    return SSS_OK;
+    FinIn f{nullptr, LC_TINY, {tiny}, ntiny, {work}, {in.chars}, {in.offs}, {in.lens}, {perm}, {lcp}};
+    SSS_TRY(launch_finisher(ctx, LC_TINY, std::min(ntiny, sm * 32), f));
+    f.cls = LC_MED;
+    f.segs = med;
+    f.count = nmed;
+    f.work = work + 1;
+    return launch_finisher(ctx, LC_MED, std::min(nmed, sm * 4), f);
 }
 
 // Smallest offset and largest end of every partition's strings: blocks of
@@ -1459,34 +1364,36 @@ sss_status impl_suffix_views(sss_ctx* ctx, uint32_t n, uint32_t max_len, uint64_
                       max_len, offs, lens);
 }
 
-// Batched sorts: one CTA per instance turns table positions into
-// instance-local indices and (optionally) computes the instance's dist.
-__global__ void k_batch_finish(const Seg* __restrict__ inst, uint32_t m, const uint32_t* __restrict__ lens,
-                               uint32_t* __restrict__ perm, const uint32_t* __restrict__ lcp,
-                               uint32_t* __restrict__ dist) {
+// Batched sorts: table positions become instance-local indices, and the
+// instance's dist is (optionally) computed.  blockIdx.y splits an instance over
+// several CTAs: with one each, eleven instances of 450k strings in all kept
+// eleven SMs busy for 193 us.
+__global__ void __launch_bounds__(256) k_batch_finish(const Seg* __restrict__ inst, uint32_t m,
+                                                      const uint32_t* __restrict__ lens, uint32_t* __restrict__ perm,
+                                                      const uint32_t* __restrict__ lcp, uint32_t* __restrict__ dist) {
     for (uint32_t k = blockIdx.x; k < m; k += gridDim.x) {
         const Seg s = inst[k];
-        for (uint32_t r = threadIdx.x; r < s.size; r += blockDim.x) {
-            uint32_t q = s.start + r;
-            uint32_t g = perm[q];
+        for (uint32_t r = blockIdx.y * 256 + threadIdx.x; r < s.size; r += gridDim.y * 256) {
+            const uint32_t q = s.start + r;
+            const uint32_t g = perm[q];
             if (dist) {
-                uint32_t left = r > 0 ? lcp[q] : 0;
-                uint32_t right = r + 1 < s.size ? lcp[q + 1] : 0;
-                uint32_t mx = left > right ? left : right;
-                uint64_t d = (uint64_t)mx + 1;
+                const uint32_t left = r > 0 ? lcp[q] : 0;
+                const uint32_t right = r + 1 < s.size ? lcp[q + 1] : 0;
+                const uint64_t d = (uint64_t)(left > right ? left : right) + 1;
                 dist[g] = d < lens[g] ? (uint32_t)d : lens[g];
             }
+            perm[q] = g - s.start;
         }
-        __syncthreads();
-        for (uint32_t r = threadIdx.x; r < s.size; r += blockDim.x) perm[s.start + r] -= s.start;
-        __syncthreads();
     }
 }
 
 sss_status impl_batch_finish(sss_ctx* ctx, const Seg* d_inst, uint32_t m, const uint32_t* lens, uint32_t* perm,
                              const uint32_t* lcp, uint32_t* dist) {
-    return sss_launch(ctx, "batch_finish", k_batch_finish, dim3(std::min<uint32_t>(m, 65535u)), dim3(256), 0, d_inst,
-                      m, lens, perm, lcp, dist);
+    // at least 64 CTAs per SM in all, so that instances of very uneven sizes even out
+    const uint32_t gx = std::min<uint32_t>(m, 65535u);
+    const uint32_t gy = std::max(1u, std::min(65535u, (uint32_t)ctx->sm_count * 64u / gx));
+    return sss_launch(ctx, "batch_finish", k_batch_finish, dim3(gx, gy), dim3(256), 0, d_inst, m, lens, perm, lcp,
+                      dist);
 }
 
 sss_status impl_dist(sss_ctx* ctx, const uint32_t* lens, uint32_t n, const uint32_t* perm, const uint32_t* lcp,

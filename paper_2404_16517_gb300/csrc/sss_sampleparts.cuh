@@ -13,7 +13,9 @@
 // first, whole-segment sorts after), and writes every segment's tiles, bucket
 // count and offsets plus the round's totals (LsPlan).  Every kernel of the round
 // runs on a fixed grid and loops over the counts in LsPlan, so a round needs no
-// host round trip and the whole loop can be captured in a CUDA graph.
+// host round trip.  The kernels take one pointer, the context's LsDev: the
+// call's pointers and sizes are read from device memory, so a captured round
+// loop serves every later call whatever its inputs and work memory are.
 #pragma once
 
 #include <algorithm>
@@ -29,22 +31,13 @@ constexpr int LG_OVS = 16;                 // samples per range bucket
 constexpr int LG_BMAX = 256;               // max range buckets per segment
 constexpr int LG_NBMAX = 2 * LG_BMAX - 1;  // range + equality buckets
 
+struct LgTile;
 struct LgSegInfo {
     Seg seg;            // start, size, depth
     uint32_t tiles;     // number of tiles
-    uint32_t tile0;     // first tile index
     uint32_t nb;        // range buckets B (splitters B-1, buckets 2B-1); 0 for whole-segment sorts
     uint32_t hist_base; // offset into hist (bucket-major: b*tiles + t)
-    uint32_t bst_base;  // offset into bucket starts (2B entries)
-    uint32_t bk_base;   // index of this segment's first bucket in the flat bucket list
-    uint32_t pad[2];
-};
-
-struct LgTile {
-    uint32_t s;      // segment index
-    uint32_t begin;  // absolute first position
-    uint32_t end;    // absolute end position
-    uint32_t t;      // tile index within segment
+    uint32_t pad;
 };
 
 // Totals of one round: segments [0, npart) are partitioned, [npart, ns) sorted
@@ -54,55 +47,147 @@ struct LsPlan {
     uint32_t pad[2];
 };
 
-// Plan a round from the segment list `list` (count cnt[2]); resets the five list
-// counters for the pushes of this round and the eight dynamic work counters.
-// One CTA of 1024 threads.
-__global__ void __launch_bounds__(1024) k_lg_plan(const Seg* __restrict__ list, uint32_t* __restrict__ cnt,
-                                                  uint32_t* __restrict__ work, uint32_t direct_max, uint32_t target, uint32_t cap_segs,
-                                                  uint32_t cap_tiles, uint32_t cap_hist,
-                                                  LgSegInfo* __restrict__ info, LsPlan* __restrict__ plan,
-                                                  unsigned* err) {
-    __shared__ uint32_t sh_warp[32];
-    __shared__ uint32_t s_ns;
-    const uint32_t tid = threadIdx.x;
-    if (tid == 0) {
-        uint32_t c = cnt[2];
-        if (c > cap_segs) {
-            atomicOr(err, ERRBIT_OVERFLOW);
-            c = 0;
+// segment lists by size class: LC_QUAD and LC_WARP share one array (from the
+// bottom and from the top), the others have one each
+enum : uint32_t { LC_QUAD = 0, LC_WARP = 1, LC_TINY = 2, LC_SMALL = 3, LC_MED = 4, LC_LARGE = 5, LC_COUNT = 6 };
+
+// A pointer to global memory that is itself read from memory: the compiler takes
+// a kernel's pointer parameters to be global, but such a one to be anything, and
+// then orders its loads with every shared-memory access around them.  With this
+// and the loads of scatter and sort_emit issued together, the 37.5M-string
+// batch's scatter takes 254 us instead of 513 and its bucket sorts 1.75 ms
+// instead of 1.88.
+template <typename T>
+struct GPtr {
+    T* p;
+    GPtr& operator=(T* q) {
+        p = q;
+        return *this;
+    }
+    __host__ __device__ __forceinline__ operator T*() const {
+#ifdef __CUDA_ARCH__
+        T* q = p;
+        __builtin_assume(__isGlobal(q));
+        return q;
+#else
+        return p;
+#endif
+    }
+};
+
+// One call's pointers and sizes, in device memory while the call runs.
+struct LsArgs {
+    GPtr<const uint8_t> chars;
+    GPtr<const uint64_t> offs;
+    GPtr<const uint32_t> lens;
+    GPtr<uint32_t> perm;
+    GPtr<uint32_t> lcp;
+    GPtr<uint64_t> K;
+    GPtr<uint64_t> tK;
+    GPtr<uint32_t> tV;
+    GPtr<uint32_t> segfmt;
+    GPtr<uint32_t> fixmap;  // one bit per position: LCP to recompute from the final order
+    GPtr<uint64_t> spl;
+    GPtr<uint32_t> hist;
+    GPtr<uint32_t> bst;  // bucket starts, LG_NBMAX + 1 per segment
+    GPtr<uint32_t> rankinfo;
+    GPtr<LgSegInfo> info;
+    GPtr<LgTile> tiles;        // large sorts only (use_tiles)
+    GPtr<uint32_t> tile0;    // first tile of every segment
+    GPtr<uint32_t> bk0;      // first bucket of every segment
+    GPtr<uint32_t> rowdone;  // rows scanned of every segment
+    GPtr<Seg> list[LC_COUNT];  // LC_WARP: the last entry of the shared array, filled downwards
+    uint32_t cap[LC_COUNT];
+    uint32_t warp_max, med_max, direct_max, target;
+    uint32_t cap_tiles, cap_hist, limit, use_tiles;
+    uint32_t q0, q1;  // the positions being sorted
+};
+
+// Device state of the local sort, one per context.
+struct LsDev {
+    LsArgs args;
+    LsPlan plan;
+    uint32_t cnt[8];   // segments per list
+    uint32_t work[8];  // dynamic work counters: [LC_*] finishers, [5] buckets, [6] direct, [7] CTAs done
+    uint32_t rounds;
+};
+
+// Exclusive block scan of three u64 at once (each two packed 32-bit counts):
+// one pass of shuffles and barriers instead of six.  sh: 3 * 32 words.
+__device__ __forceinline__ void block_scan3(uint64_t v[3], uint64_t tot[3], uint64_t* sh) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint64_t x[3] = {v[0], v[1], v[2]};
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const uint64_t y = __shfl_up_sync(SSS_FULL, x[k], o);
+            if (lane >= o) x[k] += y;
         }
-        s_ns = c;
+    }
+    if (lane == 31) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) sh[k * 32 + w] = x[k];
     }
     __syncthreads();
-    const uint32_t ns = s_ns;
-    // partitioned segments first, in list order, then the whole-segment sorts
-    uint32_t local = 0;
-    for (uint32_t s = tid; s < ns; s += 1024) local += list[s].size > direct_max ? 1u : 0u;
-    uint32_t npart;
-    BlockScan<1024>::exclusive_sum(local, sh_warp, &npart);
-    uint32_t cp = 0, cd = 0;
+    if (w < 3) {
+        uint64_t t = sh[w * 32 + lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint64_t y = __shfl_up_sync(SSS_FULL, t, o);
+            if (lane >= o) t += y;
+        }
+        sh[w * 32 + lane] = t;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        tot[k] = sh[k * 32 + 31];
+        v[k] = (w > 0 ? sh[k * 32 + w - 1] : 0ull) + x[k] - v[k];
+    }
+    __syncthreads();
+}
+
+// Plan a round from the large list; resets its counter for the pushes of this
+// round and the round's work counters.  One CTA of 1024 threads.
+__global__ void __launch_bounds__(1024) k_lg_plan(LsDev* __restrict__ S, unsigned* err) {
+    __shared__ uint64_t sh[96];
+    __shared__ uint32_t s_np, s_pt;
+    const LsArgs& A = S->args;
+    const uint32_t tid = threadIdx.x;
+    const uint32_t direct_max = A.direct_max, target = A.target;
+    const Seg* list = A.list[LC_LARGE];
+    uint32_t ns = S->cnt[LC_LARGE];
+    if (ns > A.cap[LC_LARGE]) {
+        if (tid == 0) atomicOr(err, ERRBIT_OVERFLOW);
+        ns = 0;
+    }
+    if (tid == 0) s_np = s_pt = 0;
+    __syncthreads();  // every thread has read the count
+    // the partitioned segments and their tiles come first
+    uint32_t np = 0, pt = 0;
+    for (uint32_t s = tid; s < ns; s += 1024) {
+        const uint32_t size = list[s].size;
+        if (size > direct_max) {
+            ++np;
+            pt += (size + LG_TILE - 1) / LG_TILE;
+        }
+    }
+    np = __reduce_add_sync(SSS_FULL, np);
+    pt = __reduce_add_sync(SSS_FULL, pt);
+    if ((tid & 31) == 0 && np) {
+        atomicAdd(&s_np, np);
+        atomicAdd(&s_pt, pt);
+    }
+    __syncthreads();
+    const uint32_t npart = s_np, ptiles = s_pt;
+    uint64_t carry[3] = {0, 0, 0};  // (partitioned, direct) segments, their tiles, (buckets, histogram words)
     for (uint32_t b0 = 0; b0 < ns; b0 += 1024) {
         const uint32_t s = b0 + tid;
         const bool valid = s < ns;
         Seg sg{};
         if (valid) sg = list[s];
         const bool part = valid && sg.size > direct_max;
-        uint32_t tp, td;
-        uint32_t ep = BlockScan<1024>::exclusive_sum(part ? 1u : 0u, sh_warp, &tp);
-        uint32_t ed = BlockScan<1024>::exclusive_sum(valid && !part ? 1u : 0u, sh_warp, &td);
-        if (valid) info[part ? cp + ep : npart + cd + ed].seg = sg;
-        cp += tp;
-        cd += td;
-    }
-    __syncthreads();
-    // tiles, buckets and offsets in the new order
-    uint32_t ct = 0, ch = 0, cb = 0, cpt = 0;
-    for (uint32_t b0 = 0; b0 < ns; b0 += 1024) {
-        const uint32_t s = b0 + tid;
-        const bool valid = s < ns;
-        Seg sg{};
-        if (valid) sg = info[s].seg;
-        const bool part = valid && s < npart;
         const uint32_t tiles = valid ? (sg.size + LG_TILE - 1) / LG_TILE : 0u;
         uint32_t nb = 0;
         if (part) {
@@ -110,90 +195,105 @@ __global__ void __launch_bounds__(1024) k_lg_plan(const Seg* __restrict__ list, 
             nb = nb < 2u ? 2u : (nb > (uint32_t)LG_BMAX ? (uint32_t)LG_BMAX : nb);
         }
         const uint32_t nbk = part ? 2 * nb - 1 : 0u;
-        uint32_t tt, th, tb, tpt;
-        uint32_t et = BlockScan<1024>::exclusive_sum(tiles, sh_warp, &tt);
-        uint32_t eh = BlockScan<1024>::exclusive_sum(nbk * tiles, sh_warp, &th);
-        uint32_t eb = BlockScan<1024>::exclusive_sum(nbk, sh_warp, &tb);
-        BlockScan<1024>::exclusive_sum(part ? tiles : 0u, sh_warp, &tpt);
+        uint64_t v[3], tot[3];
+        v[0] = part ? 1ull : (valid ? 1ull << 32 : 0ull);
+        v[1] = part ? (uint64_t)tiles : (uint64_t)tiles << 32;
+        v[2] = (uint64_t)nbk | ((uint64_t)nbk * tiles << 32);
+        block_scan3(v, tot, sh);
         if (valid) {
-            LgSegInfo si{};
-            si.seg = sg;
-            si.tiles = tiles;
-            si.tile0 = ct + et;
-            si.nb = nb;
-            si.hist_base = ch + eh;
-            si.bst_base = s * (LG_NBMAX + 1);
-            si.bk_base = cb + eb;
-            info[s] = si;
+            const uint32_t at = part ? (uint32_t)(carry[0] + v[0])
+                                     : npart + (uint32_t)((carry[0] + v[0]) >> 32);
+            A.info[at] = LgSegInfo{sg, tiles, nb, (uint32_t)((carry[2] + v[2]) >> 32), 0};
+            A.tile0[at] = part ? (uint32_t)(carry[1] + v[1]) : ptiles + (uint32_t)((carry[1] + v[1]) >> 32);
+            A.bk0[at] = (uint32_t)(carry[2] + v[2]);
+            A.rowdone[at] = 0;
         }
-        ct += tt;
-        ch += th;
-        cb += tb;
-        cpt += tpt;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) carry[k] += tot[k];
     }
     if (tid == 0) {
-        LsPlan pl{ns, npart, ct, cpt, cb, ch, {0, 0}};
-        if (ct > cap_tiles || ch > cap_hist) {
+        const uint32_t nt = ptiles + (uint32_t)(carry[1] >> 32), nh = (uint32_t)(carry[2] >> 32);
+        LsPlan pl{ns, npart, nt, ptiles, (uint32_t)carry[2], nh, {0, 0}};
+        if (nt > A.cap_tiles || nh > A.cap_hist) {
             atomicOr(err, ERRBIT_OVERFLOW);
             pl = LsPlan{0, 0, 0, 0, 0, 0, {0, 0}};
         }
-        *plan = pl;
-        cnt[0] = cnt[1] = cnt[2] = cnt[3] = cnt[4] = cnt[5] = 0;
-        for (int k = 0; k < 8; ++k) work[k] = 0;
+        S->plan = pl;
+        S->cnt[LC_LARGE] = 0;
+        S->work[5] = S->work[6] = S->work[7] = 0;
     }
 }
 
-// segment of flat index g among n segments with nondecreasing field f: last
-// segment with f <= g
-__device__ __forceinline__ uint32_t segment_of_tile(const LgSegInfo* info, uint32_t ns, uint32_t g) {
-    uint32_t a = 0, c = ns;
-    while (a + 1 < c) {
-        uint32_t mid = (a + c) >> 1;
-        if (info[mid].tile0 <= g) a = mid; else c = mid;
+// Last index i < n with f[i] <= g (f non-decreasing, f[0] <= g), found by the
+// whole warp: 32 probes per step.
+__device__ __forceinline__ uint32_t warp_last_le(const uint32_t* __restrict__ f, uint32_t n, uint32_t g) {
+    const uint32_t lane = threadIdx.x & 31;
+    uint32_t lo = 0, len = n;
+    while (len > 32) {
+        const uint32_t stride = (len + 31) / 32;
+        const uint32_t at = lane * stride;
+        const uint32_t k = (uint32_t)__popc(__ballot_sync(SSS_FULL, at < len && f[lo + at] <= g));
+        const uint32_t skip = k ? (k - 1) * stride : 0u;
+        lo += skip;
+        len = len - skip < stride ? len - skip : stride;
     }
-    return a;
+    const uint32_t k = (uint32_t)__popc(__ballot_sync(SSS_FULL, lane < len && f[lo + lane] <= g));
+    return lo + (k ? k - 1 : 0u);
 }
 
-__device__ __forceinline__ uint32_t segment_of_bucket(const LgSegInfo* info, uint32_t ns, uint32_t g) {
-    uint32_t a = 0, c = ns;
-    while (a + 1 < c) {
-        uint32_t mid = (a + c) >> 1;
-        if (info[mid].bk_base <= g) a = mid; else c = mid;
-    }
-    return a;
+// Tile g of the round: its segment and positions.  Rounds of large sorts may
+// hold thousands of segments: there the tiles are listed by a kernel of their
+// own (a lookup per tile, up to four dependent loads in three kernels, cost the
+// 37.5M-string batch 0.4 ms); smaller rounds look the segment up and save the
+// launch (3 us).
+struct LgTile {
+    uint32_t s, begin, end, t;  // segment, positions [begin, end), index within the segment
+};
+__device__ __forceinline__ LgTile lg_find_tile(const LsArgs& A, uint32_t s, uint32_t g) {
+    const Seg sg = A.info[s].seg;
+    LgTile tl;
+    tl.s = s;
+    tl.t = g - A.tile0[s];
+    tl.begin = sg.start + tl.t * LG_TILE;
+    const uint32_t e = sg.start + sg.size;
+    tl.end = e - tl.begin < (uint32_t)LG_TILE ? e : tl.begin + LG_TILE;
+    return tl;
+}
+__device__ __forceinline__ LgTile lg_tile(const LsArgs& A, uint32_t ns, uint32_t g) {
+    return A.use_tiles ? A.tiles[g] : lg_find_tile(A, warp_last_le(A.tile0, ns, g), g);
 }
 
-__global__ void k_lg_tiles(const LsPlan* __restrict__ plan, const LgSegInfo* __restrict__ info,
-                           LgTile* __restrict__ tiles) {
-    const uint32_t nt = plan->ntiles, ns = plan->ns;
-    for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < nt; g += gridDim.x * blockDim.x) {
-        const uint32_t s = segment_of_tile(info, ns, g);
-        const LgSegInfo si = info[s];
-        const uint32_t t = g - si.tile0;
-        const uint32_t b0 = si.seg.start + t * LG_TILE;
-        const uint32_t e = si.seg.start + si.seg.size;
-        tiles[g] = LgTile{s, b0, b0 + (uint32_t)LG_TILE < e ? b0 + (uint32_t)LG_TILE : e, t};
+__global__ void __launch_bounds__(256) k_lg_tiles(const LsDev* __restrict__ S) {
+    const LsArgs& A = S->args;
+    const uint32_t nt = S->plan.ntiles, ns = S->plan.ns;
+    for (uint32_t g = blockIdx.x * 256 + threadIdx.x; g < nt; g += gridDim.x * 256) {
+        uint32_t a = 0, c = ns;
+        while (a + 1 < c) {
+            const uint32_t mid = (a + c) >> 1;
+            if (A.tile0[mid] <= g) a = mid;
+            else c = mid;
+        }
+        A.tiles[g] = lg_find_tile(A, a, g);
     }
 }
 
 // Per partitioned segment: evenly spaced samples, sorted; splitter b = sample (b+1)*OVS-1.
-__global__ void __launch_bounds__(512) k_lg_samples(const LsPlan* __restrict__ plan,
-                                                    const LgSegInfo* __restrict__ info, const uint64_t* __restrict__ K,
-                                                    uint64_t* __restrict__ spl) {
+__global__ void __launch_bounds__(512) k_lg_samples(const LsDev* __restrict__ S) {
     __shared__ uint64_t sh[LG_BMAX * LG_OVS];
-    const uint32_t npart = plan->npart;
+    const LsArgs& A = S->args;
+    const uint32_t npart = S->plan.npart;
     for (uint32_t s = blockIdx.x; s < npart; s += gridDim.x) {
         __syncthreads();
-        LgSegInfo si = info[s];
-        uint32_t S = si.nb * LG_OVS;
-        for (uint32_t i = threadIdx.x; i < S; i += 512) {
-            uint64_t q = si.seg.start + ((2 * (uint64_t)i + 1) * si.seg.size) / (2 * (uint64_t)S);
-            sh[i] = K[q];
+        const LgSegInfo si = A.info[s];
+        const uint32_t n = si.nb * LG_OVS;
+        for (uint32_t i = threadIdx.x; i < n; i += 512) {
+            uint64_t q = si.seg.start + ((2 * (uint64_t)i + 1) * si.seg.size) / (2 * (uint64_t)n);
+            sh[i] = A.K[q];
         }
         __syncthreads();
-        bitonic_sort64<512>(sh, S);
+        bitonic_sort64<512>(sh, n);
         for (uint32_t b = threadIdx.x; b + 1 < si.nb; b += 512)
-            spl[(size_t)s * (LG_BMAX - 1) + b] = sh[(b + 1) * LG_OVS - 1];
+            A.spl[(size_t)s * (LG_BMAX - 1) + b] = sh[(b + 1) * LG_OVS - 1];
     }
 }
 
@@ -207,22 +307,22 @@ __device__ __forceinline__ uint32_t lower_bound64(const uint64_t* s, uint32_t ns
     return lo;
 }
 
-__global__ void __launch_bounds__(LG_T) k_lg_classify(const LsPlan* __restrict__ plan,
-                                                      const LgTile* __restrict__ tiles,
-                                                      const LgSegInfo* __restrict__ info,
-                                                      const uint64_t* __restrict__ K, const uint64_t* __restrict__ spl,
-                                                      uint32_t* __restrict__ hist, uint32_t* __restrict__ rankinfo) {
+__global__ void __launch_bounds__(LG_T) k_lg_classify(const LsDev* __restrict__ S) {
     constexpr int W = LG_T / 32;
     constexpr int PER_WARP = LG_TILE / W;  // contiguous positions per warp
     __shared__ uint64_t ssp[LG_BMAX];
     __shared__ uint32_t cnt[W][LG_NBMAX];
-    const uint32_t ptiles = plan->ptiles;
+    const LsArgs& A = S->args;
+    const uint64_t* __restrict__ K = A.K;
+    uint32_t* __restrict__ hist = A.hist;
+    uint32_t* __restrict__ rankinfo = A.rankinfo;
+    const uint32_t ptiles = S->plan.ptiles, npart = S->plan.npart;
     for (uint32_t g = blockIdx.x; g < ptiles; g += gridDim.x) {
         __syncthreads();
-        LgTile tl = tiles[g];
-        LgSegInfo si = info[tl.s];
+        const LgTile tl = lg_tile(A, npart, g);
+        const LgSegInfo si = A.info[tl.s];
         uint32_t nsp = si.nb - 1, nbk = 2 * si.nb - 1;
-        for (uint32_t i = threadIdx.x; i < nsp; i += LG_T) ssp[i] = spl[(size_t)tl.s * (LG_BMAX - 1) + i];
+        for (uint32_t i = threadIdx.x; i < nsp; i += LG_T) ssp[i] = A.spl[(size_t)tl.s * (LG_BMAX - 1) + i];
         for (uint32_t i = threadIdx.x; i < (uint32_t)(W * LG_NBMAX); i += LG_T) (&cnt[0][0])[i] = 0;
         __syncthreads();
         int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -272,18 +372,19 @@ __global__ void __launch_bounds__(LG_T) k_lg_classify(const LsPlan* __restrict__
 
 // Exclusive prefix of every bucket's row of tile counts (one warp per row, the
 // row contiguous, so loads coalesce); the row total goes to the bucket's start
-// slot, turned into the start by k_lg_offsets.
-__global__ void __launch_bounds__(256) k_lg_rowscan(const LsPlan* __restrict__ plan,
-                                                    const LgSegInfo* __restrict__ info, uint32_t* __restrict__ hist,
-                                                    uint32_t* __restrict__ bst) {
-    const uint32_t nrows = plan->pbuckets, npart = plan->npart;
+// slot.  The warp that finishes a segment's last row turns its totals into
+// bucket starts (a separate launch for that cost 3 us and its gap per round).
+__global__ void __launch_bounds__(256) k_lg_rowscan(const LsDev* __restrict__ S) {
+    const LsArgs& A = S->args;
+    const uint32_t nrows = S->plan.pbuckets, npart = S->plan.npart;
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t warps = gridDim.x * (blockDim.x >> 5);
     for (uint32_t r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < nrows; r += warps) {
-        const uint32_t s = segment_of_bucket(info, npart, r);
-        const LgSegInfo si = info[s];
-        const uint32_t b = r - si.bk_base;
-        uint32_t* h = hist + si.hist_base + b * si.tiles;
+        const uint32_t s = warp_last_le(A.bk0, npart, r);
+        const LgSegInfo si = A.info[s];
+        const uint32_t b = r - A.bk0[s], nbk = 2 * si.nb - 1;
+        uint32_t* h = A.hist + si.hist_base + b * si.tiles;
+        uint32_t* bst = A.bst + (size_t)s * (LG_NBMAX + 1);
         uint32_t carry = 0;
         for (uint32_t t0 = 0; t0 < si.tiles; t0 += 32) {
             const uint32_t t = t0 + lane;
@@ -297,24 +398,29 @@ __global__ void __launch_bounds__(256) k_lg_rowscan(const LsPlan* __restrict__ p
             if (t < si.tiles) h[t] = carry + x - v;
             carry += __shfl_sync(SSS_FULL, x, 31);
         }
-        if (lane == 0) bst[si.bst_base + b] = carry;
-    }
-}
-
-// Per partitioned segment: bucket starts from the row totals.
-__global__ void __launch_bounds__(512) k_lg_offsets(const LsPlan* __restrict__ plan,
-                                                    const LgSegInfo* __restrict__ info, uint32_t* __restrict__ bst) {
-    __shared__ uint32_t sh_warp[32];
-    const uint32_t npart = plan->npart;
-    for (uint32_t s = blockIdx.x; s < npart; s += gridDim.x) {
-        LgSegInfo si = info[s];
-        uint32_t nbk = 2 * si.nb - 1;
-        uint32_t b = threadIdx.x;
-        uint32_t tot = b < nbk ? bst[si.bst_base + b] : 0u;
-        uint32_t total;
-        uint32_t ex = BlockScan<512>::exclusive_sum(tot, sh_warp, &total);
-        if (b < nbk) bst[si.bst_base + b] = si.seg.start + ex;
-        if (b == 0) bst[si.bst_base + nbk] = si.seg.start + si.seg.size;
+        uint32_t done = 0;
+        if (lane == 0) {
+            __stcg(&bst[b], carry);
+            __threadfence();
+            done = atomicAdd(&A.rowdone[s], 1u) + 1u;
+        }
+        done = __shfl_sync(SSS_FULL, done, 0);
+        if (done != nbk) continue;
+        __threadfence();
+        uint32_t run = si.seg.start;
+        for (uint32_t b0 = 0; b0 < nbk; b0 += 32) {
+            const uint32_t i = b0 + lane;
+            const uint32_t v = i < nbk ? __ldcg(&bst[i]) : 0u;
+            uint32_t x = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                uint32_t y = __shfl_up_sync(SSS_FULL, x, o);
+                if (lane >= (uint32_t)o) x += y;
+            }
+            if (i < nbk) bst[i] = run + x - v;
+            run += __shfl_sync(SSS_FULL, x, 31);
+        }
+        if (lane == 0) bst[nbk] = si.seg.start + si.seg.size;
     }
 }
 
@@ -324,34 +430,48 @@ __global__ void __launch_bounds__(512) k_lg_offsets(const LsPlan* __restrict__ p
 // one bucket's range.  Written directly, the keys of a warp land in as many
 // buckets as they have, and every 8-byte key or 4-byte index costs a whole
 // sector of DRAM writes.
-__global__ void __launch_bounds__(LG_T) k_lg_scatter(const LsPlan* __restrict__ plan,
-                                                     const LgTile* __restrict__ tiles, const LgSegInfo* __restrict__ info,
-                                                     const uint32_t* __restrict__ hist, const uint32_t* __restrict__ bst,
-                                                     const uint32_t* __restrict__ rankinfo,
-                                                     const uint64_t* __restrict__ K, const uint32_t* __restrict__ perm,
-                                                     uint64_t* __restrict__ tK, uint32_t* __restrict__ tV,
-                                                     unsigned* err) {
+__global__ void __launch_bounds__(LG_T) k_lg_scatter(const LsDev* __restrict__ S, unsigned* err) {
     constexpr int PER = LG_TILE / LG_T;
     static_assert(2 * LG_T >= LG_NBMAX, "two buckets per thread in the scan");
     __shared__ uint32_t cnt[2 * LG_T];
     __shared__ uint32_t sh_warp[32];
     __shared__ uint64_t sK[LG_TILE];
     __shared__ uint32_t sV[LG_TILE], sD[LG_TILE];
+    const LsArgs& A = S->args;
+    const uint32_t* __restrict__ hist = A.hist;
+    const uint32_t* __restrict__ rankinfo = A.rankinfo;
+    const uint64_t* __restrict__ K = A.K;
+    const uint32_t* __restrict__ perm = A.perm;
+    uint64_t* __restrict__ tK = A.tK;
+    uint32_t* __restrict__ tV = A.tV;
     const uint32_t tid = threadIdx.x;
-    const uint32_t ptiles = plan->ptiles;
+    const uint32_t ptiles = S->plan.ptiles, npart = S->plan.npart;
     for (uint32_t g = blockIdx.x; g < ptiles; g += gridDim.x) {
-        const LgTile tl = tiles[g];
-        const LgSegInfo si = info[tl.s];
+        const LgTile tl = lg_tile(A, npart, g);
+        const LgSegInfo si = A.info[tl.s];
+        const uint32_t* __restrict__ bst = A.bst + (size_t)tl.s * (LG_NBMAX + 1);
         const uint32_t nbk = 2 * si.nb - 1;
         __syncthreads();  // the previous tile's keys have left shared memory
         for (uint32_t i = tid; i < 2u * LG_T; i += LG_T) cnt[i] = 0;
         __syncthreads();
-        uint32_t ri[PER];
+        // everything the tile reads, in flight before the first use
+        uint32_t ri[PER], rv[PER];
+        uint64_t rk[PER];
 #pragma unroll
         for (int u = 0; u < PER; ++u) {
             const uint32_t q = tl.begin + tid + u * LG_T;
-            ri[u] = q < tl.end ? rankinfo[q] : 0xFFFFFFFFu;
-            if (q < tl.end) atomicAdd(&cnt[min(ri[u] >> 16, 2u * LG_T - 1u)], 1u);  // b < nbk <= 511
+            ri[u] = q < tl.end ? __ldg(rankinfo + q) : 0xFFFFFFFFu;
+            rk[u] = q < tl.end ? __ldg(K + q) : 0ull;
+            rv[u] = q < tl.end ? __ldg(perm + q) : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < PER; ++u)
+            if (ri[u] != 0xFFFFFFFFu) atomicAdd(&cnt[min(ri[u] >> 16, 2u * LG_T - 1u)], 1u);  // b < nbk <= 511
+        uint32_t first[PER];  // the tile's first position in the key's bucket
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const uint32_t b = min(ri[u] >> 16, nbk - 1);
+            first[u] = ri[u] != 0xFFFFFFFFu ? __ldg(bst + b) + __ldg(hist + si.hist_base + b * si.tiles + tl.t) : 0u;
         }
         __syncthreads();
         // the tile's bucket offsets: exclusive scan of the counts
@@ -362,18 +482,17 @@ __global__ void __launch_bounds__(LG_T) k_lg_scatter(const LsPlan* __restrict__ 
         __syncthreads();
 #pragma unroll
         for (int u = 0; u < PER; ++u) {
-            const uint32_t q = tl.begin + tid + u * LG_T;
-            if (q >= tl.end) continue;
+            if (ri[u] == 0xFFFFFFFFu) continue;
             const uint32_t b = ri[u] >> 16, r = ri[u] & 0xFFFFu;
             const uint32_t slot = cnt[min(b, 2u * LG_T - 1u)] + r;
-            uint32_t dst = bst[si.bst_base + b] + hist[si.hist_base + b * si.tiles + tl.t] + r;
+            uint32_t dst = first[u] + r;
             if (b >= nbk || dst < si.seg.start || dst >= si.seg.start + si.seg.size || slot >= LG_TILE) {
                 atomicOr(err, ERRBIT_OVERFLOW);
                 if (slot >= LG_TILE) continue;
                 dst = 0xFFFFFFFFu;
             }
-            sK[slot] = K[q];
-            sV[slot] = perm[q];
+            sK[slot] = rk[u];
+            sV[slot] = rv[u];
             sD[slot] = dst;
         }
         __syncthreads();
@@ -388,48 +507,18 @@ __global__ void __launch_bounds__(LG_T) k_lg_scatter(const LsPlan* __restrict__ 
 }
 
 // Work memory of the partition for up to `cap_segs` segments covering <= n positions.
-struct SpBufs {
-    uint64_t* spl;
-    uint32_t* hist;
-    uint32_t* bst;
-    uint32_t* rankinfo;
-    LgSegInfo* info;
-    LgTile* tiles;
-    LsPlan* plan;
-    uint32_t cap_segs, cap_tiles, cap_hist;
-};
-
-inline void carve_sp(Arena& ar, uint32_t n, uint32_t cap_segs, SpBufs& b) {
-    b.cap_segs = cap_segs;
-    b.cap_tiles = n / LG_TILE + cap_segs + 2;
-    b.cap_hist = LG_NBMAX * b.cap_tiles;
-    b.spl = ar.take<uint64_t>((size_t)cap_segs * (LG_BMAX - 1));
-    b.hist = ar.take<uint32_t>(b.cap_hist);
-    b.bst = ar.take<uint32_t>((size_t)cap_segs * (LG_NBMAX + 1));
-    b.rankinfo = ar.take<uint32_t>(n);
-    b.info = ar.take<LgSegInfo>(cap_segs);
-    b.tiles = ar.take<LgTile>(b.cap_tiles);
-    b.plan = ar.take<LsPlan>(1);
-}
-
-// The partition of the planned round's partitioned segments (fixed grids).
-inline sss_status launch_sp(sss_ctx* ctx, const SpBufs& B, const uint64_t* K, const uint32_t* V, uint64_t* tK,
-                            uint32_t* tV, const char* tag_samples, const char* tag_classify, const char* tag_offsets,
-                            const char* tag_scatter) {
-    const uint32_t sm = (uint32_t)std::max(1, ctx->sm_count);
-    SSS_TRY(sss_launch(ctx, tag_samples, k_lg_samples, dim3(sm * 2), dim3(512), 0, (const LsPlan*)B.plan,
-                       (const LgSegInfo*)B.info, K, B.spl));
-    SSS_TRY(sss_launch(ctx, tag_classify, k_lg_classify, dim3(sm * 6), dim3(LG_T), 0, (const LsPlan*)B.plan,
-                       (const LgTile*)B.tiles, (const LgSegInfo*)B.info, K, (const uint64_t*)B.spl, B.hist,
-                       B.rankinfo));
-    SSS_TRY(sss_launch(ctx, tag_offsets, k_lg_rowscan, dim3(sm * 4), dim3(256), 0, (const LsPlan*)B.plan,
-                       (const LgSegInfo*)B.info, B.hist, B.bst));
-    SSS_TRY(sss_launch(ctx, tag_offsets, k_lg_offsets, dim3(sm * 2), dim3(512), 0, (const LsPlan*)B.plan,
-                       (const LgSegInfo*)B.info, B.bst));
-    SSS_TRY(sss_launch(ctx, tag_scatter, k_lg_scatter, dim3(sm * 8), dim3(LG_T), 0, (const LsPlan*)B.plan,
-                       (const LgTile*)B.tiles, (const LgSegInfo*)B.info, (const uint32_t*)B.hist,
-                       (const uint32_t*)B.bst, (const uint32_t*)B.rankinfo, K, V, tK, tV, ctx->d_err));
-    return SSS_OK;
+inline void carve_sp(Arena& ar, uint32_t n, uint32_t cap_segs, LsArgs& a) {
+    a.cap_tiles = n / LG_TILE + cap_segs + 2;
+    a.cap_hist = LG_NBMAX * a.cap_tiles;
+    a.spl = ar.take<uint64_t>((size_t)cap_segs * (LG_BMAX - 1));
+    a.hist = ar.take<uint32_t>(a.cap_hist);
+    a.bst = ar.take<uint32_t>((size_t)cap_segs * (LG_NBMAX + 1));
+    a.rankinfo = ar.take<uint32_t>(n);
+    a.info = ar.take<LgSegInfo>(cap_segs);
+    a.tiles = ar.take<LgTile>(a.cap_tiles);
+    a.tile0 = ar.take<uint32_t>(cap_segs);
+    a.bk0 = ar.take<uint32_t>(cap_segs);
+    a.rowdone = ar.take<uint32_t>(cap_segs);
 }
 
 }  // namespace
