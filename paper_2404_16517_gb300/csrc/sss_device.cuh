@@ -946,3 +946,282 @@ __device__ void block_merge_sort128_fit(uint64_t* sHi, uint64_t* sLo, uint32_t c
     }
     block_merge_sort128<THREADS, ITEMS>(sHi, sLo, count);
 }
+
+// ---------------------------------------------------------------------------
+// Block sort of reference-split keys by bucket and rank.
+//
+// The bits of a segment's keys that vary are few and, packed together, nearly
+// dense: the heads (side, v) span a short range on each side of the reference,
+// and the characters use a handful of bits per byte (5 for A-Z).  The key's head
+// counted from the smallest one of its side, followed by the varying character
+// bits, is an order-preserving number whose top bits spread the keys over about
+// two buckets per key.  Where that leaves them in clusters (skewed characters,
+// a dominant head), the next bits split every bucket again into as many as it
+// holds keys.  A key's rank inside its bucket is counted against the bucket's
+// other members (a handful) by the next 32 varying bits, which are mostly all
+// that is left, and its slot.  That needs keys that spread: the caller keeps the
+// merge sort (1,300 instructions a key) for those that do not (many equal keys).
+//
+// sK/sV: the keys and indices, each thread having written the slots
+// threadIdx.x + t * THREADS below m <= THREADS * ITEMS (no barrier needed); f:
+// the segment's key format.  They stay where they are: returns true with the
+// slots in (key, index) order in sP[0, m), after a barrier; false when a key
+// would be compared with more than BUCKET_MOST others on average.  sC: NB 16-bit
+// counters; sR: m words of 64 bits, sP: m of 16.
+constexpr uint32_t BUCKET_GOOD = 12;  // average comparisons per key that end the splitting
+constexpr uint32_t BUCKET_MOST = 48;
+
+template <int THREADS, int ITEMS, int NB>
+__device__ __forceinline__ bool block_bucket_sort(const uint64_t* sK, const uint32_t* sV, uint16_t* sC, uint64_t* sR,
+                                                  uint16_t* sP, uint32_t m, uint32_t f) {
+    constexpr int WARPS = THREADS / 32, PER = NB / 2 / THREADS;  // PER words of two counters a thread
+    static_assert(WARPS >= 8, "one warp per reduced quantity");
+    static_assert(NB <= 8192 && THREADS * ITEMS <= NB && (NB & (NB - 1)) == 0, "bucket number and slot share a word");
+    static_assert(PER >= 1, "a word of counters per thread");
+    __shared__ uint32_t s_red[8][32];
+    __shared__ uint32_t s_warp[32];
+    __shared__ uint32_t s_sq;
+    uint32_t* sW = reinterpret_cast<uint32_t*>(sC);
+    const uint32_t tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const uint32_t vb = f & 31u;
+    const uint32_t vcap = (1u << vb) - 1u;
+    // smallest and largest head of side 0 and of side 2 (side 1 has one head),
+    // and the character bits that vary (a key without characters, its string
+    // ended, sorts below the others with its bits all 0: it need not count)
+    uint32_t b[ITEMS], cw[ITEMS];  // the head (side, vk), then the bucket; the character bits at hand
+    uint32_t q[8] = {~0u, 0u, ~0u, 0u, 0u, 0u, ~0u, ~0u};
+#pragma unroll
+    for (int t = 0; t < ITEMS; ++t) {
+        b[t] = cw[t] = 0;
+        if (tid + t * THREADS >= m) continue;
+        const uint64_t k = sK[tid + t * THREADS];
+        const uint64_t ch = k << (2 + vb);
+        b[t] = (uint32_t)(k >> (62 - vb));
+        cw[t] = (uint32_t)(ch >> 32);
+        const uint32_t side = b[t] >> vb, vk = b[t] & vcap;
+        if (side == 0) {
+            q[0] = min(q[0], vk);
+            q[1] = max(q[1], vk);
+        } else if (side == 2) {
+            q[2] = min(q[2], vk);
+            q[3] = max(q[3], vk);
+        }
+        if (ch) {
+            q[4] |= cw[t];
+            q[5] |= (uint32_t)ch;
+            q[6] &= cw[t];
+            q[7] &= (uint32_t)ch;
+        } else if (side != 1) {
+            q[5] |= 1u;  // (no character bit: the low 2 + vb bits of ch are 0)
+        }
+    }
+    q[0] = __reduce_min_sync(SSS_FULL, q[0]);
+    q[1] = __reduce_max_sync(SSS_FULL, q[1]);
+    q[2] = __reduce_min_sync(SSS_FULL, q[2]);
+    q[3] = __reduce_max_sync(SSS_FULL, q[3]);
+    q[4] = __reduce_or_sync(SSS_FULL, q[4]);
+    q[5] = __reduce_or_sync(SSS_FULL, q[5]);
+    q[6] = __reduce_and_sync(SSS_FULL, q[6]);
+    q[7] = __reduce_and_sync(SSS_FULL, q[7]);
+    if (lane == 0) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s_red[i][w] = q[i];
+    }
+    for (uint32_t i = tid; i < (uint32_t)NB / 2; i += THREADS) sW[i] = 0;
+    if (tid == 0) s_sq = 0;
+    __syncthreads();
+    if (w < 8) {
+        uint32_t x = s_red[w][lane < (uint32_t)WARPS ? lane : 0u];
+        x = (w == 0 || w == 2) ? __reduce_min_sync(SSS_FULL, x)
+            : w < 4            ? __reduce_max_sync(SSS_FULL, x)
+            : w < 6            ? __reduce_or_sync(SSS_FULL, x)
+                               : __reduce_and_sync(SSS_FULL, x);
+        if (lane == 0) s_red[w][0] = x;
+    }
+    // slots in index order (as every caller's are; checked): then equal keys go by slot
+    bool ordered = true;
+    for (uint32_t j = tid + 1; j < m; j += THREADS) ordered = ordered && sV[j - 1] < sV[j];
+    ordered = __syncthreads_and(ordered) != 0;
+    const uint32_t min0 = s_red[0][0], min2 = s_red[2][0];
+    const uint32_t r0 = s_red[1][0] >= min0 ? s_red[1][0] - min0 + 1 : 0u;
+    const uint32_t r2 = s_red[3][0] >= min2 ? s_red[3][0] - min2 + 1 : 0u;
+    const uint32_t hb = 32u - (uint32_t)__clz((int)(r0 + r2));  // bits of the heads 0 .. r0 + r2
+    uint32_t B = 1;  // about two buckets per key
+    while ((1u << B) < 2u * m && (1u << B) < (uint32_t)NB) ++B;
+    // the top B bits of (head, varying character bits)
+#pragma unroll
+    for (int t = 0; t < ITEMS; ++t) {
+        if ((uint32_t)(t * THREADS) >= m) break;
+        const uint32_t side = b[t] >> vb, vk = b[t] & vcap;
+        const uint32_t h = side == 0 ? vk - min0 : (side == 1 ? r0 : r0 + 1u + vk - min2);
+        b[t] = hb > B ? h >> (hb - B) : h;
+    }
+    // the varying bits of cw not used yet, and of the low word when it is next
+    uint32_t vw = s_red[4][0] & ~s_red[6][0], vlo = s_red[5][0] & ~s_red[7][0] & ~1u;
+    // shift up to `need` (<= 32) of them into dst
+    const auto shift_in = [&](uint32_t (&dst)[ITEMS], uint32_t need) {
+        uint32_t got = 0;
+        while (got < need) {
+            if (vw == 0) {
+                if (vlo == 0) break;
+                vw = vlo;
+                vlo = 0;
+#pragma unroll
+                for (int t = 0; t < ITEMS; ++t)
+                    if (tid + t * THREADS < m) cw[t] = (uint32_t)(sK[tid + t * THREADS] << (2 + vb));
+            }
+            const uint32_t lead = (uint32_t)__clz((int)vw);
+            const uint32_t run = (uint32_t)__clz((int)~(vw << lead));  // a run of varying bits
+            const uint32_t take = run < need - got ? run : need - got;
+#pragma unroll
+            for (int t = 0; t < ITEMS; ++t) {
+                if ((uint32_t)(t * THREADS) >= m) break;  // (uniform: a short segment's idle items cost nothing)
+                dst[t] = (take < 32u ? dst[t] << take : 0u) | ((cw[t] << lead) >> (32 - take));
+            }
+            got += take;
+            vw &= lead + take < 32u ? ~0u >> (lead + take) : 0u;
+        }
+        return got;
+    };
+    if (hb < B) shift_in(b, B - hb);
+    // the bits that decide inside a bucket, left-aligned: the next varying ones,
+    // or the top of the key where a bucket may hold several heads
+    uint32_t res[ITEMS], avail = 0;
+#pragma unroll
+    for (int t = 0; t < ITEMS; ++t) res[t] = 0;
+    if (hb > B) {
+#pragma unroll
+        for (int t = 0; t < ITEMS; ++t)
+            if (tid + t * THREADS < m) res[t] = (uint32_t)(sK[tid + t * THREADS] >> 32);
+    } else {
+        avail = shift_in(res, 32);
+#pragma unroll
+        for (int t = 0; t < ITEMS; ++t) res[t] = avail ? res[t] << (32 - avail) : 0u;
+    }
+    // equal there and in the bucket means equal keys
+    const bool whole = hb <= B && (vw | vlo) == 0 && (s_red[5][0] & 1u) == 0;
+    // Within a bucket the next bits y are scaled to its size c: slot (y * c) >> bits.
+    // The slot holds a range of y; what orders its keys first is the remainder of
+    // y * c, which the following level takes in front of its own bits (10, then 9
+    // more: with c <= 2^13 the product fits 32 bits).
+    uint32_t rem[ITEMS], used = 0;
+#pragma unroll
+    for (int t = 0; t < ITEMS; ++t) rem[t] = 0;
+    uint32_t sq = 0;
+    for (uint32_t level = 0;; ++level) {
+        // count the buckets, scan the counts
+#pragma unroll
+        for (int t = 0; t < ITEMS; ++t) {
+            if ((uint32_t)(t * THREADS) >= m) break;
+            if (tid + t * THREADS >= m) continue;
+            const uint32_t sh = (b[t] & 1u) * 16u;
+            b[t] |= atomicAdd(&sW[b[t] >> 1], 1u << sh) >> sh << 16;  // the key's place in its bucket
+        }
+        __syncthreads();
+        uint32_t sum = 0, mysq = 0;
+#pragma unroll
+        for (int t = 0; t < PER; ++t) {
+            const uint32_t x = sW[tid * PER + t], c0 = x & 0xFFFFu, c1 = x >> 16;
+            mysq += c0 * c0 + c1 * c1;
+            sum += c0 + c1;
+        }
+        mysq = __reduce_add_sync(SSS_FULL, mysq);
+        if (lane == 0) atomicAdd(&s_sq, mysq);
+        uint32_t at = BlockScan<THREADS>::exclusive_sum(sum, s_warp, nullptr);
+#pragma unroll
+        for (int t = 0; t < PER; ++t) {
+            const uint32_t x = sW[tid * PER + t], mid = at + (x & 0xFFFFu);
+            sW[tid * PER + t] = at | mid << 16;
+            at = mid + (x >> 16);
+        }
+        __syncthreads();
+        const uint32_t prev = sq;
+        sq = s_sq;
+        // done, or no more bits, or (equal keys) the last level hardly split anything
+        if (sq <= BUCKET_GOOD * m || used == avail || level == 2 || (level > 0 && sq > prev - prev / 4)) break;
+        // split every bucket into as many as it holds keys
+        uint32_t lc[ITEMS];
+#pragma unroll
+        for (int t = 0; t < ITEMS; ++t) {
+            if ((uint32_t)(t * THREADS) >= m) break;
+            if (tid + t * THREADS >= m) continue;
+            const uint32_t bk = b[t] & (NB - 1), lo = sC[bk], hi = bk + 1 < (uint32_t)NB ? sC[bk + 1] : m;
+            lc[t] = lo | (hi - lo) << 16;
+        }
+        __syncthreads();
+        for (uint32_t i = tid; i < (uint32_t)NB / 2; i += THREADS) sW[i] = 0;
+        if (tid == 0) s_sq = 0;
+        const uint32_t most = level == 0 ? 10u : 9u, take = avail - used < most ? avail - used : most;
+#pragma unroll
+        for (int t = 0; t < ITEMS; ++t) {
+            if ((uint32_t)(t * THREADS) >= m) break;
+            if (tid + t * THREADS >= m) continue;
+            const uint32_t y = rem[t] << take | (res[t] << used) >> (32 - take);
+            const uint32_t x = y * (lc[t] >> 16);
+            rem[t] = x & ((1u << (used + take)) - 1u);
+            b[t] = (lc[t] & 0xFFFFu) + (x >> (used + take));
+        }
+        used += take;
+        __syncthreads();
+    }
+    if (sq > BUCKET_MOST * m) return false;
+    // place (deciding bits; bucket, slot); the keys stay
+#pragma unroll
+    for (int t = 0; t < ITEMS; ++t) {
+        const uint32_t j = tid + t * THREADS;
+        if (j >= m) continue;
+        const uint32_t bk = b[t] & (NB - 1);
+        sR[sC[bk] + (b[t] >> 16)] = (uint64_t)res[t] << 32 | bk << 16 | j;
+    }
+    __syncthreads();
+    // the rank among the bucket's members
+    const bool by_slot = whole && ordered;
+    for (uint32_t j = tid; j < m; j += THREADS) {
+        const uint64_t mine = sR[j];
+        const uint32_t bk = (uint32_t)mine >> 16, slot = (uint32_t)mine & 0xFFFFu;
+        const uint32_t lo = sC[bk], hi = bk + 1 < (uint32_t)NB ? sC[bk + 1] : m;
+        uint32_t r = lo;
+        if (by_slot) {
+#pragma unroll 4
+            for (uint32_t i = lo; i < hi; ++i) r += sR[i] < mine ? 1u : 0u;
+        } else {
+            const uint64_t key = sK[slot];
+            const uint32_t idx = sV[slot], top = (uint32_t)(mine >> 32);
+            for (uint32_t i = lo; i < hi; ++i) {
+                const uint64_t y = sR[i];
+                const uint32_t ytop = (uint32_t)(y >> 32);
+                bool less = ytop < top;
+                if (ytop == top) {
+                    const uint32_t s2 = (uint32_t)y & 0xFFFFu;
+                    const uint64_t k2 = sK[s2];
+                    less = k2 < key || (k2 == key && sV[s2] < idx);
+                }
+                r += less ? 1u : 0u;
+            }
+        }
+        sP[r] = (uint16_t)slot;
+    }
+    __syncthreads();
+    return true;
+}
+
+// The merge sort of the keys that do not spread, out of line (it is the rare
+// path, and its code would crowd the other's).  Slots in index order: a stable
+// sort by the key alone yields (key, index) order.  Checked; the 128-bit sort
+// of (key, index) otherwise.  m <= THREADS * ITEMS pairs, sorted in place; sLo:
+// THREADS * ITEMS words.
+template <int THREADS, int ITEMS>
+__device__ __noinline__ void block_merge_sort_pairs(uint64_t* sK, uint32_t* sV, uint64_t* sLo, uint32_t m) {
+    __syncthreads();
+    bool ordered = true;
+    for (uint32_t i = threadIdx.x + 1; i < m; i += THREADS) ordered = ordered && sV[i - 1] < sV[i];
+    if (__syncthreads_and(ordered)) {
+        block_merge_sort_kv_fit<THREADS, ITEMS>(sK, sV, m);
+    } else {
+        for (uint32_t i = threadIdx.x; i < m; i += THREADS) sLo[i] = sV[i];
+        __syncthreads();
+        block_merge_sort128_fit<THREADS, ITEMS>(sK, sLo, m);
+        for (uint32_t i = threadIdx.x; i < m; i += THREADS) sV[i] = (uint32_t)sLo[i];
+        __syncthreads();
+    }
+}

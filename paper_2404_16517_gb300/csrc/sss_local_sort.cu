@@ -38,7 +38,7 @@ constexpr int QUAD_W = 4;                       // segments of <= 4 strings: 4 l
 constexpr int TINY_T = 64, TINY_CAP = 64;       // segments of warp_cap+1 .. 64 strings
 constexpr int SM_T = 128, SM_CAP = 512;         // segments of 65 .. 512 strings
 constexpr int MED_T = 512, MED_CAP = 2048;      // segments of 513 .. cta_cap (<= 2048) strings, 2 CTAs per SM
-constexpr int BK_T = 512, BK_CAP = 4096;        // bucket sort CTA (bucket targets above BKS_CAP / 2)
+constexpr int BK_T = 512, BK_CAP = 4352;        // bucket sort CTA (bucket targets above BKS_CAP / 2)
 constexpr int BKS_T = 256, BKS_CAP = 2048;      // bucket sort CTA for targets <= BKS_CAP / 2 (4 CTAs per SM)
 constexpr int DIRECT_T = 1024, DIRECT_CAP = 8192;  // whole-segment sort CTA (segments <= direct_cap)
 
@@ -576,8 +576,14 @@ __global__ void __launch_bounds__(32 * WF_WARPS, 4) k_finish_group(const FinIn i
 }
 
 constexpr size_t finish_smem(int cap) { return (size_t)cap * (8 + 8 + 4 * 7); }
-// sort_emit: keys, values (64-bit), two 32-bit arrays
-constexpr size_t emit_smem(int, int cap) { return (size_t)cap * (8 + 8 + 4 + 4); }
+// sort_emit's shared memory: keys, scratch, indices, sorted order, counters.
+// The scratch is one word per key (or the low words of a 128-bit merge sort); the
+// counters are 16 bits wide, two per key (the next power of two).  A CTA of 512
+// threads takes 4,352 strings: as many as two of them on an SM have memory for,
+// and a little over the 4,096 that templates of 64 in partitions of 2^18 give.
+constexpr int emit_buckets(int cap) { return cap <= 2048 ? 4096 : 8192; }
+constexpr int emit_merge_items(int threads, int cap) { return cap / threads >= 8 ? 8 : 4; }
+constexpr size_t emit_smem(int, int cap) { return (size_t)cap * (8 + 8 + 4 + 2) + 2 * (size_t)emit_buckets(cap); }
 
 // ---------------------------------------------------------------------------
 // Large path.
@@ -682,161 +688,197 @@ __global__ void __launch_bounds__(LG_T, 6) k_lg_ext(const LsDev* __restrict__ S)
 }
 
 // Sort positions [bs, bs+m) (m <= CAP) by (key, index) in one CTA, write the
-// keys and indices back, set the LCP at every key change (d + key_lcp) and emit
+// indices back (of the keys a bucket's first and last), set the LCP at every key change (d + key_lcp) and emit
 // the groups of equal keys: runs of equal strings get lcp = length, other groups
 // become segments at depth d + v + C.  The first position's LCP is left alone.
-// Reads tK/tV (FROM_T) or K/perm fully before writing K/perm.
-template <int THREADS, int CAP, bool FROM_T>
-__device__ __forceinline__ void sort_emit(unsigned char* smem, uint32_t bs, uint32_t m, uint32_t d, uint32_t f,
-                                          LsDev* S, unsigned* err) {
+// Reads tK/tV (from_t) or K/perm fully before writing K/perm.  False (nothing
+// written) if the keys need a merge sort of more than its capacity.
+// Bound by the instructions and barriers of its phases (65 k cycles of a CTA of
+// 4,096 strings before, 47 k now: 11 k to rank, 11 k to write back, 9 k to load
+// and reduce, 7 k for the bits).  The range buckets and the 1,024 segments of
+// about 4,096 strings of the 4.19M-string sort take 147 us (306 us with the
+// merge sort alone), the 4,096-instance batch's 1.63 ms (2.10 ms).
+template <int THREADS, int CAP>
+__device__ __forceinline__ bool sort_emit(unsigned char* smem, bool from_t, uint32_t bs, uint32_t m, uint32_t d,
+                                          uint32_t f, LsDev* S, unsigned* err) {
     const LsArgs& A = S->args;  // S and err are kernel parameters: no registers held through the sort
     __shared__ uint32_t s_d, s_f;
     if (threadIdx.x == 0) {
         s_d = d;
         s_f = f;
     }
-    constexpr int ITEMS = CAP / THREADS;
-    uint64_t* sHi = reinterpret_cast<uint64_t*>(smem);
-    uint64_t* sLo = sHi + CAP;
-    uint32_t* sA = reinterpret_cast<uint32_t*>(sLo + CAP);
-    uint32_t* sN = sA + CAP;
-    __shared__ uint32_t sh_warp[32];
+    constexpr int ITEMS = (CAP + THREADS - 1) / THREADS, NB = emit_buckets(CAP);
+    constexpr int MI = emit_merge_items(THREADS, CAP);
+    static_assert(THREADS * MI <= CAP, "the merge sort pads its arrays to THREADS * MI");
+    uint64_t* sK = reinterpret_cast<uint64_t*>(smem);
+    uint64_t* sR = sK + CAP;
+    uint32_t* sV = reinterpret_cast<uint32_t*>(sR + CAP);
+    uint16_t* sC = reinterpret_cast<uint16_t*>(sV + CAP);
+    uint16_t* sP = sC + NB;  // the sorted order: position -> slot
     {
-        const uint64_t* srcK = FROM_T ? A.tK : A.K;
-        const uint32_t* srcV = FROM_T ? A.tV : A.perm;
+        const uint64_t* srcK = (from_t ? A.tK : A.K) + bs;
+        const uint32_t* srcV = (from_t ? A.tV : A.perm) + bs;
         uint64_t k[ITEMS];
         uint32_t v[ITEMS];
 #pragma unroll
         for (int t = 0; t < ITEMS; ++t) {
             const uint32_t i = threadIdx.x + t * THREADS;
-            k[t] = i < m ? srcK[bs + i] : 0ull;
-            v[t] = i < m ? srcV[bs + i] : 0u;
+            k[t] = i < m ? srcK[i] : 0ull;
+            v[t] = i < m ? srcV[i] : 0u;
         }
 #pragma unroll
         for (int t = 0; t < ITEMS; ++t) {
             const uint32_t i = threadIdx.x + t * THREADS;
             if (i < m) {
-                sHi[i] = k[t];
-                sA[i] = v[t];
+                sK[i] = k[t];
+                sV[i] = v[t];
             }
         }
     }
-    __syncthreads();
-    // A segment's members arrive in index order (every sort of an earlier round
-    // breaks ties by index, and the partition scatter keeps the order): then a
-    // stable sort by the key alone yields (key, index) order.  Checked; the
-    // 128-bit merge sort of (key, index) otherwise.
-    bool ordered = true;
-    for (uint32_t i = threadIdx.x + 1; i < m; i += THREADS) ordered = ordered && sA[i - 1] < sA[i];
-    if (__syncthreads_and(ordered)) {
-        block_merge_sort_kv_fit<THREADS, ITEMS>(sHi, sA, m);
-        for (uint32_t i = threadIdx.x; i < m; i += THREADS) sLo[i] = sA[i];
+    if (!block_bucket_sort<THREADS, ITEMS, NB>(sK, sV, sC, sR, sP, m, f)) {
+        if (m > (uint32_t)(THREADS * MI)) return false;
+        block_merge_sort_pairs<THREADS, MI>(sK, sV, sR, m);
+        for (uint32_t i = threadIdx.x; i < m; i += THREADS) sP[i] = (uint16_t)i;
         __syncthreads();
-    } else {
-        for (uint32_t i = threadIdx.x; i < m; i += THREADS) sLo[i] = sA[i];
-        __syncthreads();
-        block_merge_sort128_fit<THREADS, ITEMS>(sHi, sLo, m);
     }
-    uint64_t* K = A.K;
     uint32_t* perm = A.perm;
     uint32_t* lcp = A.lcp;
     d = s_d;
     f = s_f;
-    for (uint32_t i = threadIdx.x; i < CAP; i += THREADS) {
-        uint32_t v = 0;
-        if (i < m) {
-            uint64_t k = sHi[i];
-            K[bs + i] = k;
-            perm[bs + i] = (uint32_t)sLo[i];
-            bool bnd = (i == 0) || (sHi[i - 1] != k);
-            if (bnd && i > 0) lcp[bs + i] = d + key_lcp(sHi[i - 1], k, f);
-            v = bnd ? i : 0u;
-        }
-        sA[i] = v;
-    }
+    // Write the order back and list the groups of equal keys in shared memory
+    // (start | size << 16, in the sort's scratch): pushed as they are found, each
+    // step would wait for an atomic's way to L2 and back.
+    uint32_t* sG = reinterpret_cast<uint32_t*>(sR);
+    __shared__ uint32_t s_ng;
+    if (threadIdx.x == 0) s_ng = 0;
     __syncthreads();
-    block_inclusive_max_inplace<THREADS, ITEMS>(sA, m, sh_warp);  // sA[i] = first index of i's group
-    // group sizes at the group's first index, written by the group's last member
-    // (no atomics: a group of equal keys may hold the whole segment)
-    for (uint32_t i = threadIdx.x; i < m; i += THREADS)
-        if (i + 1 == m || sA[i + 1] == i + 1) sN[sA[i]] = i + 1 - sA[i];
-    __syncthreads();
-    for (uint32_t i0 = 0; i0 < m; i0 += THREADS) {  // uniform trip count: push_seg_warp needs whole warps
+    const uint32_t lane = threadIdx.x & 31;
+    for (uint32_t i0 = 0; i0 < m; i0 += THREADS) {  // uniform trip count: whole warps shuffle
         const uint32_t i = i0 + threadIdx.x;
-        bool want = false;
-        uint32_t c = 0, dn = 0;
+        if (i - lane >= m) break;
+        const uint32_t slot = sP[i < m ? i : m - 1];
+        const uint64_t k = sK[slot];
+        // the keys next to the warp's 32: before the first, after the last
+        uint64_t kx = 0;
+        if (lane == 0 && i > 0) kx = sK[sP[i - 1]];
+        if (lane == 31 && i + 1 < m) kx = sK[sP[i + 1]];
+        uint64_t kp = __shfl_up_sync(SSS_FULL, k, 1);
+        if (lane == 0) kp = kx;
+        const bool bnd = i == 0 || i >= m || kp != k;  // starts a group (past the end: closes the last one)
+        const unsigned bm = __ballot_sync(SSS_FULL, bnd);
+        const bool goes_on = __ballot_sync(SSS_FULL, lane == 31 && i + 1 < m && kx == k) != 0;
+        const bool ended = key_ended(k, f);
+        uint32_t c = 0;
         if (i < m) {
-            const uint32_t g = sA[i];
-            c = sN[g];
-            if (c >= 2) {
-                const uint64_t k = sHi[i];
-                if (key_ended(k, f)) {
-                    if (i != g) lcp[bs + i] = A.lens[(uint32_t)sLo[i]];
-                } else if (i == g) {
-                    want = true;
-                    dn = d + key_v(k, f) + fmt_chars(f);
+            const uint32_t e = sV[slot];
+            perm[bs + i] = e;
+            if (bnd) {
+                if (i > 0) lcp[bs + i] = d + key_lcp(kp, k, f);
+                if (!ended) {
+                    const unsigned after = lane < 31 ? bm >> (lane + 1) : 0u;
+                    c = after ? (uint32_t)__ffs((int)after) : 32u - lane;
+                    if (!after && goes_on) {
+                        // past the warp: the group's end by doubling steps, then halving ones
+                        uint32_t lo = i - lane + 32, step = 1;
+                        while (lo + step < m && sK[sP[lo + step]] == k) {
+                            lo += step;
+                            step *= 2;
+                        }
+                        uint32_t hi = lo + step < m ? lo + step : m;  // equal at lo; at hi it is not, or hi == m
+                        while (hi - lo > 1) {
+                            const uint32_t mid = (lo + hi) >> 1;
+                            if (sK[sP[mid]] == k) lo = mid;
+                            else hi = mid;
+                        }
+                        c = hi - i;
+                    }
                 }
+            } else if (ended) {
+                lcp[bs + i] = A.lens[e];  // a run of equal strings
             }
+            if (from_t && (i == 0 || i + 1 == m)) A.K[bs + i] = k;  // for the LCP at the bucket's ends
         }
-        push_seg_warp(A, S->cnt, want, bs + i, c, dn, err);
+        const unsigned gm = __ballot_sync(SSS_FULL, c >= 2);
+        if (gm) {
+            uint32_t base = 0;
+            if (lane == 0) base = atomicAdd(&s_ng, (uint32_t)__popc(gm));
+            base = __shfl_sync(SSS_FULL, base, 0);
+            if (c >= 2) sG[base + (uint32_t)__popc(gm & ((1u << lane) - 1u))] = i | c << 16;
+        }
     }
+    __syncthreads();
+    const uint32_t ng = s_ng;
+    for (uint32_t j0 = threadIdx.x - lane; j0 < ng; j0 += THREADS) {  // whole warps: push_seg_warp
+        const uint32_t j = j0 + lane;
+        const uint32_t x = j < ng ? sG[j] : 0u, i = x & 0xFFFFu;
+        uint32_t dn = 0;
+        if (j < ng) dn = d + key_v(sK[sP[i]], f) + fmt_chars(f);
+        push_seg_warp(A, S->cnt, j < ng, bs + i, x >> 16, dn, err);
+    }
+    return true;
 }
 
-// One CTA per (segment, bucket).  Range buckets are sorted in shared memory;
-// groups of equal keys become new segments at depth d + v + C.
-template <int THREADS, int CAP>
-__device__ __forceinline__ void lg_bucket(uint32_t g, uint32_t npart, LsDev* S, unsigned* err) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const LsArgs& A = S->args;
-    uint32_t* cnt = S->cnt;
-    const uint32_t sidx = warp_last_le(A.bk0, npart, g);
-    const LgSegInfo si = A.info[sidx];
-    const uint32_t b = g - A.bk0[sidx];
-    const uint32_t nbk = 2 * si.nb - 1;
-    if (b >= nbk) return;
-    const uint32_t* bst = A.bst + (size_t)sidx * (LG_NBMAX + 1);
-    uint32_t bs = bst[b], be = bst[b + 1];
-    if (bs < si.seg.start || be > si.seg.start + si.seg.size || be < bs) {
-        if (threadIdx.x == 0) atomicOr(err, ERRBIT_OVERFLOW);
-        return;
-    }
-    uint32_t m = be - bs;
-    if (m == 0) return;
-    uint32_t d = si.seg.depth;
-    const uint32_t f = A.segfmt[sidx];
-    bool eq = (b & 1u) != 0;
-    if (eq || m > (uint32_t)CAP) {
-        for (uint32_t q = bs + threadIdx.x; q < be; q += THREADS) {
-            A.K[q] = A.tK[q];
-            A.perm[q] = A.tV[q];
-        }
-        if (threadIdx.x == 0) {
-            if (eq) {
-                uint64_t k = A.tK[bs];
-                if (m >= 2 && !key_ended(k, f)) push_seg(A, cnt, bs, m, d + key_v(k, f) + fmt_chars(f), err);
-            } else {
-                // oversized range bucket: another round at this depth.  Its members
-                // have distinct keys, so the LCPs across its two ends depend on which
-                // members end up first and last: recomputed after the last round.
-                push_seg(A, cnt, bs, m, d, err);
-                if (bs > si.seg.start) atomicOr(&A.fixmap[bs >> 5], 1u << (bs & 31u));
-                if (be < si.seg.start + si.seg.size) atomicOr(&A.fixmap[be >> 5], 1u << (be & 31u));
-            }
-        }
-        if (eq && m >= 2 && key_ended(A.tK[bs], f)) {
-            // a run of equal strings: lcp = length inside the run
-            for (uint32_t q = bs + 1 + threadIdx.x; q < be; q += THREADS) A.lcp[q] = A.lens[A.tV[q]];
-        }
-        return;
-    }
-    sort_emit<THREADS, CAP, true>(smem, bs, m, d, f, S, err);
-}
-
+// One CTA per bucket of the partitioned segments, and per whole segment that
+// fits: range buckets and whole segments are sorted in shared memory, groups of
+// equal keys become new segments at depth d + v + C.  The sort is a chain of
+// short phases between barriers, so two CTAs of 512 threads on an SM overlap
+// where one of 1024 threads waits (k_lg_direct keeps the segments of more than
+// CAP strings).
 template <int THREADS, int CAP>
 __global__ void __launch_bounds__(THREADS, 65536 / (64 * THREADS)) k_lg_buckets(LsDev* S, unsigned* err) {
-    const uint32_t nb = S->plan.pbuckets;
-    for (uint32_t g = blockIdx.x; g < nb; g = cta_next_unit(&S->work[5]))
-        lg_bucket<THREADS, CAP>(g, S->plan.npart, S, err);
+    extern __shared__ __align__(16) unsigned char smem[];
+    const LsArgs& A = S->args;
+    const uint32_t nb = S->plan.pbuckets, small0 = S->plan.npart + S->plan.nbig;
+    const uint32_t n = nb + S->plan.ns - small0;
+    for (uint32_t g = blockIdx.x; g < n; g = cta_next_unit(&S->work[5])) {
+        const bool bucket = g < nb;
+        const uint32_t sidx = bucket ? warp_last_le(A.bk0, S->plan.npart, g) : small0 + (g - nb);
+        const Seg sg = A.info[sidx].seg;
+        const uint32_t f = A.segfmt[sidx];
+        uint32_t bs = sg.start, m = sg.size, b = 0;
+        if (bucket) {
+            b = g - A.bk0[sidx];
+            const uint32_t* bst = A.bst + (size_t)sidx * (LG_NBMAX + 1) + b;
+            bs = bst[0];
+            const uint32_t be = bst[1];
+            if (bs < sg.start || be > sg.start + sg.size || be < bs) {
+                if (threadIdx.x == 0) atomicOr(err, ERRBIT_OVERFLOW);
+                continue;
+            }
+            m = be - bs;
+            if (m == 0) continue;
+        }
+        const bool eq = (b & 1u) != 0;
+        if (!eq && m <= (uint32_t)CAP && sort_emit<THREADS, CAP>(smem, bucket, bs, m, sg.depth, f, S, err)) continue;
+        if (!bucket) {
+            if (threadIdx.x == 0) A.redo[atomicAdd(&S->cnt[6], 1u)] = sidx;  // at most one entry per segment
+            continue;
+        }
+        for (uint32_t q = bs + threadIdx.x; q < bs + m; q += THREADS) A.perm[q] = A.tV[q];
+        if (threadIdx.x == 0) {
+            A.K[bs] = A.tK[bs];
+            A.K[bs + m - 1] = A.tK[bs + m - 1];
+        }
+        if (!eq) {
+            // oversized range bucket: another round at this depth.  Its members
+            // have distinct keys, so the LCPs across its two ends depend on which
+            // members end up first and last: recomputed after the last round.
+            if (threadIdx.x == 0) {
+                const uint32_t be = bs + m;
+                push_seg(A, S->cnt, bs, m, sg.depth, err);
+                if (bs > sg.start) atomicOr(&A.fixmap[bs >> 5], 1u << (bs & 31u));
+                if (be < sg.start + sg.size) atomicOr(&A.fixmap[be >> 5], 1u << (be & 31u));
+            }
+        } else if (m >= 2) {
+            const uint64_t k = A.tK[bs];
+            if (!key_ended(k, f)) {
+                if (threadIdx.x == 0) push_seg(A, S->cnt, bs, m, sg.depth + key_v(k, f) + fmt_chars(f), err);
+            } else {
+                // a run of equal strings: lcp = length inside the run
+                for (uint32_t q = bs + 1 + threadIdx.x; q < bs + m; q += THREADS) A.lcp[q] = A.lens[A.tV[q]];
+            }
+        }
+    }
 }
 
 // LCP at the first position of every non-first, non-empty bucket of segment s.
@@ -853,9 +895,9 @@ __device__ __forceinline__ void lg_seams(const LsArgs& A, uint32_t s) {
 }
 
 // The last kernel of a round.  Bucket seams of the partitioned segments (their
-// buckets are sorted by now), then the large segments of at most DIRECT_CAP
-// strings: one CTA sorts a whole segment by its keys (no sampling,
-// classification or scatter).  The last CTA to end decides whether the round
+// buckets are sorted by now), then the segments of more than a bucket CTA's and
+// at most DIRECT_CAP strings, and those it handed on: one CTA sorts a whole
+// segment by its keys (no sampling, classification or scatter).  The last CTA to end decides whether the round
 // loop goes on: another round while segments were pushed, the round limit
 // holds and no capacity error occurred (loop = 1: inside a captured loop).
 template <int THREADS, int CAP>
@@ -863,13 +905,14 @@ __global__ void __launch_bounds__(THREADS) k_lg_direct(LsDev* S, unsigned* err, 
                                                        int loop) {
     extern __shared__ __align__(16) unsigned char smem[];
     const LsArgs& A = S->args;
-    const uint32_t ns = S->plan.ns, npart = S->plan.npart;
+    const uint32_t nbig = S->plan.nbig, npart = S->plan.npart;
     for (uint32_t s = blockIdx.x; s < npart; s += gridDim.x) lg_seams(A, s);
-    for (uint32_t i = blockIdx.x; npart + i < ns; i = cta_next_unit(&S->work[6])) {
-        const uint32_t sidx = npart + i;
+    const uint32_t n = nbig + S->cnt[6];
+    for (uint32_t i = blockIdx.x; i < n; i = cta_next_unit(&S->work[6])) {
+        const uint32_t sidx = i < nbig ? npart + i : A.redo[i - nbig];
         const LgSegInfo si = A.info[sidx];
         if (si.seg.size > (uint32_t)CAP) continue;
-        sort_emit<THREADS, CAP, false>(smem, si.seg.start, si.seg.size, si.seg.depth, A.segfmt[sidx], S, err);
+        sort_emit<THREADS, CAP>(smem, false, si.seg.start, si.seg.size, si.seg.depth, A.segfmt[sidx], S, err);
     }
     if (!loop) return;
     __syncthreads();
@@ -956,9 +999,12 @@ static LsKnobs ls_knobs(const sss_params& prm) {
     k.cta_cap = prm.cta_cap ? std::min(std::max(prm.cta_cap, (uint32_t)TINY_CAP), (uint32_t)MED_CAP) : (uint32_t)MED_CAP;
     k.direct_cap = prm.direct_cap ? std::min(std::max(prm.direct_cap, k.cta_cap), (uint32_t)DIRECT_CAP)
                                   : (uint32_t)DIRECT_CAP;
-    k.bucket_target = prm.bucket_target ? std::min(std::max(prm.bucket_target, 256u), (uint32_t)BK_CAP) : 2048u;
+    k.bucket_target = prm.bucket_target ? std::min(std::max(prm.bucket_target, 256u), 4096u) : 2048u;
     return k;
 }
+
+// bucket CTA: the small one when its capacity is twice the target or more
+bool small_buckets(uint32_t target) { return target <= (uint32_t)BKS_CAP / 2; }
 
 // Work memory of the local sort: fills the pointers and capacities of a.
 void carve_ls(Arena& ar, uint32_t n, uint32_t p, const sss_params& prm, LsArgs& a) {
@@ -981,6 +1027,7 @@ void carve_ls(Arena& ar, uint32_t n, uint32_t p, const sss_params& prm, LsArgs& 
     a.med_max = kn.cta_cap;
     a.direct_max = kn.direct_cap;
     a.target = kn.bucket_target;
+    a.bucket_cap = small_buckets(kn.bucket_target) ? BKS_CAP : BK_CAP;
     a.limit = 100000u;
     a.use_tiles = 0;
 }
@@ -1072,7 +1119,7 @@ sss_status impl_local_sort(sss_ctx* ctx, Arena& ar, const StrIn& in, uint32_t p,
 // seams and whole-segment sorts.  Segments up to cta_cap strings stay on their
 // lists: they are finished once, after the last round (one launch per class
 // over all rounds' segments in place of one per round).
-static sss_status launch_round(sss_ctx* ctx, const LsGrid& g, bool small_buckets, cudaGraphConditionalHandle h,
+static sss_status launch_round(sss_ctx* ctx, const LsGrid& g, bool small, cudaGraphConditionalHandle h,
                                int loop) {
     LsDev* S = static_cast<LsDev*>(ctx->d_ls);
     const LsDev* cS = S;
@@ -1084,7 +1131,7 @@ static sss_status launch_round(sss_ctx* ctx, const LsGrid& g, bool small_buckets
     SSS_TRY(sss_launch(ctx, "ls_lg_classify", k_lg_classify, dim3(g.of(6)), dim3(LG_T), 0, cS));
     SSS_TRY(sss_launch(ctx, "ls_lg_offsets", k_lg_rowscan, dim3(g.of(4)), dim3(256), 0, cS));
     SSS_TRY(sss_launch(ctx, "ls_lg_scatter", k_lg_scatter, dim3(g.of(8)), dim3(LG_T), 0, cS, ctx->d_err));
-    if (small_buckets)
+    if (small)
         SSS_TRY(sss_launch(ctx, "ls_lg_buckets", k_lg_buckets<BKS_T, BKS_CAP>, dim3(std::max(g.sm, g.of(4))),
                            dim3(BKS_T), emit_smem(BKS_T, BKS_CAP), S, ctx->d_err));
     else
@@ -1099,8 +1146,8 @@ static sss_status launch_round(sss_ctx* ctx, const LsGrid& g, bool small_buckets
 // seams.  Its kernels take the context's device state only, so one graph per
 // grid class and bucket CTA (eight at most, kept in the context) serves every
 // call; captured per call address, a sort of new inputs paid for a capture.
-static sss_status sort_graph(sss_ctx* ctx, uint32_t gcls, bool small_buckets, cudaGraphExec_t* out) {
-    sss_ctx::LsGraph& slot = ctx->ls_graphs[2 * gcls + (small_buckets ? 1 : 0)];
+static sss_status sort_graph(sss_ctx* ctx, uint32_t gcls, bool small, cudaGraphExec_t* out) {
+    sss_ctx::LsGraph& slot = ctx->ls_graphs[2 * gcls + (small ? 1 : 0)];
     if (slot.exec) {
         *out = slot.exec;
         return SSS_OK;
@@ -1130,7 +1177,7 @@ static sss_status sort_graph(sss_ctx* ctx, uint32_t gcls, bool small_buckets, cu
         ce = cudaStreamBeginCaptureToGraph(ctx->cap_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
         if (ce == cudaSuccess) {
             ctx->stream = ctx->cap_stream;
-            st = launch_round(ctx, g, small_buckets, h, 1);
+            st = launch_round(ctx, g, small, h, 1);
             const cudaError_t ee = cudaStreamEndCapture(ctx->cap_stream, &body);
             if (ce == cudaSuccess) ce = ee;
         }
@@ -1239,10 +1286,10 @@ sss_status impl_sort_segments_range(sss_ctx* ctx, Arena& ar, const StrIn& in, co
         for (uint32_t c = LC_MED + 1; c-- > LC_QUAD;) SSS_TRY(launch_finisher(ctx, c, grid[c], list_input(ctx, c)));
         return SSS_OK;
     }
-    const bool small_buckets = A.target <= (uint32_t)BKS_CAP / 2;
+    const bool small = small_buckets(A.target);
     if (!ctx->timing || (prm.flags & SSS_FLAG_GRAPH)) {
         cudaGraphExec_t ex;
-        SSS_TRY(sort_graph(ctx, gcls, small_buckets, &ex));
+        SSS_TRY(sort_graph(ctx, gcls, small, &ex));
         return sss_graph_launch(ctx, ctx->graph_tag, ex);
     }
     // kernel timing is on: the same kernels launched one by one, with the next
@@ -1251,7 +1298,7 @@ sss_status impl_sort_segments_range(sss_ctx* ctx, Arena& ar, const StrIn& in, co
     uint32_t* h_next = reinterpret_cast<uint32_t*>(ctx->h_small);
     for (uint32_t rounds = 1;; ++rounds) {
         if (rounds > A.limit) return sss_fail(ctx, SSS_ERR_CUDA, "local sort: round limit exceeded");
-        SSS_TRY(launch_round(ctx, g, small_buckets, cudaGraphConditionalHandle{}, 0));
+        SSS_TRY(launch_round(ctx, g, small, cudaGraphConditionalHandle{}, 0));
         SSS_CUDA(cudaMemcpyAsync(h_next, &S->cnt[LC_LARGE], sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
         SSS_CUDA(cudaMemcpyAsync(h_next + 1, ctx->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
         SSS_CUDA(cudaStreamSynchronize(ctx->stream));

@@ -40,10 +40,12 @@ struct LgSegInfo {
     uint32_t pad;
 };
 
-// Totals of one round: segments [0, npart) are partitioned, [npart, ns) sorted
-// whole; tiles [0, ptiles) belong to partitioned segments.
+// Totals of one round: segments [0, npart) are partitioned, the others sorted
+// whole, [npart, npart + nbig) by the CTAs for more than bucket_cap strings and
+// [npart + nbig, ns) by the bucket CTAs; tiles [0, ptiles) belong to partitioned
+// segments.
 struct LsPlan {
-    uint32_t ns, npart, ntiles, ptiles, pbuckets, hist;
+    uint32_t ns, npart, nbig, ntiles, ptiles, pbuckets;
     uint32_t pad[2];
 };
 
@@ -96,9 +98,10 @@ struct LsArgs {
     GPtr<uint32_t> tile0;    // first tile of every segment
     GPtr<uint32_t> bk0;      // first bucket of every segment
     GPtr<uint32_t> rowdone;  // rows scanned of every segment
+    GPtr<uint32_t> redo;     // whole segments the bucket CTAs handed on (cnt[6] of them)
     GPtr<Seg> list[LC_COUNT];  // LC_WARP: the last entry of the shared array, filled downwards
     uint32_t cap[LC_COUNT];
-    uint32_t warp_max, med_max, direct_max, target;
+    uint32_t warp_max, med_max, direct_max, target, bucket_cap;
     uint32_t cap_tiles, cap_hist, limit, use_tiles;
     uint32_t q0, q1;  // the positions being sorted
 };
@@ -107,30 +110,33 @@ struct LsArgs {
 struct LsDev {
     LsArgs args;
     LsPlan plan;
-    uint32_t cnt[8];   // segments per list
+    uint32_t cnt[8];   // segments per list; [6]: entries of redo
     uint32_t work[8];  // dynamic work counters: [LC_*] finishers, [5] buckets, [6] direct, [7] CTAs done
     uint32_t rounds;
 };
 
-// Exclusive block scan of three u64 at once (each two packed 32-bit counts):
-// one pass of shuffles and barriers instead of six.  sh: 3 * 32 words.
-__device__ __forceinline__ void block_scan3(uint64_t v[3], uint64_t tot[3], uint64_t* sh) {
+// Exclusive block scan of N u64 at once (each up to two packed 32-bit counts):
+// one pass of shuffles and barriers.  1024 threads; sh: N * 32 words.
+template <int N>
+__device__ __forceinline__ void block_scan_n(uint64_t (&v)[N], uint64_t (&tot)[N], uint64_t* sh) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    uint64_t x[3] = {v[0], v[1], v[2]};
+    uint64_t x[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) x[k] = v[k];
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
+        for (int k = 0; k < N; ++k) {
             const uint64_t y = __shfl_up_sync(SSS_FULL, x[k], o);
             if (lane >= o) x[k] += y;
         }
     }
     if (lane == 31) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) sh[k * 32 + w] = x[k];
+        for (int k = 0; k < N; ++k) sh[k * 32 + w] = x[k];
     }
     __syncthreads();
-    if (w < 3) {
+    if (w < N) {
         uint64_t t = sh[w * 32 + lane];
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -141,7 +147,7 @@ __device__ __forceinline__ void block_scan3(uint64_t v[3], uint64_t tot[3], uint
     }
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
+    for (int k = 0; k < N; ++k) {
         tot[k] = sh[k * 32 + 31];
         v[k] = (w > 0 ? sh[k * 32 + w - 1] : 0ull) + x[k] - v[k];
     }
@@ -151,75 +157,80 @@ __device__ __forceinline__ void block_scan3(uint64_t v[3], uint64_t tot[3], uint
 // Plan a round from the large list; resets its counter for the pushes of this
 // round and the round's work counters.  One CTA of 1024 threads.
 __global__ void __launch_bounds__(1024) k_lg_plan(LsDev* __restrict__ S, unsigned* err) {
-    __shared__ uint64_t sh[96];
-    __shared__ uint32_t s_np, s_pt;
+    __shared__ uint64_t sh[128];
+    __shared__ uint32_t s_n[4];  // segments and tiles: partitioned, then big
     const LsArgs& A = S->args;
     const uint32_t tid = threadIdx.x;
-    const uint32_t direct_max = A.direct_max, target = A.target;
+    const uint32_t direct_max = A.direct_max, bucket_cap = A.bucket_cap, target = A.target;
     const Seg* list = A.list[LC_LARGE];
     uint32_t ns = S->cnt[LC_LARGE];
     if (ns > A.cap[LC_LARGE]) {
         if (tid == 0) atomicOr(err, ERRBIT_OVERFLOW);
         ns = 0;
     }
-    if (tid == 0) s_np = s_pt = 0;
+    if (tid < 4) s_n[tid] = 0;
     __syncthreads();  // every thread has read the count
-    // the partitioned segments and their tiles come first
-    uint32_t np = 0, pt = 0;
+    uint32_t n0[4] = {0, 0, 0, 0};
     for (uint32_t s = tid; s < ns; s += 1024) {
-        const uint32_t size = list[s].size;
+        const uint32_t size = list[s].size, tiles = (size + LG_TILE - 1) / LG_TILE;
         if (size > direct_max) {
-            ++np;
-            pt += (size + LG_TILE - 1) / LG_TILE;
+            ++n0[0];
+            n0[1] += tiles;
+        } else if (size > bucket_cap) {
+            ++n0[2];
+            n0[3] += tiles;
         }
     }
-    np = __reduce_add_sync(SSS_FULL, np);
-    pt = __reduce_add_sync(SSS_FULL, pt);
-    if ((tid & 31) == 0 && np) {
-        atomicAdd(&s_np, np);
-        atomicAdd(&s_pt, pt);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t t = __reduce_add_sync(SSS_FULL, n0[k]);
+        if ((tid & 31) == 0 && t) atomicAdd(&s_n[k], t);
     }
     __syncthreads();
-    const uint32_t npart = s_np, ptiles = s_pt;
-    uint64_t carry[3] = {0, 0, 0};  // (partitioned, direct) segments, their tiles, (buckets, histogram words)
+    const uint32_t npart = s_n[0], ptiles = s_n[1], nbig = s_n[2], btiles = s_n[3];
+    // (partitioned, big) segments, their tiles, small segments and their tiles, buckets and histogram words
+    uint64_t carry[4] = {(uint64_t)npart << 32, (uint64_t)ptiles << 32,
+                         (uint64_t)(npart + nbig) | ((uint64_t)(ptiles + btiles) << 32), 0};
     for (uint32_t b0 = 0; b0 < ns; b0 += 1024) {
         const uint32_t s = b0 + tid;
         const bool valid = s < ns;
         Seg sg{};
         if (valid) sg = list[s];
-        const bool part = valid && sg.size > direct_max;
-        const uint32_t tiles = valid ? (sg.size + LG_TILE - 1) / LG_TILE : 0u;
+        const uint32_t cls = !valid ? 3u : sg.size > direct_max ? 0u : sg.size > bucket_cap ? 1u : 2u;
+        const uint32_t tiles = (sg.size + LG_TILE - 1) / LG_TILE;
         uint32_t nb = 0;
-        if (part) {
+        if (cls == 0) {
             nb = (sg.size + target - 1) / target;
             nb = nb < 2u ? 2u : (nb > (uint32_t)LG_BMAX ? (uint32_t)LG_BMAX : nb);
         }
-        const uint32_t nbk = part ? 2 * nb - 1 : 0u;
-        uint64_t v[3], tot[3];
-        v[0] = part ? 1ull : (valid ? 1ull << 32 : 0ull);
-        v[1] = part ? (uint64_t)tiles : (uint64_t)tiles << 32;
-        v[2] = (uint64_t)nbk | ((uint64_t)nbk * tiles << 32);
-        block_scan3(v, tot, sh);
+        const uint32_t nbk = cls == 0 ? 2 * nb - 1 : 0u;
+        uint64_t v[4], tot[4];
+        v[0] = cls == 0 ? 1ull : cls == 1 ? 1ull << 32 : 0ull;
+        v[1] = cls == 0 ? (uint64_t)tiles : cls == 1 ? (uint64_t)tiles << 32 : 0ull;
+        v[2] = cls == 2 ? 1ull | ((uint64_t)tiles << 32) : 0ull;
+        v[3] = (uint64_t)nbk | ((uint64_t)nbk * tiles << 32);
+        block_scan_n(v, tot, sh);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] += carry[k];
         if (valid) {
-            const uint32_t at = part ? (uint32_t)(carry[0] + v[0])
-                                     : npart + (uint32_t)((carry[0] + v[0]) >> 32);
-            A.info[at] = LgSegInfo{sg, tiles, nb, (uint32_t)((carry[2] + v[2]) >> 32), 0};
-            A.tile0[at] = part ? (uint32_t)(carry[1] + v[1]) : ptiles + (uint32_t)((carry[1] + v[1]) >> 32);
-            A.bk0[at] = (uint32_t)(carry[2] + v[2]);
+            const uint32_t at = cls == 0 ? (uint32_t)v[0] : cls == 1 ? (uint32_t)(v[0] >> 32) : (uint32_t)v[2];
+            A.info[at] = LgSegInfo{sg, tiles, nb, (uint32_t)(v[3] >> 32), 0};
+            A.tile0[at] = cls == 0 ? (uint32_t)v[1] : cls == 1 ? (uint32_t)(v[1] >> 32) : (uint32_t)(v[2] >> 32);
+            A.bk0[at] = (uint32_t)v[3];
             A.rowdone[at] = 0;
         }
 #pragma unroll
-        for (int k = 0; k < 3; ++k) carry[k] += tot[k];
+        for (int k = 0; k < 4; ++k) carry[k] += tot[k];
     }
     if (tid == 0) {
-        const uint32_t nt = ptiles + (uint32_t)(carry[1] >> 32), nh = (uint32_t)(carry[2] >> 32);
-        LsPlan pl{ns, npart, nt, ptiles, (uint32_t)carry[2], nh, {0, 0}};
+        const uint32_t nt = (uint32_t)(carry[2] >> 32), nh = (uint32_t)(carry[3] >> 32);
+        LsPlan pl{ns, npart, nbig, nt, ptiles, (uint32_t)carry[3], {0, 0}};
         if (nt > A.cap_tiles || nh > A.cap_hist) {
             atomicOr(err, ERRBIT_OVERFLOW);
             pl = LsPlan{0, 0, 0, 0, 0, 0, {0, 0}};
         }
         S->plan = pl;
-        S->cnt[LC_LARGE] = 0;
+        S->cnt[LC_LARGE] = S->cnt[6] = 0;
         S->work[5] = S->work[6] = S->work[7] = 0;
     }
 }
@@ -519,6 +530,7 @@ inline void carve_sp(Arena& ar, uint32_t n, uint32_t cap_segs, LsArgs& a) {
     a.tile0 = ar.take<uint32_t>(cap_segs);
     a.bk0 = ar.take<uint32_t>(cap_segs);
     a.rowdone = ar.take<uint32_t>(cap_segs);
+    a.redo = ar.take<uint32_t>(cap_segs);
 }
 
 }  // namespace
