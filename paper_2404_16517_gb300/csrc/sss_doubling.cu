@@ -21,8 +21,11 @@
 // Work per round: position q starts a group from the round whose L exceeds its
 // local LCP, k*(q) = bit length of lcp[q]; positions are bucketed once by k*
 // (and equal strings by the round that covers their length), so a round only
-// touches its reps, the positions that become reps next round and the equal
-// strings that end this round -- not all n positions.
+// touches its reps -- the survivors of the previous round, which resume their
+// own state, and the fresh ones of its bucket -- and the equal strings that end
+// this round, not all n positions.  A string's approx starts as its length and
+// is written again when it retires; the top bit of its position's length then
+// marks it as done (lengths are below 2^31).
 //
 // Duplicate detection, two exact variants:
 //  * sort (the appendix's route): the (key, rep) pairs are bucketed by the key's
@@ -30,9 +33,13 @@
 //    equal neighbours mark duplicates; a bucket larger than shared memory (only
 //    with many equal keys) is sorted in chunks and cross-checked by binary search.
 //  * hash table (default; the single-shot filter of the appendix with the full
-//    64-bit key stored, so there are no false positives): keys are inserted into
-//    an open-addressing table of >= 2x slots with atomicCAS, a second insert of a
-//    key marks its slot, and each rep reads its slot's mark.
+//    64-bit key compared, so there are no false positives): an open-addressing
+//    table of >= 2x slots holds the number of the rep that took the slot
+//    (atomicCAS); a rep that finds one with its own key marks both.  With the
+//    number in the slot (4 bytes) instead of the key (8 and a mark) nothing is
+//    looked up again: for 4.19M reps the insertion, the retirement, the copy of
+//    the fresh reps and the final pass took 77 + 86 + 27 + 34 us with keys; now
+//    insertion and retirement are all, 78 + 55 us.
 #include <algorithm>
 #include <mutex>
 #include <vector>
@@ -44,7 +51,10 @@ namespace {
 
 constexpr uint64_t P61 = (1ull << 61) - 1;
 constexpr uint64_t GAMMA = 0x9E3779B97F4A7C15ull;
-constexpr uint32_t ACTIVE = 0xFFFFFFFFu;
+constexpr uint32_t ACTIVE = 0xFFFFFFFFu;  // noalloc variant: no approx yet
+constexpr uint32_t DONE_BIT = 0x80000000u;  // of a position's length: retired
+constexpr uint32_t NO_REP = 0xFFFFFFFFu;   // empty table slot
+constexpr uint8_t DUP_SKIP = 2;             // dup[]: not a rep (done before its round)
 constexpr int DD_T = 512, DD_CAP = 4096;  // dedupe bucket CTA
 constexpr int HB_MAX = 13;                // max top bits for bucketing (8192 buckets)
 constexpr int KBINS = 34;                 // rounds 0..33 for the per-position round buckets
@@ -166,10 +176,21 @@ __device__ __forceinline__ uint32_t klen_of(uint32_t len, uint32_t kmin) {
     return k > kmin ? k : kmin;
 }
 
-// per-position state; counts of the round buckets
-__global__ void k_pd_init(PdIn in, const uint32_t* __restrict__ lens, uint32_t* __restrict__ apos,
-                          uint32_t* __restrict__ lpos, uint32_t* __restrict__ hlen, uint32_t* __restrict__ cnt_ks,
-                          uint32_t* __restrict__ cnt_kl, uint32_t kmin) {
+// The reps of a round: the previous round's survivors, then the fresh ones.
+struct PdReps {
+    const uint32_t* surv;
+    uint32_t ns;
+    const uint32_t* fresh;
+    uint32_t n;  // both together
+};
+__device__ __forceinline__ uint32_t rep_of(const PdReps& r, uint32_t j) {
+    return j < r.ns ? r.surv[j] : r.fresh[j - r.ns];
+}
+
+// per-position lengths, approx = length; counts of the round buckets
+__global__ void k_pd_init(PdIn in, const uint32_t* __restrict__ lens, uint32_t* __restrict__ lpos,
+                          uint32_t* __restrict__ approx, uint32_t* __restrict__ cnt_ks, uint32_t* __restrict__ cnt_kl,
+                          uint32_t kmin) {
     __shared__ uint32_t hs[KBINS], hl[KBINS];
     for (int i = threadIdx.x; i < KBINS; i += blockDim.x) hs[i] = hl[i] = 0;
     __syncthreads();
@@ -178,9 +199,8 @@ __global__ void k_pd_init(PdIn in, const uint32_t* __restrict__ lens, uint32_t* 
     uint32_t ks = 0, kl = 0;
     if (live) {
         uint32_t len = lens[ord_of(in, q)];
-        apos[q] = ACTIVE;
         lpos[q] = len;
-        hlen[q] = 0;
+        approx[q] = lens[q];
         ks = kstar_of(in, q, kmin);
         kl = klen_of(len, kmin);
     }
@@ -301,49 +321,12 @@ __device__ __forceinline__ uint64_t fold_words(uint64_t h, const uint8_t* s, uin
     return h;
 }
 
-// B1: the key of rep q.  Horner resumes from the L/2-prefix state of the
-// previous round: the rep's own state, or (for a position that starts a group
-// only from this round on) the state of its previous group start q', which
-// shares that prefix.  Such a position also shares its first minlcp[q]
-// characters with q': the whole words among them are read from q''s string,
-// which every member of the group reads (so from L2), and only the rest from
-// its own.  States are double-buffered by round parity.  prevstart and minlcp
-// are optional (a new rep then hashes its prefix from the first word).
-// (The state pointers carry no __restrict__: k_pd_cta_rounds reads in one
-// round the states it wrote in the previous one, so they must not take the
-// read-only cache path.)
-__device__ __forceinline__ uint64_t pd_rep_key(const PdIn& in, uint32_t q, const uint32_t* __restrict__ lpos,
-                                               const uint64_t* hst_in, const uint32_t* hlen_in, uint64_t* hst_out,
-                                               uint32_t* hlen_out, const uint32_t* __restrict__ prevstart,
-                                               const uint32_t* __restrict__ minlcp, uint64_t L, uint64_t B) {
-    uint32_t s = ord_of(in, q);
-    uint32_t len = lpos[q];
-    uint32_t le = L < len ? (uint32_t)L : len;
-    const uint8_t* str = in.chars + in.offs[s];
-    uint64_t h = 0;
-    uint32_t w0 = 0, wsh = 0;
-    const uint8_t* sstr = str;
-    if (L >= 16) {
-        uint32_t src = q;
-        if (hlen_in[q] != (uint32_t)(L / 2) && prevstart) src = prevstart[q];
-        if (hlen_in[src] == (uint32_t)(L / 2)) {
-            h = hst_in[src];
-            w0 = (uint32_t)(L / 16);
-        }
-        if (src != q && minlcp) {
-            const uint32_t ml = minlcp[q];
-            wsh = (ml < le ? ml : le) / 8;
-            sstr = in.chars + in.offs[ord_of(in, src)];
-        }
-    }
-    wsh = wsh > w0 ? wsh : w0;
-    uint32_t nw = (le + 7) / 8;
-    const uint64_t B2 = mulmod61(B, B);
-    h = fold_words(h, sstr, w0, wsh, 8 * wsh, B, B2);  // whole words shared with the group start
-    h = fold_words(h, str, wsh, nw, le, B, B2);
-    hst_out[q] = h;
-    hlen_out[q] = le;
-    return smix64(h ^ ((uint64_t)le * GAMMA));
+__device__ __forceinline__ uint64_t pd_key(uint64_t h, uint32_t le) { return smix64(h ^ ((uint64_t)le * GAMMA)); }
+
+// B1: the hash state of a rep's prefix of le characters, resumed from the state
+// h of its first 8 * w0 characters.
+__device__ __forceinline__ uint64_t pd_state(const uint8_t* str, uint32_t le, uint64_t h, uint32_t w0, uint64_t B) {
+    return fold_words(h, str, w0, (le + 7) / 8, le, B, mulmod61(B, B));
 }
 
 // (a - b) mod P for a, b < P
@@ -354,7 +337,7 @@ __device__ __forceinline__ uint64_t submod61(uint64_t a, uint64_t b) { return a 
 // Horner values differ by the Horner fold of the limb differences over words
 // wsh .. nw-1 alone (the polynomial is linear in the limbs, and every limb
 // keeps its power of B).
-__device__ __forceinline__ uint64_t pd_key_from_start(const uint8_t* str, const uint8_t* sstr, uint32_t le,
+__device__ __forceinline__ uint64_t pd_state_from_start(const uint8_t* str, const uint8_t* sstr, uint32_t le,
                                                       uint32_t wsh, uint64_t hsrc, uint64_t B, uint64_t B2) {
     const uint32_t nw = (le + 7) / 8;
     uint64_t D = 0;
@@ -370,43 +353,74 @@ __device__ __forceinline__ uint64_t pd_key_from_start(const uint8_t* str, const 
     return h >= P61 ? h - P61 : h;
 }
 
-// Phase 0: every rep.  When new reps resume from their group starts (prevstart
-// given), phase 1 hashes the reps that resume their own L/2 state (the group
-// starts that are still reps) and phase 2 the others; a rep of phase 2 whose
-// group start has just been hashed to the same length finishes from that hash
-// (pd_key_from_start) instead of folding the words they share.
-__global__ void k_pd_hash(PdIn in, const uint32_t* __restrict__ reps, uint32_t nreps, const uint32_t* __restrict__ lpos,
-                          const uint64_t* __restrict__ hst_in, const uint32_t* __restrict__ hlen_in,
-                          uint64_t* hst_out, uint32_t* hlen_out, const uint32_t* __restrict__ prevstart,
-                          const uint32_t* __restrict__ minlcp, uint64_t* __restrict__ K, uint32_t* __restrict__ V,
-                          uint64_t L, uint64_t B, int phase) {
-    uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= nreps) return;
-    uint32_t q = reps[j];
-    if (phase != 0) {
-        const bool own = L >= 16 && hlen_in[q] == (uint32_t)(L / 2);
-        if ((phase == 1) != own) return;
-        if (phase == 2 && prevstart && minlcp) {
-            const uint32_t src = prevstart[q];
-            const uint32_t len = lpos[q];
-            const uint32_t le = L < len ? (uint32_t)L : len;
-            if (src != q && hlen_out[src] == le) {
-                const uint32_t ml = minlcp[q];
-                const uint32_t wsh = (ml < le ? ml : le) / 8;
-                const uint64_t B2 = mulmod61(B, B);
-                const uint64_t h = pd_key_from_start(in.chars + in.offs[ord_of(in, q)],
-                                                     in.chars + in.offs[ord_of(in, src)], le, wsh, hst_out[src], B,
-                                                     B2);
+struct PsPair {
+    uint32_t s;  // last group start + 1 (0: none yet)
+    uint32_t m;  // min run_lcp since it
+};
+__device__ __forceinline__ PsPair ps_then(PsPair a, PsPair b) {
+    return b.s ? b : PsPair{a.s, a.m < b.m ? a.m : b.m};
+}
+// The scan of previous group starts (k_pd_ps_tiles): per position within its
+// tile of 4096, and the carry into every tile.
+struct PsScan {
+    const uint32_t* s;
+    const uint32_t* m;
+    const PsPair* carry;
+};
+
+// B1: the keys of reps j0 .. j1 (survivors or fresh ones, not both).  States are
+// double-buffered by round parity.  A survivor resumes its own L/2-prefix state
+// of the previous round.  A fresh rep q starts a group only from this round on:
+// its previous group start q', whose L/2-prefix it shares, was a rep of the
+// previous round (they share L/2 characters, so q' was neither alone nor
+// shorter).  With the scan of previous starts given (survivors hashed by an
+// earlier launch), q finishes from the start's state of this round if both test
+// the same length (pd_state_from_start), else resumes the start's L/2 state,
+// reading the whole words it shares with q' from q''s string, which every member
+// of the group reads (so from L2).  Without the scan it starts from the first
+// word.
+__global__ void k_pd_hash(PdIn in, PdReps reps, uint32_t j0, uint32_t j1, const uint32_t* __restrict__ lpos,
+                          const uint64_t* __restrict__ hst_in, uint64_t* hst_out, PsScan ps, uint64_t* __restrict__ K,
+                          uint8_t* __restrict__ dup, uint64_t L, uint64_t B) {
+    const uint32_t j = j0 + blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= j1) return;
+    const uint32_t q = rep_of(reps, j);
+    const uint32_t len = lpos[q];
+    if (len & DONE_BIT) {  // an equal string that ended before its round
+        dup[j] = DUP_SKIP;
+        return;
+    }
+    dup[j] = 0;
+    const uint32_t le = L < len ? (uint32_t)L : len;
+    const uint8_t* str = in.chars + in.offs[ord_of(in, q)];
+    uint64_t h = 0;
+    uint32_t w0 = 0;
+    if (j < reps.ns) {
+        if (L >= 16) {
+            h = hst_in[q];
+            w0 = (uint32_t)(L / 16);
+        }
+    } else if (ps.s) {
+        const PsPair r = ps_then(ps.carry[q / 4096], PsPair{ps.s[q], ps.m[q]});
+        const uint32_t src = r.s ? r.s - 1 : q;  // (an earlier start always exists)
+        if (src != q) {
+            const uint8_t* sstr = in.chars + in.offs[ord_of(in, src)];
+            const uint32_t ls = lpos[src];
+            const uint32_t wsh = (r.m < le ? r.m : le) / 8;  // whole words shared with the start
+            if (!(ls & DONE_BIT) && (L < ls ? (uint32_t)L : ls) == le) {
+                h = pd_state_from_start(str, sstr, le, wsh, hst_out[src], B, mulmod61(B, B));
                 hst_out[q] = h;
-                hlen_out[q] = le;
-                K[j] = smix64(h ^ ((uint64_t)le * GAMMA));
-                V[j] = q;
+                K[j] = pd_key(h, le);
                 return;
             }
+            w0 = (uint32_t)(L / 16);
+            h = fold_words(hst_in[src], sstr, w0, wsh, 8 * wsh, B, mulmod61(B, B));
+            w0 = wsh > w0 ? wsh : w0;
         }
     }
-    K[j] = pd_rep_key(in, q, lpos, hst_in, hlen_in, hst_out, hlen_out, prevstart, minlcp, L, B);
-    V[j] = q;
+    h = pd_state(str, le, h, w0, B);
+    hst_out[q] = h;
+    K[j] = pd_key(h, le);
 }
 
 // prevstart[q] = last position q' <= q that starts a group in round k-1
@@ -415,14 +429,7 @@ __global__ void k_pd_hash(PdIn in, const uint32_t* __restrict__ reps, uint32_t n
 // pairs (last start + 1, min since it) with the operator
 //     (s1, m1) then (s2, m2) = s2 ? (s2, m2) : (s1, min(m1, m2)):
 // tiles of 4096 positions (4 per thread, warp shuffles, warp totals in shared
-// memory), then the carry of earlier tiles.
-struct PsPair {
-    uint32_t s;  // last group start + 1 (0: none yet)
-    uint32_t m;  // min run_lcp since it
-};
-__device__ __forceinline__ PsPair ps_then(PsPair a, PsPair b) {
-    return b.s ? b : PsPair{a.s, a.m < b.m ? a.m : b.m};
-}
+// memory), then the carry of earlier tiles, which the reader adds.
 
 __global__ void __launch_bounds__(1024) k_pd_ps_tiles(PdIn in, uint32_t kprev, uint32_t kmin,
                                                       uint32_t* __restrict__ out_s, uint32_t* __restrict__ out_m,
@@ -514,22 +521,15 @@ __global__ void __launch_bounds__(1024) k_pd_ps_carry(PsPair* __restrict__ tagg,
     }
 }
 
-__global__ void k_pd_ps_apply(uint32_t n, uint32_t* __restrict__ out_s, uint32_t* __restrict__ out_m,
-                              const PsPair* __restrict__ tagg) {
-    const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n) return;
-    const PsPair r = ps_then(tagg[q / 4096], PsPair{out_s[q], out_m[q]});
-    out_s[q] = r.s ? r.s - 1 : q;  // no earlier start (cannot happen): itself
-    out_m[q] = r.s ? r.m : 0u;
-}
-
 // B2: bucket the keys by their top bits
-__global__ void k_pd_hist(const uint64_t* __restrict__ K, uint32_t m, uint32_t bits, uint32_t* __restrict__ hist) {
+__global__ void k_pd_hist(const uint64_t* __restrict__ K, const uint8_t* __restrict__ dup, uint32_t m, uint32_t bits,
+                          uint32_t* __restrict__ hist) {
     __shared__ uint32_t sh[1u << HB_MAX];
     uint32_t nb = 1u << bits;
     for (uint32_t i = threadIdx.x; i < nb; i += blockDim.x) sh[i] = 0;
     __syncthreads();
     for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < m; j += gridDim.x * blockDim.x) {
+        if (dup[j] == DUP_SKIP) continue;
         uint32_t b = bits ? (uint32_t)(K[j] >> (64 - bits)) : 0u;
         atomicAdd(&sh[b], 1u);
     }
@@ -564,16 +564,16 @@ __global__ void __launch_bounds__(1024) k_pd_scan(uint32_t* __restrict__ hist, u
     if (threadIdx.x == 0) bstart[nb] = total;
 }
 
-__global__ void k_pd_scatter(const uint64_t* __restrict__ K, const uint32_t* __restrict__ V, uint32_t m, uint32_t bits,
+__global__ void k_pd_scatter(const uint64_t* __restrict__ K, const uint8_t* __restrict__ dup, uint32_t m, uint32_t bits,
                              const uint32_t* __restrict__ bstart, uint32_t* __restrict__ cursor,
                              uint64_t* __restrict__ tK, uint32_t* __restrict__ tV) {
     uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= m) return;
+    if (j >= m || dup[j] == DUP_SKIP) return;
     uint64_t k = K[j];
     uint32_t b = bits ? (uint32_t)(k >> (64 - bits)) : 0u;
     uint32_t dst = bstart[b] + atomicAdd(&cursor[b], 1u);
     tK[dst] = k;
-    tV[dst] = V[j];
+    tV[dst] = j;
 }
 
 __device__ __forceinline__ bool bsearch64(const uint64_t* a, uint32_t m, uint64_t k) {
@@ -587,7 +587,7 @@ __device__ __forceinline__ bool bsearch64(const uint64_t* a, uint32_t m, uint64_
     return false;
 }
 
-// B3: one CTA per bucket; dupf[rep position] = key occurs more than once
+// B3: one CTA per bucket; dupf[rep number] = key occurs more than once
 __global__ void __launch_bounds__(DD_T) k_pd_buckets(const uint32_t* __restrict__ bstart, uint64_t* __restrict__ tK,
                                                      uint32_t* __restrict__ tV, uint8_t* __restrict__ dupf) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -663,23 +663,24 @@ __global__ void __launch_bounds__(DD_T) k_pd_buckets(const uint32_t* __restrict_
     }
 }
 
-// B2/B3, hash-table variant: insert every rep key; a second copy marks the slot
-__global__ void k_pd_ht_insert(const uint64_t* __restrict__ K, uint32_t m, unsigned long long* __restrict__ tab,
-                               uint8_t* __restrict__ mark, uint32_t tmask, uint32_t* __restrict__ zero_cnt,
-                               unsigned* err) {
-    uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= m) return;
-    uint64_t k = K[j];
-    if (k == 0) {  // 0 marks an empty slot: count zero keys apart
-        atomicAdd(zero_cnt, 1u);
-        return;
-    }
+// B2/B3, hash-table variant: every rep takes a slot with its number; one that
+// finds a rep with its own key marks both.  A slot's bits above the number's ib
+// hold the key's top ones: only where they agree is the other key looked up
+// (78 us for 4.19M reps; 93 us when every collision reads a key).
+__global__ void k_pd_ht_insert(const uint64_t* __restrict__ K, uint32_t m, uint32_t* __restrict__ tab, uint32_t tmask,
+                               uint32_t ib, uint8_t* dup, unsigned* err) {
+    const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= m || dup[j] == DUP_SKIP) return;
+    const uint64_t k = K[j];
+    const uint32_t tag = ib < 32u ? (uint32_t)(k >> (32u + ib)) << ib : 0u;
+    const uint32_t imask = ib < 32u ? (1u << ib) - 1u : ~0u;
     uint32_t h = (uint32_t)k & tmask;
     for (uint32_t i = 0; i <= tmask; ++i) {
-        unsigned long long old = atomicCAS(&tab[h], 0ull, (unsigned long long)k);
-        if (old == 0ull) return;
-        if (old == k) {
-            mark[h] = 1;
+        const uint32_t old = atomicCAS(&tab[h], NO_REP, tag | j);
+        if (old == NO_REP) return;
+        if ((old & ~imask) == tag && K[old & imask] == k) {
+            dup[old & imask] = 1;
+            dup[j] = 1;
             return;
         }
         h = (h + 1) & tmask;
@@ -701,75 +702,52 @@ __device__ __forceinline__ bool ht_dup(const unsigned long long* tab, const uint
 }
 
 // B4: retire the reps whose group is one string with a unique key (or whose
-// length <= L); survivors stay reps next round.
-__global__ void __launch_bounds__(PD_T) k_pd_retire(PdIn in, const uint32_t* __restrict__ reps, uint32_t nreps,
-                            const uint32_t* __restrict__ lpos, const uint64_t* __restrict__ K,
-                            const uint8_t* __restrict__ dupf, const unsigned long long* __restrict__ tab,
-                            const uint8_t* __restrict__ mark, uint32_t tmask, const uint32_t* __restrict__ zero_cnt,
-                            uint32_t* __restrict__ apos, uint32_t* __restrict__ reps_next,
-                            uint32_t* __restrict__ cnt, uint64_t L, int use_ht) {
-    uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+// length <= L); the others survive into the next round.
+__global__ void __launch_bounds__(PD_T) k_pd_retire(PdIn in, PdReps reps, uint32_t* __restrict__ lpos,
+                                                    const uint8_t* __restrict__ dupf, uint32_t* __restrict__ approx,
+                                                    uint32_t* __restrict__ surv_next, uint32_t* __restrict__ cnt,
+                                                    uint64_t L) {
+    const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
     bool keep = false;
     uint32_t q = 0, retired = 0;
-    if (j < nreps) {
-        q = reps[j];
-        uint32_t len = lpos[q];
-        bool single = true;
-        if (in.run_lcp) {
-            uint32_t pe = part_end_of(q, in.n, in.p);
-            single = !(q + 1 < pe && in.run_lcp[q + 1] >= L);
-        }
-        bool dup = !single;
-        if (!dup) dup = use_ht ? ht_dup(tab, mark, tmask, *zero_cnt, K[j]) : (dupf[q] != 0);
-        if (!dup || (uint64_t)len <= L) {
-            apos[q] = (uint64_t)len < L ? len : (uint32_t)L;
-            retired = 1;
-        } else {
-            keep = true;
+    if (j < reps.n) {
+        const uint8_t df = dupf[j];
+        if (df != DUP_SKIP) {
+            q = rep_of(reps, j);
+            const uint32_t len = lpos[q];
+            bool dup = df != 0;
+            if (!dup && in.run_lcp)
+                dup = q + 1 < part_end_of(q, in.n, in.p) && in.run_lcp[q + 1] >= L;  // not alone in its group
+            if (!dup || (uint64_t)len <= L) {
+                if (L < len) approx[ord_of(in, q)] = (uint32_t)L;
+                lpos[q] = len | DONE_BIT;
+                retired = 1;
+            } else {
+                keep = true;
+            }
         }
     }
     __shared__ uint32_t sh[PD_T / 32];
-    block_append<PD_T>(keep, q, reps_next, &cnt[0], sh);
+    block_append<PD_T>(keep, q, surv_next, &cnt[0], sh);
     block_count<PD_T>(retired, &cnt[1], sh);
 }
 
 // strings equal to their local predecessor whose whole length is tested this
 // round: duplicates that retire with approx = len
-__global__ void __launch_bounds__(PD_T) k_pd_retire_equal(const uint32_t* __restrict__ list, uint32_t m, const uint32_t* __restrict__ lpos,
-                                  uint32_t* __restrict__ apos, uint32_t* __restrict__ cnt) {
+__global__ void __launch_bounds__(PD_T) k_pd_retire_equal(const uint32_t* __restrict__ list, uint32_t m,
+                                                          uint32_t* __restrict__ lpos, uint32_t* __restrict__ cnt) {
     uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
     uint32_t retired = 0;
     if (j < m) {
         uint32_t q = list[j];
-        if (apos[q] == ACTIVE) {
-            apos[q] = lpos[q];
+        const uint32_t len = lpos[q];
+        if (!(len & DONE_BIT)) {
+            lpos[q] = len | DONE_BIT;
             retired = 1;
         }
     }
     __shared__ uint32_t sh[PD_T / 32];
     block_count<PD_T>(retired, &cnt[1], sh);
-}
-
-// positions that start a group from the next round on become reps (if active)
-__global__ void __launch_bounds__(PD_T) k_pd_newreps(const uint32_t* __restrict__ list, uint32_t m, const uint32_t* __restrict__ apos,
-                             uint32_t* __restrict__ reps_next, uint32_t* __restrict__ cnt) {
-    uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-    bool want = false;
-    uint32_t q = 0;
-    if (j < m) {
-        q = list[j];
-        want = apos[q] == ACTIVE;
-    }
-    __shared__ uint32_t sh[PD_T / 32];
-    block_append<PD_T>(want, q, reps_next, &cnt[0], sh);
-}
-
-__global__ void k_pd_final(PdIn in, const uint32_t* __restrict__ apos, const uint32_t* __restrict__ lpos,
-                           uint32_t* __restrict__ approx) {
-    uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= in.n) return;
-    uint32_t a = apos[q];
-    approx[ord_of(in, q)] = a == ACTIVE ? lpos[q] : a;
 }
 
 // Offsets of the per-position round buckets (by the round a position starts a
@@ -780,40 +758,47 @@ struct PdOffs {
 };
 
 // Rounds k0..k1 in one CTA, for rounds whose reps number at most CR_CAP: the
-// same steps as k_pd_hash, k_pd_ht_insert, k_pd_retire, k_pd_retire_equal and
-// k_pd_newreps, with the hash table, the keys and the rep lists in shared
-// memory and __syncthreads between the steps instead of kernel boundaries and a
-// host round trip.  The host picks k1 so that no round holds more than CR_CAP
-// reps (the reps of round k are at most the reps of round k0 plus the
-// positions whose group starts in rounds k0+1..k).  On return the next round's
-// reps are in reps_out, their count in cnt[0], and cnt[1] has grown by the
-// strings retired.  States are read and written in the global double buffers
-// with the same round parity as the per-round kernels.
+// same steps as k_pd_hash, k_pd_ht_insert, k_pd_retire and k_pd_retire_equal,
+// with the hash table, the keys and the rep lists in shared memory and
+// __syncthreads between the steps instead of kernel boundaries and a host round
+// trip.  The host picks k1 so that no round holds more than CR_CAP reps (the
+// reps of round k are at most the reps of round k0 plus the positions whose
+// group starts in rounds k0+1..k).  A list holds a round's survivors first, then
+// the fresh reps.  On return the survivors are in surv_out, their count in
+// cnt[0], and cnt[1] has grown by the strings retired.  States are read and
+// written in the global double buffers with the same round parity as the
+// per-round kernels.
 constexpr int CR_T = 1024, CR_CAP = 4096;
 constexpr size_t CR_SMEM = (size_t)CR_CAP * 8 + (size_t)2 * CR_CAP * 8 + (size_t)2 * CR_CAP * 4 + (size_t)2 * CR_CAP;
 
-__global__ void __launch_bounds__(CR_T) k_pd_cta_rounds(PdIn in, const uint32_t* __restrict__ reps0, uint32_t nreps0,
-                                                         uint32_t k0, uint32_t k1, uint32_t kmin, uint32_t kmax,
-                                                         const PdOffs off, const uint32_t* __restrict__ list_ks,
-                                                         const uint32_t* __restrict__ list_kl,
-                                                         const uint32_t* __restrict__ lpos, uint64_t* hst,
-                                                         uint32_t* hlen, uint64_t* hst2, uint32_t* hlen2,
-                                                         uint32_t* apos, uint32_t* __restrict__ reps_out,
-                                                         uint32_t* __restrict__ cnt, uint64_t B, unsigned* err) {
+__global__ void __launch_bounds__(CR_T) k_pd_cta_rounds(PdIn in, const PdReps reps0, uint32_t k0, uint32_t k1,
+                                                         uint32_t kmin, const PdOffs off,
+                                                         const uint32_t* __restrict__ list_ks,
+                                                         const uint32_t* __restrict__ list_kl, uint32_t* lpos,
+                                                         uint64_t* hst, uint64_t* hst2, uint32_t* __restrict__ approx,
+                                                         uint32_t* __restrict__ surv_out, uint32_t* __restrict__ cnt,
+                                                         uint64_t B, unsigned* err) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t* sK = reinterpret_cast<uint64_t*>(smem);                                // CR_CAP keys
     unsigned long long* tab = reinterpret_cast<unsigned long long*>(sK + CR_CAP);    // 2 CR_CAP slots
     uint32_t* lst0 = reinterpret_cast<uint32_t*>(tab + 2 * CR_CAP);                  // CR_CAP
     uint32_t* lst1 = lst0 + CR_CAP;                                                  // CR_CAP
     uint8_t* mark = reinterpret_cast<uint8_t*>(lst1 + CR_CAP);                       // 2 CR_CAP
-    __shared__ uint32_t s_n[2], s_zero, s_ret, s_ovf;
+    __shared__ uint32_t s_n[2], s_ns, s_zero, s_ret, s_ovf;
     const uint32_t tid = threadIdx.x;
-    const uint32_t n0 = nreps0 < (uint32_t)CR_CAP ? nreps0 : (uint32_t)CR_CAP;
-    for (uint32_t i = tid; i < n0; i += CR_T) lst0[i] = reps0[i];
     if (tid == 0) {
-        s_n[0] = n0;
+        s_n[0] = s_ns = reps0.ns < (uint32_t)CR_CAP ? reps0.ns : (uint32_t)CR_CAP;
         s_ret = 0;
-        s_ovf = nreps0 > (uint32_t)CR_CAP;
+        s_ovf = reps0.n > (uint32_t)CR_CAP;
+    }
+    __syncthreads();
+    for (uint32_t i = tid; i < s_ns; i += CR_T) lst0[i] = reps0.surv[i];
+    for (uint32_t i = reps0.ns + tid; i < reps0.n; i += CR_T) {
+        const uint32_t q = rep_of(reps0, i);
+        if (lpos[q] & DONE_BIT) continue;
+        const uint32_t at = atomicAdd(&s_n[0], 1u);
+        if (at < (uint32_t)CR_CAP) lst0[at] = q;
+        else s_ovf = 1;
     }
     __syncthreads();
     uint32_t cur = 0;
@@ -821,7 +806,7 @@ __global__ void __launch_bounds__(CR_T) k_pd_cta_rounds(PdIn in, const uint32_t*
         const uint64_t L = 1ull << k;
         uint32_t* lc = cur ? lst1 : lst0;
         uint32_t* ln = cur ? lst0 : lst1;
-        const uint32_t nr = s_n[cur];
+        const uint32_t nr = s_n[cur] < (uint32_t)CR_CAP ? s_n[cur] : (uint32_t)CR_CAP, ns = s_ns;
         uint32_t T = 1024;
         while (T < 2u * nr) T <<= 1;
         const uint32_t tmask = T - 1;
@@ -836,27 +821,30 @@ __global__ void __launch_bounds__(CR_T) k_pd_cta_rounds(PdIn in, const uint32_t*
         __syncthreads();
         const bool odd = ((k - kmin) & 1u) != 0;
         const uint64_t* hs_in = odd ? hst2 : hst;
-        const uint32_t* hl_in = odd ? hlen2 : hlen;
         uint64_t* hs_out = odd ? hst : hst2;
-        uint32_t* hl_out = odd ? hlen : hlen2;
         // keys of the reps, inserted into the table (a second copy marks its slot)
         for (uint32_t j = tid; j < nr; j += CR_T) {
-            const uint64_t key =
-                pd_rep_key(in, lc[j], lpos, hs_in, hl_in, hs_out, hl_out, nullptr, nullptr, L, B);
+            const uint32_t q = lc[j], len = lpos[q];
+            const uint32_t le = L < len ? (uint32_t)L : len;
+            const bool own = j < ns && L >= 16;  // a survivor resumes its L/2-prefix state
+            const uint64_t h = pd_state(in.chars + in.offs[ord_of(in, q)], le, own ? hs_in[q] : 0ull,
+                                        own ? (uint32_t)(L / 16) : 0u, B);
+            hs_out[q] = h;
+            const uint64_t key = pd_key(h, le);
             sK[j] = key;
             if (key == 0) {
                 atomicAdd(&s_zero, 1u);
                 continue;
             }
-            uint32_t h = (uint32_t)key & tmask;
+            uint32_t t = (uint32_t)key & tmask;
             for (uint32_t i = 0; i <= tmask; ++i) {
-                const unsigned long long old = atomicCAS(&tab[h], 0ull, (unsigned long long)key);
+                const unsigned long long old = atomicCAS(&tab[t], 0ull, (unsigned long long)key);
                 if (old == 0ull) break;
                 if (old == key) {
-                    mark[h] = 1;
+                    mark[t] = 1;
                     break;
                 }
-                h = (h + 1) & tmask;
+                t = (t + 1) & tmask;
             }
         }
         __syncthreads();
@@ -870,24 +858,10 @@ __global__ void __launch_bounds__(CR_T) k_pd_cta_rounds(PdIn in, const uint32_t*
                 const uint32_t pe = part_end_of(q, in.n, in.p);
                 dup = q + 1 < pe && in.run_lcp[q + 1] >= L;
             }
-            if (!dup) {
-                const uint64_t key = sK[j];
-                if (key == 0) {
-                    dup = s_zero > 1;
-                } else {
-                    uint32_t h = (uint32_t)key & tmask;
-                    for (uint32_t i = 0; i <= tmask; ++i) {
-                        const uint64_t t = tab[h];
-                        if (t == key) {
-                            dup = mark[h] != 0;
-                            break;
-                        }
-                        h = (h + 1) & tmask;
-                    }
-                }
-            }
+            if (!dup) dup = ht_dup(tab, mark, tmask, s_zero, sK[j]);
             if (!dup || (uint64_t)len <= L) {
-                apos[q] = (uint64_t)len < L ? len : (uint32_t)L;
+                if (L < len) approx[ord_of(in, q)] = (uint32_t)L;
+                lpos[q] = len | DONE_BIT;
                 atomicAdd(&s_ret, 1u);
             } else {
                 const uint32_t at = atomicAdd(&s_n[cur ^ 1], 1u);
@@ -898,18 +872,21 @@ __global__ void __launch_bounds__(CR_T) k_pd_cta_rounds(PdIn in, const uint32_t*
         // strings equal to their local predecessor whose whole length is tested now
         for (uint32_t j = off.kl[k] + tid; j < off.kl[k + 1]; j += CR_T) {
             const uint32_t q = list_kl[j];
-            if (apos[q] == ACTIVE) {
-                apos[q] = lpos[q];
+            const uint32_t len = lpos[q];
+            if (!(len & DONE_BIT)) {
+                lpos[q] = len | DONE_BIT;
                 atomicAdd(&s_ret, 1u);
             }
         }
         __syncthreads();
+        if (tid == 0) s_ns = s_n[cur ^ 1];
+        __syncthreads();
         // positions that start a group from the next round on become reps
-        // (after the last round k1 the host appends them)
+        // (after the last round k1 they are the caller's)
         if (k < k1) {
             for (uint32_t j = off.ks[k + 1] + tid; j < off.ks[k + 2]; j += CR_T) {
                 const uint32_t q = list_ks[j];
-                if (apos[q] == ACTIVE) {
+                if (!(lpos[q] & DONE_BIT)) {
                     const uint32_t at = atomicAdd(&s_n[cur ^ 1], 1u);
                     if (at < (uint32_t)CR_CAP) ln[at] = q;
                     else s_ovf = 1;
@@ -921,7 +898,7 @@ __global__ void __launch_bounds__(CR_T) k_pd_cta_rounds(PdIn in, const uint32_t*
     }
     const uint32_t nr = s_n[cur] < (uint32_t)CR_CAP ? s_n[cur] : (uint32_t)CR_CAP;
     const uint32_t* lc = cur ? lst1 : lst0;
-    for (uint32_t j = tid; j < nr; j += CR_T) reps_out[j] = lc[j];
+    for (uint32_t j = tid; j < nr; j += CR_T) surv_out[j] = lc[j];
     if (tid == 0) {
         cnt[0] = nr;
         cnt[1] += s_ret;
@@ -930,23 +907,17 @@ __global__ void __launch_bounds__(CR_T) k_pd_cta_rounds(PdIn in, const uint32_t*
 }
 
 struct PdBufs {
-    uint32_t* apos;
     uint32_t* lpos;
-    uint32_t* hlen;
     uint64_t* hst;
-    uint32_t* hlen2;
     uint64_t* hst2;
     uint32_t* prevstart;
     uint32_t* minlcp;
     PsPair* tagg;
     uint32_t* list_ks;
     uint32_t* list_kl;
-    uint32_t* reps[2];
-    unsigned long long* tab;
-    uint8_t* mark;
-    uint32_t tcap;
+    uint32_t* surv[2];
+    uint32_t* tab;
     uint64_t* K;
-    uint32_t* V;
     uint64_t* tK;
     uint32_t* tV;
     uint8_t* dupf;
@@ -957,21 +928,17 @@ struct PdBufs {
 };
 
 void carve_pd(Arena& ar, uint32_t n, PdBufs& b) {
-    b.apos = ar.take<uint32_t>(n);
     b.lpos = ar.take<uint32_t>(n);
-    b.hlen = ar.take<uint32_t>(n);
     b.hst = ar.take<uint64_t>(n);
-    b.hlen2 = ar.take<uint32_t>(n);
     b.hst2 = ar.take<uint64_t>(n);
     b.prevstart = ar.take<uint32_t>(n);
     b.minlcp = ar.take<uint32_t>(n);
     b.tagg = ar.take<PsPair>(n / 4096 + 2);
     b.list_ks = ar.take<uint32_t>(n);
     b.list_kl = ar.take<uint32_t>(n);
-    b.reps[0] = ar.take<uint32_t>(n);
-    b.reps[1] = ar.take<uint32_t>(n);
+    b.surv[0] = ar.take<uint32_t>(n);
+    b.surv[1] = ar.take<uint32_t>(n);
     b.K = ar.take<uint64_t>(n);
-    b.V = ar.take<uint32_t>(n);
     b.tK = ar.take<uint64_t>(n);
     b.tV = ar.take<uint32_t>(n);
     b.dupf = ar.take<uint8_t>(n);
@@ -979,10 +946,9 @@ void carve_pd(Arena& ar, uint32_t n, PdBufs& b) {
     b.bstart = ar.take<uint32_t>((1u << HB_MAX) + 1);
     b.cursor = ar.take<uint32_t>((1u << HB_MAX) + 1);
     b.cnt = ar.take<uint32_t>(8 + 4 * KBINS);
-    b.tcap = 1024;
-    while (b.tcap < 2ull * n) b.tcap <<= 1;
-    b.tab = ar.take<unsigned long long>(b.tcap);
-    b.mark = ar.take<uint8_t>(b.tcap);
+    size_t slots = 1024;
+    while (slots < 2ull * n) slots <<= 1;
+    b.tab = ar.take<uint32_t>(slots);
 }
 
 uint64_t host_smix(uint64_t z) { return smix64(z); }
@@ -1019,23 +985,21 @@ sss_status impl_dist_prefix(sss_ctx* ctx, Arena& ar, const StrIn& sin, const uin
     void* pin;
     SSS_TRY(sss_pinned(ctx, sizeof(uint32_t) * (8 + 4 * KBINS), &pin));
     uint32_t* h = static_cast<uint32_t*>(pin);
-    uint32_t* cnt = B.cnt;                  // [0] reps next, [1] retired, [2] zero keys
+    uint32_t* cnt = B.cnt;                  // [0] survivors, [1] retired
     uint32_t* cnt_ks = B.cnt + 8;           // KBINS
     uint32_t* cnt_kl = cnt_ks + KBINS;      // KBINS
     uint32_t* cur_ks = cnt_kl + KBINS;      // KBINS
     uint32_t* cur_kl = cur_ks + KBINS;      // KBINS
 
     SSS_CUDA(cudaMemsetAsync(B.cnt, 0, sizeof(uint32_t) * (8 + 4 * KBINS), ctx->stream));
-    SSS_CUDA(cudaMemsetAsync(B.hlen2, 0, sizeof(uint32_t) * n, ctx->stream));
-    SSS_TRY(sss_launch(ctx, "pd_init", k_pd_init, dim3((n + 255) / 256), dim3(256), 0, in, sin.lens, B.apos, B.lpos,
-                       B.hlen, cnt_ks, cnt_kl, kmin));
-    if (kmin > kmax) {
-        return sss_launch(ctx, "pd_final", k_pd_final, dim3((n + 255) / 256), dim3(256), 0, in,
-                          (const uint32_t*)B.apos, (const uint32_t*)B.lpos, approx);
-    }
+    SSS_TRY(sss_launch(ctx, "pd_init", k_pd_init, dim3((n + 255) / 256), dim3(256), 0, in, sin.lens, B.lpos, approx,
+                       cnt_ks, cnt_kl, kmin));
+    if (kmin > kmax) return SSS_OK;  // no rounds: approx = length
     SSS_CUDA(cudaMemcpyAsync(h, cnt_ks, sizeof(uint32_t) * 2 * KBINS, cudaMemcpyDeviceToHost, ctx->stream));
     SSS_CUDA(cudaStreamSynchronize(ctx->stream));
-    uint32_t ks_off[KBINS + 1], kl_off[KBINS + 1];
+    PdOffs offs;
+    uint32_t* ks_off = offs.ks;
+    uint32_t* kl_off = offs.kl;
     ks_off[0] = kl_off[0] = 0;
     for (int i = 0; i < KBINS; ++i) {
         ks_off[i + 1] = ks_off[i] + h[i];
@@ -1049,125 +1013,88 @@ sss_status impl_dist_prefix(sss_ctx* ctx, Arena& ar, const StrIn& sin, const uin
     SSS_TRY(sss_upload(ctx, cur_ks, h, sizeof(uint32_t) * 2 * KBINS));
     SSS_TRY(sss_launch(ctx, "pd_lists", k_pd_lists, dim3((n + 256 * PL_ITEMS - 1) / (256 * PL_ITEMS)), dim3(256), 0,
                        in, (const uint32_t*)B.lpos, cur_ks, cur_kl, B.list_ks, B.list_kl, kmin));
-    // the first round's reps are the positions that start a group at L = 2^kmin
-    const uint32_t* reps = B.list_ks + ks_off[kmin];
-    uint32_t nreps = ks_off[kmin + 1] - ks_off[kmin];
-    uint32_t retired = 0;
+    const uint32_t* surv = B.surv[1];
+    uint32_t ns = 0, retired = 0;
     int nxt = 0;
-    PdOffs offs;
-    for (int i = 0; i <= KBINS; ++i) {
-        offs.ks[i] = ks_off[i];
-        offs.kl[i] = kl_off[i];
-    }
     const bool cta_rounds = use_ht && !(prm.flags & SSS_FLAG_NO_CTA_ROUNDS);
     for (uint32_t k = kmin; k <= kmax && retired < n; ++k) {
         const uint64_t L = 1ull << k;
-        uint32_t tmask = 0;
-        if (cta_rounds && nreps <= (uint32_t)CR_CAP) {
-            // this round and the following ones while their reps stay few: one
-            // CTA; the reps that join in the round after the last one are
-            // appended by k_pd_newreps (they may be many)
+        const uint32_t nf = ks_off[k + 1] - ks_off[k];  // fresh reps (the ones done by now skip the round)
+        const PdReps reps{surv, ns, B.list_ks + ks_off[k], ns + nf};
+        if (cta_rounds && reps.n <= (uint32_t)CR_CAP) {
+            // this round and the following ones while their reps stay few: one CTA
             uint32_t k1 = k;
-            while (k1 < kmax && (uint64_t)nreps + (ks_off[k1 + 2] - ks_off[k + 1]) <= (uint64_t)CR_CAP) ++k1;
+            while (k1 < kmax && (uint64_t)reps.n + (ks_off[k1 + 2] - ks_off[k + 1]) <= (uint64_t)CR_CAP) ++k1;
             if (!g_cr_attr[ctx->device & 63]) {
                 SSS_CUDA(cudaFuncSetAttribute(k_pd_cta_rounds, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)CR_SMEM));
                 g_cr_attr[ctx->device & 63] = true;
             }
-            SSS_TRY(sss_launch(ctx, "pd_cta_rounds", k_pd_cta_rounds, dim3(1), dim3(CR_T), CR_SMEM, in, reps, nreps,
-                               k, k1, kmin, kmax, offs, (const uint32_t*)B.list_ks, (const uint32_t*)B.list_kl,
-                               (const uint32_t*)B.lpos, B.hst, B.hlen, B.hst2, B.hlen2, B.apos, B.reps[nxt], cnt, Bh,
-                               ctx->d_err));
-            if (k1 < kmax) {
-                const uint32_t nn = ks_off[k1 + 2] - ks_off[k1 + 1];
-                SSS_TRY(sss_launch(ctx, "pd_newreps", k_pd_newreps, dim3((nn + PD_T - 1) / PD_T), dim3(PD_T), 0,
-                                   (const uint32_t*)(B.list_ks + ks_off[k1 + 1]), nn, (const uint32_t*)B.apos,
-                                   B.reps[nxt], cnt));
-            }
-            SSS_CUDA(cudaMemcpyAsync(h, cnt, sizeof(uint32_t) * 2, cudaMemcpyDeviceToHost, ctx->stream));
-            SSS_CUDA(cudaStreamSynchronize(ctx->stream));
-            nreps = h[0];
-            retired = h[1];
-            reps = B.reps[nxt];
-            nxt ^= 1;
+            SSS_TRY(sss_launch(ctx, "pd_cta_rounds", k_pd_cta_rounds, dim3(1), dim3(CR_T), CR_SMEM, in, reps, k, k1,
+                               kmin, offs, (const uint32_t*)B.list_ks, (const uint32_t*)B.list_kl, B.lpos, B.hst,
+                               B.hst2, approx, B.surv[nxt], cnt, Bh, ctx->d_err));
             k = k1;
-            continue;
-        }
-        if (nreps > 0) {
-            // many positions start a group only from this round on: locate their
-            // previous group start, whose L/2-prefix state they share
-            const uint32_t nnew = k > kmin ? ks_off[k + 1] - ks_off[k] : 0;
-            const uint32_t* ps = nullptr;
-            if (run_lcp && k >= 4 && k > kmin && nnew > n / 16) {
-                uint32_t nt = (n + 4095) / 4096;
-                SSS_TRY(sss_launch(ctx, "pd_prevstart", k_pd_ps_tiles, dim3(nt), dim3(1024), 0, in, k - 1, kmin,
-                                   B.prevstart, B.minlcp, B.tagg));
-                SSS_TRY(sss_launch(ctx, "pd_prevstart_carry", k_pd_ps_carry, dim3(1), dim3(1024), 0, B.tagg, nt));
-                SSS_TRY(sss_launch(ctx, "pd_prevstart_apply", k_pd_ps_apply, dim3((n + 255) / 256), dim3(256), 0, n,
-                                   B.prevstart, B.minlcp, (const PsPair*)B.tagg));
-                ps = B.prevstart;
+        } else {
+            if (reps.n > 0) {
+                // many fresh reps: locate their previous group starts, whose state they share
+                PsScan ps{nullptr, nullptr, nullptr};
+                if (run_lcp && k >= 4 && k > kmin && nf > n / 16) {
+                    const uint32_t nt = (n + 4095) / 4096;
+                    SSS_TRY(sss_launch(ctx, "pd_prevstart", k_pd_ps_tiles, dim3(nt), dim3(1024), 0, in, k - 1, kmin,
+                                       B.prevstart, B.minlcp, B.tagg));
+                    SSS_TRY(sss_launch(ctx, "pd_prevstart_carry", k_pd_ps_carry, dim3(1), dim3(1024), 0, B.tagg, nt));
+                    ps = PsScan{B.prevstart, B.minlcp, B.tagg};
+                }
+                const bool odd = ((k - kmin) & 1u) != 0;
+                const uint64_t* hs_in = odd ? B.hst2 : B.hst;
+                uint64_t* hs_out = odd ? B.hst : B.hst2;
+                // with previous starts the survivors go first: the fresh reps finish from their states
+                const uint32_t cut[3] = {0, ps.s ? ns : reps.n, reps.n};
+                for (int i = 0; i < 2; ++i)
+                    if (cut[i + 1] > cut[i])
+                        SSS_TRY(sss_launch(ctx, "pd_hash", k_pd_hash, dim3((cut[i + 1] - cut[i] + 255) / 256),
+                                           dim3(256), 0, in, reps, cut[i], cut[i + 1], (const uint32_t*)B.lpos, hs_in,
+                                           hs_out, ps, B.K, B.dupf, L, Bh));
+                if (use_ht) {
+                    uint32_t T = 1024;
+                    while (T < 2ull * reps.n) T <<= 1;
+                    uint32_t ib = 1;  // reps.n < 2^ib: no number of all ones, so no slot like an empty one
+                    while (ib < 32 && (reps.n >> ib) != 0) ++ib;
+                    SSS_CUDA(cudaMemsetAsync(B.tab, 0xFF, sizeof(uint32_t) * T, ctx->stream));
+                    SSS_TRY(sss_launch(ctx, "pd_ht_insert", k_pd_ht_insert, dim3((reps.n + 255) / 256), dim3(256), 0,
+                                       (const uint64_t*)B.K, reps.n, B.tab, T - 1, ib, B.dupf, ctx->d_err));
+                } else {
+                    uint32_t bits = 0;
+                    while (bits < (uint32_t)HB_MAX && ((uint64_t)reps.n >> bits) > 1024) ++bits;
+                    uint32_t nb = 1u << bits;
+                    SSS_CUDA(cudaMemsetAsync(B.hist, 0, sizeof(uint32_t) * (nb + 1), ctx->stream));
+                    uint32_t hgrid = std::min<uint32_t>((reps.n + 4095) / 4096, 2u * (uint32_t)ctx->sm_count);
+                    SSS_TRY(sss_launch(ctx, "pd_hist", k_pd_hist, dim3(hgrid), dim3(512), 0, (const uint64_t*)B.K,
+                                       (const uint8_t*)B.dupf, reps.n, bits, B.hist));
+                    SSS_TRY(sss_launch(ctx, "pd_scan", k_pd_scan, dim3(1), dim3(1024), 0, B.hist, nb, B.bstart,
+                                       B.cursor));
+                    SSS_TRY(sss_launch(ctx, "pd_scatter", k_pd_scatter, dim3((reps.n + 255) / 256), dim3(256), 0,
+                                       (const uint64_t*)B.K, (const uint8_t*)B.dupf, reps.n, bits,
+                                       (const uint32_t*)B.bstart, B.cursor, B.tK, B.tV));
+                    SSS_TRY(sss_launch(ctx, "pd_buckets", k_pd_buckets, dim3(nb), dim3(DD_T),
+                                       (size_t)DD_CAP * (8 + 8 + 1), (const uint32_t*)B.bstart, B.tK, B.tV, B.dupf));
+                }
             }
-            const bool odd = ((k - kmin) & 1u) != 0;
-            uint64_t* hs_in = odd ? B.hst2 : B.hst;
-            uint32_t* hl_in = odd ? B.hlen2 : B.hlen;
-            uint64_t* hs_out = odd ? B.hst : B.hst2;
-            uint32_t* hl_out = odd ? B.hlen : B.hlen2;
-            // with previous starts: the surviving group starts first, then the new
-            // reps, which can finish from their start's hash
-            for (int phase = ps ? 1 : 0; phase <= (ps ? 2 : 0); ++phase)
-                SSS_TRY(sss_launch(ctx, "pd_hash", k_pd_hash, dim3((nreps + 255) / 256), dim3(256), 0, in, reps,
-                                   nreps, (const uint32_t*)B.lpos, (const uint64_t*)hs_in, (const uint32_t*)hl_in,
-                                   hs_out, hl_out, ps, ps ? (const uint32_t*)B.minlcp : (const uint32_t*)nullptr,
-                                   B.K, B.V, L, Bh, phase));
-            if (use_ht) {
-                uint32_t T = 1024;
-                while (T < 2ull * nreps) T <<= 1;
-                tmask = T - 1;
-                SSS_CUDA(cudaMemsetAsync(B.tab, 0, sizeof(unsigned long long) * T, ctx->stream));
-                SSS_CUDA(cudaMemsetAsync(B.mark, 0, T, ctx->stream));
-                SSS_CUDA(cudaMemsetAsync(&cnt[2], 0, sizeof(uint32_t), ctx->stream));
-                SSS_TRY(sss_launch(ctx, "pd_ht_insert", k_pd_ht_insert, dim3((nreps + 255) / 256), dim3(256), 0,
-                                   (const uint64_t*)B.K, nreps, B.tab, B.mark, tmask, &cnt[2], ctx->d_err));
-            } else {
-                uint32_t bits = 0;
-                while (bits < (uint32_t)HB_MAX && ((uint64_t)nreps >> bits) > 1024) ++bits;
-                uint32_t nb = 1u << bits;
-                SSS_CUDA(cudaMemsetAsync(B.hist, 0, sizeof(uint32_t) * (nb + 1), ctx->stream));
-                uint32_t hgrid = std::min<uint32_t>((nreps + 4095) / 4096, 2u * (uint32_t)ctx->sm_count);
-                SSS_TRY(sss_launch(ctx, "pd_hist", k_pd_hist, dim3(hgrid), dim3(512), 0, (const uint64_t*)B.K, nreps,
-                                   bits, B.hist));
-                SSS_TRY(sss_launch(ctx, "pd_scan", k_pd_scan, dim3(1), dim3(1024), 0, B.hist, nb, B.bstart,
-                                   B.cursor));
-                SSS_TRY(sss_launch(ctx, "pd_scatter", k_pd_scatter, dim3((nreps + 255) / 256), dim3(256), 0,
-                                   (const uint64_t*)B.K, (const uint32_t*)B.V, nreps, bits,
-                                   (const uint32_t*)B.bstart, B.cursor, B.tK, B.tV));
-                SSS_TRY(sss_launch(ctx, "pd_buckets", k_pd_buckets, dim3(nb), dim3(DD_T),
-                                   (size_t)DD_CAP * (8 + 8 + 1), (const uint32_t*)B.bstart, B.tK, B.tV, B.dupf));
-            }
-        }
-        SSS_CUDA(cudaMemsetAsync(&cnt[0], 0, sizeof(uint32_t), ctx->stream));
-        SSS_TRY(sss_launch(ctx, "pd_retire", k_pd_retire, dim3((nreps + PD_T - 1) / PD_T), dim3(PD_T), 0, in, reps, nreps,
-                           (const uint32_t*)B.lpos, (const uint64_t*)B.K, (const uint8_t*)B.dupf,
-                           (const unsigned long long*)B.tab, (const uint8_t*)B.mark, tmask,
-                           (const uint32_t*)&cnt[2], B.apos, B.reps[nxt], cnt, L, (int)use_ht));
-        uint32_t ne = kl_off[k + 1] - kl_off[k];
-        SSS_TRY(sss_launch(ctx, "pd_retire_equal", k_pd_retire_equal, dim3((ne + PD_T - 1) / PD_T), dim3(PD_T), 0,
-                           (const uint32_t*)(B.list_kl + kl_off[k]), ne, (const uint32_t*)B.lpos, B.apos, cnt));
-        if (k < kmax) {
-            uint32_t nn = ks_off[k + 2] - ks_off[k + 1];
-            SSS_TRY(sss_launch(ctx, "pd_newreps", k_pd_newreps, dim3((nn + PD_T - 1) / PD_T), dim3(PD_T), 0,
-                               (const uint32_t*)(B.list_ks + ks_off[k + 1]), nn, (const uint32_t*)B.apos,
-                               B.reps[nxt], cnt));
+            SSS_CUDA(cudaMemsetAsync(&cnt[0], 0, sizeof(uint32_t), ctx->stream));
+            SSS_TRY(sss_launch(ctx, "pd_retire", k_pd_retire, dim3((reps.n + PD_T - 1) / PD_T), dim3(PD_T), 0, in,
+                               reps, B.lpos, (const uint8_t*)B.dupf, approx, B.surv[nxt], cnt, L));
+            const uint32_t ne = kl_off[k + 1] - kl_off[k];
+            SSS_TRY(sss_launch(ctx, "pd_retire_equal", k_pd_retire_equal, dim3((ne + PD_T - 1) / PD_T), dim3(PD_T), 0,
+                               (const uint32_t*)(B.list_kl + kl_off[k]), ne, B.lpos, cnt));
         }
         SSS_CUDA(cudaMemcpyAsync(h, cnt, sizeof(uint32_t) * 2, cudaMemcpyDeviceToHost, ctx->stream));
         SSS_CUDA(cudaStreamSynchronize(ctx->stream));
-        nreps = h[0];
+        ns = h[0];
         retired = h[1];
-        reps = B.reps[nxt];
+        surv = B.surv[nxt];
         nxt ^= 1;
     }
-    return sss_launch(ctx, "pd_final", k_pd_final, dim3((n + 255) / 256), dim3(256), 0, in, (const uint32_t*)B.apos,
-                      (const uint32_t*)B.lpos, approx);
+    return SSS_OK;
 }
 
 // ---------------------------------------------------------------------------
