@@ -443,64 +443,8 @@ __device__ void block_inclusive_max_inplace(uint32_t* a, uint32_t count, uint32_
     __syncthreads();
 }
 
-// ---------------------------------------------------------------------------
-// In-shared-memory bitonic sort of `count` 128-bit keys (hi, lo), ascending,
-// padded to the next power of two with all-ones keys (count <= CAP).
 __device__ __forceinline__ bool key128_less(uint64_t ah, uint64_t al, uint64_t bh, uint64_t bl) {
     return ah < bh || (ah == bh && al < bl);
-}
-
-template <int THREADS>
-__device__ void bitonic_sort128(uint64_t* hi, uint64_t* lo, uint32_t count) {
-    uint32_t P = 1;
-    while (P < count) P <<= 1;
-    for (uint32_t i = count + threadIdx.x; i < P; i += THREADS) {
-        hi[i] = ~0ull;
-        lo[i] = ~0ull;
-    }
-    __syncthreads();
-    for (uint32_t k = 2; k <= P; k <<= 1) {
-        for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-            for (uint32_t t = threadIdx.x; t < P / 2; t += THREADS) {
-                // t-th compare-exchange pair of this stage
-                uint32_t i = 2 * j * (t / j) + (t % j);
-                uint32_t ixj = i + j;
-                bool up = (i & k) == 0;
-                uint64_t ah = hi[i], al = lo[i], bh = hi[ixj], bl = lo[ixj];
-                bool sw = up ? key128_less(bh, bl, ah, al) : key128_less(ah, al, bh, bl);
-                if (sw) {
-                    hi[i] = bh;
-                    lo[i] = bl;
-                    hi[ixj] = ah;
-                    lo[ixj] = al;
-                }
-            }
-            __syncthreads();
-        }
-    }
-}
-
-template <int THREADS>
-__device__ void bitonic_sort64(uint64_t* a, uint32_t count) {
-    uint32_t P = 1;
-    while (P < count) P <<= 1;
-    for (uint32_t i = count + threadIdx.x; i < P; i += THREADS) a[i] = ~0ull;
-    __syncthreads();
-    for (uint32_t k = 2; k <= P; k <<= 1) {
-        for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-            for (uint32_t t = threadIdx.x; t < P / 2; t += THREADS) {
-                uint32_t i = 2 * j * (t / j) + (t % j);
-                uint32_t ixj = i + j;
-                bool up = (i & k) == 0;
-                uint64_t x = a[i], y = a[ixj];
-                if (up ? (y < x) : (x < y)) {
-                    a[i] = y;
-                    a[ixj] = x;
-                }
-            }
-            __syncthreads();
-        }
-    }
 }
 
 // ---------------------------------------------------------------------------

@@ -1127,7 +1127,7 @@ static sss_status launch_round(sss_ctx* ctx, const LsGrid& g, bool small, cudaGr
     if (g.div == 1)
         SSS_TRY(sss_launch(ctx, "ls_lg_tiles", k_lg_tiles, dim3(g.of(4)), dim3(256), 0, cS));
     SSS_TRY(sss_launch(ctx, "ls_lg_ext", k_lg_ext, dim3(g.of(6)), dim3(LG_T), 0, cS));
-    SSS_TRY(sss_launch(ctx, "ls_lg_samples", k_lg_samples, dim3(g.of(2)), dim3(512), 0, cS));
+    SSS_TRY(sss_launch(ctx, "ls_lg_samples", k_lg_samples, dim3(std::max(g.sm, g.of(4))), dim3(SP_T), 0, cS));
     SSS_TRY(sss_launch(ctx, "ls_lg_classify", k_lg_classify, dim3(g.of(6)), dim3(LG_T), 0, cS));
     SSS_TRY(sss_launch(ctx, "ls_lg_offsets", k_lg_rowscan, dim3(g.of(4)), dim3(256), 0, cS));
     SSS_TRY(sss_launch(ctx, "ls_lg_scatter", k_lg_scatter, dim3(g.of(8)), dim3(LG_T), 0, cS, ctx->d_err));

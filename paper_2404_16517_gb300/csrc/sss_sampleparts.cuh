@@ -288,25 +288,101 @@ __global__ void __launch_bounds__(256) k_lg_tiles(const LsDev* __restrict__ S) {
     }
 }
 
-// Per partitioned segment: evenly spaced samples, sorted; splitter b = sample (b+1)*OVS-1.
-__global__ void __launch_bounds__(512) k_lg_samples(const LsDev* __restrict__ S) {
+// Splitters of the partitioned segments: of n = nb * LG_OVS evenly spaced
+// samples (ties by number) the ones of rank (b+1)*OVS - 1.  Ranks by comparing
+// all pairs: a unit is two buckets' worth of samples (32, one per lane) of a
+// segment, its 16 warps share out the others.  A segment of 4,096 samples is
+// then 128 units on as many CTAs (10 us); one CTA sorting them in shared memory
+// (a bitonic network, 78 steps) took 40 us with every other SM idle.
+constexpr int SP_T = 512;
+__global__ void __launch_bounds__(SP_T) k_lg_samples(const LsDev* __restrict__ S) {
     __shared__ uint64_t sh[LG_BMAX * LG_OVS];
+    __shared__ uint32_t s_rank[2 * LG_OVS];
     const LsArgs& A = S->args;
     const uint32_t npart = S->plan.npart;
-    for (uint32_t s = blockIdx.x; s < npart; s += gridDim.x) {
-        __syncthreads();
-        const LgSegInfo si = A.info[s];
-        const uint32_t n = si.nb * LG_OVS;
-        for (uint32_t i = threadIdx.x; i < n; i += 512) {
-            uint64_t q = si.seg.start + ((2 * (uint64_t)i + 1) * si.seg.size) / (2 * (uint64_t)n);
-            sh[i] = A.K[q];
+    const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    // the segments' range buckets, numbered through: (bk0[s] + s) / 2 precede segment s
+    const uint32_t total = (S->plan.pbuckets + npart) / 2;
+    // a CTA's units lie side by side: mostly one segment, whose samples stay
+    const uint32_t per = 2 * ((total + 2 * gridDim.x - 1) / (2 * gridDim.x));
+    const uint32_t last = (blockIdx.x + 1) * per < total ? (blockIdx.x + 1) * per : total;
+    uint32_t loaded = 0xFFFFFFFFu;
+    for (uint32_t x = blockIdx.x * per; x < last;) {
+        const uint32_t end = x + 2 < last ? x + 2 : last;
+        uint32_t s = 0;  // last s with (bk0[s] + s) / 2 <= x
+        for (uint32_t len = npart; len > 0;) {
+            const uint32_t stride = (len + 31) / 32, at = lane * stride;
+            const bool le = at < len && (A.bk0[s + at] + s + at) / 2 <= x;
+            const uint32_t k = (uint32_t)__popc(__ballot_sync(SSS_FULL, le));
+            const uint32_t skip = k ? (k - 1) * stride : 0u;
+            s += skip;
+            len = stride == 1 ? 0u : (len - skip < stride ? len - skip : stride);
         }
+        const LgSegInfo si = A.info[s];
+        const uint32_t r = x - (A.bk0[s] + s) / 2;  // bucket within the segment
+        if (si.nb <= SP_T / LG_OVS && (per >= 8 || si.nb <= 8)) {
+            // few samples, and segments enough for every CTA: a thread per sample, by
+            // the unit of the segment's first bucket
+            if (r == 0) {
+                const uint32_t n = si.nb * LG_OVS;
+                __syncthreads();
+                uint64_t mine = 0;
+                if (threadIdx.x < n) {
+                    mine = A.K[si.seg.start + ((2 * (uint64_t)threadIdx.x + 1) * si.seg.size) / (2 * (uint64_t)n)];
+                    sh[threadIdx.x] = mine;
+                }
+                __syncthreads();
+                if (threadIdx.x < n) {
+                    const uint32_t wb = threadIdx.x - lane, we = wb + 32 < n ? wb + 32 : n;
+                    uint32_t rank = 0;
+#pragma unroll 8
+                    for (uint32_t i = 0; i < wb; ++i) rank += sh[i] <= mine ? 1u : 0u;
+                    for (uint32_t i = wb; i < we; ++i) rank += sh[i] < mine + (i < threadIdx.x ? 1ull : 0ull) ? 1u : 0u;
+#pragma unroll 8
+                    for (uint32_t i = we; i < n; ++i) rank += sh[i] < mine ? 1u : 0u;
+                    if (rank % LG_OVS == LG_OVS - 1 && rank / LG_OVS + 1 < si.nb)
+                        A.spl[(size_t)s * (LG_BMAX - 1) + rank / LG_OVS] = mine;
+                }
+                loaded = 0xFFFFFFFFu;
+            }
+            x += si.nb - r;
+            continue;
+        }
+        const uint32_t cnt = end - x < si.nb - r ? end - x : si.nb - r;
+        const uint32_t n = si.nb * LG_OVS;
         __syncthreads();
-        bitonic_sort64<512>(sh, n);
-        for (uint32_t b = threadIdx.x; b + 1 < si.nb; b += 512)
-            A.spl[(size_t)s * (LG_BMAX - 1) + b] = sh[(b + 1) * LG_OVS - 1];
+        if (s != loaded) {
+            for (uint32_t i = threadIdx.x; i < n; i += SP_T) {
+                const uint64_t q = si.seg.start + ((2 * (uint64_t)i + 1) * si.seg.size) / (2 * (uint64_t)n);
+                sh[i] = A.K[q];
+            }
+            loaded = s;
+        }
+        if (threadIdx.x < 2 * LG_OVS) s_rank[threadIdx.x] = 0;
+        __syncthreads();
+        const uint32_t me = r * LG_OVS + lane;  // sample of this lane (lanes past cnt buckets idle)
+        const bool have = lane < cnt * LG_OVS;
+        const uint64_t mine = have ? sh[me] : 0ull;
+        const uint32_t i0 = w * si.nb, i1 = i0 + si.nb;  // this warp's share: n / 16 samples
+        uint32_t c = 0;
+        if (i1 <= r * LG_OVS || i0 > r * LG_OVS + 31u) {
+            // all before the lanes' samples (equal ones go first) or all after (they do not)
+            const uint64_t lim = mine + (i1 <= r * LG_OVS ? 1ull : 0ull);
+#pragma unroll 8
+            for (uint32_t i = i0; i < i1; ++i) c += sh[i] < lim ? 1u : 0u;
+        } else {
+            for (uint32_t i = i0; i < i1; ++i) c += sh[i] < mine + (i < me ? 1ull : 0ull) ? 1u : 0u;
+        }
+        if (have && c) atomicAdd(&s_rank[lane], c);
+        __syncthreads();
+        if (w == 0 && have) {
+            const uint32_t rank = s_rank[lane], b = rank / LG_OVS;
+            if (rank % LG_OVS == LG_OVS - 1 && b + 1 < si.nb) A.spl[(size_t)s * (LG_BMAX - 1) + b] = mine;
+        }
+        x += cnt;
     }
 }
+static_assert(SP_T / 32 == LG_OVS, "a warp's share of the samples is nb");
 
 // first splitter >= k (lower bound) among nsp sorted splitters
 __device__ __forceinline__ uint32_t lower_bound64(const uint64_t* s, uint32_t nsp, uint64_t k) {
@@ -396,18 +472,30 @@ __global__ void __launch_bounds__(256) k_lg_rowscan(const LsDev* __restrict__ S)
         const uint32_t b = r - A.bk0[s], nbk = 2 * si.nb - 1;
         uint32_t* h = A.hist + si.hist_base + b * si.tiles;
         uint32_t* bst = A.bst + (size_t)s * (LG_NBMAX + 1);
+        // 8 x 32 counts in flight: a 4M-string segment has 4,096 per row, and 32 a
+        // time they took 50 us
         uint32_t carry = 0;
-        for (uint32_t t0 = 0; t0 < si.tiles; t0 += 32) {
-            const uint32_t t = t0 + lane;
-            const uint32_t v = t < si.tiles ? h[t] : 0u;
-            uint32_t x = v;
+        for (uint32_t t0 = 0; t0 < si.tiles; t0 += 256) {
+            uint32_t v[8], x[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const uint32_t t = t0 + 32 * c + lane;
+                x[c] = v[c] = t < si.tiles ? h[t] : 0u;
+            }
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                uint32_t y = __shfl_up_sync(SSS_FULL, x, o);
-                if (lane >= (uint32_t)o) x += y;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const uint32_t y = __shfl_up_sync(SSS_FULL, x[c], o);
+                    if (lane >= (uint32_t)o) x[c] += y;
+                }
             }
-            if (t < si.tiles) h[t] = carry + x - v;
-            carry += __shfl_sync(SSS_FULL, x, 31);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const uint32_t t = t0 + 32 * c + lane;
+                if (t < si.tiles) h[t] = carry + x[c] - v[c];
+                carry += __shfl_sync(SSS_FULL, x[c], 31);
+            }
         }
         uint32_t done = 0;
         if (lane == 0) {
