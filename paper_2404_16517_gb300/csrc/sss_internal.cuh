@@ -186,6 +186,12 @@ sss_status impl_sort_segments(sss_ctx* ctx, Arena& ar, const StrIn& in, const st
 // lcp is initialised and written (other positions keep their contents).
 sss_status impl_sort_segments_range(sss_ctx* ctx, Arena& ar, const StrIn& in, const std::vector<Seg>& init,
                                     const sss_params& prm, uint32_t* perm, uint32_t* lcp, uint32_t q0, uint32_t q1);
+// Refining a sorted order group by group (see sss_local_sort.cu).
+sss_status impl_groups_begin(sss_ctx* ctx, Arena ar, const StrIn& in, const sss_params& prm, uint32_t* perm,
+                             uint32_t* lcp, const uint32_t* group_start, const uint32_t* d_groups,
+                             const uint32_t** d_counts);
+sss_status impl_groups_sort(sss_ctx* ctx, Arena ar, const StrIn& in, const sss_params& prm, uint32_t* perm,
+                            uint32_t* lcp, const uint32_t* counts);
 // Character extent [lo, hi) of every partition's strings: out[2i] = smallest
 // offset, out[2i+1] = largest offset + length (~0, 0 for an empty partition).
 sss_status impl_part_extents(sss_ctx* ctx, const StrIn& in, uint32_t p, unsigned long long* out);

@@ -126,7 +126,8 @@ __device__ __forceinline__ uint32_t ref_pick(uint32_t start, uint32_t cnt, uint3
 }
 
 // Start of a sort: the call's arguments into the context's device state,
-// identity order and LCP 0 over positions q0 .. q1, no LCPs to recompute, and
+// identity order and LCP 0 over positions q0 .. q1 (or both as they are, with
+// A.keep), no LCPs to recompute, and
 // the given initial segments (`table`, in device memory, goes through
 // k_ls_classify instead) on their lists.  One launch in place of an upload per
 // list, two memsets and the identity kernel.
@@ -145,7 +146,7 @@ __global__ void __launch_bounds__(BG_T) k_ls_begin(LsDev* __restrict__ S, const 
 #pragma unroll
     for (uint32_t k = 0; k < BG_PER; ++k) {
         const uint32_t i = base + k * BG_T;
-        if (i < q1 - q0) {
+        if (i < q1 - q0 && !A.keep) {
             A.perm[q0 + i] = q0 + i;
             A.lcp[q0 + i] = 0;
         }
@@ -1226,13 +1227,11 @@ sss_status impl_sort_segments(sss_ctx* ctx, Arena& ar, const StrIn& in, const st
     return impl_sort_segments_range(ctx, ar, in, init, prm, perm, lcp, 0, in.n);
 }
 
-sss_status impl_sort_segments_range(sss_ctx* ctx, Arena& ar, const StrIn& in, const std::vector<Seg>& init,
-                                    const sss_params& prm, uint32_t* perm, uint32_t* lcp, uint32_t q0, uint32_t q1) {
-    const uint32_t n = in.n;
-    if (n == 0 || q1 <= q0) return SSS_OK;
-    const uint32_t nr = q1 - q0;
+// The call's arguments for a sort of positions [q0, q1) with work memory from ar.
+static LsArgs ls_args(sss_ctx* ctx, Arena& ar, const StrIn& in, const sss_params& prm, uint32_t* perm, uint32_t* lcp,
+                      uint32_t q0, uint32_t q1) {
     LsArgs A{};
-    carve_ls(ar, n, 1, prm, A);
+    carve_ls(ar, in.n, 1, prm, A);
     A.chars = in.chars;
     A.offs = in.offs;
     A.lens = in.lens;
@@ -1240,8 +1239,56 @@ sss_status impl_sort_segments_range(sss_ctx* ctx, Arena& ar, const StrIn& in, co
     A.lcp = lcp;
     A.q0 = q0;
     A.q1 = q1;
-    const uint32_t gcls = ls_grid_class(nr);
-    A.use_tiles = ls_grid(ctx, gcls).div == 1;
+    A.use_tiles = ls_grid(ctx, ls_grid_class(q1 - q0)).div == 1;
+    return A;
+}
+
+// Sort the segments on the lists (`have` of each class): the rounds while there
+// are large ones, the finishers, the seams.
+static sss_status run_sort(sss_ctx* ctx, const LsArgs& A, const sss_params& prm, const uint32_t (&have)[LC_COUNT]) {
+    LsDev* S = static_cast<LsDev*>(ctx->d_ls);
+    if (have[LC_LARGE] == 0) {
+        // nothing for the rounds: the finishers over the initial segments
+        const uint32_t sm = (uint32_t)std::max(1, ctx->sm_count);
+        const uint32_t qpb = WF_WARPS * (32 / QUAD_W);
+        const uint32_t grid[5] = {std::min((have[LC_QUAD] + qpb - 1) / qpb, sm * 8),
+                                  std::min((have[LC_WARP] + WF_WARPS - 1) / WF_WARPS, sm * 16),
+                                  std::min(have[LC_TINY], sm * 32), std::min(have[LC_SMALL], sm * 16),
+                                  std::min(have[LC_MED], sm * 4)};
+        for (uint32_t c = LC_MED + 1; c-- > LC_QUAD;) SSS_TRY(launch_finisher(ctx, c, grid[c], list_input(ctx, c)));
+        return SSS_OK;
+    }
+    const uint32_t gcls = ls_grid_class(A.q1 - A.q0);
+    const bool small = small_buckets(A.target);
+    if (!ctx->timing || (prm.flags & SSS_FLAG_GRAPH)) {
+        cudaGraphExec_t ex;
+        SSS_TRY(sort_graph(ctx, gcls, small, &ex));
+        return sss_graph_launch(ctx, ctx->graph_tag, ex);
+    }
+    // kernel timing is on: the same kernels launched one by one, with the next
+    // round's segment count and the error word read back after every round
+    const LsGrid g = ls_grid(ctx, gcls);
+    uint32_t* h_next = reinterpret_cast<uint32_t*>(ctx->h_small);
+    for (uint32_t rounds = 1;; ++rounds) {
+        if (rounds > A.limit) return sss_fail(ctx, SSS_ERR_CUDA, "local sort: round limit exceeded");
+        SSS_TRY(launch_round(ctx, g, small, cudaGraphConditionalHandle{}, 0));
+        SSS_CUDA(cudaMemcpyAsync(h_next, &S->cnt[LC_LARGE], sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
+        SSS_CUDA(cudaMemcpyAsync(h_next + 1, ctx->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
+        SSS_CUDA(cudaStreamSynchronize(ctx->stream));
+        if (h_next[1] & ERRBIT_OVERFLOW) return sss_fail(ctx, SSS_ERR_CUDA, "local sort: device capacity check failed");
+        if (h_next[0] == 0) break;
+    }
+    for (uint32_t c = LC_QUAD; c <= LC_MED; ++c)
+        SSS_TRY(launch_finisher(ctx, c, finisher_grid(g, c), list_input(ctx, c)));
+    return sss_launch(ctx, "ls_fix_seams", k_fix_seams, dim3(g.of(4)), dim3(256), 0, (const LsDev*)S);
+}
+
+sss_status impl_sort_segments_range(sss_ctx* ctx, Arena& ar, const StrIn& in, const std::vector<Seg>& init,
+                                    const sss_params& prm, uint32_t* perm, uint32_t* lcp, uint32_t q0, uint32_t q1) {
+    const uint32_t n = in.n;
+    if (n == 0 || q1 <= q0) return SSS_OK;
+    const uint32_t nr = q1 - q0;
+    const LsArgs A = ls_args(ctx, ar, in, prm, perm, lcp, q0, q1);
     SSS_TRY(set_ls_attributes(ctx));
     LsDev* S = static_cast<LsDev*>(ctx->d_ls);
 
@@ -1275,39 +1322,52 @@ sss_status impl_sort_segments_range(sss_ctx* ctx, Arena& ar, const StrIn& in, co
                            dim3(std::min((m + BG_T - 1) / BG_T, (uint32_t)ctx->sm_count)), dim3(BG_T), 0, S,
                            (const Seg*)table, m, ctx->d_err));
     }
-    if (have[LC_LARGE] == 0) {
-        // nothing for the rounds: the finishers over the initial segments
-        const uint32_t sm = (uint32_t)std::max(1, ctx->sm_count);
-        const uint32_t qpb = WF_WARPS * (32 / QUAD_W);
-        const uint32_t grid[5] = {std::min((have[LC_QUAD] + qpb - 1) / qpb, sm * 8),
-                                  std::min((have[LC_WARP] + WF_WARPS - 1) / WF_WARPS, sm * 16),
-                                  std::min(have[LC_TINY], sm * 32), std::min(have[LC_SMALL], sm * 16),
-                                  std::min(have[LC_MED], sm * 4)};
-        for (uint32_t c = LC_MED + 1; c-- > LC_QUAD;) SSS_TRY(launch_finisher(ctx, c, grid[c], list_input(ctx, c)));
-        return SSS_OK;
+    return run_sort(ctx, A, prm, have);
+}
+
+
+// Refining a sorted order: groups of positions (their strings in index order)
+// that are sorted by other strings, in place.  group_start[g], g < *d_groups, is
+// the first position of group g, the next one's start its end (n for the last).
+// impl_groups_begin puts the groups of two or more on the lists, whose counts
+// (six words at *d_counts, in device memory) the caller reads back and gives to
+// impl_groups_sort.
+__global__ void __launch_bounds__(BG_T) k_ls_groups(LsDev* __restrict__ S, const uint32_t* __restrict__ group_start,
+                                                    const uint32_t* __restrict__ d_groups, unsigned* err) {
+    const uint32_t m = *d_groups, n = S->args.q1;
+    for (uint32_t k0 = blockIdx.x * BG_T; k0 < m; k0 += gridDim.x * BG_T) {
+        const uint32_t k = k0 + threadIdx.x;
+        uint32_t start = 0, size = 0;
+        if (k < m) {
+            start = group_start[k];
+            size = (k + 1 < m ? group_start[k + 1] : n) - start;
+        }
+        push_seg_warp(S->args, S->cnt, size >= 2, start, size, 0, err);
     }
-    const bool small = small_buckets(A.target);
-    if (!ctx->timing || (prm.flags & SSS_FLAG_GRAPH)) {
-        cudaGraphExec_t ex;
-        SSS_TRY(sort_graph(ctx, gcls, small, &ex));
-        return sss_graph_launch(ctx, ctx->graph_tag, ex);
-    }
-    // kernel timing is on: the same kernels launched one by one, with the next
-    // round's segment count and the error word read back after every round
-    const LsGrid g = ls_grid(ctx, gcls);
-    uint32_t* h_next = reinterpret_cast<uint32_t*>(ctx->h_small);
-    for (uint32_t rounds = 1;; ++rounds) {
-        if (rounds > A.limit) return sss_fail(ctx, SSS_ERR_CUDA, "local sort: round limit exceeded");
-        SSS_TRY(launch_round(ctx, g, small, cudaGraphConditionalHandle{}, 0));
-        SSS_CUDA(cudaMemcpyAsync(h_next, &S->cnt[LC_LARGE], sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
-        SSS_CUDA(cudaMemcpyAsync(h_next + 1, ctx->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
-        SSS_CUDA(cudaStreamSynchronize(ctx->stream));
-        if (h_next[1] & ERRBIT_OVERFLOW) return sss_fail(ctx, SSS_ERR_CUDA, "local sort: device capacity check failed");
-        if (h_next[0] == 0) break;
-    }
-    for (uint32_t c = LC_QUAD; c <= LC_MED; ++c)
-        SSS_TRY(launch_finisher(ctx, c, finisher_grid(g, c), list_input(ctx, c)));
-    return sss_launch(ctx, "ls_fix_seams", k_fix_seams, dim3(g.of(4)), dim3(256), 0, (const LsDev*)S);
+}
+
+sss_status impl_groups_begin(sss_ctx* ctx, Arena ar, const StrIn& in, const sss_params& prm, uint32_t* perm,
+                             uint32_t* lcp, const uint32_t* group_start, const uint32_t* d_groups,
+                             const uint32_t** d_counts) {
+    LsArgs A = ls_args(ctx, ar, in, prm, perm, lcp, 0, in.n);
+    A.keep = 1;
+    SSS_TRY(set_ls_attributes(ctx));
+    LsDev* S = static_cast<LsDev*>(ctx->d_ls);
+    const uint32_t sm = (uint32_t)std::max(1, ctx->sm_count);
+    SSS_TRY(sss_launch(ctx, "ls_init", k_ls_begin, dim3(std::min((in.n + 8191) / 8192, sm * 4)), dim3(BG_T), 0, S, A,
+                       LsInit{}, ctx->d_err));
+    SSS_TRY(sss_launch(ctx, "ls_classify", k_ls_groups, dim3(std::min((in.n + BG_T - 1) / BG_T, sm * 8)), dim3(BG_T),
+                       0, S, group_start, d_groups, ctx->d_err));
+    *d_counts = S->cnt;
+    return SSS_OK;
+}
+
+sss_status impl_groups_sort(sss_ctx* ctx, Arena ar, const StrIn& in, const sss_params& prm, uint32_t* perm,
+                            uint32_t* lcp, const uint32_t* counts) {
+    const LsArgs A = ls_args(ctx, ar, in, prm, perm, lcp, 0, in.n);  // as in the device state
+    uint32_t have[LC_COUNT];
+    std::copy(counts, counts + LC_COUNT, have);
+    return run_sort(ctx, A, prm, have);
 }
 
 size_t ls_dev_bytes() { return sizeof(LsDev); }

@@ -104,6 +104,7 @@ struct LsArgs {
     uint32_t warp_max, med_max, direct_max, target, bucket_cap;
     uint32_t cap_tiles, cap_hist, limit, use_tiles;
     uint32_t q0, q1;  // the positions being sorted
+    uint32_t keep;    // the order given in perm is kept (else it starts as the identity)
 };
 
 // Device state of the local sort, one per context.

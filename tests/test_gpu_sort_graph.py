@@ -97,3 +97,20 @@ def test_contexts_side_by_side():
         c.sync()
         _check(s, sss.u32(o[0]), sss.u32(o[1]))
         c.close()
+
+
+# periods that leave groups of equal ranks in every size class (pairs to > 2,048)
+@pytest.mark.parametrize("period,copies,max_len", [(700, 2, 0), (250, 30, 0), (100, 70, 1000), (20, 700, 0), (3, 2900, 0),
+                                                   (7, 1300, 129)])
+def test_suffix_groups_of_every_class(period, copies, max_len):
+    """The rank doubling of the suffix sort refines groups in place."""
+    import paper_2404_16517_gb300 as sss
+    r = np.random.default_rng(period)
+    text = np.tile(r.integers(65, 70, period).astype(np.uint8), copies)
+    text[-5:] = 80
+    n = text.shape[0]
+    lens = np.arange(n, 0, -1).astype(np.uint32)
+    ss = datagen.StringSet(text, np.arange(n, dtype=np.uint64), np.minimum(lens, max_len or n).astype(np.uint32))
+    sa, lcp = sss.sss_suffix_sort(torch.from_numpy(text).cuda(), max_len)
+    sss.context().sync()
+    _check(ss, sss.u32(sa), sss.u32(lcp))
