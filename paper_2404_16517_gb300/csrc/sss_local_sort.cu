@@ -589,88 +589,81 @@ constexpr size_t emit_smem(int, int cap) { return (size_t)cap * (8 + 8 + 4 + 2) 
 // ---------------------------------------------------------------------------
 // Large path.
 // the uncached LCP scan, kept out of line: it is the rare path of k_lg_ext
-// (shared prefixes longer than the 512 cached reference characters)
+// (strings that go on past the 1,024 cached reference characters)
 __device__ __noinline__ uint32_t lcp_full_w_outline(const uint8_t* a, uint32_t la, const uint8_t* b, uint32_t lb,
                                                     uint32_t d, uint64_t* w) {
     return lcp_full_w(a, la, b, lb, d, w);
 }
 
-// A tile of k_lg_ext.  What the member loop needs of the call and the tile sits
+// The round's tiles, and every segment's reference (a warp each): the longest of
+// REF_CAND pseudo-random members (the earliest candidate on ties).  A member's
+// LCP with the reference is capped by the reference's length, so a short
+// reference leaves every longer member that shares its whole remainder in one
+// group, and an input whose shared prefixes grow with the length (nested copies
+// of one template) then sheds only a fraction of the segment per round.
+__global__ void __launch_bounds__(256) k_lg_tiles(const LsDev* __restrict__ S) {
+    const LsArgs& A = S->args;
+    const uint32_t nt = S->plan.ntiles, ns = S->plan.ns;
+    const uint32_t gt = blockIdx.x * 256 + threadIdx.x, nthreads = gridDim.x * 256, lane = threadIdx.x & 31;
+    for (uint32_t s = gt >> 5; s < ns; s += nthreads >> 5) {
+        constexpr uint32_t REF_CAND = 8;
+        const Seg sg = A.info[s].seg;
+        uint64_t best = 0, off = 0;
+        uint32_t pos = sg.start;
+        if (lane < REF_CAND) {
+            pos = sg.start + ref_pick(sg.start, sg.size, sg.depth, lane);
+            const uint32_t e = A.perm[pos];
+            best = ((uint64_t)A.lens[e] << 32) | (uint64_t)(REF_CAND - lane);
+            off = A.offs[e];
+        }
+        uint64_t win = best;
+#pragma unroll
+        for (uint32_t o = REF_CAND / 2; o > 0; o >>= 1) {
+            const uint64_t x = __shfl_xor_sync(SSS_FULL, win, o);
+            win = x > win ? x : win;
+        }
+        if (lane < REF_CAND && best == win) {
+            const uint32_t rl = (uint32_t)(best >> 32), f = key_fmt(rl, sg.depth);
+            A.ref[s] = LgRef{{A.chars + off}, rl, f, pos, 0};
+            A.segfmt[s] = f;
+        }
+    }
+    for (uint32_t g = gt; g < nt; g += nthreads) {
+        uint32_t a = 0, c = ns;
+        while (a + 1 < c) {
+            const uint32_t mid = (a + c) >> 1;
+            if (A.tile0[mid] <= g) a = mid;
+            else c = mid;
+        }
+        const Seg sg = A.info[a].seg;
+        const uint32_t t = g - A.tile0[a], begin = sg.start + t * LG_TILE, e = sg.start + sg.size;
+        A.tiles[g] = LgTile{a, begin, e - begin < (uint32_t)LG_TILE ? e : begin + LG_TILE, t};
+    }
+}
+
+// Keys: every member's LCP with its segment's reference from the depth on, and
+// its next characters.  What the member loop needs of the call and the tile sits
 // in shared memory: in registers next to the word stream it spills at the six
-// CTAs per SM this kernel lives on.
+// CTAs per SM this kernel lives on.  It is a chain of dependent gathers, bound by
+// latency until enough are in flight, so a unit is a whole tile (four members a
+// thread) only where there are two tiles or more per CTA; below that a quarter
+// tile.  Strings that go on past the cached reference characters are compared
+// with the reference in memory, twice the loads.  300,007 strings of 16 to 1,000
+// characters: 168 us with whole tiles (293 of them on 912 CTAs) and 512 cached
+// characters, 104 us with quarter tiles, 57 us with 1,024 cached characters too.
 struct ExtTile {
     GPtr<const uint8_t> chars;
     GPtr<const uint64_t> offs;
     GPtr<const uint32_t> lens;
     GPtr<const uint32_t> perm;
     GPtr<uint64_t> K;
-    GPtr<const uint8_t> rs;  // the reference and its length
-    uint32_t rl, f, refpos, end;
+    LgRef ref;
+    uint32_t depth, begin, end;
 };
-__device__ __forceinline__ void lg_ext_tile(uint32_t sidx, const Seg seg, uint32_t begin, ExtTile& P,
-                                            uint32_t* segfmt) {
-    constexpr uint32_t NREF = 68;  // 64 words (512 chars) plus a 4-word block of slack
-    __shared__ uint64_t refw[NREF];
-    const uint32_t d = seg.depth;
-    // The reference of a large segment: the longest of REF_CAND pseudo-random
-    // members (the earliest candidate on ties).  A member's LCP with the
-    // reference is capped by the reference's length, so a short reference
-    // leaves every longer member that shares its whole remainder in one group,
-    // and an input whose shared prefixes grow with the length (nested copies of
-    // one template) then sheds only a fraction of the segment per round.
-    if (threadIdx.x < 32) {
-        constexpr uint32_t REF_CAND = 8;
-        const uint32_t t = threadIdx.x;
-        uint64_t best = 0;
-        uint32_t pos = seg.start;
-        if (t < REF_CAND) {
-            pos = seg.start + ref_pick(seg.start, seg.size, d, t);
-            best = ((uint64_t)P.lens[P.perm[pos]] << 32) | (uint64_t)(REF_CAND - t);
-        }
-#pragma unroll
-        for (uint32_t o = 16; o > 0; o >>= 1) {
-            uint64_t ob = __shfl_xor_sync(SSS_FULL, best, o);
-            best = ob > best ? ob : best;
-        }
-        const uint32_t win = REF_CAND - (uint32_t)best;  // the winning candidate's t
-        const uint32_t wpos = __shfl_sync(SSS_FULL, pos, win);
-        if (t == 0) {
-            const uint32_t r = P.perm[wpos];
-            const uint32_t rl = (uint32_t)(best >> 32);
-            const uint32_t f = key_fmt(rl, d);
-            P.rs.p = P.chars + P.offs[r];
-            P.rl = rl;
-            P.f = f;
-            P.refpos = wpos;
-            P.end = min(begin + (uint32_t)LG_TILE, seg.start + seg.size);
-            if (begin == seg.start) segfmt[sidx] = f;
-        }
-    }
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < NREF; i += LG_T) refw[i] = load_word_be(P.rs, P.rl, d + 8 * i);
-    __syncthreads();
-    for (uint32_t q = begin + threadIdx.x; q < P.end; q += LG_T) {
-        const uint32_t rl = P.rl;
-        uint64_t w;
-        uint32_t v;
-        if (q == P.refpos) {
-            v = rl > d ? rl - d : 0u;
-            v = v < VCAP ? v : VCAP;
-            w = load_word_be(P.rs, rl, d + v);
-        } else {
-            uint32_t e = P.perm[q];
-            uint32_t le = P.lens[e];
-            uint32_t mlen = le < rl ? le : rl;
-            v = (mlen <= d + 8 * (NREF - 4)) ? lcp_full_w_ref(P.chars + P.offs[e], le, rl, refw, d, &w)
-                                             : lcp_full_w_outline(P.chars + P.offs[e], le, P.rs, rl, d, &w);
-        }
-        uint32_t rho = (v >> 3) < NREF ? (uint32_t)(refw[v >> 3] >> (56 - 8 * (v & 7))) & 0xFFu
-                                       : (uint32_t)(load_word_be(P.rs, rl, d + v) >> 56);
-        P.K[q] = ref_key(v, w, rho, P.f);
-    }
-}
 
 __global__ void __launch_bounds__(LG_T, 6) k_lg_ext(const LsDev* __restrict__ S) {
+    constexpr uint32_t NREF = 132;  // 128 words (1,024 characters) plus a 4-word block of slack
+    __shared__ uint64_t refw[NREF];
     __shared__ ExtTile P;
     const LsArgs& A = S->args;
     if (threadIdx.x == 0) {
@@ -680,11 +673,41 @@ __global__ void __launch_bounds__(LG_T, 6) k_lg_ext(const LsDev* __restrict__ S)
         P.perm.p = A.perm;
         P.K.p = A.K;
     }
-    const uint32_t nt = S->plan.ntiles;
-    for (uint32_t g = blockIdx.x; g < nt; g += gridDim.x) {
+    const uint32_t sub = S->plan.ntiles < 2 * gridDim.x ? 2u : 0u;  // log2 of units per tile
+    for (uint32_t g = blockIdx.x; g < S->plan.ntiles << sub; g += gridDim.x) {
         __syncthreads();
-        const LgTile tl = lg_tile(A, S->plan.ns, g);
-        lg_ext_tile(tl.s, A.info[tl.s].seg, tl.begin, P, A.segfmt);
+        if (threadIdx.x == 0) {
+            const LgTile tl = A.tiles[g >> sub];
+            const uint32_t u = (uint32_t)LG_TILE >> sub, b = tl.begin + (g & ((1u << sub) - 1u)) * u;
+            P.ref = A.ref[tl.s];
+            P.depth = A.info[tl.s].seg.depth;
+            P.begin = b;
+            P.end = b + u < tl.end ? b + u : tl.end;
+        }
+        __syncthreads();
+        const uint32_t d = P.depth;
+        if (P.begin >= P.end) continue;
+        if (threadIdx.x < NREF) refw[threadIdx.x] = load_word_be(P.ref.chars, P.ref.len, d + 8 * threadIdx.x);
+        __syncthreads();
+        for (uint32_t q = P.begin + threadIdx.x; q < P.end; q += LG_T) {
+            const uint32_t rl = P.ref.len;
+            uint64_t w;
+            uint32_t v;
+            if (q == P.ref.pos) {
+                v = rl > d ? rl - d : 0u;
+                v = v < VCAP ? v : VCAP;
+                w = load_word_be(P.ref.chars, rl, d + v);
+            } else {
+                uint32_t e = P.perm[q];
+                uint32_t le = P.lens[e];
+                uint32_t mlen = le < rl ? le : rl;
+                v = (mlen <= d + 8 * (NREF - 4)) ? lcp_full_w_ref(P.chars + P.offs[e], le, rl, refw, d, &w)
+                                                 : lcp_full_w_outline(P.chars + P.offs[e], le, P.ref.chars, rl, d, &w);
+            }
+            uint32_t rho = (v >> 3) < NREF ? (uint32_t)(refw[v >> 3] >> (56 - 8 * (v & 7))) & 0xFFu
+                                           : (uint32_t)(load_word_be(P.ref.chars, rl, d + v) >> 56);
+            P.K[q] = ref_key(v, w, rho, P.ref.fmt);
+        }
     }
 }
 
@@ -1030,7 +1053,6 @@ void carve_ls(Arena& ar, uint32_t n, uint32_t p, const sss_params& prm, LsArgs& 
     a.target = kn.bucket_target;
     a.bucket_cap = small_buckets(kn.bucket_target) ? BKS_CAP : BK_CAP;
     a.limit = 100000u;
-    a.use_tiles = 0;
 }
 
 // Grid sizes follow the number of strings in four steps: a launch of more CTAs
@@ -1125,9 +1147,8 @@ static sss_status launch_round(sss_ctx* ctx, const LsGrid& g, bool small, cudaGr
     LsDev* S = static_cast<LsDev*>(ctx->d_ls);
     const LsDev* cS = S;
     SSS_TRY(sss_launch(ctx, "ls_lg_plan", k_lg_plan, dim3(1), dim3(1024), 0, S, ctx->d_err));
-    if (g.div == 1)
-        SSS_TRY(sss_launch(ctx, "ls_lg_tiles", k_lg_tiles, dim3(g.of(4)), dim3(256), 0, cS));
-    SSS_TRY(sss_launch(ctx, "ls_lg_ext", k_lg_ext, dim3(g.of(6)), dim3(LG_T), 0, cS));
+    SSS_TRY(sss_launch(ctx, "ls_lg_tiles", k_lg_tiles, dim3(g.of(4)), dim3(256), 0, cS));
+    SSS_TRY(sss_launch(ctx, "ls_lg_ext", k_lg_ext, dim3(g.div == 8 ? 3 * g.sm : 6 * g.sm), dim3(LG_T), 0, cS));
     SSS_TRY(sss_launch(ctx, "ls_lg_samples", k_lg_samples, dim3(std::max(g.sm, g.of(4))), dim3(SP_T), 0, cS));
     SSS_TRY(sss_launch(ctx, "ls_lg_classify", k_lg_classify, dim3(g.of(6)), dim3(LG_T), 0, cS));
     SSS_TRY(sss_launch(ctx, "ls_lg_offsets", k_lg_rowscan, dim3(g.of(4)), dim3(256), 0, cS));
@@ -1239,7 +1260,6 @@ static LsArgs ls_args(sss_ctx* ctx, Arena& ar, const StrIn& in, const sss_params
     A.lcp = lcp;
     A.q0 = q0;
     A.q1 = q1;
-    A.use_tiles = ls_grid(ctx, ls_grid_class(q1 - q0)).div == 1;
     return A;
 }
 

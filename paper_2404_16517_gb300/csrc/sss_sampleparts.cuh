@@ -32,6 +32,7 @@ constexpr int LG_BMAX = 256;               // max range buckets per segment
 constexpr int LG_NBMAX = 2 * LG_BMAX - 1;  // range + equality buckets
 
 struct LgTile;
+struct LgRef;
 struct LgSegInfo {
     Seg seg;            // start, size, depth
     uint32_t tiles;     // number of tiles
@@ -94,7 +95,8 @@ struct LsArgs {
     GPtr<uint32_t> bst;  // bucket starts, LG_NBMAX + 1 per segment
     GPtr<uint32_t> rankinfo;
     GPtr<LgSegInfo> info;
-    GPtr<LgTile> tiles;        // large sorts only (use_tiles)
+    GPtr<LgTile> tiles;
+    GPtr<LgRef> ref;    // reference of every segment
     GPtr<uint32_t> tile0;    // first tile of every segment
     GPtr<uint32_t> bk0;      // first bucket of every segment
     GPtr<uint32_t> rowdone;  // rows scanned of every segment
@@ -102,7 +104,7 @@ struct LsArgs {
     GPtr<Seg> list[LC_COUNT];  // LC_WARP: the last entry of the shared array, filled downwards
     uint32_t cap[LC_COUNT];
     uint32_t warp_max, med_max, direct_max, target, bucket_cap;
-    uint32_t cap_tiles, cap_hist, limit, use_tiles;
+    uint32_t cap_tiles, cap_hist, limit;
     uint32_t q0, q1;  // the positions being sorted
     uint32_t keep;    // the order given in perm is kept (else it starts as the identity)
 };
@@ -253,41 +255,18 @@ __device__ __forceinline__ uint32_t warp_last_le(const uint32_t* __restrict__ f,
     return lo + (k ? k - 1 : 0u);
 }
 
-// Tile g of the round: its segment and positions.  Rounds of large sorts may
-// hold thousands of segments: there the tiles are listed by a kernel of their
-// own (a lookup per tile, up to four dependent loads in three kernels, cost the
-// 37.5M-string batch 0.4 ms); smaller rounds look the segment up and save the
-// launch (3 us).
+// Tile of the round: its segment and positions.  Listed by a kernel: a lookup
+// per tile (up to four dependent loads in each of three kernels) cost the batch of
+// 37.5M strings 0.4 ms.
 struct LgTile {
     uint32_t s, begin, end, t;  // segment, positions [begin, end), index within the segment
 };
-__device__ __forceinline__ LgTile lg_find_tile(const LsArgs& A, uint32_t s, uint32_t g) {
-    const Seg sg = A.info[s].seg;
-    LgTile tl;
-    tl.s = s;
-    tl.t = g - A.tile0[s];
-    tl.begin = sg.start + tl.t * LG_TILE;
-    const uint32_t e = sg.start + sg.size;
-    tl.end = e - tl.begin < (uint32_t)LG_TILE ? e : tl.begin + LG_TILE;
-    return tl;
-}
-__device__ __forceinline__ LgTile lg_tile(const LsArgs& A, uint32_t ns, uint32_t g) {
-    return A.use_tiles ? A.tiles[g] : lg_find_tile(A, warp_last_le(A.tile0, ns, g), g);
-}
 
-__global__ void __launch_bounds__(256) k_lg_tiles(const LsDev* __restrict__ S) {
-    const LsArgs& A = S->args;
-    const uint32_t nt = S->plan.ntiles, ns = S->plan.ns;
-    for (uint32_t g = blockIdx.x * 256 + threadIdx.x; g < nt; g += gridDim.x * 256) {
-        uint32_t a = 0, c = ns;
-        while (a + 1 < c) {
-            const uint32_t mid = (a + c) >> 1;
-            if (A.tile0[mid] <= g) a = mid;
-            else c = mid;
-        }
-        A.tiles[g] = lg_find_tile(A, a, g);
-    }
-}
+// A segment's reference member: its characters, length, key format and position.
+struct LgRef {
+    GPtr<const uint8_t> chars;
+    uint32_t len, fmt, pos, pad;
+};
 
 // Splitters of the partitioned segments: of n = nb * LG_OVS evenly spaced
 // samples (ties by number) the ones of rank (b+1)*OVS - 1.  Ranks by comparing
@@ -404,10 +383,10 @@ __global__ void __launch_bounds__(LG_T) k_lg_classify(const LsDev* __restrict__ 
     const uint64_t* __restrict__ K = A.K;
     uint32_t* __restrict__ hist = A.hist;
     uint32_t* __restrict__ rankinfo = A.rankinfo;
-    const uint32_t ptiles = S->plan.ptiles, npart = S->plan.npart;
+    const uint32_t ptiles = S->plan.ptiles;
     for (uint32_t g = blockIdx.x; g < ptiles; g += gridDim.x) {
         __syncthreads();
-        const LgTile tl = lg_tile(A, npart, g);
+        const LgTile tl = A.tiles[g];
         const LgSegInfo si = A.info[tl.s];
         uint32_t nsp = si.nb - 1, nbk = 2 * si.nb - 1;
         for (uint32_t i = threadIdx.x; i < nsp; i += LG_T) ssp[i] = A.spl[(size_t)tl.s * (LG_BMAX - 1) + i];
@@ -545,9 +524,9 @@ __global__ void __launch_bounds__(LG_T) k_lg_scatter(const LsDev* __restrict__ S
     uint64_t* __restrict__ tK = A.tK;
     uint32_t* __restrict__ tV = A.tV;
     const uint32_t tid = threadIdx.x;
-    const uint32_t ptiles = S->plan.ptiles, npart = S->plan.npart;
+    const uint32_t ptiles = S->plan.ptiles;
     for (uint32_t g = blockIdx.x; g < ptiles; g += gridDim.x) {
-        const LgTile tl = lg_tile(A, npart, g);
+        const LgTile tl = A.tiles[g];
         const LgSegInfo si = A.info[tl.s];
         const uint32_t* __restrict__ bst = A.bst + (size_t)tl.s * (LG_NBMAX + 1);
         const uint32_t nbk = 2 * si.nb - 1;
@@ -616,6 +595,7 @@ inline void carve_sp(Arena& ar, uint32_t n, uint32_t cap_segs, LsArgs& a) {
     a.rankinfo = ar.take<uint32_t>(n);
     a.info = ar.take<LgSegInfo>(cap_segs);
     a.tiles = ar.take<LgTile>(a.cap_tiles);
+    a.ref = ar.take<LgRef>(cap_segs);
     a.tile0 = ar.take<uint32_t>(cap_segs);
     a.bk0 = ar.take<uint32_t>(cap_segs);
     a.rowdone = ar.take<uint32_t>(cap_segs);

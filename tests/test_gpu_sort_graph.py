@@ -114,3 +114,23 @@ def test_suffix_groups_of_every_class(period, copies, max_len):
     sa, lcp = sss.sss_suffix_sort(torch.from_numpy(text).cuda(), max_len)
     sss.context().sync()
     _check(ss, sss.u32(sa), sss.u32(lcp))
+
+
+# shared prefixes around the cached reference characters, units of a quarter and
+# of a whole tile
+@pytest.mark.parametrize("n", [3000, 40000])
+@pytest.mark.parametrize("shared", [500, 1015, 1024, 1031, 2100])
+def test_keys_past_the_cached_reference(n, shared):
+    import paper_2404_16517_gb300 as sss
+    r = np.random.default_rng(n + shared)
+    lens = (shared - 9 + r.integers(0, 30, n)).astype(np.uint32)
+    offs = np.zeros(n, np.uint64)
+    offs[1:] = np.cumsum(lens[:-1].astype(np.uint64))
+    chars = r.integers(65, 69, int(lens.astype(np.int64).sum()) + 1).astype(np.uint8)
+    t = r.integers(65, 91, shared).astype(np.uint8)
+    chars[offs.astype(np.int64)[:, None] + np.arange(shared - 12)[None, :]] = t[:shared - 12]
+    ss = datagen.StringSet(chars, offs, lens)
+    d = sss.to_device(ss)
+    perm, lcp, _, _ = sss.sss_sort(*d)
+    sss.context().sync()
+    _check(ss, sss.u32(perm), sss.u32(lcp))
