@@ -76,7 +76,7 @@ __device__ __forceinline__ int cmp_from4(const uint8_t* a, uint32_t la, const ui
     return la < lb ? -1 : (la > lb ? 1 : 0);
 }
 
-// The same comparison by a whole warp: lane k tests the word at d + 256*i + 8k,
+// cmp_from by a whole warp: lane k tests the word at d + 256*i + 8k,
 // a ballot finds the first differing word.  Every lane gets the result.
 __device__ __forceinline__ int warp_cmp_from(const uint8_t* a, uint32_t la, const uint8_t* b, uint32_t lb, uint32_t d,
                                              uint32_t* l) {
@@ -740,16 +740,29 @@ __global__ void k_d2_samples(const uint32_t* __restrict__ run_perm, Strs S, cons
     s_lens[g] = tlen(S, s);
 }
 
-__global__ void k_d2_subspl(const BucketInfo* __restrict__ bi, uint32_t p, uint32_t nss,
+// A sub-splitter as k_d2_bounds needs it: its bucket, string, truncated length,
+// and sorted rank, itself and past the samples equal to it (which are <= it too).
+struct SubSpl {
+    uint64_t off;
+    uint32_t j, len, rank, rend;
+};
+
+__global__ void k_d2_subspl(const BucketInfo* __restrict__ bi, uint32_t p, uint32_t nss, Strs S,
                             const uint32_t* __restrict__ smp, const uint32_t* __restrict__ sperm,
-                            uint32_t* __restrict__ subspl) {
+                            const uint32_t* __restrict__ s2lcp, const uint32_t* __restrict__ s2lens,
+                            uint32_t* __restrict__ subspl, SubSpl* __restrict__ info) {
     uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= nss) return;
     uint32_t j = last_le(&bi[0].ss0, p, m, sizeof(BucketInfo) / 4, 0);
     // skip buckets without sub-splitters that share ss0
     while (j + 1 < p && bi[j + 1].ss0 <= m) ++j;
-    uint32_t k = m - bi[j].ss0;
-    subspl[m] = smp[sperm[bi[j].sbase + D2_OVS * (k + 1) - 1]];
+    const BucketInfo B = bi[j];
+    const uint32_t rank = B.sbase + D2_OVS * (m - B.ss0 + 1) - 1, rlim = B.sbase + B.nsmp;
+    const uint32_t f = smp[sperm[rank]], fl = tlen(S, f);
+    uint32_t rend = rank;
+    while (rend + 1 < rlim && s2lcp[rend + 1] >= fl && s2lens[sperm[rend + 1]] == fl) ++rend;
+    subspl[m] = f;
+    info[m] = SubSpl{S.offs[f], j, fl, rank, rend};
 }
 
 // Sorted rank of every second-level sample: srank[sperm[x]] = x.
@@ -766,39 +779,38 @@ __global__ void k_d2_srank(const uint32_t* __restrict__ sperm, uint32_t S2, uint
 // ranked at or before R_end (R extended over the following samples equal to
 // the sub-splitter, which are <= it too), sample a - 1 is <= the sub-splitter
 // and sample a is larger: the count lies in [a*step, (a+1)*step - 1] (or up to
-// the piece's end past its last sample).  A binary search over the samples'
-// ranks finds a; then a window of at most 32 strings is compared a lane per
-// string, a wider one searched.
-__global__ void k_d2_bounds(const uint32_t* __restrict__ run_perm, Strs S, const BucketInfo* __restrict__ bi,
-                            uint32_t p, uint32_t nss, const uint32_t* __restrict__ pstart,
-                            const uint32_t* __restrict__ psz, const uint32_t* __restrict__ pso,
-                            const uint32_t* __restrict__ subspl, const uint32_t* __restrict__ sperm,
-                            const uint32_t* __restrict__ srank, const uint32_t* __restrict__ s2lcp,
-                            const uint32_t* __restrict__ s2lens, uint32_t step, uint32_t* __restrict__ sb) {
+// the piece's end past its last sample).  A search over the samples' ranks finds
+// a.  The strings of that window are compared a lane each, 32 characters; from
+// the first one on in a narrow window (large p: few strings between samples), else
+// from what the window's two samples share with the sub-splitter, which is in the
+// sorted samples' LCP array (a minimum over the ranks between), and eight evenly
+// spaced strings first.  Where some share those 32 characters too, the whole warp
+// compares, halving their number.  Bound by the latency of dependent gathers, of
+// which the sub-splitter's own are done once per sub-splitter: 86 us on 4.19M
+// strings with p = 16 and 94 us on the length-skewed set; a binary search by the
+// whole warp, after a lookup of the bucket in every warp, took 108 and 153 us.
+// (2.1M suffix views with p = 64, narrow windows: 148 us either way.)
+__global__ void k_d2_bounds(const uint32_t* __restrict__ run_perm, Strs S, uint32_t p, uint32_t nss,
+                            const uint32_t* __restrict__ pstart, const uint32_t* __restrict__ psz,
+                            const uint32_t* __restrict__ pso, const SubSpl* __restrict__ info,
+                            const uint32_t* __restrict__ srank, const uint32_t* __restrict__ s2lcp, uint32_t step,
+                            uint32_t* __restrict__ sb) {
     uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (g >= nss * p) return;
-    uint32_t m = g / p, i = g % p;
-    uint32_t j = last_le(&bi[0].ss0, p, m, sizeof(BucketInfo) / 4, 0);
-    while (j + 1 < p && bi[j + 1].ss0 <= m) ++j;
-    const BucketInfo B = bi[j];
-    const uint32_t k = m - B.ss0;
-    const uint32_t f = subspl[m];
-    const uint8_t* fs = S.chars + S.offs[f];
-    const uint32_t fl = tlen(S, f);
-    // R_end: the sub-splitter's sorted rank, past the samples equal to it
-    uint32_t rend = B.sbase + D2_OVS * (k + 1) - 1;
-    const uint32_t rlim = B.sbase + B.nsmp;
-    while (rend + 1 < rlim && s2lcp[rend + 1] >= fl && s2lens[sperm[rend + 1]] == fl) ++rend;
+    const uint32_t m = g / p, i = g % p;
+    const SubSpl F = info[m];
+    const uint8_t* fs = S.chars + F.off;
+    const uint32_t fl = F.len, pc = F.j * p + i;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t n_i = psz[pc], q0 = pstart[pc], g0 = pso[pc], c = pso[pc + 1] - g0;
     // a: the piece's samples ranked <= R_end (their ranks grow with their
     // positions): 32 evenly spaced samples per ballot narrow the range until it
     // fits one ballot
-    const uint32_t lane = threadIdx.x & 31;
-    const uint32_t g0 = pso[j * p + i], c = pso[j * p + i + 1] - g0;
     uint32_t klo = 0, khi = c;
     while (khi - klo > 32) {
         const uint32_t stride = (khi - klo + 31) / 32;
         const uint32_t t = klo + lane * stride;
-        const uint32_t k = (uint32_t)__popc(__ballot_sync(SSS_FULL, t < khi && srank[g0 + t] <= rend));
+        const uint32_t k = (uint32_t)__popc(__ballot_sync(SSS_FULL, t < khi && srank[g0 + t] <= F.rend));
         if (k == 0) {
             khi = klo;
         } else {
@@ -808,59 +820,63 @@ __global__ void k_d2_bounds(const uint32_t* __restrict__ run_perm, Strs S, const
         }
     }
     const uint32_t ka =
-        klo + (uint32_t)__popc(__ballot_sync(SSS_FULL, klo + lane < khi && srank[g0 + klo + lane] <= rend));
-    const uint32_t n_i = psz[j * p + i];
-    const uint32_t wa = ka * step, wb = ka < c ? (ka + 1) * step - 1 : n_i;
-    const uint32_t q0 = pstart[j * p + i];
-    uint32_t cnt = wa;
-    if (wb - wa <= 32) {
-        // a narrow window (large p: few strings between samples), a lane per
-        // string; the strings <= the sub-splitter form a prefix.  First their
-        // first 32 characters only: enough when neighbours differ early
-        const uint32_t q = wa + lane;
-        const uint32_t e = q < wb ? run_perm[q0 + q] : 0u;
+        klo + (uint32_t)__popc(__ballot_sync(SSS_FULL, klo + lane < khi && srank[g0 + klo + lane] <= F.rend));
+    // the strings <= the sub-splitter form a prefix of [a, b)
+    uint32_t a = ka * step, b = ka < c ? (ka + 1) * step - 1 : n_i;
+    uint32_t d = 0;  // characters that all of them share with it, as far as known
+    bool known = false;
+    while (a < b) {
+        const uint32_t n = b - a;
+        if (!known && n > 32 && ka > 0 && ka < c) {
+            // sample ka - 1 is below the sub-splitter or equal to it, sample ka above it
+            const uint32_t ra = srank[g0 + ka - 1], rb = srank[g0 + ka];  // ra <= R_end < rb
+            uint32_t x = fl;
+            for (uint32_t t = ra + 1 + lane; t <= rb; t += 32) x = min(x, s2lcp[t]);
+            d = __reduce_min_sync(SSS_FULL, x);
+            known = true;
+        }
+        // a lane per string, or eight that part the window in nine
+        const uint32_t lanes = n <= 32 ? n : 8u;
+        const uint32_t q = n <= 32 ? a + lane : a + (uint32_t)(((uint64_t)(lane + 1) * n) / 9u);
+        uint32_t e = 0, el = 0;
+        uint64_t eo = 0;
         bool le = false, dec = true;
-        if (q < wb) le = cmp_from4(S.chars + S.offs[e], tlen(S, e), fs, fl, 0, &dec) <= 0;
-        if (__ballot_sync(SSS_FULL, !dec) != 0) {
-            // some strings share 32+ characters with the sub-splitter: compare
-            // from the LCP that every string between the window's neighbours
-            // shares with it (the shorter of the neighbours' LCPs with it)
-            uint32_t dl = 0, dh = 0;
-            if (wa > 0) {
-                const uint32_t en = run_perm[q0 + wa - 1];
-                warp_cmp_from(S.chars + S.offs[en], tlen(S, en), fs, fl, 0, &dl);
-            }
-            if (wb < n_i) {
-                const uint32_t en = run_perm[q0 + wb];
-                warp_cmp_from(S.chars + S.offs[en], tlen(S, en), fs, fl, 0, &dh);
-            }
-            const uint32_t d = wa > 0 && wb < n_i ? (dl < dh ? dl : dh) : 0u;
-            if (q < wb) {
+        if (lane < lanes) {
+            e = run_perm[q0 + q];
+            el = tlen(S, e);
+            eo = S.offs[e];
+            le = cmp_from4(S.chars + eo, el, fs, fl, d, &dec) <= 0;
+        }
+        uint32_t cnt = (uint32_t)__popc(__ballot_sync(SSS_FULL, le && dec));
+        const uint32_t und = __ballot_sync(SSS_FULL, !dec);
+        if (und) {
+            // the undecided lanes lie between the smaller strings and the larger ones
+            uint32_t lo = (uint32_t)__ffs((int)und) - 1, hi = 32u - (uint32_t)__clz((int)und);
+            uint32_t ll = d + 32, lh = d + 32;  // shared with the ends of the range
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi) >> 1;
+                const uint64_t mo = __shfl_sync(SSS_FULL, eo, mid);
+                const uint32_t ml = __shfl_sync(SSS_FULL, el, mid);
                 uint32_t l;
-                le = cmp_from(S.chars + S.offs[e], tlen(S, e), fs, fl, d, &l) <= 0;
+                if (warp_cmp_from(S.chars + mo, ml, fs, fl, ll < lh ? ll : lh, &l) <= 0) {
+                    lo = mid + 1;
+                    ll = l;
+                } else {
+                    hi = mid;
+                    lh = l;
+                }
             }
+            cnt = lo;
         }
-        cnt = wa + (uint32_t)__popc(__ballot_sync(SSS_FULL, le));
-    } else {
-        // a wider window: binary search with warp-wide comparisons that carry the
-        // LCP with both ends (fewer strings fetched than a lane per string)
-        uint32_t a = wa, b = wb, la = 0, lb = 0;
-        while (a < b) {
-            const uint32_t mid = (a + b) >> 1;
-            const uint32_t e = run_perm[q0 + mid];
-            uint32_t l;
-            const int cmp = warp_cmp_from(S.chars + S.offs[e], tlen(S, e), fs, fl, la < lb ? la : lb, &l);
-            if (cmp <= 0) {
-                a = mid + 1;
-                la = l;
-            } else {
-                b = mid;
-                lb = l;
-            }
+        if (n <= 32) {
+            a += cnt;
+            break;
         }
-        cnt = a;
+        const uint32_t na = cnt > 0 ? a + (uint32_t)(((uint64_t)cnt * n) / 9u) + 1 : a;
+        b = cnt < lanes ? a + (uint32_t)(((uint64_t)(cnt + 1) * n) / 9u) : b;
+        a = na;
     }
-    if (lane == 0) sb[g] = cnt;
+    if (lane == 0) sb[g] = a;
 }
 
 __device__ __forceinline__ uint32_t bucket_of_sub(const BucketInfo* bi, uint32_t p, uint32_t b) {
@@ -966,14 +982,15 @@ __device__ __forceinline__ uint32_t sub_uref(const BucketInfo& B, uint32_t b, co
 // Side 0 members come before side 1, side 1 before side 2; members of
 // different sides have lcp c.
 
-// c = lcp(L, U) of every sub-bucket (one thread each): between two sub-splitters
-// of a bucket, the minimum of the sorted samples' LCP array over the samples
-// from one to the other; next to a level-1 splitter, a direct comparison; 0
-// next to a missing splitter.
+// c = lcp(L, U) of every sub-bucket, a warp each: between two sub-splitters of a
+// bucket, the minimum of the sorted samples' LCP array over the samples from one
+// to the other; next to a level-1 splitter, a comparison by the whole warp (by
+// one thread it took 51 us where the strings share 992 characters, now 7); 0 next
+// to a missing splitter.
 __global__ void k_d2_cb(Strs S, const BucketInfo* __restrict__ bi, uint32_t p, uint32_t nsb,
                         const uint32_t* __restrict__ subspl, const uint32_t* __restrict__ s2lcp,
                         uint32_t* __restrict__ cb) {
-    const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (b >= nsb) return;
     const uint32_t j = bucket_of_sub(bi, p, b);
     const BucketInfo B = bi[j];
@@ -984,13 +1001,13 @@ __global__ void k_d2_cb(Strs S, const BucketInfo* __restrict__ bi, uint32_t p, u
         c = 0;
     } else if (k >= 1 && k + 1 < B.nsb) {
         // sub-splitters k-1 and k: sorted samples sbase + D2_OVS*k - 1 and sbase + D2_OVS*(k+1) - 1
-        const uint32_t t0 = B.sbase + D2_OVS * k - 1, t1 = B.sbase + D2_OVS * (k + 1) - 1;
-        c = 0xFFFFFFFFu;
-        for (uint32_t t = t0 + 1; t <= t1; ++t) c = s2lcp[t] < c ? s2lcp[t] : c;
+        static_assert(D2_OVS <= 32, "a lane per sample");
+        const uint32_t t0 = B.sbase + D2_OVS * k - 1;
+        c = __reduce_min_sync(SSS_FULL, lane < D2_OVS ? s2lcp[t0 + 1 + lane] : 0xFFFFFFFFu);
     } else {
-        cmp_from(S.chars + S.offs[L], tlen(S, L), S.chars + S.offs[U], tlen(S, U), 0, &c);
+        warp_cmp_from(S.chars + S.offs[L], tlen(S, L), S.chars + S.offs[U], tlen(S, U), 0, &c);
     }
-    cb[b] = c;
+    if (lane == 0) cb[b] = c;
 }
 
 // Decode each slice once, one warp per slice, 32 records at a time:
@@ -1375,6 +1392,7 @@ struct MgBufs {
     uint32_t* s2lcp;
     uint32_t* s2rank;  // sorted rank of every second-level sample
     uint32_t* subspl;
+    SubSpl* sinfo;
     uint32_t* sb;
     uint32_t* ssz;
     uint64_t* soff;
@@ -1457,6 +1475,7 @@ void carve_mg(Arena& ar, uint32_t n, uint32_t p, uint32_t v, uint64_t nrecchars,
     b.s2lcp = ar.take<uint32_t>(b.cap_s2);
     b.s2rank = ar.take<uint32_t>(b.cap_s2);
     b.subspl = ar.take<uint32_t>(b.cap_nsb);
+    b.sinfo = ar.take<SubSpl>(b.cap_nsb);
     b.sb = ar.take<uint32_t>(nslices);
     b.ssz = ar.take<uint32_t>(nslices);
     b.soff = ar.take<uint64_t>(nslices + 1);
@@ -1821,16 +1840,14 @@ sss_status impl_merge(sss_ctx* ctx, char* ws, size_t ws_bytes, const StrIn& in, 
         SSS_TRY(ss);
     }
     if (NSS > 0) {
-        SSS_TRY(sss_launch(ctx, "d2_subspl", k_d2_subspl, dim3((NSS + 255) / 256), dim3(256), 0,
-                           (const BucketInfo*)b.binfo, p, NSS, (const uint32_t*)b.smp2, (const uint32_t*)b.s2perm,
-                           b.subspl));
+        SSS_TRY(sss_launch(ctx, "d2_subspl", k_d2_subspl, dim3((NSS + 63) / 64), dim3(64), 0,
+                           (const BucketInfo*)b.binfo, p, NSS, S, (const uint32_t*)b.smp2, (const uint32_t*)b.s2perm,
+                           (const uint32_t*)b.s2lcp, (const uint32_t*)b.s2lens, b.subspl, b.sinfo));
         SSS_TRY(sss_launch(ctx, "d2_srank", k_d2_srank, dim3((S2 + 255) / 256), dim3(256), 0,
                            (const uint32_t*)b.s2perm, S2, b.s2rank));
         SSS_TRY(sss_launch(ctx, "d2_bounds", k_d2_bounds, dim3((NSS * p * 32 + 127) / 128), dim3(128), 0, run_perm,
-                           S, (const BucketInfo*)b.binfo, p, NSS, (const uint32_t*)b.pstart, (const uint32_t*)b.psz,
-                           (const uint32_t*)b.pso, (const uint32_t*)b.subspl, (const uint32_t*)b.s2perm,
-                           (const uint32_t*)b.s2rank, (const uint32_t*)b.s2lcp, (const uint32_t*)b.s2lens, step,
-                           b.sb));
+                           S, p, NSS, (const uint32_t*)b.pstart, (const uint32_t*)b.psz, (const uint32_t*)b.pso,
+                           (const SubSpl*)b.sinfo, (const uint32_t*)b.s2rank, (const uint32_t*)b.s2lcp, step, b.sb));
     }
     SSS_TRY(sss_launch(ctx, "d2_slices", k_d2_slices, dim3((nslices + 255) / 256), dim3(256), 0,
                        (const BucketInfo*)b.binfo, p, NSB, (const uint32_t*)b.sb, (const uint32_t*)b.psz, b.ssz));
@@ -1853,7 +1870,7 @@ sss_status impl_merge(sss_ctx* ctx, char* ws, size_t ws_bytes, const StrIn& in, 
                            (const BucketInfo*)b.binfo, p, NSB, (const uint64_t*)b.soff, (const uint32_t*)b.subspl,
                            b.rr, b.rs, b.rk));
     } else {
-        SSS_TRY(sss_launch(ctx, "d2_cb", k_d2_cb, dim3((NSB + 255) / 256), dim3(256), 0, S,
+        SSS_TRY(sss_launch(ctx, "d2_cb", k_d2_cb, dim3((NSB + 7) / 8), dim3(256), 0, S,
                            (const BucketInfo*)b.binfo, p, NSB, (const uint32_t*)b.subspl, (const uint32_t*)b.s2lcp,
                            b.cb));
         SSS_TRY(sss_launch(ctx, "d2_recdec", k_d2_recdec, dim3((nslices * 32 + 255) / 256), dim3(256), 0, run_perm,

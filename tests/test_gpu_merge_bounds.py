@@ -1,0 +1,36 @@
+"""Sub-splitter bounds of the merge: windows on both sides of a lane per string
+(p small and large), strings that share more with a sub-splitter than a lane
+compares, many equal strings, pieces with few samples or none."""
+import numpy as np
+import pytest
+
+import datagen
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _set(kind, n, r):
+    tail = r.integers(65, 91, (n, 6)).astype(np.uint8)
+    if kind == "templates":  # shared prefixes of up to 300 characters, three of them
+        t = r.integers(65, 91, (3, 300)).astype(np.uint8)
+        pick, cut = r.integers(0, 3, n), r.integers(250, 301, n)
+        return [t[p, :c].tobytes() + x.tobytes() for p, c, x in zip(pick, cut, tail)]
+    if kind == "equal":      # long equal strings, a few hundred distinct ones
+        base = [b"L" * 90 + bytes(r.integers(65, 68, 5).astype(np.uint8)) for _ in range(300)]
+        return [base[i] for i in r.integers(0, 300, n)]
+    return [x.tobytes()[:int(l)] for x, l in zip(tail, r.integers(1, 7, n))]  # short ones
+
+
+@pytest.mark.parametrize("kind", ["templates", "equal", "short"])
+@pytest.mark.parametrize("n,p", [(9001, 2), (20011, 4), (40009, 16), (30011, 64), (3001, 100)])
+def test_merge_windows(kind, n, p):
+    import paper_2404_16517_gb300 as sss
+    ss = datagen.from_strings(_set(kind, n, np.random.default_rng(n + p)))
+    chars, offs, lens = sss.to_device(ss)
+    perm, lcp, _, _ = sss.sss_sort(chars, offs, lens, p)
+    sss.context().sync()
+    want = oracle.sort(ss)
+    assert np.array_equal(sss.u32(perm), want)
+    assert np.array_equal(sss.u32(lcp), oracle.lcp_array(ss, want))
