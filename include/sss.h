@@ -90,10 +90,11 @@ typedef struct sss_params {
     uint64_t hash_seed; /* seed of the prefix hash (default 0) */
     /* Tuning knobs of the local sort and merge: they change speed, never results.
      * 0 selects the default; other values are clamped into the stated range. */
-    uint32_t cta_cap;       /* largest segment finished inside one CTA, 64..2048 (default 2048) */
+    uint32_t cta_cap;       /* largest segment finished inside one CTA, 64..2048 (default 2048
+                               where every segment fits that, else 256) */
     uint32_t merge_ms;      /* merge segment spacing, a power of two 8..1024 (default 32) */
     uint32_t direct_cap;    /* largest segment of the multi-CTA path sorted whole by one CTA,
-                               cta_cap..8192 (default 8192) */
+                               cta_cap..8192 (default 8192 above 2^22 strings, else 4352) */
     uint32_t bucket_target; /* target size of a sampled-partition range bucket, 256..4096
                                (default 2048) */
     uint32_t warp_cap;      /* largest segment finished by one warp, 2..32 (default 32) */

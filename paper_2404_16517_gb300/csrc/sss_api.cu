@@ -317,8 +317,8 @@ static sss_params resolve_params(const sss_params* p) {
     sss_params_default(&r);
     if (p) r = *p;
     if (r.v == 0) r.v = 2;
-    r.cta_cap = clamp_or(r.cta_cap, 2048, 64, 2048);
-    r.direct_cap = clamp_or(r.direct_cap, 8192, r.cta_cap, 8192);
+    r.cta_cap = clamp_or(r.cta_cap, 0, 64, 2048);  // 0: chosen by the call's sizes
+    r.direct_cap = clamp_or(r.direct_cap, 0, std::max(r.cta_cap, 64u), 8192);
     r.bucket_target = clamp_or(r.bucket_target, 2048, 256, 4096);
     r.warp_cap = clamp_or(r.warp_cap, 32, 2, 32);
     return r;

@@ -104,7 +104,7 @@ struct LsArgs {
     GPtr<Seg> list[LC_COUNT];  // LC_WARP: the last entry of the shared array, filled downwards
     uint32_t cap[LC_COUNT];
     uint32_t warp_max, med_max, direct_max, target, bucket_cap;
-    uint32_t cap_tiles, cap_hist, limit;
+    uint32_t cap_tiles, cap_hist, cap_part, limit;
     uint32_t q0, q1;  // the positions being sorted
     uint32_t keep;    // the order given in perm is kept (else it starts as the identity)
 };
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(1024) k_lg_plan(LsDev* __restrict__ S, unsigne
     if (tid == 0) {
         const uint32_t nt = (uint32_t)(carry[2] >> 32), nh = (uint32_t)(carry[3] >> 32);
         LsPlan pl{ns, npart, nbig, nt, ptiles, (uint32_t)carry[3], {0, 0}};
-        if (nt > A.cap_tiles || nh > A.cap_hist) {
+        if (nt > A.cap_tiles || nh > A.cap_hist || npart > A.cap_part) {
             atomicOr(err, ERRBIT_OVERFLOW);
             pl = LsPlan{0, 0, 0, 0, 0, 0, {0, 0}};
         }
@@ -585,13 +585,15 @@ __global__ void __launch_bounds__(LG_T) k_lg_scatter(const LsDev* __restrict__ S
     }
 }
 
-// Work memory of the partition for up to `cap_segs` segments covering <= n positions.
-inline void carve_sp(Arena& ar, uint32_t n, uint32_t cap_segs, LsArgs& a) {
+// Work memory of the partition for up to `cap_segs` segments covering <= n
+// positions, `cap_part` of them partitioned (those come first).
+inline void carve_sp(Arena& ar, uint32_t n, uint32_t cap_segs, uint32_t cap_part, LsArgs& a) {
     a.cap_tiles = n / LG_TILE + cap_segs + 2;
-    a.cap_hist = LG_NBMAX * a.cap_tiles;
-    a.spl = ar.take<uint64_t>((size_t)cap_segs * (LG_BMAX - 1));
+    a.cap_hist = LG_NBMAX * (n / LG_TILE + cap_part + 2);
+    a.cap_part = cap_part;
+    a.spl = ar.take<uint64_t>((size_t)cap_part * (LG_BMAX - 1));
     a.hist = ar.take<uint32_t>(a.cap_hist);
-    a.bst = ar.take<uint32_t>((size_t)cap_segs * (LG_NBMAX + 1));
+    a.bst = ar.take<uint32_t>((size_t)cap_part * (LG_NBMAX + 1));
     a.rankinfo = ar.take<uint32_t>(n);
     a.info = ar.take<LgSegInfo>(cap_segs);
     a.tiles = ar.take<LgTile>(a.cap_tiles);
