@@ -919,7 +919,6 @@ template <int THREADS, int ITEMS, int NB>
 __device__ __forceinline__ bool block_bucket_sort(const uint64_t* sK, const uint32_t* sV, uint16_t* sC, uint64_t* sR,
                                                   uint16_t* sP, uint32_t m, uint32_t f) {
     constexpr int WARPS = THREADS / 32, PER = NB / 2 / THREADS;  // PER words of two counters a thread
-    static_assert(WARPS >= 8, "one warp per reduced quantity");
     static_assert(NB <= 8192 && THREADS * ITEMS <= NB && (NB & (NB - 1)) == 0, "bucket number and slot share a word");
     static_assert(PER >= 1, "a word of counters per thread");
     __shared__ uint32_t s_red[8][32];
@@ -974,13 +973,13 @@ __device__ __forceinline__ bool block_bucket_sort(const uint64_t* sK, const uint
     for (uint32_t i = tid; i < (uint32_t)NB / 2; i += THREADS) sW[i] = 0;
     if (tid == 0) s_sq = 0;
     __syncthreads();
-    if (w < 8) {
-        uint32_t x = s_red[w][lane < (uint32_t)WARPS ? lane : 0u];
-        x = (w == 0 || w == 2) ? __reduce_min_sync(SSS_FULL, x)
-            : w < 4            ? __reduce_max_sync(SSS_FULL, x)
-            : w < 6            ? __reduce_or_sync(SSS_FULL, x)
+    for (uint32_t i = w; i < 8; i += WARPS) {  // a warp per quantity
+        uint32_t x = s_red[i][lane < (uint32_t)WARPS ? lane : 0u];
+        x = (i == 0 || i == 2) ? __reduce_min_sync(SSS_FULL, x)
+            : i < 4            ? __reduce_max_sync(SSS_FULL, x)
+            : i < 6            ? __reduce_or_sync(SSS_FULL, x)
                                : __reduce_and_sync(SSS_FULL, x);
-        if (lane == 0) s_red[w][0] = x;
+        if (lane == 0) s_red[i][0] = x;
     }
     // slots in index order (as every caller's are; checked): then equal keys go by slot
     bool ordered = true;

@@ -48,3 +48,19 @@ def test_sizes_and_distributions(kind, n):
         sss.context().sync()
         assert np.array_equal(sss.u32(perm), want)
         assert np.array_equal(sss.u32(lcp), wl)
+
+
+# the CTA finisher's first iteration (65 .. 2,048 strings), as the only segment of a
+# call (its 128- and 512-thread instances) and as partitions beside others
+@pytest.mark.parametrize("kind", ["uniform", "bytes", "skewed", "equal", "staircase", "ended"])
+@pytest.mark.parametrize("n", [65, 127, 511, 512, 513, 1000, 2047, 2048])
+def test_finisher_sizes_and_distributions(kind, n):
+    import paper_2404_16517_gb300 as sss
+    ss = datagen.from_strings(_strings(kind, n, np.random.default_rng(n + 1)))
+    chars, offs, lens = sss.to_device(ss)
+    for p in (1, 3):
+        rp, rl = sss.sss_local_sort(chars, offs, lens, p)
+        sss.context().sync()
+        want, wl = oracle.local_sort(ss, p)
+        assert np.array_equal(sss.u32(rp), want)
+        assert np.array_equal(sss.u32(rl), wl)
