@@ -74,7 +74,7 @@ int sss_stat_index(sss_ctx* ctx, const char* name) {
 }
 
 sss_status sss_graph_launch(sss_ctx* ctx, const char* name, cudaGraphExec_t exec) {
-    int st = sss_stat_index(ctx, name);
+    int st = sss_stat_index(ctx, ctx->tag ? ctx->tag : name);
     bool timed = sss_timing_on(ctx, st);
     cudaEvent_t a = nullptr, b = nullptr;
     if (timed) {

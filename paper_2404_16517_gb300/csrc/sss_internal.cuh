@@ -94,9 +94,9 @@ struct sss_ctx {
     };
     static constexpr int LS_GRAPHS = 8;
     LsGraph ls_graphs[LS_GRAPHS];
-    // kernel-statistics name of the next round-loop graph launches (timed like a
-    // kernel when timing is on); set by a caller for its own sorts
-    const char* graph_tag = "ls_graph";
+    // one kernel-statistics name for all launches (instead of their own), set by a
+    // stage around the sorts of its samples
+    const char* tag = nullptr;
     // sss_sort_host: the stream that uploads characters while stage A runs, and
     // one event per uploaded chunk
     cudaStream_t copy_stream = nullptr;
@@ -143,7 +143,7 @@ template <typename... KArgs, typename... Args>
 sss_status sss_launch(sss_ctx* ctx, const char* name, void (*kernel)(KArgs...), dim3 grid, dim3 block,
                       size_t smem, Args... args) {
     if (grid.x == 0 || grid.y == 0 || grid.z == 0) return SSS_OK;
-    int st = sss_stat_index(ctx, name);
+    int st = sss_stat_index(ctx, ctx->tag && !ctx->capturing ? ctx->tag : name);
     bool timed = !ctx->capturing && sss_timing_on(ctx, st);  // no event nodes inside a captured loop
     cudaEvent_t a = nullptr, b = nullptr;
     if (timed) {

@@ -1343,7 +1343,7 @@ static sss_status run_sort(sss_ctx* ctx, const LsArgs& A, const sss_params& prm,
     if (!ctx->timing || (prm.flags & SSS_FLAG_GRAPH)) {
         cudaGraphExec_t ex;
         SSS_TRY(sort_graph(ctx, gcls, small, &ex));
-        return sss_graph_launch(ctx, ctx->graph_tag, ex);
+        return sss_graph_launch(ctx, "ls_graph", ex);
     }
     // kernel timing is on: the same kernels launched one by one, with the next
     // round's segment count and the error word read back after every round
@@ -1368,18 +1368,17 @@ sss_status impl_sort_segments_range(sss_ctx* ctx, Arena& ar, const StrIn& in, co
     const uint32_t n = in.n;
     if (n == 0 || q1 <= q0) return SSS_OK;
     const uint32_t nr = q1 - q0;
+    const LsKnobs kn = ls_knobs(prm, n, false);
+    SSS_TRY(set_ls_attributes(ctx));
     if (init.size() == 1 && init[0].start == q0 && init[0].size == nr && nr > (uint32_t)TINY_CAP &&
-        nr <= ls_knobs(prm, n, false).cta_cap && ls_knobs(prm, n, false).warp_cap < nr) {
+        nr <= kn.cta_cap && nr > kn.warp_cap)
         // one segment for one CTA: a single launch, nothing to prepare
-        SSS_TRY(set_ls_attributes(ctx));
         return launch_finisher(ctx, nr <= (uint32_t)SM_CAP ? LC_SMALL : LC_MED, 1,
                                FinIn{nullptr, LC_MED, {nullptr}, 1, {nullptr}, {in.chars}, {in.offs}, {in.lens}, {perm},
                                      {lcp}, init[0]});
-    }
     bool rounds = false;  // a segment that the CTA finisher cannot take
-    for (const Seg& s : init) rounds = rounds || s.size > ls_knobs(prm, n, false).cta_cap;
+    for (const Seg& s : init) rounds = rounds || s.size > kn.cta_cap;
     const LsArgs A = ls_args(ar, in, prm, rounds, perm, lcp, q0, q1);
-    SSS_TRY(set_ls_attributes(ctx));
     LsDev* S = static_cast<LsDev*>(ctx->d_ls);
 
     // initial segments (partitions or instances), counted by size class

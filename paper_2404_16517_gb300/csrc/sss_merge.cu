@@ -132,6 +132,42 @@ __global__ void k_c_samples(const uint32_t* __restrict__ run_perm, uint32_t n, u
     if (g == 0) *cnt = 0;
 }
 
+// The splitters of ns samples (offsets and lengths in s_offs, s_lens), ties by
+// sample number: a CTA ranks a sample against all the others, a warp per pair, and
+// the sample of rank j ns / p - 1 is splitter j.  Bound by the latency of comparing
+// strings that share long prefixes: 7 us for the 12 samples of p = 4 on templates of
+// 500 characters, where the sort (three launches) took 33, 8 for the 48 of p = 16
+// (41), 16 for the 192 of p = 64 on suffix views (33).
+constexpr uint32_t C_RANK_MAX = 256;  // 65,536 pairs: 7 for every warp that the SMs hold
+constexpr int C_RANK_T = 512;
+
+__global__ void __launch_bounds__(C_RANK_T) k_c_rank(const uint8_t* __restrict__ chars,
+                                                     const uint64_t* __restrict__ s_offs,
+                                                     const uint32_t* __restrict__ s_lens,
+                                                     const uint32_t* __restrict__ smp, uint32_t ns, uint32_t p,
+                                                     uint32_t* __restrict__ spl) {
+    __shared__ uint32_t sh_rank;
+    const uint32_t s = blockIdx.x, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) sh_rank = 0;
+    __syncthreads();
+    const uint8_t* a = chars + s_offs[s];
+    const uint32_t la = s_lens[s];
+    uint32_t smaller = 0;
+    for (uint32_t t = threadIdx.x >> 5; t < ns; t += C_RANK_T / 32) {
+        if (t == s) continue;
+        uint32_t l;
+        const int c = warp_cmp_from(chars + s_offs[t], s_lens[t], a, la, 0, &l);
+        smaller += c < 0 || (c == 0 && t < s) ? 1u : 0u;
+    }
+    if (lane == 0 && smaller) atomicAdd(&sh_rank, smaller);
+    __syncthreads();
+    for (uint32_t j = threadIdx.x + 1; j < p; j += C_RANK_T) {
+        const uint32_t k = (uint32_t)(((uint64_t)j * ns) / p);  // the splitter is the k-th smallest sample
+        if (k == sh_rank + 1) spl[j - 1] = smp[s];
+        if (k == 0 && s == 0) spl[j - 1] = MINF;
+    }
+}
+
 __global__ void k_c_splitters(const uint32_t* __restrict__ smp, const uint32_t* __restrict__ sperm, uint32_t ns,
                               uint32_t p, uint32_t* __restrict__ spl) {
     uint32_t j = blockIdx.x * blockDim.x + threadIdx.x + 1;
@@ -1584,13 +1620,22 @@ static sss_status run_partition(sss_ctx* ctx, const StrIn& in, const uint32_t* t
         SSS_TRY(sss_launch(ctx, "c_samples", k_c_samples, dim3((tot + 127) / 128), dim3(128), 0, run_perm, n, p, v, S,
                            b.smp, b.s_offs, b.s_lens, b.cnt));
     }
-    // sort the samples (views of the same characters, truncated) with stage A;
-    // equal truncated samples keep sample order, which is input-index order
-    StrIn sin{in.chars, in.n_chars, b.s_offs, b.s_lens, ns};
-    Arena sub = b.sub;
-    SSS_TRY(impl_local_sort(ctx, sub, sin, 1, sss_params{}, b.s_perm, b.s_lcp));
-    SSS_TRY(sss_launch(ctx, "c_splitters", k_c_splitters, dim3((p + 127) / 128), dim3(128), 0, (const uint32_t*)b.smp,
-                       (const uint32_t*)b.s_perm, ns, p, b.spl));
+    if (ns > 0 && ns <= C_RANK_MAX) {
+        SSS_TRY(sss_launch(ctx, "c_rank", k_c_rank, dim3(ns), dim3(C_RANK_T), 0, in.chars, (const uint64_t*)b.s_offs,
+                           (const uint32_t*)b.s_lens, (const uint32_t*)b.smp, ns, p, b.spl));
+    } else {
+        // sort the samples (views of the same characters, truncated) with stage A;
+        // equal truncated samples keep sample order, which is input-index order
+        StrIn sin{in.chars, in.n_chars, b.s_offs, b.s_lens, ns};
+        Arena sub = b.sub;
+        const char* tag = ctx->tag;
+        ctx->tag = "c_sample_sort";  // stage C's time in the statistics
+        const sss_status ss = impl_local_sort(ctx, sub, sin, 1, sss_params{}, b.s_perm, b.s_lcp);
+        ctx->tag = tag;
+        SSS_TRY(ss);
+        SSS_TRY(sss_launch(ctx, "c_splitters", k_c_splitters, dim3((p + 127) / 128), dim3(128), 0,
+                           (const uint32_t*)b.smp, (const uint32_t*)b.s_perm, ns, p, b.spl));
+    }
     uint32_t nb = p * (p + 1);
     SSS_TRY(sss_launch(ctx, "c_bounds", k_c_bounds, dim3((nb * 32 + 127) / 128), dim3(128), 0, run_perm, n, p, S,
                        (const uint32_t*)b.spl, b.bounds));
@@ -1829,14 +1874,15 @@ sss_status impl_merge(sss_ctx* ctx, char* ws, size_t ws_bytes, const StrIn& in, 
                            b.s2offs, b.s2lens));
         StrIn sin{in.chars, in.n_chars, b.s2offs, b.s2lens, S2};
         Arena sub = b.sub2;
-        // the samples' round loop as a cached graph: a sort this small is bound by
-        // the host's launches and per-round synchronisation otherwise
+        // (One segment: one per bucket, in order as they are, compares the strings in
+        // p CTAs instead of on every SM.  1.05M strings, p = 4: 120 us against 186 in
+        // four segments; 4.19M, p = 16: 140 against 182.)
         sss_params sp{};
-        sp.flags = SSS_FLAG_GRAPH;
-        const char* tag = ctx->graph_tag;
-        ctx->graph_tag = "d2_sample_sort";  // stage D's time in the statistics
+        sp.flags = SSS_FLAG_GRAPH;  // with kernel timing on, too
+        const char* tag = ctx->tag;
+        ctx->tag = "d2_sample_sort";  // stage D's time in the statistics
         const sss_status ss = impl_local_sort(ctx, sub, sin, 1, sp, b.s2perm, b.s2lcp);
-        ctx->graph_tag = tag;
+        ctx->tag = tag;
         SSS_TRY(ss);
     }
     if (NSS > 0) {

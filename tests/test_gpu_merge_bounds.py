@@ -34,3 +34,24 @@ def test_merge_windows(kind, n, p):
     want = oracle.sort(ss)
     assert np.array_equal(sss.u32(perm), want)
     assert np.array_equal(sss.u32(lcp), oracle.lcp_array(ss, want))
+
+
+# stage C alone: samples ranked in pairs (to 256) and sorted (above), runs around the
+# 33-way split, with and without truncation
+@pytest.mark.parametrize("kind", ["templates", "equal", "short"])
+@pytest.mark.parametrize("n,p,v", [(5, 8, 2), (64, 2, 1), (33 * 4, 4, 2), (34 * 4 + 1, 4, 3), (20011, 16, 15),
+                                   (20011, 16, 16), (9001, 64, 3), (70001, 3, 2)])
+def test_partition(kind, n, p, v):
+    import paper_2404_16517_gb300 as sss
+    ss = datagen.from_strings(_set(kind, n, np.random.default_rng(n + p + v)))
+    rp, _ = oracle.local_sort(ss, p)
+    chars, offs, lens = sss.to_device(ss)
+    t_rp = torch.from_numpy(rp.view(np.int32)).cuda()
+    for tr in (None, oracle.doubling(ss, 0, oracle.default_kmax(ss), 0)):
+        _, want_spl = oracle.splitters(ss, oracle.samples(rp, n, p, v), p, tr)
+        want_b = oracle.bounds(ss, rp, p, want_spl, tr)
+        t_tr = None if tr is None else torch.from_numpy(tr.view(np.int32)).cuda()
+        spl, bnd = sss.sss_partition(chars, offs, lens, t_rp, p, trunc=t_tr, prm=sss.params(v=v))
+        sss.context().sync()
+        assert np.array_equal(sss.u32(spl), want_spl)
+        assert np.array_equal(sss.u32(bnd).reshape(-1), want_b.reshape(-1))
