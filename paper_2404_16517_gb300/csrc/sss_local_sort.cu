@@ -1421,17 +1421,45 @@ sss_status impl_sort_segments_range(sss_ctx* ctx, Arena& ar, const StrIn& in, co
 // impl_groups_begin puts the groups of two or more on the lists, whose counts
 // (six words at *d_counts, in device memory) the caller reads back and gives to
 // impl_groups_sort.
+//
+// The counters take one atomic per list and CTA of 1,024 groups: with one per list
+// and warp, hundreds of thousands of groups took 20 us of serial atomics.
 __global__ void __launch_bounds__(BG_T) k_ls_groups(LsDev* __restrict__ S, const uint32_t* __restrict__ group_start,
                                                     const uint32_t* __restrict__ d_groups, unsigned* err) {
-    const uint32_t m = *d_groups, n = S->args.q1;
-    for (uint32_t k0 = blockIdx.x * BG_T; k0 < m; k0 += gridDim.x * BG_T) {
-        const uint32_t k = k0 + threadIdx.x;
-        uint32_t start = 0, size = 0;
-        if (k < m) {
-            start = group_start[k];
-            size = (k + 1 < m ? group_start[k + 1] : n) - start;
+    constexpr uint32_t PER = 4;
+    __shared__ uint32_t s_cnt[LC_COUNT], s_base[LC_COUNT];
+    const LsArgs& A = S->args;
+    const uint32_t m = *d_groups, n = A.q1, lane = threadIdx.x & 31;
+    for (uint64_t k0 = (uint64_t)blockIdx.x * BG_T * PER; k0 < m; k0 += (uint64_t)gridDim.x * BG_T * PER) {
+        uint32_t start[PER], size[PER], cls[PER], place[PER];
+#pragma unroll
+        for (uint32_t t = 0; t < PER; ++t) {
+            const uint64_t k = k0 + t * BG_T + threadIdx.x;
+            start[t] = k < m ? group_start[k] : 0u;
+            size[t] = k + 1 < m ? group_start[k + 1] : k < m ? n : 0u;
         }
-        push_seg_warp(S->args, S->cnt, size >= 2, start, size, 0, err);
+        __syncthreads();
+        if (threadIdx.x < LC_COUNT) s_cnt[threadIdx.x] = 0;
+        __syncthreads();
+#pragma unroll
+        for (uint32_t t = 0; t < PER; ++t) {
+            size[t] -= start[t];
+            cls[t] = size[t] >= 2 ? seg_class(A, size[t]) : (uint32_t)LC_COUNT;
+            const unsigned peers = __match_any_sync(SSS_FULL, cls[t]);
+            const int leader = __ffs((int)peers) - 1;
+            uint32_t base = 0;
+            if ((int)lane == leader && cls[t] < LC_COUNT) base = atomicAdd(&s_cnt[cls[t]], (uint32_t)__popc(peers));
+            place[t] = __shfl_sync(SSS_FULL, base, leader) + (uint32_t)__popc(peers & ((1u << lane) - 1u));
+        }
+        __syncthreads();
+        if (threadIdx.x < LC_COUNT) {
+            const uint32_t c = s_cnt[threadIdx.x];
+            s_base[threadIdx.x] = c ? atomicAdd(&S->cnt[threadIdx.x], c) : 0u;
+        }
+        __syncthreads();
+#pragma unroll
+        for (uint32_t t = 0; t < PER; ++t)
+            if (cls[t] < LC_COUNT) put_seg(A, cls[t], s_base[cls[t]] + place[t], Seg{start[t], size[t], 0, 0}, err);
     }
 }
 
@@ -1445,7 +1473,7 @@ sss_status impl_groups_begin(sss_ctx* ctx, Arena ar, const StrIn& in, const sss_
     const uint32_t sm = (uint32_t)std::max(1, ctx->sm_count);
     SSS_TRY(sss_launch(ctx, "ls_init", k_ls_begin, dim3(std::min((in.n + 8191) / 8192, sm * 4)), dim3(BG_T), 0, S, A,
                        LsInit{}, ctx->d_err));
-    SSS_TRY(sss_launch(ctx, "ls_classify", k_ls_groups, dim3(std::min((in.n + BG_T - 1) / BG_T, sm * 8)), dim3(BG_T),
+    SSS_TRY(sss_launch(ctx, "ls_classify", k_ls_groups, dim3(std::min((in.n + 4 * BG_T - 1) / (4 * BG_T), sm * 8)), dim3(BG_T),
                        0, S, group_start, d_groups, ctx->d_err));
     *d_counts = S->cnt;
     return SSS_OK;
@@ -1563,22 +1591,30 @@ sss_status impl_suffix_views(sss_ctx* ctx, uint32_t n, uint32_t max_len, uint64_
 // Batched sorts: table positions become instance-local indices, and the
 // instance's dist is (optionally) computed.  blockIdx.y splits an instance over
 // several CTAs: with one each, eleven instances of 450k strings in all kept
-// eleven SMs busy for 193 us.
+// eleven SMs busy for 193 us.  Eight positions of a thread are in flight: 38.7M
+// positions in 4,096 instances took 129 us one at a time, 58 us (5.3 TB/s) so.
 __global__ void __launch_bounds__(256) k_batch_finish(const Seg* __restrict__ inst, uint32_t m,
                                                       const uint32_t* __restrict__ lens, uint32_t* __restrict__ perm,
                                                       const uint32_t* __restrict__ lcp, uint32_t* __restrict__ dist) {
+    constexpr uint32_t PER = 8, SPAN = 256 * PER;
     for (uint32_t k = blockIdx.x; k < m; k += gridDim.x) {
         const Seg s = inst[k];
-        for (uint32_t r = blockIdx.y * 256 + threadIdx.x; r < s.size; r += gridDim.y * 256) {
-            const uint32_t q = s.start + r;
-            const uint32_t g = perm[q];
-            if (dist) {
-                const uint32_t left = r > 0 ? lcp[q] : 0;
-                const uint32_t right = r + 1 < s.size ? lcp[q + 1] : 0;
-                const uint64_t d = (uint64_t)(left > right ? left : right) + 1;
-                dist[g] = d < lens[g] ? (uint32_t)d : lens[g];
+        for (uint64_t r0 = (uint64_t)blockIdx.y * SPAN + threadIdx.x; r0 < s.size; r0 += (uint64_t)gridDim.y * SPAN) {
+            uint32_t g[PER];
+#pragma unroll
+            for (uint32_t t = 0; t < PER; ++t) g[t] = r0 + t * 256 < s.size ? perm[s.start + r0 + t * 256] : 0u;
+#pragma unroll
+            for (uint32_t t = 0; t < PER; ++t) {
+                if (r0 + t * 256 >= s.size) break;
+                const uint32_t r = (uint32_t)r0 + t * 256, q = s.start + r;
+                if (dist) {
+                    const uint32_t left = r > 0 ? lcp[q] : 0;
+                    const uint32_t right = r + 1 < s.size ? lcp[q + 1] : 0;
+                    const uint64_t d = (uint64_t)(left > right ? left : right) + 1;
+                    dist[g[t]] = d < lens[g[t]] ? (uint32_t)d : lens[g[t]];
+                }
+                perm[q] = g[t] - s.start;
             }
-            perm[q] = g - s.start;
         }
     }
 }
