@@ -182,13 +182,28 @@ __global__ void k_c_chartot(Strs S, uint32_t n, uint32_t p, unsigned long long* 
     const uint32_t i = blockIdx.y;
     const uint32_t lo = part_lo(n, p, i), hi = part_lo(n, p, i + 1);
     uint64_t v = 0;
-    for (uint32_t q = lo + blockIdx.x * blockDim.x + threadIdx.x; q < hi; q += gridDim.x * blockDim.x) v += tlen(S, q);
+    constexpr uint32_t PER = 8;  // lengths in flight
+    for (uint64_t q0 = lo + (uint64_t)blockIdx.x * blockDim.x * PER + threadIdx.x; q0 < hi;
+         q0 += (uint64_t)gridDim.x * blockDim.x * PER) {
+        uint32_t l[PER];
+#pragma unroll
+        for (uint32_t k = 0; k < PER; ++k) {
+            const uint64_t q = q0 + k * blockDim.x;
+            l[k] = q < hi ? tlen(S, (uint32_t)q) : 0u;
+        }
+#pragma unroll
+        for (uint32_t k = 0; k < PER; ++k) v += l[k];
+    }
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(SSS_FULL, v, o);
     if ((threadIdx.x & 31) == 0 && v) atomicAdd(&tot[i], (unsigned long long)v);
 }
 
 // P[q] = characters of the run positions before q (runs in position order), in
-// three passes over chunks of CP_CHUNK positions
+// three passes over chunks of CP_CHUNK positions.  A warp's lanes take consecutive
+// positions, so the run is read, and P written, in whole lines, and a thread's 16
+// gathers are in flight together (first and last pass on 4.19M strings: 26 and
+// 45 us with 16 consecutive positions a thread, 24 and 31 us so, which is the rate
+// of the gathers).
 constexpr uint32_t CP_T = 256, CP_PER = 16, CP_CHUNK = CP_T * CP_PER;
 
 __device__ __forceinline__ uint64_t cp_block_excl(uint64_t v, uint64_t* wt, uint64_t* total) {
@@ -216,10 +231,15 @@ __device__ __forceinline__ uint64_t cp_block_excl(uint64_t v, uint64_t* wt, uint
 __global__ void __launch_bounds__(CP_T) k_c_psum(Strs S, const uint32_t* __restrict__ run_perm, uint32_t n,
                                                   uint64_t* __restrict__ csum) {
     __shared__ uint64_t wt[CP_T / 32], tot;
-    const uint64_t q0 = (uint64_t)blockIdx.x * CP_CHUNK + (uint64_t)threadIdx.x * CP_PER;
+    const uint64_t q0 = (uint64_t)blockIdx.x * CP_CHUNK + threadIdx.x;
+    uint32_t l[CP_PER];
+#pragma unroll
+    for (uint32_t k = 0; k < CP_PER; ++k) l[k] = q0 + k * CP_T < n ? run_perm[q0 + k * CP_T] : 0u;
+#pragma unroll
+    for (uint32_t k = 0; k < CP_PER; ++k) l[k] = q0 + k * CP_T < n ? tlen(S, l[k]) : 0u;
     uint64_t v = 0;
-    for (uint32_t k = 0; k < CP_PER; ++k)
-        if (q0 + k < n) v += tlen(S, run_perm[q0 + k]);
+#pragma unroll
+    for (uint32_t k = 0; k < CP_PER; ++k) v += l[k];
     cp_block_excl(v, wt, &tot);
     if (threadIdx.x == 0) csum[blockIdx.x] = tot;
 }
@@ -240,20 +260,29 @@ __global__ void __launch_bounds__(CP_T) k_c_pscan(uint64_t* __restrict__ csum, u
 __global__ void __launch_bounds__(CP_T) k_c_pwrite(Strs S, const uint32_t* __restrict__ run_perm, uint32_t n,
                                                     const uint64_t* __restrict__ csum, uint64_t* __restrict__ P) {
     __shared__ uint64_t wt[CP_T / 32], tot;
-    const uint64_t q0 = (uint64_t)blockIdx.x * CP_CHUNK + (uint64_t)threadIdx.x * CP_PER;
+    const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const uint64_t q0 = (uint64_t)blockIdx.x * CP_CHUNK + (uint64_t)w * 32 * CP_PER + lane;  // the warp's first row
     uint32_t l[CP_PER];
+#pragma unroll
+    for (uint32_t k = 0; k < CP_PER; ++k) l[k] = q0 + k * 32 < n ? run_perm[q0 + k * 32] : 0u;
+#pragma unroll
+    for (uint32_t k = 0; k < CP_PER; ++k) l[k] = q0 + k * 32 < n ? tlen(S, l[k]) : 0u;
     uint64_t v = 0;
 #pragma unroll
-    for (uint32_t k = 0; k < CP_PER; ++k) {
-        l[k] = q0 + k < n ? tlen(S, run_perm[q0 + k]) : 0u;
-        v += l[k];
-    }
-    uint64_t run = csum[blockIdx.x] + cp_block_excl(v, wt, &tot);
+    for (uint32_t k = 0; k < CP_PER; ++k) v += l[k];
+    // the characters before the warp's first row
+    uint64_t run = csum[blockIdx.x] + __shfl_sync(SSS_FULL, cp_block_excl(v, wt, &tot), 0);
 #pragma unroll
     for (uint32_t k = 0; k < CP_PER; ++k) {
-        if (q0 + k < n) P[q0 + k] = run;
-        run += l[k];
-        if (q0 + k + 1 == n) P[n] = run;
+        uint64_t x = l[k];
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint64_t y = __shfl_up_sync(SSS_FULL, x, d);
+            if (lane >= (uint32_t)d) x += y;
+        }
+        const uint64_t q = q0 + k * 32;
+        if (q < n) P[q] = run + x - l[k];
+        if (q + 1 == n) P[n] = run + x;
+        run += __shfl_sync(SSS_FULL, x, 31);
     }
 }
 
