@@ -616,8 +616,8 @@ __device__ __forceinline__ void finish_group_segment(const Seg sg, uint32_t e, c
 // (counter, segment, strings, their offsets and lengths, characters), so the first
 // three of them run ahead: while a unit is sorted, the next one's strings, the
 // second's segments and the third's number are on their way; a string's offset and
-// length move with it between the lanes.  The batch of 4,096 instances: 534 -> 290 us
-// for its segments of 2 to 4 strings, 143 -> 94 for those of up to 32.
+// length move with it between the lanes.  The batch of 4,096 instances: 323 -> 290 us
+// for its segments of 2 to 4 strings, 99 -> 95 for those of up to 32.
 template <int W>
 __global__ void __launch_bounds__(32 * WF_WARPS, 4) k_finish_group(const FinIn in, unsigned* err) {
     constexpr uint32_t G = 32u / W;
