@@ -918,6 +918,38 @@ __device__ __forceinline__ bool sort_emit(unsigned char* smem, bool from_t, uint
     return true;
 }
 
+// An equality bucket, or a range bucket too large for its CTA, is copied to its
+// place as it is; in a run of equal strings (ended) the LCPs are the lengths.  Eight
+// strings of a thread in flight.
+template <int THREADS>
+__device__ __forceinline__ void copy_run(const LsArgs& A, uint32_t bs, uint32_t m, bool ended, uint32_t part,
+                                         uint32_t parts) {
+    constexpr uint32_t PER = 8;
+    for (uint64_t i0 = (uint64_t)part * THREADS * PER + threadIdx.x; i0 < m; i0 += (uint64_t)parts * THREADS * PER) {
+        uint32_t v[PER], l[PER];
+#pragma unroll
+        for (uint32_t t = 0; t < PER; ++t) v[t] = i0 + t * THREADS < m ? A.tV[bs + i0 + t * THREADS] : 0u;
+#pragma unroll
+        for (uint32_t t = 0; t < PER; ++t) l[t] = ended && i0 + t * THREADS < m ? A.lens[v[t]] : 0u;
+#pragma unroll
+        for (uint32_t t = 0; t < PER; ++t) {
+            const uint64_t i = i0 + t * THREADS;
+            if (i >= m) break;
+            A.perm[bs + i] = v[t];
+            if (ended && i > 0) A.lcp[bs + i] = l[t];
+        }
+    }
+}
+
+// A bucket of more strings than this is left to all the CTAs of the round's last
+// kernel, by an entry (start, size, ended) in memory that is free by then.  4.19M
+// suffixes of one repeated character (rounds of one bucket each): 127 ms of copies
+// by one CTA a round of 137 in all, 6.4 ms in all so.  (Each CTA reads every entry, so
+// they are few.)
+constexpr uint32_t BIG_RUN = 1u << 17;
+static_assert(sizeof(LgRef) >= sizeof(Seg) && BIG_RUN > 2 * (uint32_t)MED_CAP, "one reference per large segment");
+__device__ __forceinline__ Seg* big_runs(const LsArgs& A) { return reinterpret_cast<Seg*>(static_cast<LgRef*>(A.ref)); }
+
 // One CTA per bucket of the partitioned segments, and per whole segment that
 // fits: range buckets and whole segments are sorted in shared memory, groups of
 // equal keys become new segments at depth d + v + C.  The sort is a chain of
@@ -954,29 +986,23 @@ __global__ void __launch_bounds__(THREADS, 65536 / (64 * THREADS)) k_lg_buckets(
             if (threadIdx.x == 0) A.redo[atomicAdd(&S->cnt[6], 1u)] = sidx;  // at most one entry per segment
             continue;
         }
-        for (uint32_t q = bs + threadIdx.x; q < bs + m; q += THREADS) A.perm[q] = A.tV[q];
-        if (threadIdx.x == 0) {
-            A.K[bs] = A.tK[bs];
-            A.K[bs + m - 1] = A.tK[bs + m - 1];
-        }
+        const uint64_t k = A.tK[bs];
+        const bool ended = eq && key_ended(k, f);
+        if (m <= BIG_RUN) copy_run<THREADS>(A, bs, m, ended, 0, 1);
+        if (threadIdx.x != 0) continue;
+        if (m > BIG_RUN) big_runs(A)[atomicAdd(&S->cnt[7], 1u)] = Seg{bs, m, ended ? 1u : 0u, 0};
+        A.K[bs] = k;
+        A.K[bs + m - 1] = A.tK[bs + m - 1];
         if (!eq) {
             // oversized range bucket: another round at this depth.  Its members
             // have distinct keys, so the LCPs across its two ends depend on which
             // members end up first and last: recomputed after the last round.
-            if (threadIdx.x == 0) {
-                const uint32_t be = bs + m;
-                push_seg(A, S->cnt, bs, m, sg.depth, err);
-                if (bs > sg.start) atomicOr(&A.fixmap[bs >> 5], 1u << (bs & 31u));
-                if (be < sg.start + sg.size) atomicOr(&A.fixmap[be >> 5], 1u << (be & 31u));
-            }
-        } else if (m >= 2) {
-            const uint64_t k = A.tK[bs];
-            if (!key_ended(k, f)) {
-                if (threadIdx.x == 0) push_seg(A, S->cnt, bs, m, sg.depth + key_v(k, f) + fmt_chars(f), err);
-            } else {
-                // a run of equal strings: lcp = length inside the run
-                for (uint32_t q = bs + 1 + threadIdx.x; q < bs + m; q += THREADS) A.lcp[q] = A.lens[A.tV[q]];
-            }
+            const uint32_t be = bs + m;
+            push_seg(A, S->cnt, bs, m, sg.depth, err);
+            if (bs > sg.start) atomicOr(&A.fixmap[bs >> 5], 1u << (bs & 31u));
+            if (be < sg.start + sg.size) atomicOr(&A.fixmap[be >> 5], 1u << (be & 31u));
+        } else if (m >= 2 && !ended) {
+            push_seg(A, S->cnt, bs, m, sg.depth + key_v(k, f) + fmt_chars(f), err);
         }
     }
 }
@@ -995,11 +1021,12 @@ __device__ __forceinline__ void lg_seams(const LsArgs& A, uint32_t s) {
 }
 
 // The last kernel of a round.  Bucket seams of the partitioned segments (their
-// buckets are sorted by now), then the segments of more than a bucket CTA's and
-// at most DIRECT_CAP strings, and those it handed on: one CTA sorts a whole
-// segment by its keys (no sampling, classification or scatter).  The last CTA to end decides whether the round
-// loop goes on: another round while segments were pushed, the round limit
-// holds and no capacity error occurred (loop = 1: inside a captured loop).
+// buckets are sorted by now) and the copies of the largest buckets, then the
+// segments of more than a bucket CTA's and at most DIRECT_CAP strings, and those it
+// handed on: one CTA sorts a whole segment by its keys (no sampling, classification
+// or scatter).  The last CTA to end decides whether the round loop goes on: another
+// round while segments were pushed, the round limit holds and no capacity error
+// occurred (loop = 1: inside a captured loop).
 template <int THREADS, int CAP>
 __global__ void __launch_bounds__(THREADS) k_lg_direct(LsDev* S, unsigned* err, cudaGraphConditionalHandle h,
                                                        int loop) {
@@ -1007,6 +1034,11 @@ __global__ void __launch_bounds__(THREADS) k_lg_direct(LsDev* S, unsigned* err, 
     const LsArgs& A = S->args;
     const uint32_t nbig = S->plan.nbig, npart = S->plan.npart;
     for (uint32_t s = blockIdx.x; s < npart; s += gridDim.x) lg_seams(A, s);
+    const uint32_t nruns = S->cnt[7];
+    for (uint32_t i = 0; i < nruns; ++i) {
+        const Seg run = big_runs(A)[i];
+        copy_run<THREADS>(A, run.start, run.size, run.depth != 0, blockIdx.x, gridDim.x);
+    }
     const uint32_t n = nbig + S->cnt[6];
     for (uint32_t i = blockIdx.x; i < n; i = cta_next_unit(&S->work[6])) {
         const uint32_t sidx = i < nbig ? npart + i : A.redo[i - nbig];

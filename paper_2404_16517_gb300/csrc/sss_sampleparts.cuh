@@ -113,7 +113,7 @@ struct LsArgs {
 struct LsDev {
     LsArgs args;
     LsPlan plan;
-    uint32_t cnt[8];   // segments per list; [6]: entries of redo
+    uint32_t cnt[8];   // segments per list; [6]: entries of redo, [7]: largest buckets, copied by the round's last kernel
     uint32_t work[8];  // dynamic work counters: [LC_*] finishers, [5] buckets, [6] direct, [7] CTAs done
     uint32_t rounds;
 };
@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(1024) k_lg_plan(LsDev* __restrict__ S, unsigne
             pl = LsPlan{0, 0, 0, 0, 0, 0, {0, 0}};
         }
         S->plan = pl;
-        S->cnt[LC_LARGE] = S->cnt[6] = 0;
+        S->cnt[LC_LARGE] = S->cnt[6] = S->cnt[7] = 0;
         S->work[5] = S->work[6] = S->work[7] = 0;
     }
 }

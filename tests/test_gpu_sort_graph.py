@@ -134,3 +134,22 @@ def test_keys_past_the_cached_reference(n, shared):
     perm, lcp, _, _ = sss.sss_sort(*d)
     sss.context().sync()
     _check(ss, sss.u32(perm), sss.u32(lcp))
+
+
+# buckets of equal keys around the size that is copied by all CTAs (2^17): equal
+# strings, and strings that go on past an equal key
+@pytest.mark.parametrize("m", [(1 << 17) - 3, (1 << 17) + 2, 300007])
+@pytest.mark.parametrize("kind", ["ended", "goes on"])
+def test_largest_equality_buckets(m, kind):
+    import paper_2404_16517_gb300 as sss
+    r = np.random.default_rng(m)
+    if kind == "ended":
+        strs = [b"EQUAL"] * m + [bytes(x) for x in r.integers(65, 91, (5000, 7)).astype(np.uint8)]
+    else:  # whichever half the reference is from, the other one's keys are equal
+        t = r.integers(65, 91, (2 * m, 3)).astype(np.uint8)
+        strs = [(b"B" if i & 1 else b"C") * 20 + t[i].tobytes() for i in range(2 * m)]
+    ss = datagen.from_strings([strs[i] for i in r.permutation(len(strs))])
+    chars, offs, lens = sss.to_device(ss)
+    perm, lcp, _, _ = sss.sss_sort(chars, offs, lens)
+    sss.context().sync()
+    _check(ss, sss.u32(perm), sss.u32(lcp))
