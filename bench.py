@@ -259,7 +259,7 @@ def main():
                     choices=["all", "pdms", "batch", "serve", "charsample", "suffix", "config1", "config3", "h2d"])
     ap.add_argument("--batch-instances", type=int, default=4096)
     ap.add_argument("--no-tune", action="store_true", help="batch: skip the autotuner (default knobs)")
-    ap.add_argument("--no-graph", action="store_true", help="batch: host-driven round loop only")
+    ap.add_argument("--no-graph", action="store_true", help="launch every kernel by itself instead of the sort's graph (for profilers; slower)")
     ap.add_argument("--per-instance-steps", type=int, default=2,
                     help="timed passes of one sss_sort call per instance (0: skip that comparison)")
     ap.add_argument("--serve-requests", type=int, default=20000)
@@ -319,29 +319,15 @@ def main():
     def step(prm_=None):
         sss.sss_sort(chars, offs, lens, args.p, prm_ or prm, perm, lcp, out_dist=dist_t, out_approx=approx, ctx=ctx)
 
-    # the local sort's round loop host-driven or as one graph launch: the faster
-    # is timed below (both are reported)
-    def loop_ms(prm_, reps=5):
-        for _ in range(2):
-            step(prm_)
-        torch.cuda.synchronize()
-        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        a.record()
-        for _ in range(reps):
-            step(prm_)
-        b.record()
-        torch.cuda.synchronize()
-        return a.elapsed_time(b) / reps
-
+    # a sort is one graph launch; with kernel timing on that takes the flag, and
+    # without it every kernel is launched, and timed, by itself
     prm_host = prm
-    prm_graph = sss.params(merge_ms=args.merge_ms, flags=sss.SSS_FLAG_GRAPH)
-    round_loop = {"ms_host_loop": loop_ms(prm_host), "ms_graph": loop_ms(prm_graph)}
-    round_loop["used"] = "graph" if round_loop["ms_graph"] < round_loop["ms_host_loop"] else "host"
-    if round_loop["used"] == "graph":
-        prm = prm_graph
+    if not args.no_graph:
+        prm = sss.params(merge_ms=args.merge_ms, flags=sss.SSS_FLAG_GRAPH)
+    round_loop = {"used": "kernels" if args.no_graph else "graph"}
 
-    # warm-up; the second one with every kernel timed (host-driven, so that the
-    # kernels inside a graph launch are timed one by one) to find the dominant kernel
+    # warm-up; the second one with every kernel timed, to find the dominant kernel
+    ctx.set_timing(args.no_graph, "")
     step()
     torch.cuda.synchronize()
     ctx.reset_stats()
@@ -349,7 +335,7 @@ def main():
     step(prm_host)
     torch.cuda.synchronize()
     stats_all = ctx.kernel_stats()
-    ctx.set_timing(False)
+    ctx.set_timing(args.no_graph, "")
     for _ in range(args.warmup - 2):
         step()
     torch.cuda.synchronize()
@@ -388,7 +374,7 @@ def main():
     hbm, peak_kind = peaks()
     dstat = stats.get(dom, {"launches": 0, "total_ms": 0.0, "timed": 0})
     per_step = args.steps
-    if dstat["timed"] == 0:  # the dominant kernel ran inside the graph: its host-driven time
+    if dstat["timed"] == 0:  # the dominant kernel ran inside the graph: its time launched by itself
         dstat, per_step = stats_all.get(dom), 1
     avg_ms = dstat["total_ms"] / max(1, dstat["timed"])
     algo = algorithmic_bytes(dom, n, N, D, Dapprox, dstat["launches"] / max(1, per_step))
@@ -556,35 +542,25 @@ def bench_batch(args, dev, ctx):
                   "ms_default_knobs": ms_default, "ms_tuned_knobs": ms_tuned,
                   "fastest_on_sample_ms": table[0][0], "slowest_on_sample_ms": table[-1][0]}
 
-    # the whole sort as one CUDA graph launch, against the host-driven round loop
-    graph = None
-    if not args.no_graph:
-        prm_g = sss.params(flags=prm.flags | sss.SSS_FLAG_GRAPH, cta_cap=prm.cta_cap, direct_cap=prm.direct_cap,
-                           bucket_target=prm.bucket_target, warp_cap=prm.warp_cap)
-        ms_host = timed(prm, max(1, args.steps // 2))
-        ms_graph = timed(prm_g, max(1, args.steps // 2))
-        graph = {"ms_host_loop": ms_host, "ms_graph": ms_graph, "used": ms_graph < ms_host}
-        p_host = perm.clone()
-        run(prm_g)
-        torch.cuda.synchronize()
-        graph["outputs_identical"] = bool(torch.equal(p_host, perm))
-        if ms_graph < ms_host:
-            prm = prm_g
+    if args.no_graph:
+        ctx.set_timing(True, "")
 
     def step():
         run(prm)
 
-    # per-kernel launch counts and times from one host-driven pass (kernels
-    # inside a graph launch are not timed one by one)
-    prm_h = sss.params(flags=prm.flags & ~sss.SSS_FLAG_GRAPH, cta_cap=prm.cta_cap, direct_cap=prm.direct_cap,
-                       bucket_target=prm.bucket_target, warp_cap=prm.warp_cap)
+    # launches of a step (its graph counts as one), then every kernel of a step
+    # launched and timed by itself
+    ctx.reset_stats()
+    run(prm)
+    torch.cuda.synchronize()
+    launches = sum(v["launches"] for v in ctx.kernel_stats().values())
     ctx.reset_stats()
     ctx.set_timing(True, "")
-    run(prm_h)
+    run(prm)
     torch.cuda.synchronize()
     stats = ctx.kernel_stats()
-    ctx.set_timing(False)
-    launches = sum(v["launches"] for v in stats.values())
+    ctx.set_timing(args.no_graph, "")
+    kernels = sum(v["launches"] for v in stats.values())
     if args.breakdown:
         print_breakdown(stats, "batch")
     for _ in range(args.warmup):
@@ -606,10 +582,7 @@ def bench_batch(args, dev, ctx):
     algo = D + 20 * n
     return {"workload": f"batch_{m}_instances_2^6..2^16_len8..300_ACGT", "instances": m, "strings": n, "chars": N,
             "D_over_N": D / N, "ms_per_step": ms, "chars_per_s": N / (ms / 1e3), "strings_per_s": n / (ms / 1e3),
-            # with the graph used a step is one instance-table upload and one graph
-            # launch whose nodes run the kernels counted from the host-driven pass
-            "gpu_launches_per_step": 1 if (graph and graph["used"]) else launches,
-            "kernels_per_step": launches, "tuning": tuning, "graph": graph,
+            "gpu_launches_per_step": launches, "kernels_per_step": kernels, "tuning": tuning,
             "per_instance_calls": per,
             "speedup_vs_per_instance": (per["ms_per_step"] / ms) if per else None,
             "outputs_identical": per["outputs_identical"] if per else None,
@@ -814,9 +787,7 @@ def bench_sort_config(args, dev, ctx, workload: str, chars, offs, lens, p: int, 
     """Time sss_sort on one more string set (a sub-line of the JSON): L2
     flushed (a 256 MB write) before every step, each step timed by its own CUDA
     events on the context stream, the dominant kernel's roofline and the
-    stage-level efficiencies as for the headline.  The local sort's round loop
-    runs host-driven and as one graph launch (SSS_FLAG_GRAPH); the faster is
-    reported, both are listed."""
+    stage-level efficiencies as for the headline."""
     import torch
 
     import paper_2404_16517_gb300 as sss
@@ -824,26 +795,7 @@ def bench_sort_config(args, dev, ctx, workload: str, chars, offs, lens, p: int, 
     N = int(lens.to(torch.int64).sum().item())
     flush = torch.empty(256 << 20, dtype=torch.uint8, device=dev)
     st = torch.cuda.current_stream(dev)
-    perm0 = torch.empty(n, dtype=torch.int32, device=dev)
-    lcp0 = torch.empty(n, dtype=torch.int32, device=dev)
-
-    def loop_ms(prm_, reps):
-        for _ in range(3):
-            sss.sss_sort(chars, offs, lens, p, prm_, perm0, lcp0, ctx=ctx)
-        ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(reps)]
-        torch.cuda.synchronize()
-        for i in range(reps):
-            flush.fill_(i & 0xFF)
-            ev[i][0].record(st)
-            sss.sss_sort(chars, offs, lens, p, prm_, perm0, lcp0, ctx=ctx)
-            ev[i][1].record(st)
-        torch.cuda.synchronize()
-        return statistics.mean(a.elapsed_time(b) for a, b in ev)
-
-    ms_host = loop_ms(sss.params(), 10)
-    ms_graph = loop_ms(sss.params(flags=sss.SSS_FLAG_GRAPH), 10)
-    prm = sss.params(flags=sss.SSS_FLAG_GRAPH) if ms_graph < ms_host else sss.params()
-    del perm0, lcp0
+    prm = sss.params(flags=sss.SSS_FLAG_GRAPH)  # (one graph launch a sort with kernel timing on, too)
     perm = torch.empty(n, dtype=torch.int32, device=dev)
     lcp = torch.empty(n, dtype=torch.int32, device=dev)
     dist_t = torch.empty(n, dtype=torch.int32, device=dev)
@@ -854,8 +806,7 @@ def bench_sort_config(args, dev, ctx, workload: str, chars, offs, lens, p: int, 
 
     for _ in range(args.warmup):
         step()
-    # per-kernel times from one host-driven pass (kernels inside a graph launch
-    # are not timed one by one)
+    # every kernel's time, launched by itself
     torch.cuda.synchronize()
     ctx.reset_stats()
     ctx.set_timing(True, "")
@@ -883,7 +834,7 @@ def bench_sort_config(args, dev, ctx, workload: str, chars, offs, lens, p: int, 
     hbm, peak_kind = peaks()
     dstat = stats.get(dom, {"launches": 0, "total_ms": 0.0, "timed": 0})
     per_step = steps
-    if dstat["timed"] == 0:  # the dominant kernel ran inside the graph: its host-driven time
+    if dstat["timed"] == 0:  # the dominant kernel ran inside the graph: its time launched by itself
         dstat, per_step = stats_all.get(dom), 1
     avg_ms = dstat["total_ms"] / max(1, dstat["timed"])
     algo = algorithmic_bytes(dom, n, N, D, Dapprox, dstat["launches"] / max(1, per_step))
@@ -894,8 +845,6 @@ def bench_sort_config(args, dev, ctx, workload: str, chars, offs, lens, p: int, 
             "ms_per_step": ms_step, "chars_per_s": N / (ms_step / 1e3), "strings_per_s": n / (ms_step / 1e3),
             "D_over_N": D / max(1, N), "approx_over_N": Dapprox / max(1, N), "gpu_launches_per_step": launches,
             "kernels_per_step": kernels,
-            "round_loop": {"ms_host_loop": ms_host, "ms_graph": ms_graph,
-                           "used": "graph" if ms_graph < ms_host else "host"},
             "l2": note,
             "roofline": {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": hbm, "unit": "GB/s",
                          "frac": achieved / hbm, "peak_kind": peak_kind, "algorithmic_bytes_per_launch": algo,
