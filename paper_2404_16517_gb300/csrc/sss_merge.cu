@@ -816,7 +816,7 @@ __global__ void k_d2_subspl(const BucketInfo* __restrict__ bi, uint32_t p, uint3
                             const uint32_t* __restrict__ smp, const uint32_t* __restrict__ sperm,
                             const uint32_t* __restrict__ s2lcp, const uint32_t* __restrict__ s2lens,
                             uint32_t* __restrict__ subspl, SubSpl* __restrict__ info) {
-    uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t m = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (m >= nss) return;
     uint32_t j = last_le(&bi[0].ss0, p, m, sizeof(BucketInfo) / 4, 0);
     // skip buckets without sub-splitters that share ss0
@@ -824,10 +824,17 @@ __global__ void k_d2_subspl(const BucketInfo* __restrict__ bi, uint32_t p, uint3
     const BucketInfo B = bi[j];
     const uint32_t rank = B.sbase + D2_OVS * (m - B.ss0 + 1) - 1, rlim = B.sbase + B.nsmp;
     const uint32_t f = smp[sperm[rank]], fl = tlen(S, f);
-    uint32_t rend = rank;
-    while (rend + 1 < rlim && s2lcp[rend + 1] >= fl && s2lens[sperm[rend + 1]] == fl) ++rend;
-    subspl[m] = f;
-    info[m] = SubSpl{S.offs[f], j, fl, rank, rend};
+    uint32_t rend = rank;  // the last sample equal to it, a lane per rank
+    for (bool all = true; all;) {
+        const uint32_t t = rend + 1 + lane;
+        const uint32_t eq = __ballot_sync(SSS_FULL, t < rlim && s2lcp[t] >= fl && s2lens[sperm[t]] == fl);
+        all = eq == SSS_FULL;
+        rend += all ? 32u : (uint32_t)__ffs((int)~eq) - 1u;
+    }
+    if (lane == 0) {
+        subspl[m] = f;
+        info[m] = SubSpl{S.offs[f], j, fl, rank, rend};
+    }
 }
 
 // Sorted rank of every second-level sample: srank[sperm[x]] = x.
@@ -1096,7 +1103,20 @@ __device__ __forceinline__ uint64_t d2_mask_from(uint32_t off) { return off == 0
 // (k_d2_recdec): the slice's positions are walked in run order (coalesced reads
 // of the run, no search for the slice, the predecessor's length by a shuffle),
 // every record is written for the merge and the fallback, and the forward walk
-// of the decode runs on the values still in registers.
+// of the decode runs on the values still in registers.  Bound by the chain of
+// dependent gathers of a chunk (string, offset and length, characters), so the
+// loads of the following chunks are in flight while one is decoded: the characters
+// of the next, the offsets and lengths of the one after, the strings of the third.
+// 79 -> 69 us on 1.05M strings with p = 4 (slices of 400 records), 14.9 -> 9.4 ms on 1M equal
+// strings (a slice per run); with slices of 64 records (4.19M, p = 16) it stays at 203.
+struct RecChunk {  // a lane's record in one chunk
+    uint32_t e, lcp;  // string, run LCP
+    uint32_t tl;      // its (truncated) length
+    uint64_t off;
+    uint32_t hr;      // LCP with the predecessor in the slice
+    uint64_t x0, x1;  // the aligned words that hold the characters at hr
+};
+
 __global__ void __launch_bounds__(256) k_d2_recdec(const uint32_t* __restrict__ run_perm,
                                                    const uint32_t* __restrict__ run_lcp, Strs S,
                                                    const BucketInfo* __restrict__ bi, uint32_t p, uint32_t nsb,
@@ -1120,44 +1140,89 @@ __global__ void __launch_bounds__(256) k_d2_recdec(const uint32_t* __restrict__ 
     const uint32_t q0 = pstart[j * p + i] + lo;  // run position of the slice's first string
     const uint32_t ref = sub_ref(B, b, subspl), uref = sub_uref(B, b, subspl);
     const uint32_t c = cb[b];
-    const uint32_t ef = run_perm[q0];
-    const uint32_t tlf = tlen(S, ef);
+    // the chunk o0's loads, in three steps; past the slice's end they read nothing
+    const auto load_strings = [&](RecChunk& k, uint32_t o0) {
+        const uint32_t o = o0 + lane;
+        k.e = k.lcp = 0;
+        if (o < len) {
+            k.e = run_perm[q0 + o];
+            k.lcp = run_lcp[q0 + o];
+        }
+    };
+    const auto load_extents = [&](RecChunk& k, uint32_t o0) {
+        k.tl = 0;
+        k.off = 0;
+        if (o0 + lane < len) {
+            k.tl = tlen(S, k.e);
+            k.off = S.offs[k.e];
+        }
+    };
+    uint32_t carry_tl = 0;
+    const auto load_heads = [&](RecChunk& k, uint32_t o0) {
+        uint32_t prev_tl = __shfl_up_sync(SSS_FULL, k.tl, 1);
+        if (lane == 0) prev_tl = carry_tl;
+        carry_tl = __shfl_sync(SSS_FULL, k.tl, 31);
+        const uint32_t o = o0 + lane;
+        k.hr = 0;
+        k.x0 = k.x1 = 0;
+        if (o < len) {
+            if (o > 0) k.hr = min(k.lcp, min(k.tl, prev_tl));
+            if (k.hr < k.tl) {
+                const uintptr_t a = (uintptr_t)(S.chars + k.off + k.hr);
+                const uint64_t* w = reinterpret_cast<const uint64_t*>(a & ~uintptr_t(7));
+                k.x0 = ld_chars8<true>(w);
+                if ((a & 7) != 0 && k.tl - k.hr > 8 - (uint32_t)(a & 7)) k.x1 = ld_chars8<true>(w + 1);
+            }
+        }
+    };
+    RecChunk c0, c1, c2;
+    load_strings(c0, 0);
+    load_strings(c1, 32);
+    load_strings(c2, 64);
+    load_extents(c0, 0);
+    load_extents(c1, 32);
+    load_heads(c0, 0);
+    const uint32_t tlf = __shfl_sync(SSS_FULL, c0.tl, 0);
+    const uint64_t offf = __shfl_sync(SSS_FULL, c0.off, 0);
     uint32_t r0 = 0, ul = 0;
-    if (ref != MINF) warp_cmp_from(S.chars + S.offs[ref], tlen(S, ref), S.chars + S.offs[ef], tlf, c, &r0);
-    const uint64_t key0 = load_word_be(S.chars + S.offs[ef], tlf, r0);
+    if (ref != MINF) warp_cmp_from(S.chars + S.offs[ref], tlen(S, ref), S.chars + offf, tlf, c, &r0);
+    const uint64_t key0 = load_word_be(S.chars + offf, tlf, r0);
     // forwards: the records, then r and the characters at r
-    uint32_t carry_r = 0xFFFFFFFFu, carry_tl = 0;
+    uint32_t carry_r = 0xFFFFFFFFu;
+    RecChunk last_e = c0;
     uint64_t carry_key = 0;
     for (uint32_t o0 = 0; o0 < len; o0 += 32) {
         const uint32_t o = o0 + lane;
         const bool valid = o < len;
         const uint32_t t = s0 + o;
-        uint32_t e = 0, tl = 0;
-        if (valid) {
-            e = run_perm[q0 + o];
-            tl = tlen(S, e);
-        }
-        uint32_t prev_tl = __shfl_up_sync(SSS_FULL, tl, 1);
-        if (lane == 0) prev_tl = carry_tl;
-        carry_tl = __shfl_sync(SSS_FULL, tl, 31);
+        const RecChunk k = c0;
+        load_heads(c1, o0 + 32);
+        load_extents(c2, o0 + 64);
+        RecChunk c3;
+        load_strings(c3, o0 + 96);
         uint32_t h = 0xFFFFFFFFu;
         uint64_t hw = 0ull;
         if (valid) {
-            uint32_t hr = 0;  // the record's LCP with its predecessor (0 for the slice's first)
-            if (o > 0) {
-                hr = run_lcp[q0 + o];
-                hr = hr < tl ? hr : tl;
-                hr = hr < prev_tl ? hr : prev_tl;
+            // the 8 characters at hr, zeros past the string's end
+            uint64_t head = 0;
+            if (k.hr < k.tl) {
+                const uint32_t sh = 8 * (uint32_t)((uintptr_t)(S.chars + k.off + k.hr) & 7), rem = k.tl - k.hr;
+                head = bswap64(k.x0) << sh;
+                if (sh) head |= bswap64(k.x1) >> (64 - sh);
+                if (rem < 8) head &= ~0ull << (8 * (8 - rem));
             }
-            const uint64_t head = load_word_be<true>(S.chars + S.offs[e], tl, hr);
-            R.idx[t] = e;
-            R.h[t] = hr;
-            R.tl[t] = tl;
+            R.idx[t] = k.e;
+            R.h[t] = k.hr;
+            R.tl[t] = k.tl;
             R.head[t] = head;
-            clen[t] = tl - hr;
-            h = o == 0 ? r0 : hr;
+            clen[t] = k.tl - k.hr;
+            h = o == 0 ? r0 : k.hr;
             hw = o == 0 ? key0 : head;
         }
+        last_e = k;
+        c0 = c1;
+        c1 = c2;
+        c2 = c3;
         uint32_t r = h;
 #pragma unroll
         for (uint32_t sh = 1; sh < 32; sh <<= 1) {
@@ -1196,21 +1261,32 @@ __global__ void __launch_bounds__(256) k_d2_recdec(const uint32_t* __restrict__ 
         carry_key = __shfl_sync(SSS_FULL, key, 31);
     }
     __syncwarp();  // the records and r written above are read back below
-    const uint32_t el = R.idx[s1 - 1];
+    const int ll = (int)((len - 1) & 31u);
+    const uint32_t tll = __shfl_sync(SSS_FULL, last_e.tl, ll);
+    const uint64_t offl = __shfl_sync(SSS_FULL, last_e.off, ll);
     // u of the last record: c when its r (the last chunk's lane 31 holds it:
     // lanes past the slice's end leave the minimum alone) is larger, as
     // min(r, u) = c; else compared from c on
     if (uref != PINF && uref != MINF) {
         if (carry_r > c) ul = c;
-        else warp_cmp_from(S.chars + S.offs[uref], tlen(S, uref), S.chars + S.offs[el], tlen(S, el), c, &ul);
+        else warp_cmp_from(S.chars + S.offs[uref], tlen(S, uref), S.chars + offl, tll, c, &ul);
     }
     // backwards
     uint32_t carry_u = ul;
     const uint32_t nch = (len + 31) / 32;
+    const auto load_back = [&](uint32_t ci, uint32_t* hn, uint32_t* rn) {  // the next record's h, the record's r
+        const uint32_t t = s0 + 32 * ci + lane;
+        *hn = t + 1 < s1 ? R.h[t + 1] : 0xFFFFFFFFu;
+        *rn = t < s1 ? rv[t] : 0u;
+    };
+    uint32_t hn, rt;
+    load_back(nch - 1, &hn, &rt);
     for (uint32_t ci = nch; ci-- > 0;) {
         const uint32_t t = s0 + 32 * ci + lane;
         const bool valid = t < s1;
-        uint32_t u = valid && t + 1 < s1 ? R.h[t + 1] : 0xFFFFFFFFu;  // h of the next record
+        uint32_t u = hn;
+        const uint32_t rc = rt;
+        if (ci > 0) load_back(ci - 1, &hn, &rt);
 #pragma unroll
         for (uint32_t sh = 1; sh < 32; sh <<= 1) {
             const uint32_t y = __shfl_down_sync(SSS_FULL, u, sh);
@@ -1219,8 +1295,7 @@ __global__ void __launch_bounds__(256) k_d2_recdec(const uint32_t* __restrict__ 
         u = carry_u < u ? carry_u : u;
         carry_u = __shfl_sync(SSS_FULL, u, 0);
         if (valid) {
-            const uint32_t rt = rv[t];
-            if (rt > c) {
+            if (rc > c) {
                 rs[t] = 0;  // rv and rk hold r and the characters at r
             } else if (u > c) {
                 rs[t] = 2;
@@ -1924,7 +1999,7 @@ sss_status impl_merge(sss_ctx* ctx, char* ws, size_t ws_bytes, const StrIn& in, 
         SSS_TRY(ss);
     }
     if (NSS > 0) {
-        SSS_TRY(sss_launch(ctx, "d2_subspl", k_d2_subspl, dim3((NSS + 63) / 64), dim3(64), 0,
+        SSS_TRY(sss_launch(ctx, "d2_subspl", k_d2_subspl, dim3((NSS * 32 + 255) / 256), dim3(256), 0,
                            (const BucketInfo*)b.binfo, p, NSS, S, (const uint32_t*)b.smp2, (const uint32_t*)b.s2perm,
                            (const uint32_t*)b.s2lcp, (const uint32_t*)b.s2lens, b.subspl, b.sinfo));
         SSS_TRY(sss_launch(ctx, "d2_srank", k_d2_srank, dim3((S2 + 255) / 256), dim3(256), 0,
