@@ -55,3 +55,20 @@ def test_partition(kind, n, p, v):
         sss.context().sync()
         assert np.array_equal(sss.u32(spl), want_spl)
         assert np.array_equal(sss.u32(bnd).reshape(-1), want_b.reshape(-1))
+
+
+# a few distinct strings only: runs of equal samples longer than a warp, slices of
+# one to hundreds of chunks of 32 records
+@pytest.mark.parametrize("n,p", [(33, 2), (5000, 2), (70001, 4), (70001, 16)])
+@pytest.mark.parametrize("distinct", [1, 3])
+def test_long_equal_runs(n, p, distinct):
+    import paper_2404_16517_gb300 as sss
+    r = np.random.default_rng(n + p)
+    base = [b"M" * 30 + bytes([65 + i]) for i in range(distinct)]
+    ss = datagen.from_strings([base[i] for i in r.integers(0, distinct, n)])
+    chars, offs, lens = sss.to_device(ss)
+    perm, lcp, _, _ = sss.sss_sort(chars, offs, lens, p)
+    sss.context().sync()
+    want = oracle.sort(ss)
+    assert np.array_equal(sss.u32(perm), want)
+    assert np.array_equal(sss.u32(lcp), oracle.lcp_array(ss, want))
