@@ -954,9 +954,12 @@ __device__ __forceinline__ bool block_bucket_sort(const uint64_t* sK, const uint
             q[5] |= (uint32_t)ch;
             q[6] &= cw[t];
             q[7] &= (uint32_t)ch;
-        } else if (side != 1) {
-            q[5] |= 1u;  // (no character bit: the low 2 + vb bits of ch are 0)
         }
+        // A key without characters ties with one whose varying bits are all 0 in the
+        // same head.  On sides 0 and 2 either may come with the other; on side 1 are
+        // the strings that end where the reference does, and with characters those
+        // that go on past it (a reference of 2^vb - 1 characters).
+        if ((ch != 0) == (side == 1)) q[5] |= 1u;  // (no character bit: the low 2 + vb bits of ch are 0)
     }
     q[0] = __reduce_min_sync(SSS_FULL, q[0]);
     q[1] = __reduce_max_sync(SSS_FULL, q[1]);
