@@ -369,8 +369,9 @@ sss_status sss_local_sort(sss_ctx* ctx, const uint8_t* chars, uint64_t n_chars, 
     StrIn in{chars, n_chars, offsets, lengths, n};
     if (prm.flags & SSS_FLAG_CHECKED) SSS_TRY(checked_input(ctx, in));
     char* ws;
-    SSS_TRY(sss_workspace(ctx, need_local_sort(n, p, prm), &ws));
-    Arena ar{ws, 0, 0};
+    const size_t need = need_local_sort(n, p, prm);
+    SSS_TRY(sss_workspace(ctx, need, &ws));
+    Arena ar{ws, need, 0};
     return impl_local_sort(ctx, ar, in, p, prm, out_run_perm, out_run_lcp);
 }
 
@@ -396,8 +397,9 @@ sss_status sss_dist_prefix(sss_ctx* ctx, const uint8_t* chars, uint64_t n_chars,
     StrIn in{chars, n_chars, offsets, lengths, n};
     if (prm.flags & SSS_FLAG_CHECKED) SSS_TRY(checked_input(ctx, in));
     char* ws;
-    SSS_TRY(sss_workspace(ctx, need_dist_prefix(n), &ws));
-    Arena ar{ws, 0, 0};
+    const size_t need = need_dist_prefix(n);
+    SSS_TRY(sss_workspace(ctx, need, &ws));
+    Arena ar{ws, need, 0};
     const uint32_t* rp = (prm.flags & SSS_FLAG_NO_LOCAL_LCP_SKIP) ? nullptr : run_perm;
     const uint32_t* rl = (prm.flags & SSS_FLAG_NO_LOCAL_LCP_SKIP) ? nullptr : run_lcp;
     return impl_dist_prefix(ctx, ar, in, rp, rl, p, prm, out_approx);
@@ -414,8 +416,9 @@ sss_status sss_partition(sss_ctx* ctx, const uint8_t* chars, uint64_t n_chars, c
     sss_params prm = resolve_params(params);
     StrIn in{chars, n_chars, offsets, lengths, n};
     char* ws;
-    SSS_TRY(sss_workspace(ctx, need_partition(n, p, prm.v), &ws));
-    Arena ar{ws, 0, 0};
+    const size_t need = need_partition(n, p, prm.v);
+    SSS_TRY(sss_workspace(ctx, need, &ws));
+    Arena ar{ws, need, 0};
     return impl_partition(ctx, ar, in, trunc, run_perm, p, prm.v, prm.flags, out_splitters, out_bounds);
 }
 
@@ -493,8 +496,9 @@ sss_status sss_sort(sss_ctx* ctx, const uint8_t* chars, uint64_t n_chars, const 
     if (prm.flags & SSS_FLAG_CHECKED) SSS_TRY(checked_input(ctx, in));
     if (p == 1) {
         char* ws;
-        SSS_TRY(sss_workspace(ctx, need_local_sort(n, 1, prm), &ws));
-        Arena ar{ws, 0, 0};
+        const size_t need = need_local_sort(n, 1, prm);
+        SSS_TRY(sss_workspace(ctx, need, &ws));
+        Arena ar{ws, need, 0};
         SSS_TRY(impl_local_sort(ctx, ar, in, 1, prm, out_perm, out_lcp));
         if (out_dist) SSS_TRY(impl_dist(ctx, lengths, n, out_perm, out_lcp, out_dist));
         if (out_approx)
@@ -590,8 +594,9 @@ sss_status sss_sort_host(sss_ctx* ctx, const uint8_t* h_chars, uint64_t n_chars,
     };
     if (p == 1) {
         char* ws;
-        SSS_TRY(sss_workspace(ctx, need_local_sort(n, 1, prm), &ws));
-        Arena ar{ws, 0, 0};
+        const size_t need = need_local_sort(n, 1, prm);
+        SSS_TRY(sss_workspace(ctx, need, &ws));
+        Arena ar{ws, need, 0};
         SSS_TRY(stage_a(ar, out_perm, out_lcp));
     } else {
         SSS_TRY(run_pipeline(ctx, in, p, prm, out_perm, out_lcp, nullptr, nullptr, stage_a));

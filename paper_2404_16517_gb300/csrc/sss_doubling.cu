@@ -971,6 +971,7 @@ sss_status impl_dist_prefix(sss_ctx* ctx, Arena& ar, const StrIn& sin, const uin
     if (n == 0) return SSS_OK;
     PdBufs B;
     carve_pd(ar, n, B);
+    SSS_TRY(sss_fits(ctx, ar));
     if (!g_pd_attr[ctx->device & 63]) {
         SSS_CUDA(cudaFuncSetAttribute(k_pd_buckets, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)(DD_CAP * (8 + 8 + 1))));

@@ -28,7 +28,8 @@ struct Seg {
 
 // ---------------------------------------------------------------------------
 // Bump allocator over one device buffer.  With base == nullptr it only counts,
-// so the same carving code gives the workspace size.
+// so the same carving code gives the workspace size.  It hands out past `cap` too:
+// whoever carves checks sss_fits before the first use.
 struct Arena {
     char* base = nullptr;
     size_t cap = 0;
@@ -127,6 +128,13 @@ sss_status sss_workspace(sss_ctx* ctx, size_t bytes, char** out);
 sss_status sss_pinned(sss_ctx* ctx, size_t bytes, void** out);
 // Asynchronous upload from the pinned staging buffer (tracked by pin_event).
 sss_status sss_upload(sss_ctx* ctx, void* dst, const void* src, size_t bytes);
+
+// What was carved lies inside the buffer.
+inline sss_status sss_fits(sss_ctx* ctx, const Arena& ar) {
+    if (!ar.base || ar.off <= ar.cap) return SSS_OK;
+    return sss_fail(ctx, SSS_ERR_WORKSPACE, "work memory overrun: " + std::to_string(ar.off) + " of " +
+                                                std::to_string(ar.cap) + " bytes");
+}
 
 // Instrumentation hooks used by the launch wrapper.
 int sss_stat_index(sss_ctx* ctx, const char* name);

@@ -1132,8 +1132,10 @@ __global__ void k_check_input(const uint8_t* __restrict__ chars, uint64_t n_char
 //    CTA's 4,352 and 8,192 strings, and one CTA of 1024 threads with an SM to
 //    itself is a long chain; partitioned they use every SM (serving 468 us against
 //    397).  Above, there are enough of them (the batch: 4839 us against 4902).
+// direct_min: the smallest value of the rule for direct_cap, so that the work memory
+// never shrinks as n grows (a segment above it may be partitioned).
 struct LsKnobs {
-    uint32_t warp_cap, cta_cap, direct_cap, bucket_target;
+    uint32_t warp_cap, cta_cap, direct_cap, bucket_target, direct_min;
 };
 static LsKnobs ls_knobs(const sss_params& prm, uint32_t n, bool rounds) {
     LsKnobs k;
@@ -1142,6 +1144,7 @@ static LsKnobs ls_knobs(const sss_params& prm, uint32_t n, bool rounds) {
                             : (rounds ? 256u : (uint32_t)MED_CAP);
     const uint32_t direct = n > (1u << 22) ? (uint32_t)DIRECT_CAP : (uint32_t)BK_CAP;
     k.direct_cap = std::min(std::max(prm.direct_cap ? prm.direct_cap : direct, k.cta_cap), (uint32_t)DIRECT_CAP);
+    k.direct_min = prm.direct_cap ? k.direct_cap : (uint32_t)BK_CAP;
     k.bucket_target = prm.bucket_target ? std::min(std::max(prm.bucket_target, 256u), 4096u) : 2048u;
     return k;
 }
@@ -1165,7 +1168,7 @@ void carve_ls(Arena& ar, uint32_t n, uint32_t p, const sss_params& prm, LsArgs& 
     for (uint32_t c = LC_TINY; c <= LC_LARGE; ++c) a.list[c] = ar.take<Seg>(a.cap[c]);
     a.segfmt = ar.take<uint32_t>(a.cap[LC_LARGE]);
     a.fixmap = ar.take<uint32_t>(n / 32 + 1);
-    carve_sp(ar, n, a.cap[LC_LARGE], n / (kn.direct_cap + 1) + p + 2, a);
+    carve_sp(ar, n, a.cap[LC_LARGE], n / (kn.direct_min + 1) + p + 2, a);
     a.warp_max = kn.warp_cap;
     a.med_max = kn.cta_cap;
     a.direct_max = kn.direct_cap;
@@ -1439,6 +1442,7 @@ sss_status impl_sort_segments_range(sss_ctx* ctx, Arena& ar, const StrIn& in, co
     bool rounds = false;  // a segment that the CTA finisher cannot take
     for (const Seg& s : init) rounds = rounds || s.size > kn.cta_cap;
     const LsArgs A = ls_args(ar, in, prm, rounds, perm, lcp, q0, q1);
+    SSS_TRY(sss_fits(ctx, ar));
     LsDev* S = static_cast<LsDev*>(ctx->d_ls);
 
     // initial segments (partitions or instances), counted by size class
@@ -1527,6 +1531,7 @@ sss_status impl_groups_begin(sss_ctx* ctx, Arena ar, const StrIn& in, const sss_
                              uint32_t* lcp, const uint32_t* group_start, const uint32_t* d_groups,
                              const uint32_t** d_counts) {
     LsArgs A = ls_args(ar, in, prm, false, perm, lcp, 0, in.n);
+    SSS_TRY(sss_fits(ctx, ar));
     A.keep = 1;
     SSS_TRY(set_ls_attributes(ctx));
     LsDev* S = static_cast<LsDev*>(ctx->d_ls);

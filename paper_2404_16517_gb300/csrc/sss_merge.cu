@@ -1766,6 +1766,7 @@ sss_status impl_partition(sss_ctx* ctx, Arena& ar, const StrIn& in, const uint32
                           uint32_t p, uint32_t v, uint32_t flags, uint32_t* out_spl, uint32_t* out_bounds) {
     MgBufs b;
     carve_mg_small(ar, in.n, p, v, b);
+    SSS_TRY(sss_fits(ctx, ar));
     SSS_TRY(run_partition(ctx, in, trunc, run_perm, p, v, flags, b));
     if (p > 1 && out_spl)
         SSS_CUDA(cudaMemcpyAsync(out_spl, b.spl, sizeof(uint32_t) * (p - 1), cudaMemcpyDeviceToDevice, ctx->stream));
@@ -1884,6 +1885,7 @@ sss_status impl_merge(sss_ctx* ctx, char* ws, size_t ws_bytes, const StrIn& in, 
     Arena ar{ws, ws_bytes, 0};
     MgBufs b;
     carve_mg(ar, n, p, v, nrecchars, b);
+    SSS_TRY(sss_fits(ctx, ar));
     Strs S{in.chars, in.offs, in.lens, trunc};
     SSS_TRY(run_partition(ctx, in, trunc, run_perm, p, v, flags, b));
     const bool two_level = p <= MAX_P_TWO_LEVEL && !(flags & SSS_FLAG_MERGE_TREE);

@@ -190,7 +190,8 @@ sss_status impl_suffix_sort(sss_ctx* ctx, char* ws, size_t ws_bytes, const uint8
     uint32_t* lvbase[SX_MAXLEV];
     for (uint32_t t = 0; t < nlev; ++t) lvbase[t] = ar.take<uint32_t>(n);
     size_t sort_off = (ar.off + 255) & ~size_t(255);
-    const Arena sort_ar{ws + sort_off, need_local_sort(n, 1, prm), 0};
+    SSS_TRY(sss_fits(ctx, ar));
+    const Arena sort_ar{ws + sort_off, ws_bytes > sort_off ? ws_bytes - sort_off : 0, 0};
     const uint32_t sm = (uint32_t)std::max(1, ctx->sm_count);
     const uint32_t grid = std::min((n + 255) / 256, sm * 16);
     const uint32_t target = max_len ? std::min(max_len, n) : n;
