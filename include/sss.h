@@ -27,7 +27,8 @@
  *  - Work memory is owned by the context: it is allocated with cudaMalloc on
  *    first use and grown when a larger problem arrives, or supplied by the caller
  *    with sss_set_workspace().
- *  - A context is not thread-safe; use one context per host thread.
+ *  - A context is not thread-safe; use one context per host thread.  Its calls run
+ *    one after the other, also when they are on different streams (sss_set_stream).
  *  - Limits: n < 2^32 - 1, 1 <= p <= 1024, string lengths < 2^31.
  */
 #ifndef SSS_H
@@ -115,7 +116,12 @@ sss_status sss_create(sss_ctx** out, int device, void* cuda_stream);
 /* Destroy a context (synchronises its stream, frees its memory).  NULL is a no-op. */
 sss_status sss_destroy(sss_ctx* ctx);
 
-/* Change the stream subsequent calls enqueue on. */
+/* Change the stream subsequent calls enqueue on.  The new stream waits for the
+ * context's last call (on the device, the host does not): a context's calls run one
+ * after the other whatever their streams, as they share its work memory and device
+ * state.  Use one context per stream for calls that are to overlap.  The old stream
+ * need not exist any more.  Calls captured into a CUDA graph are outside this order:
+ * the caller lets a launch of that graph overlap none of the context's other calls. */
 sss_status sss_set_stream(sss_ctx* ctx, void* cuda_stream);
 
 /* Hand the context a caller-owned device buffer to use as work memory instead of

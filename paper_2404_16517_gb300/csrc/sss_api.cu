@@ -186,6 +186,7 @@ sss_status sss_create(sss_ctx** out, int device, void* stream) {
         return SSS_ERR_OOM;
     }
     cudaEventCreateWithFlags(&ctx->pin_event, cudaEventDisableTiming);
+    cudaEventCreateWithFlags(&ctx->call_event, cudaEventDisableTiming);
     cudaEventRecord(ctx->pin_event, ctx->stream);
     cudaDeviceSynchronize();
     *out = ctx;
@@ -216,13 +217,30 @@ sss_status sss_destroy(sss_ctx* ctx) {
     if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
     for (cudaEvent_t e : ctx->chunk_events) cudaEventDestroy(e);
     if (ctx->pin_event) cudaEventDestroy(ctx->pin_event);
+    if (ctx->call_event) cudaEventDestroy(ctx->call_event);
     delete ctx;
     return SSS_OK;
 }
 
 sss_status sss_set_stream(sss_ctx* ctx, void* stream) {
     if (!ctx) return SSS_ERR_INVALID_ARG;
-    ctx->stream = static_cast<cudaStream_t>(stream);
+    const cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (st == ctx->stream) return SSS_OK;
+    if (ctx->called) {
+        // the context's calls share its work memory and device state: the new stream
+        // waits for the last one
+        int dev = ctx->device;
+        cudaGetDevice(&dev);
+        cudaSetDevice(ctx->device);
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        cudaError_t e = cudaStreamIsCapturing(st, &cap);
+        if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone) e = cudaStreamWaitEvent(st, ctx->call_event, 0);
+        if (e != cudaSuccess) cudaGetLastError();
+        cudaSetDevice(dev);
+        if (e != cudaSuccess)
+            return sss_fail(ctx, SSS_ERR_CUDA, std::string("sss_set_stream: ") + cudaGetErrorString(e));
+    }
+    ctx->stream = st;
     return SSS_OK;
 }
 
@@ -365,6 +383,7 @@ sss_status sss_local_sort(sss_ctx* ctx, const uint8_t* chars, uint64_t n_chars, 
     if (n > 0 && (!out_run_perm || !out_run_lcp)) return sss_fail(ctx, SSS_ERR_INVALID_ARG, "outputs must be non-NULL");
     if (n == 0) return SSS_OK;
     cudaSetDevice(ctx->device);
+    const CallEnd end{ctx};
     sss_params prm = resolve_params(params);
     StrIn in{chars, n_chars, offsets, lengths, n};
     if (prm.flags & SSS_FLAG_CHECKED) SSS_TRY(checked_input(ctx, in));
@@ -381,6 +400,7 @@ sss_status sss_dist(sss_ctx* ctx, const uint32_t* lengths, uint32_t n, const uin
     if (n == 0) return SSS_OK;
     if (!lengths || !perm || !lcp || !out_dist) return sss_fail(ctx, SSS_ERR_INVALID_ARG, "NULL pointer");
     cudaSetDevice(ctx->device);
+    const CallEnd end{ctx};
     return impl_dist(ctx, lengths, n, perm, lcp, out_dist);
 }
 
@@ -393,6 +413,7 @@ sss_status sss_dist_prefix(sss_ctx* ctx, const uint8_t* chars, uint64_t n_chars,
     if (n > 0 && !out_approx) return sss_fail(ctx, SSS_ERR_INVALID_ARG, "out_approx must be non-NULL");
     if (n == 0) return SSS_OK;
     cudaSetDevice(ctx->device);
+    const CallEnd end{ctx};
     sss_params prm = resolve_params(params);
     StrIn in{chars, n_chars, offsets, lengths, n};
     if (prm.flags & SSS_FLAG_CHECKED) SSS_TRY(checked_input(ctx, in));
@@ -413,6 +434,7 @@ sss_status sss_partition(sss_ctx* ctx, const uint8_t* chars, uint64_t n_chars, c
     if (!out_bounds || (p > 1 && !out_splitters))
         return sss_fail(ctx, SSS_ERR_INVALID_ARG, "outputs must be non-NULL");
     cudaSetDevice(ctx->device);
+    const CallEnd end{ctx};
     sss_params prm = resolve_params(params);
     StrIn in{chars, n_chars, offsets, lengths, n};
     char* ws;
@@ -431,6 +453,7 @@ sss_status sss_lcp_merge(sss_ctx* ctx, const uint8_t* chars, uint64_t n_chars, c
         return sss_fail(ctx, SSS_ERR_INVALID_ARG, "NULL pointer");
     if (n == 0) return SSS_OK;
     cudaSetDevice(ctx->device);
+    const CallEnd end{ctx};
     sss_params prm = resolve_params(params);
     StrIn in{chars, n_chars, offsets, lengths, n};
     uint64_t tot = 0;
@@ -491,6 +514,7 @@ sss_status sss_sort(sss_ctx* ctx, const uint8_t* chars, uint64_t n_chars, const 
     if (n > 0 && (!out_perm || !out_lcp)) return sss_fail(ctx, SSS_ERR_INVALID_ARG, "outputs must be non-NULL");
     if (n == 0) return SSS_OK;
     cudaSetDevice(ctx->device);
+    const CallEnd end{ctx};
     sss_params prm = resolve_params(params);
     StrIn in{chars, n_chars, offsets, lengths, n};
     if (prm.flags & SSS_FLAG_CHECKED) SSS_TRY(checked_input(ctx, in));
@@ -520,6 +544,7 @@ sss_status sss_sort_host(sss_ctx* ctx, const uint8_t* h_chars, uint64_t n_chars,
         return sss_fail(ctx, SSS_ERR_INVALID_ARG, "device buffers and outputs must be non-NULL");
     if (n == 0) return SSS_OK;
     cudaSetDevice(ctx->device);
+    const CallEnd end{ctx};
     sss_params prm = resolve_params(params);
     if (prm.flags & SSS_FLAG_CHECKED)
         return sss_fail(ctx, SSS_ERR_UNIMPLEMENTED, "sss_sort_host: SSS_FLAG_CHECKED needs sss_sort");
@@ -629,6 +654,7 @@ sss_status sss_sort_batch(sss_ctx* ctx, const uint8_t* chars, uint64_t n_chars, 
         if ((uint64_t)sorted[k - 1].start + sorted[k - 1].size > sorted[k].start)
             return sss_fail(ctx, SSS_ERR_INVALID_ARG, "instances overlap");
     cudaSetDevice(ctx->device);
+    const CallEnd end{ctx};
     sss_params prm = resolve_params(params);
     StrIn in{chars, n_chars, offsets, lengths, n_table};
     if (prm.flags & SSS_FLAG_CHECKED) SSS_TRY(checked_input(ctx, in));
@@ -660,6 +686,7 @@ sss_status sss_suffix_sort(sss_ctx* ctx, const uint8_t* text, uint64_t n_text, u
     if (n_text == 0) return SSS_OK;
     if (!text || !out_sa || !out_lcp) return sss_fail(ctx, SSS_ERR_INVALID_ARG, "NULL pointer");
     cudaSetDevice(ctx->device);
+    const CallEnd end{ctx};
     sss_params prm = resolve_params(params);
     const uint32_t n = (uint32_t)n_text;
     const size_t need = sss_suffix_workspace_bytes(n_text, &prm);

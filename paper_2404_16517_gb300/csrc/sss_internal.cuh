@@ -70,6 +70,10 @@ struct sss_ctx {
     void* h_pin = nullptr;
     size_t h_pin_bytes = 0;
     cudaEvent_t pin_event = nullptr;
+    // end of the context's last call, which a call on another stream waits for
+    // (sss_set_stream)
+    cudaEvent_t call_event = nullptr;
+    bool called = false;
     // sticky device error word
     unsigned* d_err = nullptr;
     // small device scratch for counters and reductions (never inside the workspace)
@@ -135,6 +139,25 @@ inline sss_status sss_fits(sss_ctx* ctx, const Arena& ar) {
     return sss_fail(ctx, SSS_ERR_WORKSPACE, "work memory overrun: " + std::to_string(ar.off) + " of " +
                                                 std::to_string(ar.cap) + " bytes");
 }
+
+// Marks the end of a call on the context's stream when it goes out of scope.  The
+// event is recorded then, and not on the old stream when the stream is changed,
+// because that stream may be gone by then.  (A call being captured has no place on
+// the stream: whoever launches the graph orders it.)
+struct CallEnd {
+    sss_ctx* ctx;
+    ~CallEnd() {
+        cudaStreamCaptureStatus st;
+        if (cudaStreamIsCapturing(ctx->stream, &st) == cudaSuccess) {
+            if (st != cudaStreamCaptureStatusNone) return;
+            if (cudaEventRecord(ctx->call_event, ctx->stream) == cudaSuccess) {
+                ctx->called = true;
+                return;
+            }
+        }
+        cudaGetLastError();
+    }
+};
 
 // Instrumentation hooks used by the launch wrapper.
 int sss_stat_index(sss_ctx* ctx, const char* name);
