@@ -670,7 +670,7 @@ sss_status sss_sort_batch(sss_ctx* ctx, const uint8_t* chars, uint64_t n_chars, 
     SSS_TRY(sss_upload(ctx, d_inst, pin, sizeof(Seg) * m));
     size_t off = (ar.off + 255) & ~size_t(255);
     Arena sa{ws + off, need - off, 0};
-    SSS_TRY(impl_sort_segments(ctx, sa, in, segs, prm, out_perm, out_lcp));
+    SSS_TRY(impl_sort_segments(ctx, sa, in, segs, prm, out_perm, out_lcp, d_inst));
     return impl_batch_finish(ctx, d_inst, m, lengths, out_perm, out_lcp, out_dist);
 }
 

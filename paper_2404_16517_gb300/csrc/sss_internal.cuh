@@ -211,12 +211,14 @@ sss_status impl_local_sort(sss_ctx* ctx, Arena& ar, const StrIn& in, uint32_t p,
                            uint32_t* perm, uint32_t* lcp);
 size_t need_local_sort(uint32_t n, uint32_t p, const sss_params& prm);
 // Sort every given segment of positions (each starting at depth 0) independently.
+// d_init: the same segments in device memory, if the caller has them there.
 sss_status impl_sort_segments(sss_ctx* ctx, Arena& ar, const StrIn& in, const std::vector<Seg>& init,
-                              const sss_params& prm, uint32_t* perm, uint32_t* lcp);
+                              const sss_params& prm, uint32_t* perm, uint32_t* lcp, const Seg* d_init = nullptr);
 // The same for segments inside positions [q0, q1): only that range of perm and
 // lcp is initialised and written (other positions keep their contents).
 sss_status impl_sort_segments_range(sss_ctx* ctx, Arena& ar, const StrIn& in, const std::vector<Seg>& init,
-                                    const sss_params& prm, uint32_t* perm, uint32_t* lcp, uint32_t q0, uint32_t q1);
+                                    const sss_params& prm, uint32_t* perm, uint32_t* lcp, uint32_t q0, uint32_t q1,
+                                    const Seg* d_init = nullptr);
 // Refining a sorted order group by group (see sss_local_sort.cu).
 sss_status impl_groups_begin(sss_ctx* ctx, Arena ar, const StrIn& in, const sss_params& prm, uint32_t* perm,
                              uint32_t* lcp, const uint32_t* group_start, const uint32_t* d_groups,

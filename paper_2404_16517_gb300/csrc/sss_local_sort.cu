@@ -1366,8 +1366,8 @@ static sss_status sort_graph(sss_ctx* ctx, uint32_t gcls, bool small, cudaGraphE
 }
 
 sss_status impl_sort_segments(sss_ctx* ctx, Arena& ar, const StrIn& in, const std::vector<Seg>& init,
-                              const sss_params& prm, uint32_t* perm, uint32_t* lcp) {
-    return impl_sort_segments_range(ctx, ar, in, init, prm, perm, lcp, 0, in.n);
+                              const sss_params& prm, uint32_t* perm, uint32_t* lcp, const Seg* d_init) {
+    return impl_sort_segments_range(ctx, ar, in, init, prm, perm, lcp, 0, in.n, d_init);
 }
 
 // The call's arguments for a sort of positions [q0, q1) with work memory from ar.
@@ -1427,7 +1427,8 @@ static sss_status run_sort(sss_ctx* ctx, const LsArgs& A, const sss_params& prm,
 }
 
 sss_status impl_sort_segments_range(sss_ctx* ctx, Arena& ar, const StrIn& in, const std::vector<Seg>& init,
-                                    const sss_params& prm, uint32_t* perm, uint32_t* lcp, uint32_t q0, uint32_t q1) {
+                                    const sss_params& prm, uint32_t* perm, uint32_t* lcp, uint32_t q0, uint32_t q1,
+                                    const Seg* d_init) {
     const uint32_t n = in.n;
     if (n == 0 || q1 <= q0) return SSS_OK;
     const uint32_t nr = q1 - q0;
@@ -1461,9 +1462,15 @@ sss_status impl_sort_segments_range(sss_ctx* ctx, Arena& ar, const StrIn& in, co
     li.n = m <= LS_INLINE ? m : 0u;
     SSS_TRY(sss_launch(ctx, "ls_init", k_ls_begin, dim3((nr + BG_T * BG_PER - 1) / (BG_T * BG_PER)), dim3(BG_T), 0, S,
                        A, li, ctx->d_err));
-    if (m > LS_INLINE) {
-        // more than fit in the launch's arguments: through the second key array,
-        // free until the first scatter (every one holds >= 2 strings of 8 bytes there)
+    if (m > LS_INLINE && d_init) {
+        // more than fit in the launch's arguments, and in device memory already
+        const uint32_t all = (uint32_t)init.size();
+        SSS_TRY(sss_launch(ctx, "ls_classify", k_ls_classify,
+                           dim3(std::min((all + BG_T - 1) / BG_T, (uint32_t)ctx->sm_count)), dim3(BG_T), 0, S, d_init,
+                           all, ctx->d_err));
+    } else if (m > LS_INLINE) {
+        // through the second key array, free until the first scatter (every one
+        // holds >= 2 strings of 8 bytes there)
         void* pin;
         SSS_TRY(sss_pinned(ctx, sizeof(Seg) * (size_t)m, &pin));
         Seg* h = static_cast<Seg*>(pin);
