@@ -95,7 +95,8 @@ typedef struct sss_params {
                                where every segment fits that, else 256) */
     uint32_t merge_ms;      /* merge segment spacing, a power of two 8..1024 (default 32) */
     uint32_t direct_cap;    /* largest segment of the multi-CTA path sorted whole by one CTA,
-                               cta_cap..8192 (default 8192 above 2^22 strings, else 4352) */
+                               cta_cap..8192 (default 8192, but a few of more than 4352
+                               are partitioned) */
     uint32_t bucket_target; /* target size of a sampled-partition range bucket, 256..4096
                                (default 2048) */
     uint32_t warp_cap;      /* largest segment finished by one warp, 2..32 (default 32) */

@@ -1120,30 +1120,26 @@ __global__ void k_check_input(const uint8_t* __restrict__ chars, uint64_t n_char
         }
 }
 
-// The size-class knobs of the local sort for a call of n strings; 0 takes the
-// default (values are clamped by the API already).  Two defaults are rules:
+// The size-class knobs of the local sort; 0 takes the default (values are clamped
+// by the API already).  Two defaults are rules:
 //  * cta_cap: a call whose segments all fit the CTA finisher (<= 2,048 strings)
 //    runs no rounds, which cost it 28 us more (1,000 strings: 27 us against 55).
 //    With larger segments the rounds run anyway, and the bucket CTAs sort a
 //    segment of more than 256 strings faster than the finisher, whose every
 //    iteration sorts (group, key, index): 11 serving requests 397 us with 2,048,
 //    337 with 256; the 4,096-instance batch 4839 and 4804.
-//  * direct_cap: up to 2^22 strings there are few segments between the bucket
-//    CTA's 4,352 and 8,192 strings, and one CTA of 1024 threads with an SM to
-//    itself is a long chain; partitioned they use every SM (serving 468 us against
-//    397).  Above, there are enough of them (the batch: 4839 us against 4902).
-// direct_min: the smallest value of the rule for direct_cap, so that the work memory
-// never shrinks as n grows (a segment above it may be partitioned).
+//  * direct_cap: 8,192, but k_lg_plan may have the segments above direct_min, a
+//    bucket CTA's capacity, partitioned.  A given value holds as it is.
 struct LsKnobs {
     uint32_t warp_cap, cta_cap, direct_cap, bucket_target, direct_min;
 };
-static LsKnobs ls_knobs(const sss_params& prm, uint32_t n, bool rounds) {
+static LsKnobs ls_knobs(const sss_params& prm, bool rounds) {
     LsKnobs k;
     k.warp_cap = prm.warp_cap ? std::min(prm.warp_cap, 32u) : 32u;
     k.cta_cap = prm.cta_cap ? std::min(std::max(prm.cta_cap, (uint32_t)TINY_CAP), (uint32_t)MED_CAP)
                             : (rounds ? 256u : (uint32_t)MED_CAP);
-    const uint32_t direct = n > (1u << 22) ? (uint32_t)DIRECT_CAP : (uint32_t)BK_CAP;
-    k.direct_cap = std::min(std::max(prm.direct_cap ? prm.direct_cap : direct, k.cta_cap), (uint32_t)DIRECT_CAP);
+    k.direct_cap = prm.direct_cap ? std::min(std::max(prm.direct_cap, k.cta_cap), (uint32_t)DIRECT_CAP)
+                                  : (uint32_t)DIRECT_CAP;
     k.direct_min = prm.direct_cap ? k.direct_cap : (uint32_t)BK_CAP;
     k.bucket_target = prm.bucket_target ? std::min(std::max(prm.bucket_target, 256u), 4096u) : 2048u;
     return k;
@@ -1154,7 +1150,7 @@ bool small_buckets(uint32_t target) { return target <= (uint32_t)BKS_CAP / 2; }
 
 // Work memory of the local sort: fills the pointers and capacities of a.
 void carve_ls(Arena& ar, uint32_t n, uint32_t p, const sss_params& prm, LsArgs& a) {
-    const LsKnobs kn = ls_knobs(prm, n, true);  // the one with more large segments
+    const LsKnobs kn = ls_knobs(prm, true);  // the one with more large segments
     a.cap[LC_QUAD] = a.cap[LC_WARP] = n / 2 + 2;
     a.cap[LC_TINY] = n / (kn.warp_cap + 1) + 2;
     a.cap[LC_SMALL] = n / (TINY_CAP + 1) + 2;
@@ -1172,6 +1168,7 @@ void carve_ls(Arena& ar, uint32_t n, uint32_t p, const sss_params& prm, LsArgs& 
     a.warp_max = kn.warp_cap;
     a.med_max = kn.cta_cap;
     a.direct_max = kn.direct_cap;
+    a.direct_min = kn.direct_min;
     a.target = kn.bucket_target;
     a.bucket_cap = small_buckets(kn.bucket_target) ? BKS_CAP : BK_CAP;
     a.limit = 100000u;
@@ -1371,11 +1368,14 @@ sss_status impl_sort_segments(sss_ctx* ctx, Arena& ar, const StrIn& in, const st
 }
 
 // The call's arguments for a sort of positions [q0, q1) with work memory from ar.
-static LsArgs ls_args(Arena& ar, const StrIn& in, const sss_params& prm, bool rounds, uint32_t* perm, uint32_t* lcp,
-                      uint32_t q0, uint32_t q1) {
+static LsArgs ls_args(const sss_ctx* ctx, Arena& ar, const StrIn& in, const sss_params& prm, bool rounds,
+                      uint32_t* perm, uint32_t* lcp, uint32_t q0, uint32_t q1) {
     LsArgs A{};
     carve_ls(ar, in.n, 1, prm, A);
-    A.med_max = ls_knobs(prm, in.n, rounds).cta_cap;
+    A.med_max = ls_knobs(prm, rounds).cta_cap;
+    const uint32_t sm = (uint32_t)std::max(1, ctx->sm_count);
+    A.few = 2 * sm;
+    A.few_alone = sm / 8;
     A.chars = in.chars;
     A.offs = in.offs;
     A.lens = in.lens;
@@ -1432,7 +1432,7 @@ sss_status impl_sort_segments_range(sss_ctx* ctx, Arena& ar, const StrIn& in, co
     const uint32_t n = in.n;
     if (n == 0 || q1 <= q0) return SSS_OK;
     const uint32_t nr = q1 - q0;
-    const LsKnobs kn = ls_knobs(prm, n, false);
+    const LsKnobs kn = ls_knobs(prm, false);
     SSS_TRY(set_ls_attributes(ctx));
     if (init.size() == 1 && init[0].start == q0 && init[0].size == nr && nr > (uint32_t)TINY_CAP &&
         nr <= kn.cta_cap && nr > kn.warp_cap)
@@ -1442,7 +1442,7 @@ sss_status impl_sort_segments_range(sss_ctx* ctx, Arena& ar, const StrIn& in, co
                                      {lcp}, init[0]});
     bool rounds = false;  // a segment that the CTA finisher cannot take
     for (const Seg& s : init) rounds = rounds || s.size > kn.cta_cap;
-    const LsArgs A = ls_args(ar, in, prm, rounds, perm, lcp, q0, q1);
+    const LsArgs A = ls_args(ctx, ar, in, prm, rounds, perm, lcp, q0, q1);
     SSS_TRY(sss_fits(ctx, ar));
     LsDev* S = static_cast<LsDev*>(ctx->d_ls);
 
@@ -1537,7 +1537,7 @@ __global__ void __launch_bounds__(BG_T) k_ls_groups(LsDev* __restrict__ S, const
 sss_status impl_groups_begin(sss_ctx* ctx, Arena ar, const StrIn& in, const sss_params& prm, uint32_t* perm,
                              uint32_t* lcp, const uint32_t* group_start, const uint32_t* d_groups,
                              const uint32_t** d_counts) {
-    LsArgs A = ls_args(ar, in, prm, false, perm, lcp, 0, in.n);
+    LsArgs A = ls_args(ctx, ar, in, prm, false, perm, lcp, 0, in.n);
     SSS_TRY(sss_fits(ctx, ar));
     A.keep = 1;
     SSS_TRY(set_ls_attributes(ctx));
@@ -1553,7 +1553,7 @@ sss_status impl_groups_begin(sss_ctx* ctx, Arena ar, const StrIn& in, const sss_
 
 sss_status impl_groups_sort(sss_ctx* ctx, Arena ar, const StrIn& in, const sss_params& prm, uint32_t* perm,
                             uint32_t* lcp, const uint32_t* counts) {
-    const LsArgs A = ls_args(ar, in, prm, false, perm, lcp, 0, in.n);  // as in the device state
+    const LsArgs A = ls_args(ctx, ar, in, prm, false, perm, lcp, 0, in.n);  // as in the device state
     uint32_t have[LC_COUNT];
     std::copy(counts, counts + LC_COUNT, have);
     return run_sort(ctx, A, prm, have);

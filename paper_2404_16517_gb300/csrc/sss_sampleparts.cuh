@@ -104,17 +104,19 @@ struct LsArgs {
     GPtr<Seg> list[LC_COUNT];  // LC_WARP: the last entry of the shared array, filled downwards
     uint32_t cap[LC_COUNT];
     uint32_t warp_max, med_max, direct_max, target, bucket_cap;
+    uint32_t direct_min, few, few_alone;  // k_lg_plan's rule for segments of direct_min + 1 .. direct_max strings
     uint32_t cap_tiles, cap_hist, cap_part, limit;
     uint32_t q0, q1;  // the positions being sorted
     uint32_t keep;    // the order given in perm is kept (else it starts as the identity)
 };
 
-// Device state of the local sort, one per context.
+// Device state of the local sort, one per context.  (A sector each for what a kernel
+// reads once and for the counters that others change meanwhile.)
 struct LsDev {
     LsArgs args;
-    LsPlan plan;
-    uint32_t cnt[8];   // segments per list; [6]: entries of redo, [7]: largest buckets, copied by the round's last kernel
-    uint32_t work[8];  // dynamic work counters: [LC_*] finishers, [5] buckets, [6] direct, [7] CTAs done
+    alignas(32) LsPlan plan;
+    alignas(32) uint32_t cnt[8];   // segments per list; [6]: entries of redo, [7]: largest buckets, copied by the round's last kernel
+    alignas(32) uint32_t work[8];  // dynamic work counters: [LC_*] finishers, [5] buckets, [6] direct, [7] CTAs done
     uint32_t rounds;
 };
 
@@ -159,38 +161,67 @@ __device__ __forceinline__ void block_scan_n(uint64_t (&v)[N], uint64_t (&tot)[N
 
 // Plan a round from the large list; resets its counter for the pushes of this
 // round and the round's work counters.  One CTA of 1024 threads.
+//
+// Segments above direct_max strings (8,192) are partitioned.  The middle ones above
+// direct_min (4,352, a bucket CTA's capacity) are sorted whole, by a CTA that has an
+// SM to itself, except few of them.  Measured with both ways forced, us partitioned /
+// whole, by the number of middle segments:
+//  * In a round that partitions others anyway they add little to its kernels, while
+//    even one sorted whole is a kernel's time after them.  6,000 strings of 12
+//    characters beside one of 20,000: 113 / 130 (1), 126 / 136 (38), 176 / 165 (152),
+//    242 / 218 (304), 369 / 310 (608); beside one of 3,000,000: 580 / 598 (76),
+//    686 / 668 (304).  But the range buckets that a round of one large segment leaves
+//    too large, up to 256 of them, are mostly middle ones, and slower whole at any
+//    number: 1.35M suffix views 329 / 351, 2.5M 471 / 515, 4.2M 694 / 760.  The line:
+//    two segments per SM.
+//  * In a round of their own it depends on the strings.  6,000 suffix views: 111 / 107
+//    (1), 122 / 115 (11), 128 / 118 (38), 177 / 147 (152); of uneven lengths, from one
+//    template: 161 / 182 (1), 182 / 192 (11), 203 / 208 (38), 316 / 296 (152).  The
+//    line: an eighth of a segment per SM, where the two kinds balance.
 __global__ void __launch_bounds__(1024) k_lg_plan(LsDev* __restrict__ S, unsigned* err) {
     __shared__ uint64_t sh[128];
-    __shared__ uint32_t s_n[4];  // segments and tiles: partitioned, then big
+    __shared__ uint32_t s_n[6];  // segments and tiles: above direct_max, middle, others above bucket_cap
     const LsArgs& A = S->args;
     const uint32_t tid = threadIdx.x;
-    const uint32_t direct_max = A.direct_max, bucket_cap = A.bucket_cap, target = A.target;
+    const uint32_t whole_max = A.direct_max, whole_min = A.direct_min, bucket_cap = A.bucket_cap, target = A.target;
+    const uint32_t few = A.few, few_alone = A.few_alone;
     const Seg* list = A.list[LC_LARGE];
+    LgSegInfo* info = A.info;
+    uint32_t *tile0 = A.tile0, *bk0 = A.bk0, *rowdone = A.rowdone;
+    const uint32_t cap_tiles = A.cap_tiles, cap_hist = A.cap_hist, cap_part = A.cap_part;
     uint32_t ns = S->cnt[LC_LARGE];
     if (ns > A.cap[LC_LARGE]) {
         if (tid == 0) atomicOr(err, ERRBIT_OVERFLOW);
         ns = 0;
     }
-    if (tid < 4) s_n[tid] = 0;
+    if (tid < 6) s_n[tid] = 0;
     __syncthreads();  // every thread has read the count
-    uint32_t n0[4] = {0, 0, 0, 0};
+    uint32_t n0[6] = {0, 0, 0, 0, 0, 0};
     for (uint32_t s = tid; s < ns; s += 1024) {
         const uint32_t size = list[s].size, tiles = (size + LG_TILE - 1) / LG_TILE;
-        if (size > direct_max) {
+        if (size > whole_max) {
             ++n0[0];
             n0[1] += tiles;
-        } else if (size > bucket_cap) {
+        } else if (size > whole_min) {
             ++n0[2];
             n0[3] += tiles;
+        } else if (size > bucket_cap) {
+            ++n0[4];
+            n0[5] += tiles;
         }
     }
+    if ((tid & ~31u) < ns) {  // (mostly one warp has segments)
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const uint32_t t = __reduce_add_sync(SSS_FULL, n0[k]);
-        if ((tid & 31) == 0 && t) atomicAdd(&s_n[k], t);
+        for (int k = 0; k < 6; ++k) {
+            const uint32_t t = __reduce_add_sync(SSS_FULL, n0[k]);
+            if ((tid & 31) == 0 && t) atomicAdd(&s_n[k], t);
+        }
     }
     __syncthreads();
-    const uint32_t npart = s_n[0], ptiles = s_n[1], nbig = s_n[2], btiles = s_n[3];
+    const bool part_mid = s_n[2] <= (s_n[0] > 0 ? few : few_alone);
+    const uint32_t direct_max = part_mid ? whole_min : whole_max;
+    const uint32_t npart = s_n[0] + (part_mid ? s_n[2] : 0u), ptiles = s_n[1] + (part_mid ? s_n[3] : 0u);
+    const uint32_t nbig = s_n[4] + (part_mid ? 0u : s_n[2]), btiles = s_n[5] + (part_mid ? 0u : s_n[3]);
     // (partitioned, big) segments, their tiles, small segments and their tiles, buckets and histogram words
     uint64_t carry[4] = {(uint64_t)npart << 32, (uint64_t)ptiles << 32,
                          (uint64_t)(npart + nbig) | ((uint64_t)(ptiles + btiles) << 32), 0};
@@ -217,10 +248,10 @@ __global__ void __launch_bounds__(1024) k_lg_plan(LsDev* __restrict__ S, unsigne
         for (int k = 0; k < 4; ++k) v[k] += carry[k];
         if (valid) {
             const uint32_t at = cls == 0 ? (uint32_t)v[0] : cls == 1 ? (uint32_t)(v[0] >> 32) : (uint32_t)v[2];
-            A.info[at] = LgSegInfo{sg, tiles, nb, (uint32_t)(v[3] >> 32), 0};
-            A.tile0[at] = cls == 0 ? (uint32_t)v[1] : cls == 1 ? (uint32_t)(v[1] >> 32) : (uint32_t)(v[2] >> 32);
-            A.bk0[at] = (uint32_t)v[3];
-            A.rowdone[at] = 0;
+            info[at] = LgSegInfo{sg, tiles, nb, (uint32_t)(v[3] >> 32), 0};
+            tile0[at] = cls == 0 ? (uint32_t)v[1] : cls == 1 ? (uint32_t)(v[1] >> 32) : (uint32_t)(v[2] >> 32);
+            bk0[at] = (uint32_t)v[3];
+            rowdone[at] = 0;
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) carry[k] += tot[k];
@@ -228,7 +259,7 @@ __global__ void __launch_bounds__(1024) k_lg_plan(LsDev* __restrict__ S, unsigne
     if (tid == 0) {
         const uint32_t nt = (uint32_t)(carry[2] >> 32), nh = (uint32_t)(carry[3] >> 32);
         LsPlan pl{ns, npart, nbig, nt, ptiles, (uint32_t)carry[3], {0, 0}};
-        if (nt > A.cap_tiles || nh > A.cap_hist || npart > A.cap_part) {
+        if (nt > cap_tiles || nh > cap_hist || npart > cap_part) {
             atomicOr(err, ERRBIT_OVERFLOW);
             pl = LsPlan{0, 0, 0, 0, 0, 0, {0, 0}};
         }
