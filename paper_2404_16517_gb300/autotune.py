@@ -8,7 +8,9 @@ split by sampled partition into range buckets of about bucket_target strings.
 They change speed, never results.  The tuner times candidate settings on a
 sample of the caller's own workload (CUDA events on the context stream, median
 of a few runs after a warm-up) and returns the fastest; results can be cached in
-a JSON file keyed by the GPU name and a coarse signature of the workload.
+a JSON file keyed by the GPU name and a coarse signature of the workload.  The
+library's own defaults are among the candidates of the default grid, so that tuning
+does not return a setting that was slower than them.
 """
 from __future__ import annotations
 
@@ -21,22 +23,28 @@ import torch
 
 from . import Context, context, instance_table, lib, params, sss_sort, _ptr
 
+# 0: the library's choice by the call's sizes (cta_cap: 2048 or 256; direct_cap: 8192,
+# or 4352 where few segments are larger than that)
+DEFAULTS = {"bucket_target": 0, "cta_cap": 0, "direct_cap": 0, "warp_cap": 0}
 DEFAULT_GRID = {
-    "cta_cap": [512, 1024, 2048],
-    "direct_cap": [2048, 4096, 8192],
+    "cta_cap": [0, 256, 512, 1024, 2048],
+    "direct_cap": [2048, 4352, 8192],
     "bucket_target": [1024, 2048, 4096],
     "warp_cap": [16, 32],
 }
 
 
 def candidates(grid: dict | None = None) -> list[dict]:
-    """Every valid combination of the grid (direct_cap >= cta_cap)."""
+    """Every valid combination of the grid (direct_cap >= cta_cap unless either is
+    left to the library); without a grid, the library's defaults and then those of
+    DEFAULT_GRID."""
+    out = [] if grid else [dict(DEFAULTS)]
     grid = grid or DEFAULT_GRID
     keys = sorted(grid)
-    out = []
     for vals in itertools.product(*(grid[k] for k in keys)):
         c = dict(zip(keys, vals))
-        if c.get("direct_cap", 8192) < c.get("cta_cap", 2048):
+        direct = c.get("direct_cap", 0)
+        if direct and direct < c.get("cta_cap", 0):
             continue
         out.append(c)
     return out
