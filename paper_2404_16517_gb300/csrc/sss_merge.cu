@@ -867,7 +867,8 @@ __global__ void k_d2_bounds(const uint32_t* __restrict__ run_perm, Strs S, uint3
                             const uint32_t* __restrict__ pso, const SubSpl* __restrict__ info,
                             const uint32_t* __restrict__ srank, const uint32_t* __restrict__ s2lcp, uint32_t step,
                             uint32_t* __restrict__ sb) {
-    uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    // (a warp each: 2^32 threads from 134M strings on with p = 256)
+    const uint32_t g = (uint32_t)(((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (g >= nss * p) return;
     const uint32_t m = g / p, i = g % p;
     const SubSpl F = info[m];
@@ -2006,7 +2007,7 @@ sss_status impl_merge(sss_ctx* ctx, char* ws, size_t ws_bytes, const StrIn& in, 
                            (const uint32_t*)b.s2lcp, (const uint32_t*)b.s2lens, b.subspl, b.sinfo));
         SSS_TRY(sss_launch(ctx, "d2_srank", k_d2_srank, dim3((S2 + 255) / 256), dim3(256), 0,
                            (const uint32_t*)b.s2perm, S2, b.s2rank));
-        SSS_TRY(sss_launch(ctx, "d2_bounds", k_d2_bounds, dim3((NSS * p * 32 + 127) / 128), dim3(128), 0, run_perm,
+        SSS_TRY(sss_launch(ctx, "d2_bounds", k_d2_bounds, dim3((NSS * p + 3) / 4), dim3(128), 0, run_perm,
                            S, p, NSS, (const uint32_t*)b.pstart, (const uint32_t*)b.psz, (const uint32_t*)b.pso,
                            (const SubSpl*)b.sinfo, (const uint32_t*)b.s2rank, (const uint32_t*)b.s2lcp, step, b.sb));
     }
