@@ -26,7 +26,11 @@
  *    are sticky in the context and returned by sss_sync().
  *  - Work memory is owned by the context: it is allocated with cudaMalloc on
  *    first use and grown when a larger problem arrives, or supplied by the caller
- *    with sss_set_workspace().
+ *    with sss_set_workspace().  Beside it a context holds a few KB of device memory,
+ *    and up to eight CUDA graphs for its sorts, one per size class of call (to 2^17,
+ *    2^18, 2^19 strings and more, by bucket_target): each is made by the first sort
+ *    of its class that needs rounds, which takes 0.03 to 0.2 ms longer for it and,
+ *    whoever owns the work memory, up to 2 MB of the driver's device memory.
  *  - A context is not thread-safe; use one context per host thread.  Its calls run
  *    one after the other, also when they are on different streams (sss_set_stream).
  *  - Limits: n < 2^32 - 1, 1 <= p <= 1024, string lengths < 2^31.
@@ -303,9 +307,10 @@ size_t sss_batch_workspace_bytes(uint32_t n_table, uint32_t m, const sss_params*
  * characters are never copied.  The suffixes truncated to 64 characters are
  * sorted as strings by stage A (p = 1); where that leaves equal truncations,
  * prefix doubling over ranks follows: the order on the first min(2h, target)
- * characters is the order of the pairs (rank_h(i), rank_h(i + o)), o <= h,
- * sorted as 10-byte strings by stage A, until every rank is distinct or the
- * target length (max_len, else the whole suffix) is reached.  A text with
+ * characters is the order of the pairs (rank_h(i), rank_h(i + o)), o <= h.  The
+ * groups of equal first ranks are refined in place, their second ranks sorted as
+ * 5-byte strings by stage A, until every rank is distinct or the target length
+ * (max_len, else the whole suffix) is reached.  A text with
  * short repeats is done after the first sort; a text of one repeated character
  * takes log2(n / 64) rounds.  The LCPs come from the rank levels.
  * text         : DEVICE array of n_text bytes, no 0x00 byte (checked with

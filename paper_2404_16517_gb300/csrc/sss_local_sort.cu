@@ -656,8 +656,8 @@ constexpr size_t finish_smem(int cap) { return (size_t)cap * (8 + 8 + 4 * 7); }
 // sort_emit's shared memory: keys, scratch, indices, sorted order, counters.
 // The scratch is one word per key (or the low words of a 128-bit merge sort); the
 // counters are 16 bits wide, two per key (the next power of two).  A CTA of 512
-// threads takes 4,352 strings: as many as two of them on an SM have memory for,
-// and a little over the 4,096 that templates of 64 in partitions of 2^18 give.
+// threads takes 4,352 strings: as many, in steps of 256, as two of them on an SM
+// have memory for.
 constexpr int emit_buckets(int cap) { return cap <= 2048 ? 4096 : 8192; }
 constexpr int emit_merge_items(int threads, int cap) { return cap / threads >= 8 ? 8 : 4; }
 constexpr size_t emit_smem(int, int cap) { return (size_t)cap * (8 + 8 + 4 + 2) + 2 * (size_t)emit_buckets(cap); }

@@ -98,3 +98,40 @@ def test_the_second_stream_waits_on_the_device():
     for s, (perm, lcp) in zip(sets, out):
         want = oracle.sort(s)
         assert np.array_equal(sss.u32(perm), want) and np.array_equal(sss.u32(lcp), oracle.lcp_array(s, want))
+
+
+# one CTA's sort, and a few lists by their classes: the calls that need no rounds
+@pytest.mark.parametrize("p", [1, 3])
+def test_calls_without_rounds_can_be_captured(p):
+    """On the capturing stream a call neither waits for the context's earlier calls
+    nor marks its end; the graph sorts what the buffers hold when it is launched."""
+    import paper_2404_16517_gb300 as sss
+    sets = [_set(1500, s) for s in (21, 22)]
+    cap = max(s.chars.shape[0] for s in sets)
+    dev = [sss.to_device(s) for s in sets]
+    chars = torch.zeros(cap, dtype=torch.uint8, device="cuda")
+    offs, lens = torch.empty_like(dev[0][1]), torch.empty_like(dev[0][2])
+    perm = torch.empty(1500, dtype=torch.int32, device="cuda")
+    lcp = torch.empty_like(perm)
+
+    def load(d):
+        chars[:d[0].numel()].copy_(d[0])
+        offs.copy_(d[1])
+        lens.copy_(d[2])
+
+    load(dev[0])
+    sss.sss_local_sort(chars, offs, lens, p, None, perm, lcp)  # work memory and kernels
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        sss.sss_local_sort(chars, offs, lens, p, None, perm, lcp)
+    for s, d in zip(sets, dev):
+        load(d)
+        graph.replay()
+        torch.cuda.synchronize()
+        sss.context().sync()
+        want, wl = oracle.local_sort(s, p)
+        assert np.array_equal(sss.u32(perm), want)
+        assert np.array_equal(sss.u32(lcp), wl)
+        sss.sss_sort(*d, 2)  # and calls outside the graph go on
+        sss.context().sync()
